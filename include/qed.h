@@ -285,10 +285,10 @@ qed_status qed_check(qed_species* const* sp, int n_species, void* stream);
 /* ------------------------------------------------------------------------------------------
  * Batches: many independent scenarios (for example a parameter scan of collisions, or the
  * requests of a serving loop), each with its own species, field and steps, advanced together.
- * Each batch step is five launches for all scenarios: a tile schedule that lays the live
+ * Each batch step is four launches for all scenarios: a tile schedule that lays the live
  * scenarios' 256-particle tiles end to end in one tile space, the step (a persistent grid that
- * strides through that space, so every block gets an equal share in one wave), and the three
- * merge kernels (per-scenario plan, event-mask prefixes and the ordered scatter, each striding
+ * strides through that space, so every block gets an equal share in one wave), and the two
+ * merge kernels (per-scenario plan and the ordered scatter, which strides
  * through all scenarios together); qed_batch_run replays them from a captured CUDA graph.  A
  * scenario gives the same particles alone or in any mix, and, with the default grid, the same
  * ledger bit for bit as qed_run (block p of the grid takes the same tiles of the scenario either

@@ -267,12 +267,13 @@ struct qed_species {
 
 namespace {
 template <typename R>
-void carve_species(Carver& cv, SpeciesDev<R>& s, size_t cap, size_t acap, size_t words, size_t ranges) {
+void carve_species(Carver& cv, SpeciesDev<R>& s, size_t cap, size_t acap) {
   cv.add(&s.x, cap); cv.add(&s.y, cap); cv.add(&s.z, cap);
   cv.add(&s.ux, cap); cv.add(&s.uy, cap); cv.add(&s.uz, cap);
   cv.add(&s.tau, cap); cv.add(&s.id, cap);
-  cv.add(&s.evmask, words); cv.add(&s.wprefix, words);
-  cv.add(&s.rangesum, ranges); cv.add(&s.rprefix, ranges);
+  cv.add(&s.evmask, event_words(cap));
+  cv.add(&s.fine, 2 * event_fines(cap)); cv.add(&s.coarse, 2 * event_coarses(cap));
+  cv.add(&s.cprefix, event_coarses(cap));
   cv.add(&s.ax, acap); cv.add(&s.ay, acap); cv.add(&s.az, acap);
   cv.add(&s.aux, acap); cv.add(&s.auy, acap); cv.add(&s.auz, acap);
   cv.add(&s.atau, acap); cv.add(&s.aparent, acap);
@@ -363,15 +364,10 @@ extern "C" qed_status qed_species_alloc(qed_kind kind, qed_precision precision, 
   sp->precision = precision;
   sp->cap = capacity;
   sp->acap = append_capacity;
-  const size_t words = capacity / 32 + 2;
-  const size_t ranges = (words >> kRangeShift) + 2;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   sp->ledger_parts = std::max(step_grid_size(QED_MIXED), step_grid_size(QED_FP64));
   Carver cv;
-  if (precision == QED_MIXED) carve_species(cv, sp->f, capacity, std::max<size_t>(append_capacity, 1), words, ranges);
-  else carve_species(cv, sp->d, capacity, std::max<size_t>(append_capacity, 1), words, ranges);
+  if (precision == QED_MIXED) carve_species(cv, sp->f, capacity, std::max<size_t>(append_capacity, 1));
+  else carve_species(cv, sp->d, capacity, std::max<size_t>(append_capacity, 1));
   cv.add(&sp->cnt, 1);
   cv.add(&sp->ledger_part, (size_t)sp->ledger_parts * kLedgerN);
   cv.add(&sp->ledger, kLedgerN);
@@ -805,9 +801,10 @@ StepArgs<R> make_args(const qed_tables* T, qed_species* const* sp, const qed_ste
 }
 
 template <typename R>
-qed_status do_step(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t step,
+qed_status do_step(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t step, bool want,
                    cudaStream_t s) {
-  const StepArgs<R> a = make_args<R>(T, sp, p, step);
+  StepArgs<R> a = make_args<R>(T, sp, p, step);
+  a.want = want ? 1 : 0;
   const int grid = std::min(step_grid_size(sizeof(R) == 4 ? QED_MIXED : QED_FP64), sp[0]->ledger_parts);
   const size_t smem = (size_t)(a.tab.n_eta + a.tab.n_chi) * sizeof(R);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -883,6 +880,7 @@ struct qed_batch {
   void* scal = nullptr;  // StepScalars<R>[S]
   int target_blocks = 0, graph_steps = 32, max_parts = 0, fuse_k = 0;
   cudaGraphExec_t graph = nullptr;
+  int graph_launches = 0;  // kernels in the captured graph
   int graph_for_steps = 0, graph_for_target = 0, graph_for_grid = 0, graph_for_fuse = 0;
   std::vector<char> slot_grid;  // slot's field is gathered from a grid
   int grid_fields = 0;
@@ -913,10 +911,11 @@ BatchCtl<R> batch_ctl(const qed_batch* b) {
   return c;
 }
 
-void launch_batch(const qed_batch* b, cudaStream_t s) {
+// One batch step; want: the last of a call (or of a captured graph), whose ledgers can be read.
+void launch_batch(const qed_batch* b, bool want, cudaStream_t s) {
   const TableHost& h = b->tables->host;
-  if (b->precision == QED_MIXED) launch_batch_step<float>(batch_ctl<float>(b), h.p.n_eta, h.p.n_chi, s);
-  else launch_batch_step<double>(batch_ctl<double>(b), h.p.n_eta, h.p.n_chi, s);
+  if (b->precision == QED_MIXED) launch_batch_step<float>(batch_ctl<float>(b), h.p.n_eta, h.p.n_chi, want, s);
+  else launch_batch_step<double>(batch_ctl<double>(b), h.p.n_eta, h.p.n_chi, want, s);
 }
 
 void set_slot_grid(qed_batch* b, int slot, bool grid) {
@@ -940,10 +939,12 @@ qed_status ensure_graph(qed_batch* b) {
   cudaGraph_t g = nullptr;
   const cudaStream_t s = b->own;
   QED_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  for (int k = 0; k < b->graph_steps; ++k) launch_batch(b, s);
+  const uint64_t l0 = launch_count_value();
+  for (int k = 0; k < b->graph_steps; ++k) launch_batch(b, k == b->graph_steps - 1, s);
+  b->graph_launches = (int)(launch_count_value() - l0);
   cudaError_t e = cudaStreamEndCapture(s, &g);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-  count_launch(-5 * b->graph_steps);  // captured, not executed: replays are counted instead
+  count_launch(-b->graph_launches);  // captured, not executed: replays are counted instead
   e = cudaGraphInstantiate(&b->graph, g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) { b->graph = nullptr; return cuda_fail(e, "cudaGraphInstantiate"); }
@@ -1045,12 +1046,12 @@ extern "C" qed_status qed_batch_run(qed_batch* b, uint64_t n_steps, void* stream
     QED_CUDA(cudaStreamWaitEvent(b->own, b->ev_in, 0));
     for (; done + b->graph_steps <= n_steps; done += b->graph_steps) {
       QED_CUDA(cudaGraphLaunch(b->graph, b->own));
-      count_launch(5 * b->graph_steps);
+      count_launch(b->graph_launches);
     }
     QED_CUDA(cudaEventRecord(b->ev_out, b->own));
     QED_CUDA(cudaStreamWaitEvent(s, b->ev_out, 0));
   }
-  for (; done < n_steps; ++done) launch_batch(b, s);
+  for (; done < n_steps; ++done) launch_batch(b, done + 1 == n_steps, s);
   QED_CUDA(cudaGetLastError());
   return QED_OK;
 }
@@ -1138,8 +1139,9 @@ extern "C" qed_status qed_run(const qed_tables* T, qed_species* const* sp, const
   if (st != QED_OK) return st;
   NvtxRange range("qed_run");
   for (uint64_t k = 0; k < n_steps; ++k) {
-    st = sp[0]->precision == QED_MIXED ? do_step<float>(T, sp, *p, p->step + k, s)
-                                       : do_step<double>(T, sp, *p, p->step + k, s);
+    const bool want = k + 1 == n_steps;
+    st = sp[0]->precision == QED_MIXED ? do_step<float>(T, sp, *p, p->step + k, want, s)
+                                       : do_step<double>(T, sp, *p, p->step + k, want, s);
     if (st != QED_OK) return st;
   }
   QED_CUDA(cudaGetLastError());
@@ -1163,7 +1165,7 @@ qed_status run_multi(const qed_tables* T, qed_species* const* sp, const qed_step
     if (per_step > 0 || left < 2) {
       const uint64_t m = per_step > 0 ? std::min(left, per_step) : left;
       for (uint64_t k = 0; k < m; ++k) {
-        qed_status st = do_step<R>(T, sp, p, step++, s);
+        qed_status st = do_step<R>(T, sp, p, step++, k + 1 == left, s);
         if (st != QED_OK) return st;
       }
       left -= m;
@@ -1182,12 +1184,12 @@ qed_status run_multi(const qed_tables* T, qed_species* const* sp, const qed_step
     QED_CUDA(cudaStreamSynchronize(s));
     if (k > (uint32_t)K) return fail(QED_ERR_NUMERIC, "qed_run_multistep: bad probe result");
     if (k > 0) {
-      a.multi = 1;
+      a.want = k == left ? 1 : 0;
       timed = timing_events(e0, e1, g_timing_multi);
       if (timed) cudaEventRecord(e0, s);
       const int grid = launch_fused<R>(a, (int)k, true, sp[0]->first_event, sp[0]->ledger_parts, s);
       if (timed) cudaEventRecord(e1, s);
-      launch_finalize<R>(a, grid, s);
+      if (a.want) launch_ledger<R>(a, grid, s);
       step += k;
       left -= k;
     }

@@ -156,6 +156,7 @@ struct StepScalars {
   R phi_ref_mod;   // the same reduced to [-pi, pi] (carrier)
   R omega, E0, inv_len, len;
   int kind;
+  uint32_t phase[3];  // event-count buffer of e-, e+, photons (DevCounters::phase; step kernels)
   // grid gather
   const R* grid;
   size_t gN;       // values per component

@@ -47,11 +47,26 @@ struct DevCounters {
   uint32_t n_app;    // particles appended to this species' append region during the step
   uint32_t n_dead;   // converted photons held
   uint32_t err;      // latched error bits (QED_ERR_* as 1u << code)
-  uint32_t pad[3];
+  // event counts (SpeciesDev::fine, coarse) are double-buffered: a step counts in buffer `phase`,
+  // which is all zero when the step starts; its finalisation clears the entries the step before
+  // used in the other one (ext, in fine groups) and then switches
+  uint32_t phase;
+  uint32_t ext[2];
 };
 
-constexpr int kRangeShift = 8;  // one range = 256 warp chunks = 8192 parents
-constexpr int kLedgerN = 18;
+// A parent's rank among its species' parents of children is summed from three levels: whole
+// coarse groups, whole fine groups in its coarse group, whole mask words in its fine group.
+constexpr int kFineShift = 5;    // 32 mask words (1024 parents) per fine group
+constexpr int kCoarseShift = 5;  // 32 fine groups (32768 parents) per coarse group
+#ifdef __CUDACC__
+#define QED_HD __host__ __device__
+#else
+#define QED_HD
+#endif
+QED_HD constexpr uint32_t event_words(size_t cap) { return (uint32_t)(((cap >> 5) + 1 + 31) & ~size_t(31)); }
+QED_HD constexpr uint32_t event_fines(size_t cap) { return ((event_words(cap) >> kFineShift) + 31u) & ~31u; }
+QED_HD constexpr uint32_t event_coarses(size_t cap) { return ((event_fines(cap) >> kCoarseShift) + 31u) & ~31u; }
+constexpr int kLedgerN = 15;
 
 // Species arrays in precision R plus the scratch used by one step.
 template <typename R>
@@ -61,11 +76,12 @@ struct SpeciesDev {
   uint32_t* id;
   uint32_t cap;
   DevCounters* cnt;
-  // as a parent: which lanes of each 32-particle chunk created children this step
-  uint32_t* evmask;   // [cap/32 + 1]
-  uint32_t* rangesum; // [ranges]  children per range of 256 chunks (integer atomics)
-  uint32_t* rprefix;  // [ranges]  exclusive prefix of rangesum
-  uint32_t* wprefix;  // [cap/32 + 1] exclusive prefix of popc(evmask)
+  // as a parent: which lanes of each 32-particle chunk created children this step, and their
+  // number per fine and coarse group (integer atomics; two buffers each, see DevCounters::phase)
+  uint32_t* evmask;   // [event_words(cap)]
+  uint32_t* fine;     // [2 * event_fines(cap)]
+  uint32_t* coarse;   // [2 * event_coarses(cap)]
+  uint32_t* cprefix;  // [event_coarses(cap)] exclusive prefix of coarse (batches)
   // as a destination: particles created for this species during the step
   R *ax, *ay, *az, *aux, *auy, *auz;
   double* atau;
@@ -82,9 +98,8 @@ struct FinalizePlan {
   uint32_t next_id_old[3];
   uint32_t m[3];            // particles merged into each destination
   uint32_t from_electrons;  // photon children whose parents are electrons (ranked first)
-  uint32_t ranges[3];       // ranges per parent species
-  uint32_t events[3];       // events of each parent species this step
-  uint32_t pad;
+  uint32_t phase[3];        // event-count buffer each parent species used
+  uint32_t ticket;          // finalisation blocks done (the last one sets the counters)
 };
 
 // Analytic field parameters (Sec. 3.2 stand-in for the PIC gather).
@@ -115,25 +130,23 @@ struct StepArgs {
   double* ledger_part;  // [gridDim.x * kLedgerN]
   double* ledger;       // [kLedgerN]
   FinalizePlan* plan;
-  unsigned long long* work;  // [5] cumulative e+- pushes, photon pushes, particles created, and the
-                             // e+- and photon pushes made by multi-step passes (part of [0], [1])
-  int multi;                 // this finalisation follows a multi-step commit
+  unsigned long long* work;  // [6] cumulative e+- pushes, photon pushes, particles created, the e+- and
+                             // photon pushes made by multi-step passes (part of [0], [1]), and the
+                             // per-step photon pushes in a field
+  int want;                  // somebody can read this step's ledger: keep its sums
 };
 
 // What one batch step does with a slot, written by the tile schedule at the start of the step:
 // the slot's 256-particle tiles occupy [tile_base, tile_base + T[0] + T[1] + T[2]) of the batch
-// step's tile space (species in order e-, e+, photons), its event-mask ranges
-// [range_base, range_base + Rg[0] + Rg[1] + Rg[2]) of the range space; n are the particles
-// held (the step's parents).
+// step's tile space (species in order e-, e+, photons); n are the particles held (the step's
+// parents).
 struct SlotPlan {
   uint32_t live;
   uint32_t tile_base;
   uint32_t T[3];
   uint32_t n[3];
-  uint32_t range_base;
-  uint32_t Rg[3];
 };
-constexpr int kBatchTotals = 4;  // [tiles, ranges, children (after the plan), spare]
+constexpr int kBatchTotals = 4;  // [tiles, spare]
 
 // Many independent scenarios ("slots") stepped together: per-slot arguments live in device
 // memory.  The per-step path puts the tiles of all live slots in one tile space that a
@@ -163,10 +176,15 @@ struct BatchCtl {
 template <typename R>
 void launch_step(const StepArgs<R>& a, int grid, int block, size_t smem, cudaStream_t s);
 template <typename R>
-void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, cudaStream_t s);
+void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, bool want, cudaStream_t s);
 size_t step_scalars_bytes(int precision);
+// Merges the step's children into place and sets the counters; `step_grid` ledger partials are
+// reduced when a.want is set.
 template <typename R>
 void launch_finalize(const StepArgs<R>& a, int step_grid, cudaStream_t s);
+// Reduces `parts` ledger partials (after a multi-step commit).
+template <typename R>
+void launch_ledger(const StepArgs<R>& a, int parts, cudaStream_t s);
 // Multi-step pass over K <= fuse_max_steps() steps: the probe (commit = false) sets
 // *first_event to the first step with an event (K if none); the commit advances K event-free
 // steps and writes the ledger partials of the last.  Returns the grid (ledger partials) used.

@@ -1,17 +1,15 @@
 // qed_kernels.cu -- CUDA kernels of the QED Monte-Carlo step (Sec. 3) for sm_103a.
 //
 // One step = one launch of step_kernel over all three species (warp-uniform chunks of 32
-// consecutive particles, grid-stride over chunks) followed by three small finalisation
-// kernels that merge the particles created during the step in (parent species, parent
-// index) order:
-//   step_kernel     push, eta/chi, rates, tau; events collected per warp and taken 32 at a time
-//                   (ballot + one atomic per warp append), per-chunk event masks, per-block FP64
-//                   ledger partials
-//   plan_kernel     one block: scans the per-range child counts, checks capacities, writes the
-//                   merge plan and reduces the ledger partials in a fixed order
-//   prefix_kernel   exclusive prefix of the event-mask popcounts per parent species
-//   scatter_kernel  ranks every new particle by its parent's position (a counting sort on the
-//                   dense parent index), moves it into place and assigns consecutive ids
+// consecutive particles, grid-stride over chunks) followed by one finalisation kernel that merges
+// the particles created during the step in (parent species, parent index) order:
+//   step_kernel      push, eta/chi, rates, tau; events collected per warp and taken 32 at a time
+//                    (ballot + one atomic per warp append), per-chunk event masks and their counts
+//                    per group of chunks; per-block FP64 ledger partials where the step's ledger
+//                    can be read
+//   finalize_kernel  checks capacities, ranks every new particle by its parent's position (a
+//                    counting sort on the dense parent index), moves it into place and assigns
+//                    consecutive ids; the last block sets the counters
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -36,10 +34,14 @@ constexpr int kWarps = kBlock / 32;    // compute warps
 constexpr int kStepThreads = kBlock + 32;  // plus one producer warp that issues the tile copies
 
 enum LedgerSlot {
-  kN0 = 0, kN1, kN2, kE0, kE1, kE2, kEmitN, kEmitE, kDrop, kEmitDef, kPairN, kPairE, kPairDef, kOorEta, kOorChi,
-  kPushedLep, kPushedPh,  // alive particles pushed this step
-  kTauPh                  // photons pushed in a field (their optical depth changed and is stored)
+  kN0 = 0, kN1, kN2, kE0, kE1, kE2, kEmitN, kEmitE, kDrop, kEmitDef, kPairN, kPairE, kPairDef, kOorEta, kOorChi
 };
+
+// Programmatic dependent launch: a kernel's blocks may start, and run what does not depend on
+// earlier kernels, while the kernel before it drains; pdl_wait returns once that one has
+// completed and its writes are visible.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Compensated (Kahan) accumulation in the working precision.
 template <typename R>
@@ -63,7 +65,7 @@ struct Acc {
   KSum<R> emit_e, emit_def, pair_e, pair_def;
   uint32_t n[3] = {0, 0, 0};
   uint32_t oor_eta = 0, oor_chi = 0;
-  uint32_t pushed_lep = 0, pushed_ph = 0, tau_ph = 0;
+  uint32_t pushed_ph = 0, tau_ph = 0;  // photons pushed; those in a field (optical depth stored)
   uint32_t emit_n = 0, drop = 0, pair_n = 0;
 };
 
@@ -196,6 +198,14 @@ __device__ __forceinline__ void enqueue_event(EventQueue<R>& q, unsigned evm, bo
   q.count += (uint32_t)__popc(evm);
 }
 
+// Adds c (mod 2^32) to the event counts, buffer ph, of the groups that hold mask word `chunk`.
+template <typename R>
+__device__ __forceinline__ void count_events(const SpeciesDev<R>& sp, uint32_t ph, uint32_t chunk, uint32_t c) {
+  const uint32_t f = chunk >> kFineShift;
+  atomicAdd(&sp.fine[ph * event_fines(sp.cap) + f], c);
+  atomicAdd(&sp.coarse[ph * event_coarses(sp.cap) + (f >> kCoarseShift)], c);
+}
+
 // One particle of a 32-particle chunk (the whole warp calls this together).  The state comes
 // from the shared-memory tile; results are stored straight to global memory.  A particle whose
 // optical depth ran out goes to the warp's event ring; its momentum and optical depth are
@@ -217,14 +227,11 @@ __device__ __forceinline__ void lepton_chunk(const StepArgs<R>& a, const StepSca
   int oor;
   const R eta = lepton_advance<R, G, FC>(S, a.tab, lnh, kind == QED_ELECTRON ? (R)-1 : (R)1, a.dt_r, a.win_v_r, x, y,
                                          z, u, tau, gam, u2, oor);
-  if (active && oor > 0) acc.oor_eta++;
-  if (active) acc.pushed_lep++;
-
   const bool ev = active && a.emit && tau.used_up();
   const unsigned evm = __ballot_sync(kFull, ev);
   if (evm) {
     enqueue_event<R>(q, evm, ev, lane, i, x, y, z, u[0], u[1], u[2], eta);
-    if (lane == 0) atomicAdd(&sp.rangesum[chunk >> kRangeShift], (uint32_t)__popc(evm));
+    if (lane == 0) count_events(sp, S.phase[kind], chunk, (uint32_t)__popc(evm));
   }
   if (lane == 0) sp.evmask[chunk] = evm;
   if (active) {
@@ -232,8 +239,11 @@ __device__ __forceinline__ void lepton_chunk(const StepArgs<R>& a, const StepSca
     if (!ev) {
       sp.ux[i] = u[0]; sp.uy[i] = u[1]; sp.uz[i] = u[2];
       tau.store(sp.tau + i);
-      acc.e[kind].add(gam);
-      acc.n[kind]++;
+    }
+    // the ledger's sums only where somebody can read them (the last step of a run)
+    if (a.want) {
+      if (oor > 0) acc.oor_eta++;
+      if (!ev) { acc.e[kind].add(gam); acc.n[kind]++; }
     }
   }
 }
@@ -245,7 +255,8 @@ __device__ __forceinline__ void lepton_chunk(const StepArgs<R>& a, const StepSca
 // call sites cost the loop more (on GB300, 3 blocks of 288 threads per SM) than the inlined
 // code's registers do.
 template <typename R, int KIND>
-__device__ __forceinline__ void lepton_events(const StepArgs<R>& a, EventRing<R>* ring, uint32_t head, uint32_t take) {
+__device__ __forceinline__ void lepton_events(const StepArgs<R>& a, uint32_t phase, EventRing<R>* ring, uint32_t head,
+                                              uint32_t take) {
   const SpeciesDev<R>& sp = a.sp[KIND];
   const SpeciesDev<R>& dst = a.sp[2];  // photon children are appended to the photon species
   const int lane = threadIdx.x & 31;
@@ -293,13 +304,13 @@ __device__ __forceinline__ void lepton_events(const StepArgs<R>& a, EventRing<R>
     } else {
       // no photon: the event is not a child after all
       atomicAnd(&sp.evmask[i >> 5], ~(1u << (i & 31u)));
-      atomicSub(&sp.rangesum[(i >> 5) >> kRangeShift], 1u);
+      count_events(sp, phase, i >> 5, 0xffffffffu);
     }
     tau = Tau<R>::fresh(-Num<R>::log_(U[1].u));
   }
   const unsigned childm = __ballot_sync(kFull, child);
   const uint32_t nc = (uint32_t)__popc(childm);
-  {
+  if (a.want) {
     const KSum<R> se = warp_ksum<R>(emitted), sd = warp_ksum<R>(def), sg = warp_ksum<R>(ev ? gam : (R)0);
     if (lane == 0) {
       EventSums<R>& es = ring->sums;
@@ -372,7 +383,6 @@ __device__ __forceinline__ void photon_chunk(const StepArgs<R>& a, const StepSca
   R eps, ie;
   int oor;
   const R chi = photon_advance<R, G, FC>(S, a.tab, lnT, a.dt_r, a.win_v_r, x, y, z, k, tau, eps, ie, oor);
-  if (alive && oor > 0) acc.oor_chi++;
   if (alive) acc.pushed_ph++;
   // a photon outside any field keeps its optical depth: only its position is stored
   const bool tau_moves = alive && chi > (R)0;
@@ -385,17 +395,17 @@ __device__ __forceinline__ void photon_chunk(const StepArgs<R>& a, const StepSca
     enqueue_event<R>(q, evm, ev, lane, i, x, y, z, k[0], k[1], k[2], chi);
     if (lane == 0) {
       const uint32_t c = (uint32_t)__popc(evm);
-      atomicAdd(&sp.rangesum[chunk >> kRangeShift], c);
+      count_events(sp, S.phase[2], chunk, c);
       atomicAdd(&sp.cnt->n_dead, c);
     }
   }
   if (lane == 0) sp.evmask[chunk] = evm;
   if (alive) {
     sp.x[i] = x; sp.y[i] = y; sp.z[i] = z;  // k is unchanged between events
-    if (!ev) {
-      if (tau_moves) tau.store(sp.tau + i);
-      acc.e[2].add(eps);
-      acc.n[2]++;
+    if (!ev && tau_moves) tau.store(sp.tau + i);
+    if (a.want) {
+      if (oor > 0) acc.oor_chi++;
+      if (!ev) { acc.e[2].add(eps); acc.n[2]++; }
     }
   }
 }
@@ -448,7 +458,7 @@ __device__ __forceinline__ void photon_events(const StepArgs<R>& a, EventRing<R>
     tp = Tau<R>::fresh(-Num<R>::log_(U[2].u));
   }
   const unsigned evm = __ballot_sync(kFull, ev);
-  {
+  if (a.want) {
     const KSum<R> se = warp_ksum<R>(converted), sd = warp_ksum<R>(def);
     const KSum<R> s0 = warp_ksum<R>(gm), s1 = warp_ksum<R>(gp);
     if (lane == 0) {
@@ -587,13 +597,12 @@ __device__ __forceinline__ void compute_warps_sync() { asm volatile("bar.sync 1,
 // W warps take part: the whole block (CW = false, every thread calls this), or the compute warps
 // only (CW = true, synchronised by their named barrier; the producer warp holds no sums, and its
 // zeros would change nothing).
-constexpr int kCounts = 11;
+constexpr int kCounts = 8;
 template <typename R, int W, bool CW = false>
 __device__ __forceinline__ void write_ledger_partial(const Acc<R>& acc, double* ledger_part, uint32_t blk) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   KSum<R> f[7] = {acc.e[0], acc.e[1], acc.e[2], acc.emit_e, acc.emit_def, acc.pair_e, acc.pair_def};
-  uint32_t c[kCounts] = {acc.n[0], acc.n[1], acc.n[2], acc.emit_n, acc.drop, acc.pair_n, acc.oor_eta, acc.oor_chi,
-                         acc.pushed_lep, acc.pushed_ph, acc.tau_ph};
+  uint32_t c[kCounts] = {acc.n[0], acc.n[1], acc.n[2], acc.emit_n, acc.drop, acc.pair_n, acc.oor_eta, acc.oor_chi};
 #pragma unroll
   for (int q = 0; q < 7; ++q) {
     KSum<R> t = f[q];
@@ -625,7 +634,6 @@ __device__ __forceinline__ void write_ledger_partial(const Acc<R>& acc, double* 
       case kEmitN: cs = 3; break;    case kEmitE: fs = 3; break;    case kDrop: cs = 4; break;
       case kEmitDef: fs = 4; break;  case kPairN: cs = 5; break;    case kPairE: fs = 5; break;
       case kPairDef: fs = 6; break;  case kOorEta: cs = 6; break;   case kOorChi: cs = 7; break;
-      case kPushedLep: cs = 8; break; case kPushedPh: cs = 9; break; case kTauPh: cs = 10; break;
       default: break;
     }
     double t = 0.0;
@@ -641,6 +649,21 @@ __device__ __forceinline__ void write_ledger_partial(const Acc<R>& acc, double* 
     ledger_part[(size_t)blk * kLedgerN + k] = t;
   }
   if (CW) compute_warps_sync();  // s_fr and s_cr are reused by the next slot's partial
+}
+
+// The photon push counters of a block: summed over its warps in shared memory, then added to the
+// scenario's work counters (the e+- pushes follow from the particle counts).
+template <typename R>
+__device__ __forceinline__ void add_work(const Acc<R>& acc, uint32_t* s_work, int lane) {
+  const uint32_t p = __reduce_add_sync(kFull, acc.pushed_ph), t = __reduce_add_sync(kFull, acc.tau_ph);
+  if (lane == 0 && p) {
+    atomicAdd(&s_work[0], p);
+    atomicAdd(&s_work[1], t);
+  }
+}
+__device__ __forceinline__ void flush_work(uint32_t* s_work, unsigned long long* work) {
+  if (s_work[0]) atomicAdd(&work[1], (unsigned long long)s_work[0]);
+  if (s_work[1]) atomicAdd(&work[5], (unsigned long long)s_work[1]);
 }
 
 // The block's tiles of species SP, global tiles [t_lo, t_hi), with the block's tile count k
@@ -690,8 +713,8 @@ __device__ __forceinline__ bool species_tiles(const StepArgs<R>& a, const StepSc
     }
     while (q.count >= 32u || (!more && q.count > 0u)) {
       const uint32_t take = min(q.count, 32u);
-      if (SP == 0) lepton_events<R, QED_ELECTRON>(a, q.r, q.head, take);
-      else if (SP == 1) lepton_events<R, QED_POSITRON>(a, q.r, q.head, take);
+      if (SP == 0) lepton_events<R, QED_ELECTRON>(a, S.phase[0], q.r, q.head, take);
+      else if (SP == 1) lepton_events<R, QED_POSITRON>(a, S.phase[1], q.r, q.head, take);
       else photon_events<R>(a, q.r, q.head, take);
       q.head = (q.head + take) & (uint32_t)(kRing - 1);
       q.count -= take;
@@ -730,26 +753,32 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
   __shared__ StepScalars<R> S;
   __shared__ int s_abort;
 
-  const uint32_t n0 = a.sp[0].cnt->n, n1 = a.sp[1].cnt->n, n2 = a.sp[2].cnt->n;
-  const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 + kTile - 1) / kTile;
-  const uint32_t ttot = T0 + T1 + T2;
+  __shared__ uint32_t s_work[2];
+
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) {
+  // what does not depend on the step before: barriers, rate tables (fixed after their upload) and
+  // the field scalars of this step
+  if (threadIdx.x == kBlock) {
     for (int st = 0; st < kStages; ++st) {
       mbar_init(&full[st], 1);
       mbar_init(&empty[st], kWarps);
     }
     mbar_fence_init();
     s_abort = 0;
+    s_work[0] = s_work[1] = 0;
   }
-  __syncthreads();
-  if (threadIdx.x == kBlock)
-    for (uint32_t k = 0; k < (uint32_t)kStages; ++k) issue_tile(a, buf, full, k, n0, n1, n2, blk, nblk);
-  // stage the rate tables and the per-step field scalars while the first tiles load
   for (int k = threadIdx.x; k < a.tab.n_eta; k += blockDim.x) s_lnh[k] = a.tab.ln_h[k];
   for (int k = threadIdx.x; k < a.tab.n_chi; k += blockDim.x) s_lnT[k] = a.tab.ln_T[k];
   if (threadIdx.x == 0) make_scalars<R>(a.field, a.t0 + (double)a.step * a.dt, a.win_x0, a.win_v, S);
+  pdl_wait();
+  const uint32_t n0 = a.sp[0].cnt->n, n1 = a.sp[1].cnt->n, n2 = a.sp[2].cnt->n;
+  const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 + kTile - 1) / kTile;
+  const uint32_t ttot = T0 + T1 + T2;
+  if (threadIdx.x < 3) S.phase[threadIdx.x] = (threadIdx.x == 0 ? a.sp[0] : (threadIdx.x == 1 ? a.sp[1] : a.sp[2])).cnt->phase;
+  if (threadIdx.x == kBlock)
+    for (uint32_t k = 0; k < (uint32_t)kStages; ++k) issue_tile(a, buf, full, k, n0, n1, n2, blk, nblk);
   __syncthreads();
+  pdl_launch();
 
   Acc<R> acc;
   if (warp == kWarps) {
@@ -793,17 +822,18 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
     // a wait that gave up leaves the step unfinished (QED_ERR_TIMEOUT): events still in the
     // ring are not taken
     __syncwarp();
-    if (lane == 0) {
+    if (a.want && lane == 0) {
       const EventSums<R>& es = q.r->sums;
       for (int c = 0; c < 3; ++c) { acc.e[c].merge(es.e[c]); acc.n[c] += es.n[c]; }
       acc.emit_e = es.emit_e; acc.emit_def = es.emit_def;
       acc.pair_e = es.pair_e; acc.pair_def = es.pair_def;
       acc.emit_n = es.emit_n; acc.drop = es.drop; acc.pair_n = es.pair_n;
     }
+    add_work(acc, s_work, lane);
   }
   __syncthreads();
-
-  write_ledger_partial<R, kWarps + 1>(acc, a.ledger_part, blk);
+  if (threadIdx.x == 0) flush_work(s_work, a.work);
+  if (a.want) write_ledger_partial<R, kWarps + 1>(acc, a.ledger_part, blk);
 }
 
 template <typename R, bool G>
@@ -961,7 +991,6 @@ __device__ __forceinline__ void fused_body(const StepArgs<R>& a, int K, uint32_t
         tau.store(cc.tau + cc.i);
         acc.e[pos ? 1 : 0].add(gam);
         acc.n[pos ? 1 : 0]++;
-        acc.pushed_lep += (uint32_t)K;
         if (oor > 0) acc.oor_eta++;
       }
     } else if (!tau.dead()) {  // converted photons stay as holes until compaction
@@ -998,7 +1027,7 @@ __device__ __forceinline__ void fused_body(const StepArgs<R>& a, int K, uint32_t
         tau.store(cc.tau + cc.i);
         acc.e[2].add(eps);
         acc.n[2]++;
-        acc.pushed_ph += (uint32_t)K;
+        acc.pushed_ph++;
         if (oor > 0) acc.oor_chi++;
       }
     }
@@ -1007,8 +1036,22 @@ __device__ __forceinline__ void fused_body(const StepArgs<R>& a, int K, uint32_t
   }
   if (COMMIT) {
     if (bad) atomicOr(&a.sp[0].cnt->err, 1u << QED_ERR_NUMERIC);
+    __shared__ uint32_t s_pushed;
+    if (threadIdx.x == 0) s_pushed = 0;
     __syncthreads();
-    write_ledger_partial<R, kFuseThreads / 32>(acc, a.ledger_part, blk);
+    const uint32_t pushed = __reduce_add_sync(kFull, acc.pushed_ph);
+    if ((threadIdx.x & 31) == 0 && pushed) atomicAdd(&s_pushed, pushed);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const unsigned long long p = (unsigned long long)s_pushed * (unsigned long long)K;
+      if (p) { atomicAdd(&a.work[1], p); atomicAdd(&a.work[4], p); }
+      if (blk == 0) {
+        const unsigned long long l = (unsigned long long)nl * (unsigned long long)K;
+        atomicAdd(&a.work[0], l);
+        atomicAdd(&a.work[3], l);
+      }
+    }
+    if (a.want) write_ledger_partial<R, kFuseThreads / 32>(acc, a.ledger_part, blk);
   }
 }
 
@@ -1075,179 +1118,215 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
   return warp_base + inc - v;
 }
 
-template <typename R>
-__device__ __forceinline__ void plan_body(const StepArgs<R>& a, int nparts) {
-  __shared__ uint32_t s_tot[3];
-  constexpr int kPer = 8;  // range sums a thread keeps in registers (more go through memory twice)
-  for (int s = 0; s < 3; ++s) {
-    const SpeciesDev<R>& sp = a.sp[s];
-    const uint32_t words = (sp.cnt->n + 31u) >> 5;
-    const uint32_t ranges = (words + (1u << kRangeShift) - 1u) >> kRangeShift;
-    // each thread scans a contiguous segment of ranges; the loads of a segment are issued
-    // together and kept for the write-back
-    const uint32_t per = (ranges + blockDim.x - 1) / blockDim.x;
-    const uint32_t r0 = threadIdx.x * per, r1 = min(ranges, r0 + per);
-    uint32_t v[kPer];
-    uint32_t local = 0;
+// Sum of the entries [lo, hi) of a group-aligned array v (lo a multiple of 32 entries, hi - lo <= 32;
+// storage is padded to whole groups), or of their popcounts: eight independent 16-byte loads.
+template <bool POP>
+__device__ __forceinline__ uint32_t group_sum(const uint32_t* v, uint32_t lo, uint32_t hi) {
+  const uint4* p = reinterpret_cast<const uint4*>(v + lo);
+  uint32_t s = 0;
+  const uint32_t m = hi - lo;
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      v[q] = (q < (int)per && r0 + q < r1) ? sp.rangesum[r0 + q] : 0u;
-      local += v[q];
-    }
-    for (uint32_t r = r0 + kPer; r < r1; ++r) local += sp.rangesum[r];
-    uint32_t total;
-    uint32_t run = block_exclusive_scan(local, &total);
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      if (q < (int)per && r0 + q < r1) {
-        sp.rprefix[r0 + q] = run;
-        run += v[q];
-        sp.rangesum[r0 + q] = 0u;  // ready for the next step
-      }
-    }
-    for (uint32_t r = r0 + kPer; r < r1; ++r) {
-      const uint32_t c = sp.rangesum[r];
-      sp.rprefix[r] = run;
-      run += c;
-      sp.rangesum[r] = 0u;
-    }
-    if (threadIdx.x == 0) {
-      s_tot[s] = total;
-      a.plan->ranges[s] = ranges;
-      a.plan->events[s] = total;
+  for (uint32_t q = 0; q < 8; ++q) {
+    if (4 * q < m) {
+      const uint4 t = p[q];
+      s += POP ? (uint32_t)__popc(t.x) : t.x;
+      if (4 * q + 1 < m) s += POP ? (uint32_t)__popc(t.y) : t.y;
+      if (4 * q + 2 < m) s += POP ? (uint32_t)__popc(t.z) : t.z;
+      if (4 * q + 3 < m) s += POP ? (uint32_t)__popc(t.w) : t.w;
     }
   }
-  __syncthreads();
-  // destinations e-, e+, photons checked by threads 0, 1, 2 at once
-  if (threadIdx.x < 3) {
-    const int d = threadIdx.x;
-    FinalizePlan& P = *a.plan;
-    const uint32_t pairs = a.pairs ? s_tot[2] : 0u;
-    const uint32_t photons = a.emit ? s_tot[0] + s_tot[1] : 0u;
-    const SpeciesDev<R>& dst = (d == 2 && a.drain) ? a.sp[3] : (d == 0 ? a.sp[0] : (d == 1 ? a.sp[1] : a.sp[2]));
-    const SpeciesDev<R>& app = d == 0 ? a.sp[0] : (d == 1 ? a.sp[1] : a.sp[2]);  // append region owner
-    const uint32_t n_old = dst.cnt->n, next_old = dst.cnt->next_id, n_app = app.cnt->n_app;
-    P.n_old[d] = n_old;
-    P.next_id_old[d] = next_old;
-    uint32_t m = d == 2 ? photons : pairs;
-    if (n_app != m || m > app.acap) {  // an append overflowed: drop the step's children
-      atomicOr(&dst.cnt->err, 1u << QED_ERR_CAPACITY);
-      m = 0;
-    }
-    if ((uint64_t)n_old + m > dst.cap) {
-      atomicOr(&dst.cnt->err, 1u << QED_ERR_CAPACITY);
+  return s;
+}
+
+// Parents of children before parent p inside its coarse group.
+template <typename R>
+__device__ __forceinline__ uint32_t rank_in_coarse(const SpeciesDev<R>& sp, uint32_t phase, uint32_t p) {
+  const uint32_t w = p >> 5, f = w >> kFineShift;
+  const uint32_t f0 = f & ~((1u << kCoarseShift) - 1u), w0 = w & ~((1u << kFineShift) - 1u);
+  return group_sum<false>(sp.fine + phase * event_fines(sp.cap), f0, f) + group_sum<true>(sp.evmask, w0, w) +
+         (uint32_t)__popc(sp.evmask[w] & ((1u << (p & 31u)) - 1u));
+}
+
+// What the step leaves to merge, from the counters and the parents' totals (the same on every
+// thread that computes it; the error bits are set by the one with `report`).
+template <typename R>
+__device__ __forceinline__ FinalizePlan make_plan(const StepArgs<R>& a, uint32_t from_electrons, bool report) {
+  FinalizePlan P;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const SpeciesDev<R>& app = a.sp[d];  // append region owner
+    const SpeciesDev<R>& dst = (d == 2 && a.drain) ? a.sp[3] : a.sp[d];
+    P.n_old[d] = dst.cnt->n;
+    P.next_id_old[d] = dst.cnt->next_id;
+    P.phase[d] = app.cnt->phase;
+    uint32_t m = app.cnt->n_app;
+    // children beyond the append region or the destination's room: drop the step's children
+    if (m > app.acap || (uint64_t)P.n_old[d] + m > dst.cap) {
+      if (report) atomicOr(&dst.cnt->err, 1u << QED_ERR_CAPACITY);
       m = 0;
     }
     P.m[d] = m;
-    if (d == 0) P.from_electrons = s_tot[0];
   }
-  // ledger: fixed-order reduction of the per-block partials, one warp per ledger field (lane l
-  // sums partials l, l+32, ... in order, then a fixed shuffle tree): deterministic for a fixed grid
+  P.from_electrons = from_electrons;
+  P.ticket = 0;
+  return P;
+}
+
+// Child c (in destination order e-, e+, photons) of the step planned in P: its rank among the
+// destination's new particles is its parent's rank (a counting sort on the dense parent index),
+// which fixes its slot and its id.  coarse_before(s, c): children of species s's parents in the
+// coarse groups before c.
+template <typename R, typename F>
+__device__ __forceinline__ void place_child(const StepArgs<R>& a, const FinalizePlan& P, uint32_t c, F coarse_before) {
+  const uint32_t m0 = P.m[0], m1 = P.m[1];
+  const int d = c < m0 ? 0 : (c < m0 + m1 ? 1 : 2);
+  const uint32_t j = c - (d == 0 ? 0u : (d == 1 ? m0 : m0 + m1));
+  // constant indices only (no dynamic indexing of the kernel parameters)
+  const SpeciesDev<R>& app = d == 0 ? a.sp[0] : (d == 1 ? a.sp[1] : a.sp[2]);
+  const SpeciesDev<R>& dst = (d == 2 && a.drain) ? a.sp[3] : app;
+  const uint32_t par = app.aparent[j];
+  const R x = app.ax[j], y = app.ay[j], z = app.az[j], ux = app.aux[j], uy = app.auy[j], uz = app.auz[j];
+  const double tau = app.atau[j];
+  const int ps = d < 2 ? 2 : (int)(par >> 31);
+  const uint32_t p = d < 2 ? par : par & 0x7fffffffu;
+  const SpeciesDev<R>& psp = ps == 0 ? a.sp[0] : (ps == 1 ? a.sp[1] : a.sp[2]);
+  const uint32_t ph = ps == 0 ? P.phase[0] : (ps == 1 ? P.phase[1] : P.phase[2]);
+  const uint32_t rank = coarse_before(ps, p >> (5 + kFineShift + kCoarseShift)) + rank_in_coarse(psp, ph, p) +
+                        (ps == 1 ? P.from_electrons : 0u);
+  const uint32_t m = d == 0 ? m0 : (d == 1 ? m1 : P.m[2]);
+  if (rank >= m) { atomicOr(&dst.cnt->err, 1u << QED_ERR_NUMERIC); return; }
+  const uint32_t o = (d == 0 ? P.n_old[0] : (d == 1 ? P.n_old[1] : P.n_old[2])) + rank;
+  dst.x[o] = x; dst.y[o] = y; dst.z[o] = z;
+  dst.ux[o] = ux; dst.uy[o] = uy; dst.uz[o] = uz;
+  dst.tau[o] = tau;
+  dst.id[o] = (d == 0 ? P.next_id_old[0] : (d == 1 ? P.next_id_old[1] : P.next_id_old[2])) + rank;
+  if (dst.w) dst.w[o] = app.aw ? app.aw[j] : (R)1;
+}
+
+// Clears, share `i` of `n`, the event counts that the step before left in the buffer this step
+// did not use.
+template <typename R>
+__device__ __forceinline__ void clear_other_counts(const StepArgs<R>& a, const FinalizePlan& P, uint32_t i, uint32_t n) {
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    const SpeciesDev<R>& sp = a.sp[s];
+    const uint32_t o = P.phase[s] ^ 1u, ext = sp.cnt->ext[o];
+    for (uint32_t k = i; k < ext; k += n) sp.fine[o * event_fines(sp.cap) + k] = 0u;
+    for (uint32_t k = i; k < (ext + 31u) >> kCoarseShift; k += n) sp.coarse[o * event_coarses(sp.cap) + k] = 0u;
+  }
+}
+
+__device__ __forceinline__ uint32_t fines_of(uint32_t n) { return (((n + 31u) >> 5) + 31u) >> kFineShift; }
+__device__ __forceinline__ uint32_t coarses_of(uint32_t n) { return (fines_of(n) + 31u) >> kCoarseShift; }
+
+// The counters after the merge and the scenario's work counters (one thread).  n: the step's parents.
+template <typename R>
+__device__ __forceinline__ void finish_counters(const StepArgs<R>& a, const FinalizePlan& P, const uint32_t n[3]) {
+  const uint32_t emitted = a.sp[2].cnt->n_app, pairs = a.sp[0].cnt->n_app;
+  atomicAdd(&a.work[0], (unsigned long long)n[0] + n[1]);
+  if (emitted + pairs) atomicAdd(&a.work[2], (unsigned long long)emitted + 2ull * pairs);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const SpeciesDev<R>& sp = a.sp[d];
+    sp.cnt->ext[P.phase[d] ^ 1u] = 0u;
+    sp.cnt->ext[P.phase[d]] = fines_of(n[d]);
+    sp.cnt->phase = P.phase[d] ^ 1u;
+    sp.cnt->n_app = 0u;
+    const SpeciesDev<R>& dst = (d == 2 && a.drain) ? a.sp[3] : sp;
+    dst.cnt->n = P.n_old[d] + P.m[d];
+    dst.cnt->next_id = P.next_id_old[d] + P.m[d];
+  }
+}
+
+// Fixed-order reduction of the per-block ledger partials, one warp per field (lane l sums
+// partials l, l+32, ... in order, then a fixed shuffle tree): deterministic for a fixed grid.
+template <typename R>
+__device__ __forceinline__ void reduce_ledger(const StepArgs<R>& a, int nparts) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int k = warp; k < kLedgerN; k += blockDim.x >> 5) {
     double t = 0.0;
 #pragma unroll 4
     for (int p = lane; p < nparts; p += 32) t += a.ledger_part[(size_t)p * kLedgerN + k];
     for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(kFull, t, off);
-    if (lane == 0) {
-      a.ledger[k] = t;
-      // several warps update the work counters: integer atomics (order-independent)
-      if (k == kPushedLep) atomicAdd(&a.work[0], (unsigned long long)t);
-      if (!a.multi && k == kTauPh) atomicAdd(&a.work[5], (unsigned long long)t);
-      if (k == kPushedPh) atomicAdd(&a.work[1], (unsigned long long)t);
-      if (a.multi && k == kPushedLep) atomicAdd(&a.work[3], (unsigned long long)t);
-      if (a.multi && k == kPushedPh) atomicAdd(&a.work[4], (unsigned long long)t);
-      if (k == kEmitN) atomicAdd(&a.work[2], (unsigned long long)t);
-      if (k == kPairN) atomicAdd(&a.work[2], 2ull * (unsigned long long)t);
+    if (lane == 0) a.ledger[k] = t;
+  }
+}
+
+// The merge of one step.  Every block computes the plan for itself: the counters give the totals,
+// and warp s scans species s's coarse event counts (one per 32768 parents) into shared memory; a
+// child's rank is then three sums of at most 32 entries each, by its own thread.
+// Latency-bound: it moves a few MB at most, on every step of every run.  The form before it, a
+// one-block plan, a prefix over the event masks and a scatter, were three dependent launches of
+// 12, 5 and 8 us (GB300, 1e3 to 3e5 electrons); with this one, and the ledger's sums kept only
+// where they can be read, a step of 1e3 electrons went from 39.8 to 18.4 us and the 4000-step
+// collision of 1e3 electrons from 109 to 50 ms.
+constexpr int kCoarseMax = 1024;  // prefixes per species in shared memory (larger species: groups of counts)
+constexpr int kFinalThreads = 256;
+template <typename R>
+__global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const StepArgs<R> a, int nparts) {
+  __shared__ uint32_t s_pre[3][kCoarseMax];
+  __shared__ uint32_t s_from;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  pdl_wait();
+  pdl_launch();
+  const uint32_t n[3] = {a.sp[0].cnt->n, a.sp[1].cnt->n, a.sp[2].cnt->n};
+  const bool any_ph = a.sp[2].cnt->n_app != 0u, any_pair = a.sp[0].cnt->n_app != 0u;
+  uint32_t per[3];  // coarse counts per prefix entry
+#pragma unroll
+  for (int s = 0; s < 3; ++s) per[s] = (coarses_of(n[s]) + kCoarseMax - 1) / kCoarseMax;
+  if (warp < 3) {
+    const SpeciesDev<R>& sp = warp == 0 ? a.sp[0] : (warp == 1 ? a.sp[1] : a.sp[2]);
+    const uint32_t* co = sp.coarse + sp.cnt->phase * event_coarses(sp.cap);
+    const uint32_t nc = (warp < 2 ? any_ph : any_pair) ? coarses_of(warp == 0 ? n[0] : (warp == 1 ? n[1] : n[2])) : 0u;
+    const uint32_t g = warp == 0 ? per[0] : (warp == 1 ? per[1] : per[2]);
+    uint32_t run = 0;
+#pragma unroll 4
+    for (uint32_t e0 = 0; e0 * g < nc; e0 += 32) {
+      uint32_t v = 0;
+      for (uint32_t k = (e0 + lane) * g; k < min(nc, (e0 + lane + 1) * g); ++k) v += co[k];
+      uint32_t inc = v;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, inc, off);
+        if (lane >= off) inc += t;
+      }
+      if (e0 + lane < (uint32_t)kCoarseMax) s_pre[warp][e0 + lane] = run + inc - v;
+      run += __shfl_sync(kFull, inc, 31);
+    }
+    if (warp == 0 && lane == 0) s_from = run;
+  }
+  __syncthreads();
+  const FinalizePlan P = make_plan(a, s_from, blockIdx.x == 0 && threadIdx.x == 0);
+  const uint32_t tot = P.m[0] + P.m[1] + P.m[2];
+  const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  for (uint32_t c = first; c < tot; c += stride)
+    place_child<R>(a, P, c, [&](int s, uint32_t cg) {
+      const uint32_t g = s == 0 ? per[0] : (s == 1 ? per[1] : per[2]);
+      uint32_t r = s_pre[s][cg / g];
+      if (g > 1) {
+        const SpeciesDev<R>& sp = s == 0 ? a.sp[0] : (s == 1 ? a.sp[1] : a.sp[2]);
+        const uint32_t* co = sp.coarse + (s == 0 ? P.phase[0] : (s == 1 ? P.phase[1] : P.phase[2])) * event_coarses(sp.cap);
+        for (uint32_t k = cg / g * g; k < cg; ++k) r += co[k];
+      }
+      return r;
+    });
+  clear_other_counts(a, P, first, stride);
+  if (a.want && blockIdx.x == gridDim.x - 1) reduce_ledger(a, nparts);
+  // the last block to get here sets the counters: by then every block has read them
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&a.plan->ticket, 1u) == gridDim.x - 1) {
+      a.plan->ticket = 0u;
+      finish_counters(a, P, n);
     }
   }
 }
 
 template <typename R>
-__global__ void __launch_bounds__(1024) plan_kernel(const StepArgs<R> a, int nparts) {
-  plan_body<R>(a, nparts);
-}
-
-template <typename R>
-__device__ __forceinline__ void prefix_body(const StepArgs<R>& a, uint32_t bx, uint32_t gx) {
-  const uint32_t R0 = a.plan->ranges[0], R1 = a.plan->ranges[1], R2 = a.plan->ranges[2];
-  for (uint32_t g = bx; g < R0 + R1 + R2; g += gx) {
-    const int s = g < R0 ? 0 : (g < R0 + R1 ? 1 : 2);
-    const uint32_t r = g - (s == 0 ? 0u : (s == 1 ? R0 : R0 + R1));
-    const SpeciesDev<R>& sp = a.sp[s];
-    // ranges without events hold no parent of any child: their word prefixes are never read
-    // (the test is uniform across the block, as the scan below needs)
-    const uint32_t Rs = s == 0 ? R0 : (s == 1 ? R1 : R2);
-    const uint32_t r_end = r + 1 < Rs ? sp.rprefix[r + 1] : a.plan->events[s];
-    if (r_end == sp.rprefix[r]) continue;
-    const uint32_t words = (sp.cnt->n + 31u) >> 5;
-    const uint32_t w = (r << kRangeShift) + threadIdx.x;
-    const uint32_t m = w < words ? sp.evmask[w] : 0u;
-    const uint32_t ex = block_exclusive_scan((uint32_t)__popc(m), nullptr);
-    if (w < words) sp.wprefix[w] = sp.rprefix[r] + ex;
-  }
-}
-
-template <typename R>
-__global__ void __launch_bounds__(256) prefix_kernel(const StepArgs<R> a) {
-  prefix_body<R>(a, blockIdx.x, gridDim.x);
-}
-
-template <typename R>
-__device__ __forceinline__ uint32_t parent_rank(const SpeciesDev<R>& ps, uint32_t p) {
-  const uint32_t w = p >> 5, b = p & 31u;
-  return ps.wprefix[w] + (uint32_t)__popc(ps.evmask[w] & ((1u << b) - 1u));
-}
-
-// Child c (in destination order e-, e+, photons) of the step planned in P: its rank among the
-// destination's new particles is its parent's rank (a counting sort on the dense parent index),
-// which fixes its slot and its id.
-template <typename R>
-__device__ __forceinline__ void scatter_one(const StepArgs<R>& a, const FinalizePlan& P, uint32_t c) {
-  const uint32_t m0 = P.m[0], m1 = P.m[1];
-  const int d = c < m0 ? 0 : (c < m0 + m1 ? 1 : 2);
-  const uint32_t j = c - (d == 0 ? 0u : (d == 1 ? m0 : m0 + m1));
-  const SpeciesDev<R>& app = a.sp[d];
-  const SpeciesDev<R>& dst = (d == 2 && a.drain) ? a.sp[3] : a.sp[d];
-  const uint32_t par = app.aparent[j];
-  uint32_t rank;
-  if (d < 2) {
-    rank = parent_rank(a.sp[2], par);
-  } else {
-    const uint32_t pk = par >> 31;
-    rank = parent_rank(a.sp[pk], par & 0x7fffffffu) + (pk ? P.from_electrons : 0u);
-  }
-  if (rank >= P.m[d]) { atomicOr(&dst.cnt->err, 1u << QED_ERR_NUMERIC); return; }
-  const uint32_t o = P.n_old[d] + rank;
-  dst.x[o] = app.ax[j]; dst.y[o] = app.ay[j]; dst.z[o] = app.az[j];
-  dst.ux[o] = app.aux[j]; dst.uy[o] = app.auy[j]; dst.uz[o] = app.auz[j];
-  dst.tau[o] = app.atau[j];
-  dst.id[o] = P.next_id_old[d] + rank;
-  if (dst.w) dst.w[o] = app.aw ? app.aw[j] : (R)1;
-}
-
-// The counters after the merge (one thread).
-template <typename R>
-__device__ __forceinline__ void finish_counters(const StepArgs<R>& a, const FinalizePlan& P) {
-  for (int d = 0; d < 3; ++d) {
-    const SpeciesDev<R>& dst = (d == 2 && a.drain) ? a.sp[3] : a.sp[d];
-    dst.cnt->n = P.n_old[d] + P.m[d];
-    dst.cnt->next_id = P.next_id_old[d] + P.m[d];
-    a.sp[d].cnt->n_app = 0u;
-  }
-}
-
-template <typename R>
-__device__ __forceinline__ void scatter_body(const StepArgs<R>& a, uint32_t bx, uint32_t gx) {
-  const FinalizePlan P = *a.plan;
-  const uint32_t tot = P.m[0] + P.m[1] + P.m[2];
-  for (uint32_t c = bx * blockDim.x + threadIdx.x; c < tot; c += gx * blockDim.x) scatter_one<R>(a, P, c);
-  if (bx == 0 && threadIdx.x == 0) finish_counters<R>(a, P);
-}
-
-template <typename R>
-__global__ void __launch_bounds__(256) scatter_kernel(const StepArgs<R> a) {
-  scatter_body<R>(a, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(512) ledger_kernel(const StepArgs<R> a, int nparts) {
+  pdl_wait();
+  reduce_ledger(a, nparts);
 }
 
 // ----------------------------------------------------------------------------- batches
@@ -1325,13 +1404,16 @@ __device__ __forceinline__ int slot_of_block(const uint32_t* blocks, int S, uint
 
 // ---- per-step path of a batch: one tile space over all live slots
 // The tile schedule (one block) lays the live slots' tiles end to end (slot order, species order
-// inside a slot), and likewise their event-mask ranges, and evaluates every slot's per-step field
-// scalars once.
+// inside a slot) and evaluates every slot's per-step field
+// scalars once.  want: the batch call's last step (the ledgers of all live slots can be read after
+// it; a slot that ends with this step keeps its ledger too).
 template <typename R>
-__global__ void __launch_bounds__(1024) batch_tiles_kernel(const BatchCtl<R> c) {
+__global__ void __launch_bounds__(1024) batch_tiles_kernel(const BatchCtl<R> c, int want) {
+  pdl_wait();
+  pdl_launch();
   const int per = (c.S + blockDim.x - 1) / blockDim.x;
   const int s0 = threadIdx.x * per, s1 = min(c.S, s0 + per);
-  uint32_t tiles = 0, ranges = 0;
+  uint32_t tiles = 0;
   for (int sl = s0; sl < s1; ++sl) {
     SlotPlan q{};
     q.live = c.remaining[sl] > 0u ? 1u : 0u;
@@ -1340,28 +1422,24 @@ __global__ void __launch_bounds__(1024) batch_tiles_kernel(const BatchCtl<R> c) 
       for (int k = 0; k < 3; ++k) {
         q.n[k] = a.sp[k].cnt->n;
         q.T[k] = (q.n[k] + kTile - 1) / kTile;
-        const uint32_t words = (q.n[k] + 31u) >> 5;
-        q.Rg[k] = (words + (1u << kRangeShift) - 1u) >> kRangeShift;
         tiles += q.T[k];
-        ranges += q.Rg[k];
       }
-      make_scalars<R>(a.field, a.t0 + (double)a.step * a.dt, a.win_x0, a.win_v,
-                      static_cast<StepScalars<R>*>(c.scal)[sl]);
+      c.args[sl].want = want || c.remaining[sl] == 1u;
+      StepScalars<R>& S = static_cast<StepScalars<R>*>(c.scal)[sl];
+      make_scalars<R>(a.field, a.t0 + (double)a.step * a.dt, a.win_x0, a.win_v, S);
+      for (int k = 0; k < 3; ++k) S.phase[k] = a.sp[k].cnt->phase;
     }
     c.splan[sl] = q;
   }
-  uint32_t ttot, rtot;
+  uint32_t ttot;
   uint32_t tb = block_exclusive_scan(tiles, &ttot);
-  uint32_t rb = block_exclusive_scan(ranges, &rtot);
   for (int sl = s0; sl < s1; ++sl) {
     SlotPlan& q = c.splan[sl];
     q.tile_base = tb;
-    q.range_base = rb;
     tb += q.T[0] + q.T[1] + q.T[2];
-    rb += q.Rg[0] + q.Rg[1] + q.Rg[2];
     c.live[sl] = q.live;
   }
-  if (threadIdx.x == 0) { c.tot[0] = ttot; c.tot[1] = rtot; }
+  if (threadIdx.x == 0) c.tot[0] = ttot;
 }
 
 // The run of tiles of one (slot, species) that global tile g of the batch step lies in: its tiles
@@ -1465,8 +1543,8 @@ __device__ __forceinline__ void run_tiles(const StepArgs<R>& A, const StepScalar
     }
     while (q.count >= 32u || (!more && q.count > 0u)) {
       const uint32_t take = min(q.count, 32u);
-      if (SP == 0) lepton_events<R, QED_ELECTRON>(A, q.r, q.head, take);
-      else if (SP == 1) lepton_events<R, QED_POSITRON>(A, q.r, q.head, take);
+      if (SP == 0) lepton_events<R, QED_ELECTRON>(A, S.phase[0], q.r, q.head, take);
+      else if (SP == 1) lepton_events<R, QED_POSITRON>(A, S.phase[1], q.r, q.head, take);
       else photon_events<R>(A, q.r, q.head, take);
       q.head = (q.head + take) & (uint32_t)(kRing - 1);
       q.count -= take;
@@ -1509,27 +1587,30 @@ batch_step_kernel(const BatchCtl<R> c) {
   __shared__ __align__(16) StepArgs<R> A;
   __shared__ __align__(16) StepScalars<R> S;
   __shared__ int s_abort;
+  __shared__ uint32_t s_work[2];
 
   const uint32_t blk = blockIdx.x, nblk = gridDim.x;
-  const uint32_t ttot = c.tot[0];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) {
+  for (int k = threadIdx.x; k < c.tab.n_eta; k += blockDim.x) s_lnh[k] = c.tab.ln_h[k];
+  for (int k = threadIdx.x; k < c.tab.n_chi; k += blockDim.x) s_lnT[k] = c.tab.ln_T[k];
+  if (threadIdx.x == kBlock) {
     for (int st = 0; st < kStages; ++st) {
       mbar_init(&full[st], 1);
       mbar_init(&empty[st], kWarps);
     }
     mbar_fence_init();
     s_abort = 0;
+    s_work[0] = s_work[1] = 0;
   }
+  pdl_wait();
+  const uint32_t ttot = c.tot[0];
   __syncthreads();
+  pdl_launch();
   TileRun prun;  // producer's run of tiles and its arrays
   TileSrc<R> psrc{};
   if (threadIdx.x == kBlock)
     for (uint32_t k = 0; k < (uint32_t)kStages && blk + k * nblk < ttot; ++k)
       issue_batch_tile(c, buf, full, k, blk + k * nblk, prun, psrc);
-  for (int k = threadIdx.x; k < c.tab.n_eta; k += blockDim.x) s_lnh[k] = c.tab.ln_h[k];
-  for (int k = threadIdx.x; k < c.tab.n_chi; k += blockDim.x) s_lnT[k] = c.tab.ln_T[k];
-  __syncthreads();
 
   if (warp == kWarps) {
     // ---------------- producer
@@ -1564,17 +1645,25 @@ batch_step_kernel(const BatchCtl<R> c) {
   static_assert(sizeof(StepArgs<R>) % 8 == 0 && sizeof(StepScalars<R>) % 8 == 0, "8-byte words");
   auto flush_slot = [&]() {
     __syncwarp();
-    if (lane == 0) {
-      const EventSums<R>& es = q.r->sums;
-      for (int k = 0; k < 3; ++k) { acc.e[k].merge(es.e[k]); acc.n[k] += es.n[k]; }
-      acc.emit_e = es.emit_e; acc.emit_def = es.emit_def;
-      acc.pair_e = es.pair_e; acc.pair_def = es.pair_def;
-      acc.emit_n = es.emit_n; acc.drop = es.drop; acc.pair_n = es.pair_n;
-      q.r->sums = EventSums<R>{};
+    add_work(acc, s_work, lane);
+    if (A.want) {
+      if (lane == 0) {
+        const EventSums<R>& es = q.r->sums;
+        for (int k = 0; k < 3; ++k) { acc.e[k].merge(es.e[k]); acc.n[k] += es.n[k]; }
+        acc.emit_e = es.emit_e; acc.emit_def = es.emit_def;
+        acc.pair_e = es.pair_e; acc.pair_def = es.pair_def;
+        acc.emit_n = es.emit_n; acc.drop = es.drop; acc.pair_n = es.pair_n;
+        q.r->sums = EventSums<R>{};
+      }
+      __syncwarp();
+      write_ledger_partial<R, kWarps, true>(acc, A.ledger_part, part);
     }
-    __syncwarp();
-    write_ledger_partial<R, kWarps, true>(acc, A.ledger_part, part);
     acc = Acc<R>{};
+    compute_warps_sync();  // every warp has added its work
+    if (threadIdx.x == 0) {
+      flush_work(s_work, A.work);
+      s_work[0] = s_work[1] = 0;
+    }
   };
   for (uint32_t k = 0;;) {
     const uint32_t g = blk + k * nblk;
@@ -1611,68 +1700,50 @@ batch_step_kernel(const BatchCtl<R> c) {
   if (cur >= 0) flush_slot();
 }
 
-// Per-slot plan (one block per live slot): as plan_kernel, over the slot's partials
-// 0 .. min(its tiles, G) - 1.
+// Per-slot plan (one block per live slot): the exclusive prefixes of its species' coarse event
+// counts, the merge plan, the slot's ledger (from its partials 0 .. min(its tiles, G) - 1) where it
+// can be read, and the counts of the step before cleared.
 template <typename R>
-__global__ void __launch_bounds__(1024) batch_plan_kernel(const BatchCtl<R> c, int G) {
-  __shared__ __align__(16) StepArgs<R> A;
+__global__ void __launch_bounds__(256) batch_plan_kernel(const BatchCtl<R> c, int G) {
+  __shared__ uint32_t s_tot;
+  pdl_wait();
+  pdl_launch();
   const int sl = blockIdx.x;
   const SlotPlan& q = c.splan[sl];
   if (!q.live) return;
-  const uint32_t tiles = q.T[0] + q.T[1] + q.T[2];
-  load_args(A, c.args + sl);
-  plan_body<R>(A, (int)min(tiles, (uint32_t)G));
-}
-
-// Event-mask prefixes of every live slot's ranges with events, one warp per range over the
-// batch step's range space (ranges without events are never read by the scatter).
-template <typename R>
-__global__ void __launch_bounds__(256) batch_prefix_kernel(const BatchCtl<R> c) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
-  const uint32_t rtot = c.tot[1];
-  int cur = 0;
-  for (uint32_t rg = gw; rg < rtot; rg += nw) {
-    while (cur + 1 < c.S && c.splan[cur + 1].range_base <= rg) ++cur;
-    const SlotPlan& q = c.splan[cur];
-    uint32_t r = rg - q.range_base;
-    int s = 0;
-    if (r >= q.Rg[0]) { r -= q.Rg[0]; s = 1; if (r >= q.Rg[1]) { r -= q.Rg[1]; s = 2; } }
-    const StepArgs<R>& a = c.args[cur];
+  const StepArgs<R>& a = c.args[sl];
+  for (int s = 0; s < 3; ++s) {
     const SpeciesDev<R>& sp = a.sp[s];
-    const uint32_t r0 = sp.rprefix[r];
-    const uint32_t r_end = r + 1 < q.Rg[s] ? sp.rprefix[r + 1] : a.plan->events[s];
-    if (r_end == r0) continue;
-    const uint32_t words = (q.n[s] + 31u) >> 5;
-    const uint32_t w0 = (r << kRangeShift) + lane * 8u;
-    uint32_t pc[8], sum = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      pc[i] = w0 + i < words ? (uint32_t)__popc(sp.evmask[w0 + i]) : 0u;
-      sum += pc[i];
+    if ((s < 2 ? a.sp[2] : a.sp[0]).cnt->n_app == 0u) continue;  // (uniform) no child asks for it
+    const uint32_t nc = coarses_of(q.n[s]);
+    const uint32_t* co = sp.coarse + sp.cnt->phase * event_coarses(sp.cap);
+    uint32_t base = 0;
+    for (uint32_t k0 = 0; k0 < nc; k0 += blockDim.x) {
+      const uint32_t k = k0 + threadIdx.x, v = k < nc ? co[k] : 0u;
+      uint32_t tot;
+      const uint32_t ex = block_exclusive_scan(v, &tot);
+      if (k < nc) sp.cprefix[k] = base + ex;
+      base += tot;
     }
-    uint32_t inc = sum;
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t t = __shfl_up_sync(kFull, inc, off);
-      if (lane >= (uint32_t)off) inc += t;
-    }
-    uint32_t run = r0 + inc - sum;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (w0 + i < words) sp.wprefix[w0 + i] = run;
-      run += pc[i];
-    }
+    if (s == 0 && threadIdx.x == 0) s_tot = base;
   }
+  __syncthreads();
+  if (threadIdx.x == 0) *a.plan = make_plan(a, a.sp[2].cnt->n_app ? s_tot : 0u, true);
+  FinalizePlan P;
+  for (int s = 0; s < 3; ++s) P.phase[s] = a.sp[s].cnt->phase;
+  clear_other_counts(a, P, threadIdx.x, blockDim.x);
+  if (a.want) reduce_ledger(a, (int)min(q.T[0] + q.T[1] + q.T[2], (uint32_t)G));
 }
 
-// The new particles of every live slot, ranked and moved into place (scatter_one) by a grid that
+// The new particles of every live slot, ranked and moved into place (place_child) by a grid that
 // strides through all slots' children together; the first threads of block 0 then set each
 // slot's counters and advance its step.
 constexpr int kMaxScatterSlots = 4096;
 template <typename R>
 __global__ void __launch_bounds__(256) batch_scatter_kernel(const BatchCtl<R> c) {
   __shared__ uint32_t s_base[kMaxScatterSlots + 1];
+  pdl_wait();
+  pdl_launch();
   const int per = (c.S + blockDim.x - 1) / blockDim.x;
   const int s0 = threadIdx.x * per, s1 = min(c.S, s0 + per);
   uint32_t mine = 0;
@@ -1692,13 +1763,13 @@ __global__ void __launch_bounds__(256) batch_scatter_kernel(const BatchCtl<R> c)
     int lo = 0, hi = c.S;  // s_base[lo] <= ci < s_base[hi]
     while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (s_base[mid] <= ci) lo = mid; else hi = mid; }
     const StepArgs<R>& a = c.args[lo];
-    scatter_one<R>(a, *a.plan, ci - s_base[lo]);
+    place_child<R>(a, *a.plan, ci - s_base[lo], [&](int s, uint32_t cg) { return a.sp[s].cprefix[cg]; });
   }
   if (blockIdx.x == 0)
     for (int sl = threadIdx.x; sl < c.S; sl += blockDim.x) {
       if (!c.splan[sl].live) continue;
       const StepArgs<R>& a = c.args[sl];
-      finish_counters<R>(a, *a.plan);
+      finish_counters<R>(a, *a.plan, c.splan[sl].n);
       c.args[sl].step = a.step + 1;  // the slot's next step
       c.remaining[sl] -= 1u;
     }
@@ -1741,6 +1812,8 @@ __global__ void __launch_bounds__(kFuseThreads) batch_fused_kernel(const BatchCt
   const int K = s_K;
   if (K == 0) return;
   load_args(A, c.args + sl);
+  if (threadIdx.x == 0) A.want = 1;  // the stretch may use up the slot's steps
+  __syncthreads();
   const uint32_t bb = b - c.blocks[sl], nb = c.blocks[sl + 1] - c.blocks[sl];
   if (A.field.kind == QED_FIELD_PLANE_LP) fused_body<R, G, COMMIT, kFieldLP>(A, K, c.first_event + sl, bb, nb, smem_raw);
   else if (A.field.kind == QED_FIELD_PLANE_CP) fused_body<R, G, COMMIT, kFieldCP>(A, K, c.first_event + sl, bb, nb, smem_raw);
@@ -1758,9 +1831,7 @@ __global__ void __launch_bounds__(1024) batch_commit_plan_kernel(const BatchCtl<
   }
   if (k == 0) return;
   load_args(A, c.args + sl);
-  if (threadIdx.x == 0) A.multi = 1;
-  __syncthreads();
-  plan_body<R>(A, (int)(c.blocks[sl + 1] - c.blocks[sl]));  // no children: counters stay, ledger of the last step
+  reduce_ledger(A, (int)(c.blocks[sl + 1] - c.blocks[sl]));  // no children: the ledger of the stretch's last step
   __syncthreads();
   if (threadIdx.x == 0) {
     c.args[sl].step = A.step + k;
@@ -1944,6 +2015,23 @@ void count_launch(int n) { g_launches += (uint64_t)n; }
 uint64_t launch_count_value() { return g_launches.load(); }
 #endif
 
+// Launch with programmatic dependent launch: the kernel may start before the one ahead of it in
+// the stream has finished, and calls pdl_wait before it touches anything that one writes.
+template <typename... P, typename... A>
+static void launch_pdl(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
 // dynamic shared memory of the step kernel: the tile stages, the compute warps' event rings,
 // then ln h and ln T
 template <typename R>
@@ -1979,11 +2067,11 @@ void launch_step(const StepArgs<R>& a, int grid, int block, size_t smem_unused, 
   if (a.field.kind == QED_FIELD_GRID) {
     if (smem > 48 * 1024)
       cudaFuncSetAttribute(step_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    step_kernel<R, true><<<grid, kStepThreads, smem, s>>>(a);
+    launch_pdl(step_kernel<R, true>, grid, kStepThreads, smem, s, a);
   } else {
     if (smem > 48 * 1024)
       cudaFuncSetAttribute(step_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    step_kernel<R, false><<<grid, kStepThreads, smem, s>>>(a);
+    launch_pdl(step_kernel<R, false>, grid, kStepThreads, smem, s, a);
   }
   count_launch();
 }
@@ -1992,7 +2080,7 @@ void launch_step(const StepArgs<R>& a, int grid, int block, size_t smem_unused, 
 
 #if QED_PART(2)
 template <typename R>
-void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, cudaStream_t s) {
+void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, bool want, cudaStream_t s) {
   const size_t smem = step_smem<R>(n_eta, n_chi);
   if (smem + sizeof(StepArgs<R>) + sizeof(StepScalars<R>) > 40 * 1024) {
     cudaFuncSetAttribute(batch_step_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -2014,13 +2102,12 @@ void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, cudaStream_t 
     count_launch(5);
   }
   // the per-step path: one tile space over all live slots, strided by a persistent grid
-  batch_tiles_kernel<R><<<1, 1024, 0, s>>>(c);
-  if (c.grid_fields) batch_step_kernel<R, true><<<c.target_blocks, kStepThreads, smem, s>>>(c);
-  else batch_step_kernel<R, false><<<c.target_blocks, kStepThreads, smem, s>>>(c);
-  batch_plan_kernel<R><<<c.S, 1024, 0, s>>>(c, c.target_blocks);
-  batch_prefix_kernel<R><<<sm_count() * 8, 256, 0, s>>>(c);
-  batch_scatter_kernel<R><<<sm_count() * 4, 256, 0, s>>>(c);
-  count_launch(5);
+  launch_pdl(batch_tiles_kernel<R>, 1, 1024, 0, s, c, want ? 1 : 0);
+  if (c.grid_fields) launch_pdl(batch_step_kernel<R, true>, c.target_blocks, kStepThreads, smem, s, c);
+  else launch_pdl(batch_step_kernel<R, false>, c.target_blocks, kStepThreads, smem, s, c);
+  launch_pdl(batch_plan_kernel<R>, c.S, 256, 0, s, c, c.target_blocks);
+  launch_pdl(batch_scatter_kernel<R>, sm_count() * 4, 256, 0, s, c);
+  count_launch(4);
 }
 
 #endif
@@ -2075,10 +2162,14 @@ void launch_selftest_wait(uint32_t polls, uint32_t* bits, cudaStream_t s) {
 
 template <typename R>
 void launch_finalize(const StepArgs<R>& a, int step_grid, cudaStream_t s) {
-  plan_kernel<R><<<1, 1024, 0, s>>>(a, step_grid);
-  prefix_kernel<R><<<sm_count() * 4, 256, 0, s>>>(a);
-  scatter_kernel<R><<<sm_count() * 4, 256, 0, s>>>(a);
-  count_launch(3);
+  launch_pdl(finalize_kernel<R>, sm_count(), kFinalThreads, 0, s, a, step_grid);
+  count_launch();
+}
+
+template <typename R>
+void launch_ledger(const StepArgs<R>& a, int parts, cudaStream_t s) {
+  ledger_kernel<R><<<1, 512, 0, s>>>(a, parts);
+  count_launch();
 }
 
 #endif
@@ -2314,13 +2405,14 @@ void launch_merge(const SpeciesDev<R>& sp, const MergeDev& m, uint64_t* keys, ui
 #define QED_INSTANTIATE_STEP(R)                                                                                  \
   template void launch_step<R>(const StepArgs<R>&, int, int, size_t, cudaStream_t);                              \
   template void launch_finalize<R>(const StepArgs<R>&, int, cudaStream_t);                                       \
+  template void launch_ledger<R>(const StepArgs<R>&, int, cudaStream_t);                                         \
   template int launch_fused<R>(const StepArgs<R>&, int, bool, uint32_t*, int, cudaStream_t);
 QED_INSTANTIATE_STEP(float)
 QED_INSTANTIATE_STEP(double)
 #endif
 #if QED_PART(2)
-template void launch_batch_step<float>(const BatchCtl<float>&, int, int, cudaStream_t);
-template void launch_batch_step<double>(const BatchCtl<double>&, int, int, cudaStream_t);
+template void launch_batch_step<float>(const BatchCtl<float>&, int, int, bool, cudaStream_t);
+template void launch_batch_step<double>(const BatchCtl<double>&, int, int, bool, cudaStream_t);
 #endif
 #if QED_PART(3)
 #define QED_INSTANTIATE(R)                                                                                       \

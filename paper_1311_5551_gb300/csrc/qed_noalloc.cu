@@ -25,22 +25,23 @@ using namespace qedlib;
 namespace {
 
 constexpr size_t kMaxElectrons = 65536;  // per call
-constexpr size_t kWords = kMaxElectrons / 32 + 2;
-constexpr size_t kRanges = (kWords >> kRangeShift) + 2;
+constexpr size_t kWords = event_words(kMaxElectrons);
+constexpr size_t kCounts = 2 * event_fines(kMaxElectrons) + 2 * event_coarses(kMaxElectrons);  // fine, coarse
+constexpr size_t kEmptyWords = event_words(1) + 2 * event_fines(1) + 2 * event_coarses(1);
 constexpr size_t kMaxGrid = 2048;        // step-kernel blocks (ledger partials)
 constexpr size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 // layout of the scratch array (byte offsets)
 constexpr size_t kOffCounters = 0;                                           // 4 DevCounters
-constexpr size_t kOffMasks = align256(kOffCounters + 4 * sizeof(DevCounters));  // evmask, wprefix
-constexpr size_t kOffRanges = align256(kOffMasks + 2 * kWords * 4);          // rangesum, rprefix
-constexpr size_t kOffAppend = align256(kOffRanges + 2 * kRanges * 4);        // photon append region
+constexpr size_t kOffMasks = align256(kOffCounters + 4 * sizeof(DevCounters));  // evmask
+constexpr size_t kOffCounts = align256(kOffMasks + kWords * 4);              // fine, coarse
+constexpr size_t kOffAppend = align256(kOffCounts + kCounts * 4);            // photon append region
 constexpr size_t kAppendBytes = kMaxElectrons * (6 * 8 + 8 + 4) + 8 * 256;   // sized for FP64
 constexpr size_t kOffLedger = align256(kOffAppend + kAppendBytes);           // partials + ledger
 constexpr size_t kLedgerBytes = (kMaxGrid + 1) * kLedgerN * 8;
 constexpr size_t kOffPlan = align256(kOffLedger + kLedgerBytes);
 constexpr size_t kOffWork = align256(kOffPlan + sizeof(FinalizePlan));
-constexpr size_t kOffEmpty = align256(kOffWork + 5 * 8);                     // masks of the empty species
-constexpr size_t kScratchBytes = align256(kOffEmpty + 64);
+constexpr size_t kOffEmpty = align256(kOffWork + 6 * 8);                     // masks and counts of the empty species
+constexpr size_t kScratchBytes = align256(kOffEmpty + kEmptyWords * 4);
 
 // The scratch.  Host code must not pass this name to a kernel: on the host it is only a
 // stand-in for the device symbol; its device address comes from cudaGetSymbolAddress.
@@ -49,9 +50,13 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 std::mutex g_mu;
 void* g_addr[128] = {};  // device address of the scratch, per device ordinal
 
-__global__ void noalloc_begin_kernel(DevCounters* c, uint32_t n_e, const uint32_t* photon_counter) {
+// every call starts from cleared counters and event counts: the array keeps the last call's
+// contents, and an earlier call may have stopped on an error (one warp)
+__global__ void noalloc_begin_kernel(DevCounters* c, uint32_t* counts, uint32_t n_e, const uint32_t* photon_counter) {
+  for (uint32_t k = threadIdx.x; k < (uint32_t)kCounts; k += 32) counts[k] = 0u;
+  if (threadIdx.x != 0) return;
   // electrons, positrons (empty), photons (empty, receives the append), drain = caller's arrays
-  for (int k = 0; k < 4; ++k) { c[k].n = 0; c[k].next_id = 0; c[k].n_app = 0; c[k].n_dead = 0; c[k].err = 0; }
+  for (int k = 0; k < 4; ++k) c[k] = DevCounters{};
   c[0].n = n_e;
   c[3].n = photon_counter[0];
   c[3].next_id = photon_counter[1];
@@ -66,13 +71,12 @@ __global__ void noalloc_end_kernel(const DevCounters* c, uint32_t* photon_counte
 }
 
 template <typename R>
-void bind_species(SpeciesDev<R>& s, DevCounters* cnt, uint32_t* masks, uint32_t* ranges, size_t words,
-                  size_t nranges) {
+void bind_species(SpeciesDev<R>& s, DevCounters* cnt, uint32_t* masks, uint32_t* counts, size_t cap) {
   s.cnt = cnt;
   s.evmask = masks;
-  s.wprefix = masks + words;
-  s.rangesum = ranges;
-  s.rprefix = ranges + nranges;
+  s.fine = counts;
+  s.coarse = counts + 2 * event_fines(cap);
+  s.cap = (uint32_t)cap;
 }
 
 template <typename R>
@@ -80,19 +84,19 @@ qed_status run_noalloc(const TablesDev& tv, const qed_soa* e, size_t n, const qe
                        uint32_t* counter, const qed_step_params* p, unsigned char* base, cudaStream_t s) {
   DevCounters* cnt = reinterpret_cast<DevCounters*>(base + kOffCounters);
   uint32_t* masks = reinterpret_cast<uint32_t*>(base + kOffMasks);
-  uint32_t* ranges = reinterpret_cast<uint32_t*>(base + kOffRanges);
+  uint32_t* counts = reinterpret_cast<uint32_t*>(base + kOffCounts);
   uint32_t* empty = reinterpret_cast<uint32_t*>(base + kOffEmpty);
   StepArgs<R> a{};
   // electrons: the caller's arrays, updated in place
   SpeciesDev<R>& el = a.sp[0];
   el.x = (R*)e->x; el.y = (R*)e->y; el.z = (R*)e->z; el.ux = (R*)e->ux; el.uy = (R*)e->uy; el.uz = (R*)e->uz;
-  el.tau = e->tau; el.id = e->id; el.cap = (uint32_t)n; el.acap = 0;
-  bind_species(el, cnt + 0, masks, ranges, kWords, kRanges);
+  el.tau = e->tau; el.id = e->id; el.acap = 0;
+  bind_species(el, cnt + 0, masks, counts, kMaxElectrons);
   // positrons: empty (no pairs in this variant)
-  bind_species(a.sp[1], cnt + 1, empty, empty + 4, 2, 2);
+  bind_species(a.sp[1], cnt + 1, empty, empty + event_words(1), 1);
   // photons: empty, but their append region (in the scratch) collects the new photons
   SpeciesDev<R>& pg = a.sp[2];
-  bind_species(pg, cnt + 2, empty, empty + 4, 2, 2);
+  bind_species(pg, cnt + 2, empty, empty + event_words(1), 1);
   unsigned char* ap = base + kOffAppend;
   auto take = [&](size_t bytes) { unsigned char* q = ap; ap += align256(bytes); return q; };
   pg.ax = (R*)take(kMaxElectrons * sizeof(R)); pg.ay = (R*)take(kMaxElectrons * sizeof(R));
@@ -114,10 +118,7 @@ qed_status run_noalloc(const TablesDev& tv, const qed_soa* e, size_t n, const qe
   a.ledger = a.ledger_part + kMaxGrid * kLedgerN;
   a.plan = reinterpret_cast<FinalizePlan*>(base + kOffPlan);
   a.work = reinterpret_cast<unsigned long long*>(base + kOffWork);
-  // every call starts from cleared counters and range sums: the array keeps the last call's
-  // contents, and an earlier call may have stopped on an error
-  cudaMemsetAsync(ranges, 0, 2 * kRanges * 4, s);
-  noalloc_begin_kernel<<<1, 1, 0, s>>>(cnt, (uint32_t)n, counter);
+  noalloc_begin_kernel<<<1, 32, 0, s>>>(cnt, counts, (uint32_t)n, counter);
   const int grid = std::min(step_grid_size(sizeof(R) == 4 ? QED_MIXED : QED_FP64), (int)kMaxGrid);
   launch_step<R>(a, grid, 256, 0, s);
   launch_finalize<R>(a, grid, s);
