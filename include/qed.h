@@ -270,7 +270,9 @@ typedef struct {
  * (parent species, parent index) with consecutive ids.  sp[3] receives the new photons when
  * drain_photons is set (it may be NULL otherwise).  Species must share one precision. */
 qed_status qed_step(const qed_tables* tables, qed_species* const* sp, const qed_step_params* params, void* stream);
-/* n_steps consecutive steps starting at params->step. */
+/* n_steps consecutive steps starting at params->step.  In the mixed path the photons held are taken
+ * up to 16 steps at a time (photons depend on no other particle; one that converts does so at its
+ * step), with the results of the single steps. */
 qed_status qed_run(const qed_tables* tables, qed_species* const* sp, const qed_step_params* params,
                    uint64_t n_steps, void* stream);
 /* Ledger of the last step taken on these species.  Synchronises the stream. */
@@ -386,8 +388,9 @@ qed_status qed_philox(size_t n, const uint64_t* ctr, const uint64_t key[2], uint
  * pushes, out[1] photon pushes (converted photons excluded), out[2] particles created.
  * Synchronises. */
 qed_status qed_work_read(qed_species* electrons, uint64_t out[3], int reset, void* stream);
-/* As qed_work_read, plus out[3] e+- pushes and out[4] photon pushes made by multi-step passes
- * (already counted in out[0] and out[1]), and out[5] photon pushes of the per-step kernel in a
+/* As qed_work_read, plus out[3] e+- pushes and out[4] photon pushes made by passes over several
+ * steps (the multi-step passes of qed_run_multistep and, in the mixed path, the photon windows of
+ * every run of more than two steps; already counted in out[0] and out[1]), and out[5] photon pushes of the per-step kernel in a
  * field, whose optical depth changed and was written back (a photon outside every field keeps
  * its optical depth, and the step stores only its position). */
 qed_status qed_work_read_split(qed_species* electrons, uint64_t out[6], int reset, void* stream);
@@ -396,7 +399,8 @@ qed_status qed_work_read_split(qed_species* electrons, uint64_t out[6], int rese
  * and the number of launches timed since the last reset. */
 qed_status qed_timing_enable(int on);
 qed_status qed_timing_read(double* step_kernel_ms, uint64_t* launches, int reset);
-/* The same for the multi-step passes of qed_run_multistep (probe and commit launches). */
+/* The same for the passes over several steps: the probe and commit launches of qed_run_multistep
+ * and the photon windows of single-scenario runs. */
 qed_status qed_timing_read_multistep(double* ms, uint64_t* passes, int reset);
 
 /* Failure-detection self-test: runs the bounded mbarrier wait that every pipeline wait of the

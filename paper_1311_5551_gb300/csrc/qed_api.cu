@@ -267,13 +267,14 @@ struct qed_species {
 
 namespace {
 template <typename R>
-void carve_species(Carver& cv, SpeciesDev<R>& s, size_t cap, size_t acap) {
+void carve_species(Carver& cv, SpeciesDev<R>& s, size_t cap, size_t acap, bool windows) {
   cv.add(&s.x, cap); cv.add(&s.y, cap); cv.add(&s.z, cap);
   cv.add(&s.ux, cap); cv.add(&s.uy, cap); cv.add(&s.uz, cap);
   cv.add(&s.tau, cap); cv.add(&s.id, cap);
   cv.add(&s.evmask, event_words(cap));
   cv.add(&s.fine, 2 * event_fines(cap)); cv.add(&s.coarse, 2 * event_coarses(cap));
   cv.add(&s.cprefix, event_coarses(cap));
+  if (windows) { cv.add(&s.cmask, event_words(cap)); cv.add(&s.wflag, event_fines(cap)); }
   cv.add(&s.ax, acap); cv.add(&s.ay, acap); cv.add(&s.az, acap);
   cv.add(&s.aux, acap); cv.add(&s.auy, acap); cv.add(&s.auz, acap);
   cv.add(&s.atau, acap); cv.add(&s.aparent, acap);
@@ -366,8 +367,8 @@ extern "C" qed_status qed_species_alloc(qed_kind kind, qed_precision precision, 
   sp->acap = append_capacity;
   sp->ledger_parts = std::max(step_grid_size(QED_MIXED), step_grid_size(QED_FP64));
   Carver cv;
-  if (precision == QED_MIXED) carve_species(cv, sp->f, capacity, std::max<size_t>(append_capacity, 1));
-  else carve_species(cv, sp->d, capacity, std::max<size_t>(append_capacity, 1));
+  if (precision == QED_MIXED) carve_species(cv, sp->f, capacity, std::max<size_t>(append_capacity, 1), kind == QED_PHOTON);
+  else carve_species(cv, sp->d, capacity, std::max<size_t>(append_capacity, 1), false);
   cv.add(&sp->cnt, 1);
   cv.add(&sp->ledger_part, (size_t)sp->ledger_parts * kLedgerN);
   cv.add(&sp->ledger, kLedgerN);
@@ -797,14 +798,17 @@ StepArgs<R> make_args(const qed_tables* T, qed_species* const* sp, const qed_ste
   a.ledger = sp[0]->ledger;
   a.plan = sp[0]->plan;
   a.work = sp[0]->work;
+  a.win_s = -1;
   return a;
 }
 
+// One step; want: its ledger can be read.  win_s: the step's place in a photon window (-1: none).
 template <typename R>
-qed_status do_step(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t step, bool want,
-                   cudaStream_t s) {
+void do_step(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t step, bool want, int win_s,
+             cudaStream_t s) {
   StepArgs<R> a = make_args<R>(T, sp, p, step);
   a.want = want ? 1 : 0;
+  a.win_s = win_s;
   const int grid = std::min(step_grid_size(sizeof(R) == 4 ? QED_MIXED : QED_FP64), sp[0]->ledger_parts);
   const size_t smem = (size_t)(a.tab.n_eta + a.tab.n_chi) * sizeof(R);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -814,7 +818,32 @@ qed_status do_step(const qed_tables* T, qed_species* const* sp, const qed_step_p
   if (timed) cudaEventRecord(e1, s);
   launch_finalize<R>(a, grid, s);
   sp[0]->last_drain = a.drain;
-  return QED_OK;
+}
+
+// n consecutive steps; want: the last one's ledger can be read.  The mixed path takes its photons a
+// window at a time (window_kernel): from two steps on it pays at any size (one launch of a few
+// microseconds per window where there are few photons).  The FP64 path is bound by the FP64 pipe,
+// which the window's arithmetic needs as much, and keeps no room for a waiting conversion's chi.
+template <typename R>
+void do_steps(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t step, uint64_t n, bool want,
+              cudaStream_t s) {
+  const uint64_t quiet = want ? n - 1 : n;  // steps whose ledger nobody reads
+  for (uint64_t k = 0; k < n;) {
+    const int K = k < quiet ? (int)std::min<uint64_t>(kWinMax, quiet - k) : 1;
+    bool window = false;
+    if constexpr (sizeof(R) == 4) {
+      if (K >= 2) {
+        const StepArgs<R> a = make_args<R>(T, sp, p, step + k);
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        const bool timed = timing_events(e0, e1, g_timing_multi);
+        if (timed) cudaEventRecord(e0, s);
+        launch_window(a, K, s);
+        if (timed) cudaEventRecord(e1, s);
+        window = true;
+      }
+    }
+    for (int w = 0; w < K; ++w, ++k) do_step<R>(T, sp, p, step + k, want && k + 1 == n, window ? w : -1, s);
+  }
 }
 
 qed_status check_step_args(const qed_tables* T, qed_species* const* sp, const qed_step_params* p) {
@@ -1138,12 +1167,8 @@ extern "C" qed_status qed_run(const qed_tables* T, qed_species* const* sp, const
   st = sync_weights(sp, s);
   if (st != QED_OK) return st;
   NvtxRange range("qed_run");
-  for (uint64_t k = 0; k < n_steps; ++k) {
-    const bool want = k + 1 == n_steps;
-    st = sp[0]->precision == QED_MIXED ? do_step<float>(T, sp, *p, p->step + k, want, s)
-                                       : do_step<double>(T, sp, *p, p->step + k, want, s);
-    if (st != QED_OK) return st;
-  }
+  if (sp[0]->precision == QED_MIXED) do_steps<float>(T, sp, *p, p->step, n_steps, true, s);
+  else do_steps<double>(T, sp, *p, p->step, n_steps, true, s);
   QED_CUDA(cudaGetLastError());
   return QED_OK;
 }
@@ -1164,10 +1189,8 @@ qed_status run_multi(const qed_tables* T, qed_species* const* sp, const qed_step
   while (left > 0) {
     if (per_step > 0 || left < 2) {
       const uint64_t m = per_step > 0 ? std::min(left, per_step) : left;
-      for (uint64_t k = 0; k < m; ++k) {
-        qed_status st = do_step<R>(T, sp, p, step++, k + 1 == left, s);
-        if (st != QED_OK) return st;
-      }
+      do_steps<R>(T, sp, p, step, m, m == left, s);
+      step += m;
       left -= m;
       per_step = 0;
       continue;

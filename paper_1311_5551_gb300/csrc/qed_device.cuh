@@ -634,6 +634,11 @@ template <> struct Tau<float> {
   static __device__ __forceinline__ Tau fresh(float x) { return Tau{x, 0.0f}; }
   static __device__ __forceinline__ Tau infinite() { return Tau{__int_as_float(0x7f800000), 0.0f}; }
   static __device__ __forceinline__ Tau one() { return Tau{1.0f, 0.0f}; }
+  // what the 8 bytes hold between a photon window and the step that takes its conversion: that
+  // step (in the window) and chi
+  static __device__ __forceinline__ Tau window(int step, float chi) { return Tau{__int_as_float(step), chi}; }
+  __device__ __forceinline__ int window_step() const { return __float_as_int(hi); }
+  __device__ __forceinline__ float window_chi() const { return lo; }
 };
 
 // Conversions between the double tau of the C ABI and the stored representation.

@@ -52,7 +52,12 @@ struct DevCounters {
   // used in the other one (ext, in fine groups) and then switches
   uint32_t phase;
   uint32_t ext[2];
+  uint32_t win_n;    // photons the current window has advanced (the first win_n, a multiple of 1024)
+  uint32_t pad[3];
 };
+
+// Photon windows: steps a window spans at most (a converted photon's step is a bit of `wflag`).
+constexpr int kWinMax = 16;
 
 // A parent's rank among its species' parents of children is summed from three levels: whole
 // coarse groups, whole fine groups in its coarse group, whole mask words in its fine group.
@@ -82,6 +87,10 @@ struct SpeciesDev {
   uint32_t* fine;     // [2 * event_fines(cap)]
   uint32_t* coarse;   // [2 * event_coarses(cap)]
   uint32_t* cprefix;  // [event_coarses(cap)] exclusive prefix of coarse (batches)
+  // photon windows: the photons a window found to convert (one bit each) and, per fine group, at
+  // which of its steps (bit s); the groups' words are zero between windows
+  uint32_t* cmask;    // [event_words(cap)]
+  uint32_t* wflag;    // [event_fines(cap)]
   // as a destination: particles created for this species during the step
   R *ax, *ay, *az, *aux, *auy, *auz;
   double* atau;
@@ -134,6 +143,7 @@ struct StepArgs {
                              // photon pushes made by multi-step passes (part of [0], [1]), and the
                              // per-step photon pushes in a field
   int want;                  // somebody can read this step's ledger: keep its sums
+  int win_s;                 // step of the photon window this step belongs to (-1: none)
 };
 
 // What one batch step does with a slot, written by the tile schedule at the start of the step:
@@ -178,6 +188,9 @@ void launch_step(const StepArgs<R>& a, int grid, int block, size_t smem, cudaStr
 template <typename R>
 void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, bool want, cudaStream_t s);
 size_t step_scalars_bytes(int precision);
+// Advances the photons held, but for the last n mod 1024, by K <= kWinMax steps from a.step on (see
+// window_kernel).
+void launch_window(const StepArgs<float>& a, int K, cudaStream_t s);
 // Merges the step's children into place and sets the counters; `step_grid` ledger partials are
 // reduced when a.want is set.
 template <typename R>

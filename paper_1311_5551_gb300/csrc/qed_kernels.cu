@@ -557,15 +557,15 @@ __device__ __forceinline__ TileSrc<R> tile_src(const SpeciesDev<R>& p) {
 // Thread 0 issues the bulk copies of the block's k-th tile into stage k % kStages.
 template <typename R>
 __device__ __forceinline__ void issue_tile(const StepArgs<R>& a, TileBuf<R>* buf, uint64_t* bar, uint32_t k, uint32_t n0,
-                                        uint32_t n1, uint32_t n2, uint32_t blk, uint32_t nblk) {
-  const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 + kTile - 1) / kTile;
+                                        uint32_t n1, uint32_t n2, uint32_t win_n, uint32_t blk, uint32_t nblk) {
+  const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 - win_n + kTile - 1) / kTile;
   const uint32_t t = blk + k * nblk;
   if (t >= T0 + T1 + T2) return;
   int s; uint32_t j;
   decode_tile(t, T0, T1, s, j);
   const TileSrc<R> src = s == 0 ? tile_src(a.sp[0]) : (s == 1 ? tile_src(a.sp[1]) : tile_src(a.sp[2]));
   const uint32_t ns = s == 0 ? n0 : (s == 1 ? n1 : n2);
-  const uint32_t first = j * kTile;
+  const uint32_t first = (s == 2 ? win_n : 0u) + j * kTile;
   const uint32_t valid = min((uint32_t)kTile, ns - first);
   // arrays start 16-byte aligned and tiles start at multiples of 256 particles, so every source
   // is 16-byte aligned; only whole 16-byte pieces are copied (no read past the last particle),
@@ -666,8 +666,8 @@ __device__ __forceinline__ void flush_work(uint32_t* s_work, unsigned long long*
   if (s_work[1]) atomicAdd(&work[5], (unsigned long long)s_work[1]);
 }
 
-// The block's tiles of species SP, global tiles [t_lo, t_hi), with the block's tile count k
-// running on; field class FC.  Events are taken 32 at a time and all of them after the species'
+// The block's tiles of species SP, global tiles [t_lo, t_hi) over its particles [base, n), with the
+// block's tile count k running on; field class FC.  Events are taken 32 at a time and all of them after the species'
 // last tile.  False if a wait gave up (the events left in the ring are then not taken).  One loop
 // per species and field class, so no tile decodes its species or dispatches on the field (on
 // GB300 this took 10% off the head-on job's per-step kernel).  Species indices stay compile-time
@@ -675,10 +675,10 @@ __device__ __forceinline__ void flush_work(uint32_t* s_work, unsigned long long*
 template <typename R, bool G, int FC, int SP>
 __device__ __forceinline__ bool species_tiles(const StepArgs<R>& a, const StepScalars<R>& S, const R* lnh, const R* lnT,
                                               TileBuf<R>* buf, uint64_t* full, uint64_t* empty, uint32_t& k,
-                                              uint32_t blk, uint32_t nblk, uint32_t t_lo, uint32_t t_hi, uint32_t n,
-                                              int lane, int warp, Acc<R>& acc, EventQueue<R>& q) {
-  const uint32_t last = n ? (n - 1u) / (uint32_t)kTile : 0u;  // the only tile that can be ragged
-  const uint32_t valid = n - last * (uint32_t)kTile;
+                                              uint32_t blk, uint32_t nblk, uint32_t t_lo, uint32_t t_hi, uint32_t base,
+                                              uint32_t n, int lane, int warp, Acc<R>& acc, EventQueue<R>& q) {
+  const uint32_t last = n > base ? (n - base - 1u) / (uint32_t)kTile : 0u;  // the only tile that can be ragged
+  const uint32_t valid = n - base - last * (uint32_t)kTile;
   const uint32_t in_r = floor16(valid * (uint32_t)sizeof(R)) / (uint32_t)sizeof(R);
   const uint32_t in_t = floor16(valid * 8u) / 8u;
   const bool ragged = in_r < valid || in_t < valid;
@@ -693,7 +693,7 @@ __device__ __forceinline__ bool species_tiles(const StepArgs<R>& a, const StepSc
       TileBuf<R>& b = buf[st];
       if (ragged && j == last) {
         const TileSrc<R> g = tile_src(a.sp[SP]);
-        const uint32_t gi = j * kTile + r;
+        const uint32_t gi = base + j * kTile + r;
         if (r >= in_r && r < valid) {
           b.x[r] = g.x[gi]; b.y[r] = g.y[gi]; b.z[r] = g.z[gi];
           b.ux[r] = g.ux[gi]; b.uy[r] = g.uy[gi]; b.uz[r] = g.uz[gi];
@@ -701,7 +701,7 @@ __device__ __forceinline__ bool species_tiles(const StepArgs<R>& a, const StepSc
         if (r >= in_t && r < valid) b.tau[r] = g.tau[gi];
         compute_warps_sync();
       }
-      const uint32_t chunk = j * kWarps + warp;
+      const uint32_t chunk = base / 32u + j * kWarps + warp;
       if (SP == 2)
         photon_chunk<R, G, FC>(a, S, lnT, chunk, n, lane, acc, q, b.x[r], b.y[r], b.z[r], b.ux[r], b.uy[r], b.uz[r],
                                &b.tau[r]);
@@ -726,13 +726,73 @@ template <typename R, bool G, int FC>
 __device__ __forceinline__ bool species_pass(const StepArgs<R>& a, const StepScalars<R>& S, const R* lnh, const R* lnT,
                                              TileBuf<R>* buf, uint64_t* full, uint64_t* empty, uint32_t& k,
                                              uint32_t blk, uint32_t nblk, uint32_t T0, uint32_t T1, uint32_t ttot,
-                                             uint32_t n0, uint32_t n1, uint32_t n2, int lane, int warp, Acc<R>& acc,
-                                             EventQueue<R>& q) {
-  return species_tiles<R, G, FC, 0>(a, S, lnh, lnT, buf, full, empty, k, blk, nblk, 0u, T0, n0, lane, warp, acc, q) &&
-         species_tiles<R, G, FC, 1>(a, S, lnh, lnT, buf, full, empty, k, blk, nblk, T0, T0 + T1, n1, lane, warp, acc,
+                                             uint32_t n0, uint32_t n1, uint32_t n2, uint32_t win_n, int lane,
+                                             int warp, Acc<R>& acc, EventQueue<R>& q) {
+  return species_tiles<R, G, FC, 0>(a, S, lnh, lnT, buf, full, empty, k, blk, nblk, 0u, T0, 0u, n0, lane, warp, acc,
                                     q) &&
-         species_tiles<R, G, FC, 2>(a, S, lnh, lnT, buf, full, empty, k, blk, nblk, T0 + T1, ttot, n2, lane, warp, acc,
-                                    q);
+         species_tiles<R, G, FC, 1>(a, S, lnh, lnT, buf, full, empty, k, blk, nblk, T0, T0 + T1, 0u, n1, lane, warp,
+                                    acc, q) &&
+         species_tiles<R, G, FC, 2>(a, S, lnh, lnT, buf, full, empty, k, blk, nblk, T0 + T1, ttot, win_n, n2, lane,
+                                    warp, acc, q);
+}
+
+// The conversions that the photon window found for this step: the groups of 1024 photons whose
+// flag has the step's bit, one group per warp at a time (one mask word per lane).  Makes the step's
+// event-mask words and counts of the group and takes the events (photon_events), as if the photons
+// had been pushed by this step.  A converted photon waits with its step and its chi in the place of
+// its optical depth, at its position after the push.
+template <typename R>
+__device__ __forceinline__ void window_events(const StepArgs<R>& a, uint32_t phase, uint32_t win_n, uint32_t blk,
+                                              uint32_t nblk, int lane, int warp, EventQueue<R>& q) {
+  const SpeciesDev<R>& sp = a.sp[2];
+  const uint32_t groups = win_n >> 10, W = nblk * kWarps, me = blk * kWarps + warp;
+  const uint32_t bit = 1u << a.win_s;
+  for (uint32_t g0 = 0; g0 < groups; g0 += 32u * W) {
+    const uint32_t mine = g0 + (uint32_t)lane * W + me;  // neighbouring groups go to different warps
+    const uint32_t fl = mine < groups ? sp.wflag[mine] : 0u;
+    unsigned todo = __ballot_sync(kFull, (fl & bit) != 0u);
+    if ((fl & bit) && !(fl >> a.win_s >> 1)) sp.wflag[mine] = 0u;  // the group's last step with conversions
+    while (todo) {
+      const uint32_t g = g0 + (uint32_t)(__ffs(todo) - 1) * W + me;
+      todo &= todo - 1u;
+      const uint32_t w = g * 32u + (uint32_t)lane;
+      uint32_t m = 0;
+      for (uint32_t left = sp.cmask[w]; left; left &= left - 1u) {
+        const uint32_t b = (uint32_t)__ffs(left) - 1u;
+        if (Tau<R>::load(sp.tau + w * 32u + b).window_step() == a.win_s) m |= 1u << b;
+      }
+      sp.evmask[w] = m;
+      const uint32_t c = __reduce_add_sync(kFull, (uint32_t)__popc(m));
+      if (lane == 0) {
+        count_events(sp, phase, g * 32u, c);
+        atomicAdd(&sp.cnt->n_dead, c);
+      }
+      while (__any_sync(kFull, m != 0u)) {
+        const bool ev = m != 0u;
+        uint32_t i = 0;
+        R x = (R)0, y = (R)0, z = (R)0, k0 = (R)0, k1 = (R)0, k2 = (R)0, chi = (R)0;
+        if (ev) {
+          i = w * 32u + (uint32_t)__ffs(m) - 1u;
+          x = sp.x[i]; y = sp.y[i]; z = sp.z[i];
+          k0 = sp.ux[i]; k1 = sp.uy[i]; k2 = sp.uz[i];
+          chi = Tau<R>::load(sp.tau + i).window_chi();
+          m &= m - 1u;
+        }
+        enqueue_event<R>(q, __ballot_sync(kFull, ev), ev, lane, i, x, y, z, k0, k1, k2, chi);
+        __syncwarp();
+        if (q.count >= 32u) {
+          photon_events<R>(a, q.r, q.head, 32u);
+          q.head = (q.head + 32u) & (uint32_t)(kRing - 1);
+          q.count -= 32u;
+        }
+      }
+    }
+  }
+  if (q.count) {
+    photon_events<R>(a, q.r, q.head, q.count);
+    q.head = (q.head + q.count) & (uint32_t)(kRing - 1);
+    q.count = 0;
+  }
 }
 
 // The step over one scenario, run by block `blk` of the `nblk` blocks given to it: block blk
@@ -772,11 +832,12 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
   if (threadIdx.x == 0) make_scalars<R>(a.field, a.t0 + (double)a.step * a.dt, a.win_x0, a.win_v, S);
   pdl_wait();
   const uint32_t n0 = a.sp[0].cnt->n, n1 = a.sp[1].cnt->n, n2 = a.sp[2].cnt->n;
-  const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 + kTile - 1) / kTile;
+  const uint32_t win_n = sizeof(R) == 4 && a.win_s >= 0 ? a.sp[2].cnt->win_n : 0u;
+  const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 - win_n + kTile - 1) / kTile;
   const uint32_t ttot = T0 + T1 + T2;
   if (threadIdx.x < 3) S.phase[threadIdx.x] = (threadIdx.x == 0 ? a.sp[0] : (threadIdx.x == 1 ? a.sp[1] : a.sp[2])).cnt->phase;
   if (threadIdx.x == kBlock)
-    for (uint32_t k = 0; k < (uint32_t)kStages; ++k) issue_tile(a, buf, full, k, n0, n1, n2, blk, nblk);
+    for (uint32_t k = 0; k < (uint32_t)kStages; ++k) issue_tile(a, buf, full, k, n0, n1, n2, win_n, blk, nblk);
   __syncthreads();
   pdl_launch();
 
@@ -790,7 +851,7 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
         const int st = (int)(k % kStages);
         if (!mbar_wait_bounded(&empty[st], ((k / kStages) - 1u) & 1u, kWaitLimit)) { s_abort = 1; break; }
         fence_proxy_async_smem();  // the compute warps' accesses to this stage come first
-        issue_tile(a, buf, full, k, n0, n1, n2, blk, nblk);
+        issue_tile(a, buf, full, k, n0, n1, n2, win_n, blk, nblk);
       }
       if (s_abort) {
         // a wait gave up: report it, then wait (bounded) for the copies this block issued
@@ -805,19 +866,21 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
     EventQueue<R> q{ring + warp, 0u, 0u};
     if (lane == 0) q.r->sums = EventSums<R>{};
     __syncwarp();
+    if constexpr (sizeof(R) == 4)
+      if (win_n) window_events<R>(a, S.phase[2], win_n, blk, nblk, lane, warp, q);
     // one loop per species and field class: no per-tile dispatch (a grid-field instantiation
     // only ever sees the general class)
     uint32_t k = 0;
     bool ok;
     if (!G && S.kind == QED_FIELD_PLANE_LP)
       ok = species_pass<R, G, G ? kFieldAny : kFieldLP>(a, S, s_lnh, s_lnT, buf, full, empty, k, blk, nblk, T0, T1,
-                                                        ttot, n0, n1, n2, lane, warp, acc, q);
+                                                        ttot, n0, n1, n2, win_n, lane, warp, acc, q);
     else if (!G && S.kind == QED_FIELD_PLANE_CP)
       ok = species_pass<R, G, G ? kFieldAny : kFieldCP>(a, S, s_lnh, s_lnT, buf, full, empty, k, blk, nblk, T0, T1,
-                                                        ttot, n0, n1, n2, lane, warp, acc, q);
+                                                        ttot, n0, n1, n2, win_n, lane, warp, acc, q);
     else
       ok = species_pass<R, G, kFieldAny>(a, S, s_lnh, s_lnT, buf, full, empty, k, blk, nblk, T0, T1, ttot, n0, n1, n2,
-                                         lane, warp, acc, q);
+                                         win_n, lane, warp, acc, q);
     if (!ok) s_abort = 1;
     // a wait that gave up leaves the step unfinished (QED_ERR_TIMEOUT): events still in the
     // ring are not taken
@@ -1321,6 +1384,289 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const StepArgs<
       finish_counters(a, P, n);
     }
   }
+}
+
+// ----------------------------------------------------------------------------- photon windows
+// Photons depend on no other particle, and the only thing a step does with one is to convert it.  So
+// a run takes its photons several steps at a time: at the start of a window of K steps this kernel
+// advances every photon held (but for the last n mod 1024) by K steps in registers, with
+// photon_advance's own operations, and stops a photon at the step at which its optical depth runs
+// out; the K per-step kernels that follow push the leptons and the photons made since, and take the
+// conversions found for their step (window_events).  Particles, ids and order are those of the
+// per-step path: a conversion is taken at its step, and the merge ranks it by the photon's index.
+//
+// A step whose ledger can be read (the last of a run) belongs to no window: its sums are taken by
+// the per-step kernel over every photon, in its order.
+//
+// What it saves: the per-step kernel streams 44 B per photon and step and is issue-bound on the
+// bookkeeping around the field evaluation; here a photon is loaded and stored (52 B) once per K.
+// Issue-bound.  What it does about that:
+//  - What a photon keeps over the window (energy, drift velocity, the invariant's factor) is computed
+//    once; the plane wave's step-dependent phases and the T table's cells are read as pairs.
+//  - A photon whose chi stays below the table's start whatever the phase (chi_bound) has rate zero:
+//    it only drifts, as does one that stays outside the pulse.  Photon energies mix within every
+//    chunk, so the others (about half) go to a ring per warp and are stepped 32 at a time.
+//  - In a uniform field chi and the rate are constants of the photon.
+// Measured on GB300 (16 steps): 2e7 cascade photons 580 us, 36 us a step against 189 us on the
+// per-step kernel; 6e6 photons in a pulse 273 us, 17 us a step.  Whole runs: the collision of 1e6
+// electrons 367 -> 139 ms, the cascade's 50 steps 10.2 -> 4.2 ms.
+enum WindowClass { kWinLP = 0, kWinCP = 1, kWinRotating = 2, kWinUniform = 3, kWinGrid = 4 };
+
+struct WinRing {
+  uint32_t i[kRing];
+  float v[8][kRing];  // x, y, z, k, optical depth (hi, lo)
+};
+struct WinShared {
+  StepScalars<float> S[kWinMax];
+  float2 pair[kWinMax];  // per step: plane waves (phi_ref, phi_ref_mod); rotating E (E_x, E_y)
+  uint32_t pushed;
+  WinRing ring[kFuseThreads / 32];
+};
+
+// T(chi) as lookup_T, from cells (ln T_i, ln T_i+1)
+__device__ __forceinline__ float lookup_T_cells(const TabDev<float>& T, const float2* cell, float chi, int& oor) {
+  oor = 0;
+  if (!(chi >= T.chi_min)) return 0.0f;
+  if (chi > T.chi_max) { oor = 1; return T_above<float>(T, chi); }
+  int i, o; float w;
+  grid_pos(Num<float>::log_tab_(chi), T.ln_chi_min, T.inv_d_chi, T.n_chi, i, w, o);
+  const float2 c = cell[i];
+  return Num<float>::exp_tab_(Num<float>::fma_(w, c.y, (1.0f - w) * c.x));
+}
+
+// One photon of a window with its constants.
+template <int WC>
+struct WinPhoton {
+  float x, y, z, k[3], eps, ie, vx, vy, vz, hd;
+  Tau<float> tau;
+  __device__ __forceinline__ void constants(float wv) {
+    using N = Num<float>;
+    N::root_inv_(dot3<float>(k, k), eps, ie);
+    vx = N::fma_(k[0], ie, -wv); vy = k[1] * ie; vz = k[2] * ie;
+    if (WC == kWinLP || WC == kWinCP) {  // chi = hd |E| (chi_plane)
+      const float d = k[0] > 0.0f ? N::div_(N::fma_(k[1], k[1], k[2] * k[2]), eps + k[0]) : eps - k[0];
+      hd = 0.5f * d;
+    }
+  }
+  __device__ __forceinline__ void drift(float dt) {
+    using N = Num<float>;
+    x = N::fma_(dt, vx, x); y = N::fma_(dt, vy, y); z = N::fma_(dt, vz, z);
+  }
+  // a bound of chi over every phase, with room for the rounding of the phase functions
+  __device__ __forceinline__ float chi_bound(float E0) const {
+    return (WC == kWinRotating ? 0.5f * eps : hd) * fabsf(E0) * 1.0001f;
+  }
+};
+
+// Steps one photon per lane up to K steps; the step it converted at, or -1.
+template <bool G, int WC>
+__device__ __forceinline__ int window_steps(const StepArgs<float>& a, const WinShared& sh, const float2* cell, int K,
+                                            WinPhoton<WC>& p, float& chi) {
+  using N = Num<float>;
+  const float dt = a.dt_r;
+  const StepScalars<float>& S0 = sh.S[0];
+  const float om = S0.omega, len = S0.len, inv_len = S0.inv_len, E0 = S0.E0;
+  int k = 0;
+  for (; k < K; ++k) {
+    chi = 0.0f;
+    int oor;
+    if (WC == kWinLP || WC == kWinCP) {
+      // plane_at and chi_plane
+      const float2 ref = sh.pair[k];
+      float env = 1.0f;
+      bool in = true;
+      if (len > 0.0f) {
+        const float phi = N::fma_(-om, p.x, ref.x);
+        in = phi > 0.0f && phi < len;
+        const float sn = N::sin_env_((float)kPi * (phi * inv_len));
+        env = sn * sn;
+      }
+      const float amp0 = E0 * env;
+      float amp;
+      if (WC == kWinLP) {
+        float sn, cs;
+        N::carrier_(N::fma_(-om, p.x, ref.y), &sn, &cs);
+        amp = fabsf(amp0 * cs);
+      } else {
+        amp = amp0;
+      }
+      if (in) chi = p.hd * amp;
+    } else if (WC == kWinRotating) {
+      // chi_of with E = (E_x, E_y, 0), B = 0: the terms left out are exact zeros
+      const float2 E = sh.pair[k];
+      const float e0 = -(p.k[2] * E.y), e1 = p.k[2] * E.x, e2 = N::fma_(p.k[0], E.y, -(p.k[1] * E.x));
+      const float c2 = N::fma_(e0, e0, N::fma_(e1, e1, e2 * e2));
+      if (c2 > 0.0f) chi = 0.5f * N::sqrt_pos_(c2);
+    } else {
+      int fc;
+      chi = chi_at<float, G, kFieldAny>(sh.S[k], p.x, p.y, p.z, p.k, p.eps, fc);
+    }
+    if (chi > 0.0f) {
+      const float lam = (float)kAlpha * chi * p.ie * lookup_T_cells(a.tab, cell, chi, oor);
+      p.tau.sub(lam * dt);
+    }
+    p.drift(dt);
+    if (a.pairs && p.tau.used_up()) return k;
+  }
+  return -1;
+}
+
+// Writes one stepped photon back; a converted one waits for its step (window_events).
+template <int WC>
+__device__ __forceinline__ void window_store(const StepArgs<float>& a, uint32_t i, const WinPhoton<WC>& p,
+                                             const Tau<float>& tau0, int conv, float chi, int K, uint32_t& pushed) {
+  const SpeciesDev<float>& sp = a.sp[2];
+  sp.x[i] = p.x; sp.y[i] = p.y; sp.z[i] = p.z;
+  pushed += conv >= 0 ? (uint32_t)conv + 1u : (uint32_t)K;
+  if (conv >= 0) {
+    Tau<float>::window(conv, chi).store(sp.tau + i);
+    atomicOr(&sp.cmask[i >> 5], 1u << (i & 31u));
+    atomicOr(&sp.wflag[i >> 10], 1u << conv);
+  } else if (__float_as_int(p.tau.hi) != __float_as_int(tau0.hi) || __float_as_int(p.tau.lo) != __float_as_int(tau0.lo)) {
+    p.tau.store(sp.tau + i);
+  }
+}
+
+// Takes `take` (<= 32) photons from the warp's ring, one per lane.
+template <bool G, int WC>
+__device__ __forceinline__ void window_batch(const StepArgs<float>& a, const WinShared& sh, const WinRing& r,
+                                             const float2* cell, uint32_t head, uint32_t take, int K, uint32_t& pushed) {
+  const int lane = threadIdx.x & 31;
+  if ((uint32_t)lane < take) {
+    const uint32_t q = (head + (uint32_t)lane) & (uint32_t)(kRing - 1);
+    WinPhoton<WC> p;
+    p.x = r.v[0][q]; p.y = r.v[1][q]; p.z = r.v[2][q];
+    p.k[0] = r.v[3][q]; p.k[1] = r.v[4][q]; p.k[2] = r.v[5][q];
+    const Tau<float> tau0{r.v[6][q], r.v[7][q]};
+    p.tau = tau0;
+    p.constants(a.win_v_r);
+    float chi;
+    const int conv = window_steps<G, WC>(a, sh, cell, K, p, chi);
+    window_store<WC>(a, r.i[q], p, tau0, conv, chi, K, pushed);
+  }
+  __syncwarp();  // the ring slots read above may be refilled
+}
+
+template <bool G, int WC>
+__device__ __forceinline__ void window_body(const StepArgs<float>& a, int K, uint32_t blk, uint32_t nblk, WinShared& sh,
+                                            const float2* cell) {
+  const SpeciesDev<float>& sp = a.sp[2];
+  const uint32_t nwin = sp.cnt->n & ~1023u;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t nw = nblk * (kFuseThreads / 32), chunks = nwin >> 5;
+  const float dt = a.dt_r;
+  WinRing& ring = sh.ring[warp];
+  uint32_t head = 0, count = 0;  // warp-uniform
+  uint32_t pushed = 0;
+  uint32_t chunk = blk * (kFuseThreads / 32) + warp;
+  // the next chunk's state is loaded while the current one is stepped
+  PState<float> nxt{};
+  auto load = [&](uint32_t c) {
+    const uint32_t i = c * 32u + (uint32_t)lane;
+    nxt = {sp.x[i], sp.y[i], sp.z[i], sp.ux[i], sp.uy[i], sp.uz[i], sp.tau[i]};
+  };
+  if (chunk < chunks) load(chunk);
+  for (; chunk < chunks; chunk += nw) {
+    const PState<float> cur = nxt;
+    if (chunk + nw < chunks) load(chunk + nw);
+    const uint32_t i = chunk * 32u + (uint32_t)lane;
+    if (lane == 0) sp.cmask[chunk] = 0u;
+    __syncwarp();
+    WinPhoton<WC> p;
+    p.x = cur.x; p.y = cur.y; p.z = cur.z;
+    p.k[0] = cur.u0; p.k[1] = cur.u1; p.k[2] = cur.u2;
+    const Tau<float> tau0 = Tau<float>::from_stored(cur.tau);
+    p.tau = tau0;
+    const bool alive = !tau0.dead();
+    bool later = false;
+    if (alive) {
+      p.constants(a.win_v_r);
+      float chi = 0.0f;
+      int oor, conv = -1;
+      if (WC == kWinGrid) {
+        conv = window_steps<G, WC>(a, sh, cell, K, p, chi);
+      } else if (WC == kWinUniform) {
+        float amp = 0.0f, E[3], B[3];
+        const int fc = field_at<float, false>(sh.S[0], p.x, p.y, p.z, E, B, amp);
+        chi = chi_for<float>(fc, p.k, p.eps, E, B, amp);
+        float d = 0.0f;
+        if (chi > 0.0f) {
+          const float lam = (float)kAlpha * chi * p.ie * lookup_T_cells(a.tab, cell, chi, oor);
+          d = lam * dt;
+        }
+        for (int k = 0; k < K; ++k) {
+          if (chi > 0.0f) p.tau.sub(d);
+          p.drift(dt);
+          if (a.pairs && p.tau.used_up()) { conv = k; break; }
+        }
+      } else {
+        // (an optical depth that is used up already converts at the next step, field or not)
+        const bool used = tau0.used_up();
+        const bool none = !used && (WC == kWinLP || WC == kWinCP) && outside_pulse<float>(sh.S, K, p.x, p.vx, dt);
+        const bool soft = !used && p.chi_bound(sh.S[0].E0) < a.tab.chi_min;
+        if (soft && !none) p.tau.sub(0.0f);  // (the rate is zero: the value stays)
+        later = !none && !soft;
+        if (!later)
+          for (int k = 0; k < K; ++k) p.drift(dt);
+      }
+      if (!later) window_store<WC>(a, i, p, tau0, conv, chi, K, pushed);
+    }
+    if (WC != kWinGrid && WC != kWinUniform) {
+      const unsigned m = __ballot_sync(kFull, later);
+      if (later) {
+        const uint32_t q = (head + count + (uint32_t)__popc(m & ((1u << lane) - 1u))) & (uint32_t)(kRing - 1);
+        ring.i[q] = i;
+        ring.v[0][q] = cur.x; ring.v[1][q] = cur.y; ring.v[2][q] = cur.z;
+        ring.v[3][q] = cur.u0; ring.v[4][q] = cur.u1; ring.v[5][q] = cur.u2;
+        ring.v[6][q] = tau0.hi; ring.v[7][q] = tau0.lo;
+      }
+      count += (uint32_t)__popc(m);
+      __syncwarp();
+      const bool end = chunk + nw >= chunks;
+      while (count >= 32u || (end && count > 0u)) {
+        const uint32_t take = min(count, 32u);
+        window_batch<G, WC>(a, sh, ring, cell, head, take, K, pushed);
+        head = (head + take) & (uint32_t)(kRing - 1);
+        count -= take;
+      }
+    }
+  }
+  pushed = __reduce_add_sync(kFull, pushed);
+  if (lane == 0 && pushed) atomicAdd(&sh.pushed, pushed);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (sh.pushed) {
+      atomicAdd(&a.work[1], (unsigned long long)sh.pushed);
+      atomicAdd(&a.work[4], (unsigned long long)sh.pushed);
+    }
+    if (blk == 0) sp.cnt->win_n = nwin;
+  }
+}
+
+// Shared memory: WinShared, then the T table's cells (n_chi - 1 of them).
+inline size_t window_smem(int n_chi) { return sizeof(WinShared) + (size_t)n_chi * sizeof(float2); }
+
+template <bool G>
+__global__ void __launch_bounds__(kFuseThreads) window_kernel(const StepArgs<float> a, int K) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  WinShared& sh = *reinterpret_cast<WinShared*>(smem_raw);
+  float2* cell = reinterpret_cast<float2*>(smem_raw + sizeof(WinShared));
+  for (int k = threadIdx.x; k + 1 < a.tab.n_chi; k += blockDim.x) cell[k] = make_float2(a.tab.ln_T[k], a.tab.ln_T[k + 1]);
+  const int kind = a.field.kind;
+  if ((int)threadIdx.x < K) {
+    StepScalars<float>& S = sh.S[threadIdx.x];
+    make_scalars<float>(a.field, a.t0 + (double)(a.step + threadIdx.x) * a.dt, a.win_x0, a.win_v, S);
+    sh.pair[threadIdx.x] = kind == QED_FIELD_ROTATING_E ? make_float2(S.E[0], S.E[1]) : make_float2(S.phi_ref, S.phi_ref_mod);
+  }
+  if (threadIdx.x == 0) sh.pushed = 0;
+  pdl_wait();
+  __syncthreads();
+  pdl_launch();
+  if (G) window_body<G, kWinGrid>(a, K, blockIdx.x, gridDim.x, sh, cell);
+  else if (kind == QED_FIELD_PLANE_LP) window_body<G, kWinLP>(a, K, blockIdx.x, gridDim.x, sh, cell);
+  else if (kind == QED_FIELD_PLANE_CP) window_body<G, kWinCP>(a, K, blockIdx.x, gridDim.x, sh, cell);
+  else if (kind == QED_FIELD_ROTATING_E) window_body<G, kWinRotating>(a, K, blockIdx.x, gridDim.x, sh, cell);
+  else window_body<G, kWinUniform>(a, K, blockIdx.x, gridDim.x, sh, cell);
 }
 
 template <typename R>
@@ -2154,6 +2500,16 @@ int launch_fused(const StepArgs<R>& a, int K, bool commit, uint32_t* first_event
 }
 
 int fuse_max_steps() { return kMaxFuse; }
+
+void launch_window(const StepArgs<float>& a, int K, cudaStream_t s) {
+  const size_t smem = window_smem(a.tab.n_chi);
+  const auto k = a.field.kind == QED_FIELD_GRID ? window_kernel<true> : window_kernel<false>;
+  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int b = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, kFuseThreads, smem);
+  launch_pdl(k, sm_count() * std::max(b, 1), kFuseThreads, smem, s, a, K);
+  count_launch();
+}
 
 void launch_selftest_wait(uint32_t polls, uint32_t* bits, cudaStream_t s) {
   selftest_wait_kernel<<<1, 32, 0, s>>>(polls, bits);

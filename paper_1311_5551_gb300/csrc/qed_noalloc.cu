@@ -113,6 +113,7 @@ qed_status run_noalloc(const TablesDev& tv, const qed_soa* e, size_t n, const qe
   a.dt = p->dt; a.t0 = p->t0; a.win_x0 = p->window_x0; a.win_v = p->window_v;
   a.dt_r = (R)p->dt; a.win_v_r = (R)p->window_v;
   a.seed = p->seed; a.scenario = p->scenario; a.step = p->step;
+  a.win_s = -1;
   a.emit = 1; a.pairs = 0; a.drain = 1; a.recoil_energy = p->recoil_energy ? 1 : 0;
   a.ledger_part = reinterpret_cast<double*>(base + kOffLedger);
   a.ledger = a.ledger_part + kMaxGrid * kLedgerN;
