@@ -141,42 +141,99 @@ void set_tab_scalars(TabDev<R>& t, const TableHost& h) {
   t.T_at_chi_max = (R)std::exp(h.ln_T[p.n_chi - 1]);
 }
 
+// Guide of one row of n nodes for draws in [0, top]: entry b holds the first and the last bracket of
+// the draws in [b, b + 1] top/kGuide.  Bracket of v: the largest node j <= n - 2 with A[j] < v
+// (rising) or A[j] > v (falling), 0 if there is none.  A row that is not monotone has no such order:
+// all its entries span the row, which leaves the whole row to the binary search.
 template <typename R>
-void fill_image(std::vector<R>& img, const TableHost& h) {
-  img.clear();
-  auto put = [&](const std::vector<double>& v) { for (double x : v) img.push_back((R)x); };
-  put(h.ln_h); put(h.ln_T); put(h.P); put(h.Q); put(h.zeta_lo); put(h.zeta_hi); put(h.Pf);
+void guide_row(const R* A, int n, bool rising, double top, uint32_t* g) {
+  bool monotone = true;
+  for (int j = 0; j + 1 < n; ++j) monotone = monotone && (rising ? A[j] <= A[j + 1] : A[j] >= A[j + 1]);
+  if (!monotone) {
+    std::fill(g, g + kGuide, (uint32_t)(n - 2) << 16);
+    return;
+  }
+  auto bracket = [&](int edge) {
+    const R v = (R)(top * edge / kGuide);  // exact: kGuide and top are powers of two
+    int lo = 0, hi = n - 1;
+    while (hi - lo > 1) { const int mid = (lo + hi) / 2; if (rising ? A[mid] < v : A[mid] > v) lo = mid; else hi = mid; }
+    return (uint32_t)lo;
+  };
+  for (int b = 0; b < kGuide; ++b) {
+    const uint32_t u = bracket(b), v = bracket(b + 1);
+    g[b] = rising ? (u | v << 16) : (v | u << 16);
+  }
 }
 
+// The device image of the tables in precision R: values, then guides.
 template <typename R>
-void bind_image(TabDev<R>& t, const R* base, const TableHost& h) {
-  const R* p = base;
-  t.ln_h = p; p += h.ln_h.size();
-  t.ln_T = p; p += h.ln_T.size();
-  t.P = p; p += h.P.size();
-  t.Q = p; p += h.Q.size();
-  t.zeta_lo = p; p += h.zeta_lo.size();
-  t.zeta_hi = p; p += h.zeta_hi.size();
-  t.Pf = p;
-}
+struct TableImage {
+  std::vector<R> v;
+  std::vector<uint32_t> g;
+  size_t at_T, at_head, at_P2, at_Q2, at_F2, at_gQ, at_gF;
+
+  size_t begin() {  // sections start at multiples of four values (16 or 32 bytes)
+    while (v.size() % 4) v.push_back((R)0);
+    return v.size();
+  }
+  size_t pairs(const std::vector<double>& rows, int n) {
+    const size_t at = begin();
+    for (size_t k = 0; k < rows.size(); ++k) {
+      v.push_back((R)rows[k]);
+      v.push_back((R)rows[(int)(k % n) + 1 < n ? k + 1 : k]);
+    }
+    return at;
+  }
+  size_t guides(const std::vector<double>& rows, int n, bool rising, double top) {
+    const size_t at = g.size(), m = rows.size() / n;
+    g.resize(at + m * kGuide);
+    std::vector<R> row(n);
+    for (size_t r = 0; r < m; ++r) {
+      for (int j = 0; j < n; ++j) row[j] = (R)rows[r * n + j];
+      guide_row<R>(row.data(), n, rising, top, &g[at + r * kGuide]);
+    }
+    return at;
+  }
+  explicit TableImage(const TableHost& h) {
+    const int n = h.p.n_xi;
+    for (double x : h.ln_h) v.push_back((R)x);
+    at_T = begin();
+    for (double x : h.ln_T) v.push_back((R)x);
+    at_head = begin();
+    for (int i = 0; i < h.p.n_eta; ++i)
+      for (double x : {h.P[(size_t)i * n], h.Q[(size_t)(i + 1) * n - 1], h.zeta_lo[i], h.zeta_hi[i]}) v.push_back((R)x);
+    at_P2 = pairs(h.P, n);
+    at_Q2 = pairs(h.Q, n);
+    at_F2 = pairs(h.Pf, h.p.n_f);
+    guides(h.P, n, true, 0.5);
+    at_gQ = guides(h.Q, n, false, 0.5);
+    at_gF = guides(h.Pf, h.p.n_f, true, 1.0);
+  }
+  size_t value_bytes() const { return (v.size() * sizeof(R) + 255) & ~size_t(255); }
+  size_t bytes() const { return value_bytes() + ((g.size() * 4 + 255) & ~size_t(255)); }
+  cudaError_t upload(char* base, TabDev<R>& t, cudaStream_t s) const {
+    const R* p = reinterpret_cast<const R*>(base);
+    const uint32_t* q = reinterpret_cast<const uint32_t*>(base + value_bytes());
+    t.ln_h = p; t.ln_T = p + at_T; t.head = p + at_head;
+    t.P2 = p + at_P2; t.Q2 = p + at_Q2; t.F2 = p + at_F2;
+    t.gP = q; t.gQ = q + at_gQ; t.gF = q + at_gF;
+    cudaError_t e = cudaMemcpyAsync(base, v.data(), v.size() * sizeof(R), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return e;
+    return cudaMemcpyAsync(base + value_bytes(), g.data(), g.size() * 4, cudaMemcpyHostToDevice, s);
+  }
+};
 
 qed_status upload_tables(qed_tables* T, const qed_allocator* alloc, cudaStream_t s) {
   if (T->host.p.n_eta > 4096 || T->host.p.n_chi > 4096)
     return fail(QED_ERR_INVALID_ARG, "n_eta and n_chi must be <= 4096 (h and T are staged in shared memory)");
-  std::vector<double> i64;
-  std::vector<float> i32;
-  fill_image(i64, T->host);
-  fill_image(i32, T->host);
-  const size_t b64 = (i64.size() * 8 + 255) & ~size_t(255);
-  const size_t b32 = i32.size() * 4;
-  qed_status st = T->mem.get(b64 + b32, alloc, s);
+  const TableImage<double> i64(T->host);
+  const TableImage<float> i32(T->host);
+  qed_status st = T->mem.get(i64.bytes() + i32.bytes(), alloc, s);
   if (st != QED_OK) return st;
   char* base = static_cast<char*>(T->mem.ptr);
-  QED_CUDA(cudaMemcpyAsync(base, i64.data(), i64.size() * 8, cudaMemcpyHostToDevice, s));
-  QED_CUDA(cudaMemcpyAsync(base + b64, i32.data(), i32.size() * 4, cudaMemcpyHostToDevice, s));
+  QED_CUDA(i64.upload(base, T->d64, s));
+  QED_CUDA(i32.upload(base + i64.bytes(), T->d32, s));
   QED_CUDA(cudaStreamSynchronize(s));  // the host images are locals
-  bind_image(T->d64, reinterpret_cast<const double*>(base), T->host);
-  bind_image(T->d32, reinterpret_cast<const float*>(base + b64), T->host);
   set_tab_scalars(T->d64, T->host);
   set_tab_scalars(T->d32, T->host);
   return QED_OK;
@@ -907,6 +964,7 @@ struct qed_batch {
            *skip = nullptr, *span = nullptr, *tot = nullptr;
   SlotPlan* splan = nullptr;
   void* scal = nullptr;  // StepScalars<R>[S]
+  void* wscal = nullptr;  // StepScalars<float>[S * kWinMax] (mixed path)
   int target_blocks = 0, graph_steps = 32, max_parts = 0, fuse_k = 0;
   cudaGraphExec_t graph = nullptr;
   int graph_launches = 0;  // kernels in the captured graph
@@ -936,15 +994,30 @@ BatchCtl<R> batch_ctl(const qed_batch* b) {
   c.splan = b->splan;
   c.scal = b->scal;
   c.tot = b->tot;
+  c.wscal = b->wscal;
   c.tab = tab_of<R>(b->tables);
   return c;
 }
 
-// One batch step; want: the last of a call (or of a captured graph), whose ledgers can be read.
-void launch_batch(const qed_batch* b, bool want, cudaStream_t s) {
+// n batch steps, of which the last stands at `end` in its call.  The mixed path
+// takes the photons of all slots a window at a time (not beside multi-step passes, which move a slot
+// by more than one step per batch step).
+void launch_batch_steps(const qed_batch* b, int n, BatchEnd end, cudaStream_t s) {
   const TableHost& h = b->tables->host;
-  if (b->precision == QED_MIXED) launch_batch_step<float>(batch_ctl<float>(b), h.p.n_eta, h.p.n_chi, want, s);
-  else launch_batch_step<double>(batch_ctl<double>(b), h.p.n_eta, h.p.n_chi, want, s);
+  for (int k = 0; k < n;) {
+    const int W = std::min(kWinMax, n - k);
+    const BatchEnd win_end = k + W == n ? end : kBatchInside;
+    const bool window = b->precision == QED_MIXED && b->fuse_k == 0 && W >= 2;
+    if (window) launch_batch_window(batch_ctl<float>(b), h.p.n_chi, W, win_end, s);
+    for (int w = 0; w < W; ++w, ++k) {
+      const BatchEnd e = k + 1 == n ? end : kBatchInside;
+      const int win_s = window ? w : -1;
+      if (b->precision == QED_MIXED)
+        launch_batch_step<float>(batch_ctl<float>(b), h.p.n_eta, h.p.n_chi, e, W, win_end, win_s, s);
+      else
+        launch_batch_step<double>(batch_ctl<double>(b), h.p.n_eta, h.p.n_chi, e, W, win_end, win_s, s);
+    }
+  }
 }
 
 void set_slot_grid(qed_batch* b, int slot, bool grid) {
@@ -969,7 +1042,7 @@ qed_status ensure_graph(qed_batch* b) {
   const cudaStream_t s = b->own;
   QED_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
   const uint64_t l0 = launch_count_value();
-  for (int k = 0; k < b->graph_steps; ++k) launch_batch(b, k == b->graph_steps - 1, s);
+  launch_batch_steps(b, b->graph_steps, kBatchGroupEnd, s);
   b->graph_launches = (int)(launch_count_value() - l0);
   cudaError_t e = cudaStreamEndCapture(s, &g);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
@@ -1018,11 +1091,14 @@ extern "C" qed_status qed_batch_create(const qed_tables* T, qed_precision prec, 
   char* scal = nullptr;
   cv.add(&scal, step_scalars_bytes(prec) * S);
   cv.add(&b->tot, kBatchTotals);
+  char* wscal = nullptr;
+  if (prec == QED_MIXED) cv.add(&wscal, step_scalars_bytes(prec) * S * kWinMax);
   qed_status st = b->mem.get(cv.total(), alloc, s);
   if (st != QED_OK) { delete b; return st; }
   cv.bind(b->mem.ptr);
   b->args = args;
   b->scal = scal;
+  b->wscal = wscal;
   cudaError_t e = cudaMemsetAsync(b->mem.ptr, 0, cv.total(), s);
   if (e != cudaSuccess) { b->mem.release(); delete b; return cuda_fail(e, "cudaMemsetAsync"); }
   *out = b;
@@ -1073,14 +1149,21 @@ extern "C" qed_status qed_batch_run(qed_batch* b, uint64_t n_steps, void* stream
     if (st != QED_OK) return st;
     QED_CUDA(cudaEventRecord(b->ev_in, s));
     QED_CUDA(cudaStreamWaitEvent(b->own, b->ev_in, 0));
+    QED_CUDA(cudaMemsetAsync(b->tot + 1, 0, 4, b->own));
     for (; done + b->graph_steps <= n_steps; done += b->graph_steps) {
+      // the graph that ends with the call keeps the ledgers of its last step
+      if (done + b->graph_steps == n_steps) QED_CUDA(cudaMemsetAsync(b->tot + 1, 1, 4, b->own));
       QED_CUDA(cudaGraphLaunch(b->graph, b->own));
       count_launch(b->graph_launches);
     }
     QED_CUDA(cudaEventRecord(b->ev_out, b->own));
     QED_CUDA(cudaStreamWaitEvent(s, b->ev_out, 0));
   }
-  for (; done < n_steps; ++done) launch_batch(b, done + 1 == n_steps, s);
+  for (; done < n_steps;) {
+    const uint64_t m = std::min<uint64_t>(n_steps - done, 1u << 20);
+    launch_batch_steps(b, (int)m, done + m == n_steps ? kBatchCallEnd : kBatchInside, s);
+    done += m;
+  }
   QED_CUDA(cudaGetLastError());
   return QED_OK;
 }

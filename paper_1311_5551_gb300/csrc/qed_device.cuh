@@ -67,7 +67,7 @@ constexpr double kRatePhoton = kSqrt3 * kAlpha / kTwoPi;
 // ------------------------------------------------------------------ Philox4x64-10
 // Counter-based generator of Salmon, Moraes, Dror & Shaw (SC'11), 10 rounds.
 __device__ __forceinline__ void philox4x64(uint64_t c[4], uint64_t k0, uint64_t k1) {
-#pragma unroll
+#pragma unroll 1  // (events run this once per step and block: unrolled, it waits on instruction fetches)
   for (int r = 0; r < 10; ++r) {
     const uint64_t a0 = c[0], a2 = c[2];
     const uint64_t lo0 = 0xD2E7470EE14C6C93ull * a0, hi0 = __umul64hi(0xD2E7470EE14C6C93ull, a0);
@@ -512,75 +512,128 @@ __device__ __forceinline__ R lookup_T(const TabDev<R>& T, const R* lnT, R chi, i
   return Num<R>::exp_tab_(Num<R>::fma_(w, lnT[i + 1], ((R)1 - w) * lnT[i]));
 }
 
+// Node pairs (value, next value) of the inverse CDFs.
+template <typename R> struct Pair2;
+template <> struct Pair2<float> { using T = float2; };
+template <> struct Pair2<double> { using T = double2; };
 template <typename R>
-__device__ __forceinline__ R xi_node(const TabDev<R>& T, int r, int j) {
-  const R zlo = __ldg(T.zeta_lo + r), zhi = __ldg(T.zeta_hi + r);
-  const R z = zlo + (R)j * (zhi - zlo) / (R)(T.n_xi - 1);
-  return (R)1 / ((R)1 + Num<R>::exp_(-z));
+__device__ __forceinline__ typename Pair2<R>::T node_pair(const R* A, int j) {
+  return __ldg(reinterpret_cast<const typename Pair2<R>::T*>(A) + j);
 }
 
-// Invert one P_chi row: xi linear in P between the bracketing nodes; the complement Q is used
-// when U > 1/2 (the same interpolation, precise near P = 1).
+// Brackets of v in two rows of node pairs, A and A + 2 n, from their guide entries: the largest node
+// j <= n - 2 with value < v (rising rows) or > v (falling), between the guide's two; a binary search
+// where these differ.  The guide names one or two brackets for nearly every draw, so an event reads
+// 2 + 2 scattered words here, one after the other; searching the whole rows took 16 to 24, and every
+// lane of a warp reads other lines (see lepton_events for what it measured).
 template <typename R>
-__device__ R invert_xi_row(const TabDev<R>& T, int r, R U, R V) {
-  const int n = T.n_xi;
-  const R* P = T.P + (size_t)r * n;
-  const R* Q = T.Q + (size_t)r * n;
-  if (U <= __ldg(P)) return xi_node(T, r, 0);
-  if (V <= __ldg(Q + n - 1)) return xi_node(T, r, n - 1);
-  int lo = 0, hi = n - 1;
-  R frac;
-  if (U <= (R)0.5) {
-    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (__ldg(P + mid) < U) lo = mid; else hi = mid; }
-    const R p0 = __ldg(P + lo), p1 = __ldg(P + lo + 1);
-    frac = (U - p0) / (p1 - p0);
-  } else {
-    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (__ldg(Q + mid) > V) lo = mid; else hi = mid; }
-    const R q0 = __ldg(Q + lo), q1 = __ldg(Q + lo + 1);
-    frac = (q0 - V) / (q0 - q1);
+__device__ __forceinline__ void bracket2(const R* A, int n, bool rising, R v, uint32_t ga, uint32_t gb, int& ja, int& jb) {
+  const R* B = A + 2 * (size_t)n;
+  int ha = (int)(ga >> 16) + 1, hb = (int)(gb >> 16) + 1;
+  ja = (int)(ga & 0xffffu);
+  jb = (int)(gb & 0xffffu);
+  while (max(ha - ja, hb - jb) > 1) {
+    const int ma = (ja + ha) >> 1, mb = (jb + hb) >> 1;  // (a finished row's is its ja)
+    const R ta = __ldg(A + 2 * ma), tb = __ldg(B + 2 * mb);
+    if (ha - ja > 1) { if (rising ? ta < v : ta > v) ja = ma; else ha = ma; }
+    if (hb - jb > 1) { if (rising ? tb < v : tb > v) jb = mb; else hb = mb; }
   }
-  const R x0 = xi_node(T, r, lo), x1 = xi_node(T, r, lo + 1);
-  return x0 + frac * (x1 - x0);
 }
-
-// Photon energy fraction xi = 2chi/eta (Sec. 3); false when U is below the cut-off.
+// Guide entry of a draw v in [0, 1/scale].
 template <typename R>
-__device__ bool sample_xi(const TabDev<R>& T, R eta, R U, R V, R& xi) {
-  int i, o; R w;
-  grid_pos(Num<R>::log_(eta), T.ln_eta_min, T.inv_d_eta, T.n_eta, i, w, o);
-  const int n = T.n_xi;
-  const R pcut = ((R)1 - w) * __ldg(T.P + (size_t)i * n) + w * __ldg(T.P + (size_t)(i + 1) * n);
-  if (U < pcut) return false;
-  R x = ((R)1 - w) * invert_xi_row(T, i, U, V);
-  if (w > (R)0) x += w * invert_xi_row(T, i + 1, U, V);
-  if (o < 0) x *= eta / T.eta_min;  // classical scaling below the table
-  if (x > (R)1) x = (R)1;
-  xi = x;
+__device__ __forceinline__ int guide_bin(R v, R scale) { return min((int)(v * (scale * (R)kGuide)), kGuide - 1); }
+
+// Photon energy fraction xi = 2chi/eta (Sec. 3) by inverting the two bracketing P_chi rows: what
+// does not depend on the draw is loaded first (it overlaps the random numbers).
+template <typename R>
+struct XiSampler {
+  int i, o;
+  R w, p0[2], qn[2], zlo[2], zhi[2];
+
+  __device__ __forceinline__ void prepare(const TabDev<R>& T, R eta) {
+    grid_pos(Num<R>::log_(eta), T.ln_eta_min, T.inv_d_eta, T.n_eta, i, w, o);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const auto a = node_pair<R>(T.head, 2 * (i + r)), z = node_pair<R>(T.head, 2 * (i + r) + 1);
+      p0[r] = a.x; qn[r] = a.y;
+      zlo[r] = z.x; zhi[r] = z.y;
+    }
+  }
+  // false when U is below the cut-off (no photon)
+  __device__ __forceinline__ bool above_cut(R U) const { return !(U < ((R)1 - w) * p0[0] + w * p0[1]); }
+
+  // Both rows inverted and blended: xi linear in P between the bracketing nodes j, j + 1; the
+  // complement Q is used when U > 1/2 (the same interpolation, precise near P = 1).  (Loops over
+  // the rows and nodes, not unrolled: the event path is long, straight and mostly fetched anew.)
+  __device__ __forceinline__ R sample(const TabDev<R>& T, R eta, R U, R V) const {
+    const bool lower = U <= (R)0.5;
+    const int n = T.n_xi;
+    const R* A = (lower ? T.P2 : T.Q2) + 2 * (size_t)i * (size_t)n;
+    const R v = lower ? U : V;
+    const uint32_t* g = (lower ? T.gP : T.gQ) + (size_t)i * kGuide + guide_bin<R>(v, (R)2);
+    int j0, j1;
+    bracket2<R>(A, n, lower, v, __ldg(g), __ldg(g + kGuide), j0, j1);
+    const auto e0 = node_pair<R>(A, j0), e1 = node_pair<R>(A, n + j1);
+    R xr[2];
+#pragma unroll 1
+    for (int r = 0; r < 2; ++r) {
+      const R lo = r ? e1.x : e0.x, hi = r ? e1.y : e0.y;
+      const R pz = r ? p0[1] : p0[0], qz = r ? qn[1] : qn[0], zl = r ? zlo[1] : zlo[0], zh = r ? zhi[1] : zhi[0];
+      const bool lo0 = U <= pz, hi1 = !lo0 && V <= qz;
+      const int j = lo0 ? 0 : (hi1 ? n - 1 : (r ? j1 : j0));
+      R x01[2];
+#pragma unroll 1
+      for (int t = 0; t < 2; ++t) {
+        const R z = zl + (R)(j + t) * (zh - zl) / (R)(n - 1);
+        const R xx = (R)1 / ((R)1 + Num<R>::exp_(-z));
+        if (t == 0) x01[0] = xx; else x01[1] = xx;
+      }
+      const R frac = lower ? (U - lo) / (hi - lo) : (lo - V) / (lo - hi);
+      const R x = lo0 || hi1 ? x01[0] : x01[0] + frac * (x01[1] - x01[0]);
+      if (r == 0) xr[0] = x; else xr[1] = x;
+    }
+    R x = ((R)1 - w) * xr[0];
+    if (w > (R)0) x += w * xr[1];
+    if (o < 0) x *= eta / T.eta_min;  // classical scaling below the table
+    if (x > (R)1) x = (R)1;
+    return x;
+  }
+};
+
+// xi for (eta, U); false when U is below the cut-off.
+template <typename R>
+__device__ __forceinline__ bool sample_xi(const TabDev<R>& T, R eta, R U, R V, R& xi) {
+  XiSampler<R> s;
+  s.prepare(T, eta);
+  if (!s.above_cut(U)) return false;
+  xi = s.sample(T, eta, U, V);
   return true;
-}
-
-template <typename R>
-__device__ R invert_f_row(const TabDev<R>& T, int r, R V) {
-  const int n = T.n_f;
-  const R* P = T.Pf + (size_t)r * n;
-  int lo = 0, hi = n - 1;
-  while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (__ldg(P + mid) < V) lo = mid; else hi = mid; }
-  const R p0 = __ldg(P + lo), p1 = __ldg(P + lo + 1);
-  const R frac = (V - p0) / (p1 - p0);
-  const R f0 = (R)0.5 * (R)lo / (R)(n - 1), f1 = (R)0.5 * (R)(lo + 1) / (R)(n - 1);
-  return f0 + frac * (f1 - f0);
 }
 
 // Positron energy fraction f (Sec. 3, App. B): U < 1/2 maps to f <= 1/2 through V = 2U,
 // U >= 1/2 to f >= 1/2 through V = 2(1 - U).
 template <typename R>
-__device__ R sample_f(const TabDev<R>& T, R chi, R U, R Vc) {
+__device__ __forceinline__ R sample_f(const TabDev<R>& T, R chi, R U, R Vc) {
   int i, o; R w;
   grid_pos(Num<R>::log_(chi), T.ln_chi_min, T.inv_d_chi, T.n_chi, i, w, o);
   const bool lower = U < (R)0.5;
   const R V = lower ? (R)2 * U : (R)2 * Vc;
-  R fh = ((R)1 - w) * invert_f_row(T, i, V);
-  if (w > (R)0) fh += w * invert_f_row(T, i + 1, V);
+  const int n = T.n_f;
+  const R* P = T.F2 + 2 * (size_t)i * (size_t)n;
+  const uint32_t* g = T.gF + (size_t)i * kGuide + guide_bin<R>(V, (R)1);
+  int j[2];
+  bracket2<R>(P, n, true, V, __ldg(g), __ldg(g + kGuide), j[0], j[1]);
+  R fr[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int lo = j[r];
+    const auto e = node_pair<R>(P, r * n + lo);
+    const R frac = (V - e.x) / (e.y - e.x);
+    const R f0 = (R)0.5 * (R)lo / (R)(n - 1), f1 = (R)0.5 * (R)(lo + 1) / (R)(n - 1);
+    fr[r] = f0 + frac * (f1 - f0);
+  }
+  R fh = ((R)1 - w) * fr[0];
+  if (w > (R)0) fh += w * fr[1];
   return lower ? fh : (R)1 - fh;
 }
 

@@ -30,15 +30,21 @@ template <typename R>
 struct TabDev {
   const R* ln_h;     // [n_eta]
   const R* ln_T;     // [n_chi]
-  const R* P;        // [n_eta * n_xi]
-  const R* Q;        // [n_eta * n_xi]
-  const R* zeta_lo;  // [n_eta]
-  const R* zeta_hi;  // [n_eta]
-  const R* Pf;       // [n_chi * n_f]
+  // the inverse CDFs as an event reads them: one 16- or 32-byte head per eta row, the nodes in pairs
+  // (value, next value), and per row a guide (kGuide entries) from the draw to its bracket
+  const R* head;     // [n_eta * 4]  P_chi's first node, 1 - P_chi's last, zeta_lo, zeta_hi
+  const R* P2;       // [n_eta * n_xi * 2]
+  const R* Q2;       // [n_eta * n_xi * 2]
+  const R* F2;       // [n_chi * n_f * 2]
+  const uint32_t* gP;  // [n_eta * kGuide]  draws U in [0, 1/2]
+  const uint32_t* gQ;  // [n_eta * kGuide]  draws 1 - U in [0, 1/2]
+  const uint32_t* gF;  // [n_chi * kGuide]  draws V in [0, 1]
   int n_eta, n_xi, n_chi, n_f;
   R ln_eta_min, inv_d_eta, eta_min;
   R ln_chi_min, inv_d_chi, chi_min, chi_max, T_at_chi_max;
 };
+
+constexpr int kGuide = 256;  // guide entries per row: first bracket | last bracket << 16 of an equal share of the draws
 
 // Per-species counters in device memory.
 struct DevCounters {
@@ -149,14 +155,20 @@ struct StepArgs {
 // What one batch step does with a slot, written by the tile schedule at the start of the step:
 // the slot's 256-particle tiles occupy [tile_base, tile_base + T[0] + T[1] + T[2]) of the batch
 // step's tile space (species in order e-, e+, photons); n are the particles held (the step's
-// parents).
+// parents).  Inside a photon window the photon tiles start at photon win_n, and T[3] tiles without
+// particles follow, which share the conversions that the window found.
 struct SlotPlan {
   uint32_t live;
   uint32_t tile_base;
-  uint32_t T[3];
+  uint32_t T[4];
   uint32_t n[3];
+  uint32_t win_n;
 };
-constexpr int kBatchTotals = 4;  // [tiles, spare]
+constexpr int kBatchTotals = 4;  // [tiles, the group of steps under way is the call's last, spare]
+
+// Place of a batch step, or of the end of a photon window, in its call: inside; the last of a group
+// of steps (a captured graph), which tot[1] says is the call's last or not; the last of its call.
+enum BatchEnd { kBatchInside = 0, kBatchGroupEnd = 1, kBatchCallEnd = 2 };
 
 // Many independent scenarios ("slots") stepped together: per-slot arguments live in device
 // memory.  The per-step path puts the tiles of all live slots in one tile space that a
@@ -171,6 +183,7 @@ struct BatchCtl {
   SlotPlan* splan;       // [S] tile and range layout of the current batch step
   void* scal;            // [S] per-slot field scalars of the current step (StepScalars<R>)
   uint32_t* tot;         // [kBatchTotals] sizes of the current batch step's spaces
+  void* wscal;           // [S * kWinMax] field scalars of the current photon window's steps (mixed path)
   TabDev<R> tab;         // the batch's tables (shared by every slot)
   int S;                 // slots
   int target_blocks;     // step-kernel grid (blocks striding through the tile space)
@@ -186,7 +199,12 @@ struct BatchCtl {
 template <typename R>
 void launch_step(const StepArgs<R>& a, int grid, int block, size_t smem, cudaStream_t s);
 template <typename R>
-void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, bool want, cudaStream_t s);
+void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, BatchEnd end, int win_w, BatchEnd win_end, int win_s,
+                       cudaStream_t s);
+// A photon window of up to W steps in every slot (see window_kernel); the W batch steps that follow
+// are launched with win_w = W, win_end = end and win_s = 0 .. W - 1.  The call's last step belongs to
+// no window: a window that ends with it is one step shorter.
+void launch_batch_window(const BatchCtl<float>& c, int n_chi, int W, BatchEnd end, cudaStream_t s);
 size_t step_scalars_bytes(int precision);
 // Advances the photons held, but for the last n mod 1024, by K <= kWinMax steps from a.step on (see
 // window_kernel).

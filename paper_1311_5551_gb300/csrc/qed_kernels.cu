@@ -65,7 +65,7 @@ struct Acc {
   KSum<R> emit_e, emit_def, pair_e, pair_def;
   uint32_t n[3] = {0, 0, 0};
   uint32_t oor_eta = 0, oor_chi = 0;
-  uint32_t pushed_ph = 0, tau_ph = 0;  // photons pushed; those in a field (optical depth stored)
+  uint32_t pushed_ph = 0;  // photons pushed
   uint32_t emit_n = 0, drop = 0, pair_n = 0;
 };
 
@@ -142,18 +142,28 @@ __device__ __forceinline__ R lepton_advance(const StepScalars<R>& S, const TabDe
 // appends) is long next to the rest of a particle's step, and rare: a few per warp per step even
 // at the peak of a collision.  Taken where it is found, each warp with an event would run that
 // path with one lane active.  Instead every warp writes its events into a ring in shared memory
-// and takes them 32 at a time, all lanes busy: whenever 32 are waiting, before its next tile is
-// of another species, and after its last tile.  An event depends only on its particle's state
+// and takes them 32 at a time, all lanes busy, whenever 32 are waiting; what is left in the block's
+// rings after its last tile of a species is taken together, 32 per warp (drain_block: the few
+// events of eight warps fill one batch, where each warp ran the path for its own).  An event depends only on its particle's state
 // after the push (and its id and weight), so the particles get the same bits as if each event
 // were taken where it was found; only the order in which the ledger sums are accumulated changes.
 constexpr int kRing = 64;  // entries per warp: fewer than 32 waiting plus at most 32 from a chunk
 
-// The ledger sums that events add to, kept per warp beside its ring (out of the registers of
-// the hot loop) and folded into the block's ledger partial at the end.
+// A warp's ledger sums, kept beside its ring (out of the registers of the hot loop) and folded into
+// the block's ledger partial at the end.
 template <typename R>
 struct EventSums {
   KSum<R> e[3], emit_e, emit_def, pair_e, pair_def;
-  uint32_t n[3], emit_n, drop, pair_n;
+  uint32_t n[3], emit_n, drop, pair_n, oor_eta, oor_chi;
+};
+
+// A lane's ledger sums over the particles of one run of tiles (one species); folded into the warp's
+// sums after it.  The step kernels keep them only where the ledger can be read, in tile loops of
+// their own (WANT): the others have the registers.
+template <typename R>
+struct RunSums {
+  KSum<R> e;
+  uint32_t n = 0, oor = 0;
 };
 
 template <typename R>
@@ -161,6 +171,7 @@ struct __align__(16) EventRing {
   uint32_t i[kRing];  // particle index
   R v[7][kRing];      // x, y, z after the push; u after the push (photons: k); eta (photons: chi)
   EventSums<R> sums;
+  uint32_t head, count;  // of the warp's queue, where other warps read it (drain_block)
 };
 
 // Compensated warp sum of one value per lane (fixed shuffle order); lane 0 holds the result.
@@ -211,9 +222,9 @@ __device__ __forceinline__ void count_events(const SpeciesDev<R>& sp, uint32_t p
 // optical depth ran out goes to the warp's event ring; its momentum and optical depth are
 // stored when the event is taken.  The chunk's event mask counts every event as a child here;
 // an emission that yields no photon (below the energy cut) takes its bit back then.
-template <typename R, bool G, int FC>
-__device__ __forceinline__ void lepton_chunk(const StepArgs<R>& a, const StepScalars<R>& S, const R* lnh, int kind,
-                                             uint32_t chunk, uint32_t n, int lane, Acc<R>& acc, EventQueue<R>& q,
+template <typename R, bool G, int FC, int kind, bool WANT>
+__device__ __forceinline__ void lepton_chunk(const StepArgs<R>& a, const StepScalars<R>& S, const R* lnh,
+                                             uint32_t chunk, uint32_t n, int lane, RunSums<R>& sums, EventQueue<R>& q,
                                              R x, R y, R z, R v0, R v1, R v2, const double* tau_src) {
   const SpeciesDev<R>& sp = a.sp[kind];
   const uint32_t i = chunk * 32u + (uint32_t)lane;
@@ -240,28 +251,32 @@ __device__ __forceinline__ void lepton_chunk(const StepArgs<R>& a, const StepSca
       sp.ux[i] = u[0]; sp.uy[i] = u[1]; sp.uz[i] = u[2];
       tau.store(sp.tau + i);
     }
-    // the ledger's sums only where somebody can read them (the last step of a run)
-    if (a.want) {
-      if (oor > 0) acc.oor_eta++;
-      if (!ev) { acc.e[kind].add(gam); acc.n[kind]++; }
+    if (WANT) {
+      if (oor > 0) sums.oor++;
+      if (!ev) { sums.e.add(gam); sums.n++; }
     }
   }
 }
 
-// Takes `take` (<= 32) events from the ring, starting at `head`, one per lane: photon emission
+// Takes `take` (<= 32) events, one per lane (lane l: entry p of ring `src`): photon emission
 // by an e+- (Sec. 3): photon energy from the inverse CDF of P_chi, recoil, fresh optical depths
 // for the emitter and the photon, the photon appended to the photon species' append region.
-// Inlined into the tile loop: as a call, the ABI's saved registers and the spills around the
-// call sites cost the loop more (on GB300, 3 blocks of 288 threads per SM) than the inlined
-// code's registers do.
-template <typename R, int KIND>
-__device__ __forceinline__ void lepton_events(const StepArgs<R>& a, uint32_t phase, EventRing<R>* ring, uint32_t head,
-                                              uint32_t take) {
-  const SpeciesDev<R>& sp = a.sp[KIND];
+// A chain of dependent loads and special functions, with scattered table reads: its latency counts
+// in small runs, its loads in large ones.  The loads that need no random number come first, the append
+// slots are asked for before the energies are searched, both table rows are searched at once and
+// from a guide (bracket2), and the block's events share batches.  On GB300 200 steps of 1e3
+// electrons went from 3.69 to 3.01 ms (searched in whole rows: 3.35), 100 steps of 1e4 on the FP64
+// path, where every batch costs the slow pipe, from 5.77 to 4.20, a step of 1e6 electrons in a pulse
+// from 50.8 to 45.5 us (guide alone).
+// Inlined, once per kernel for either lepton: as a call, the ABI's saved registers and the spills
+// around the call site cost the loop more (on GB300, 3 blocks of 288 threads per SM).
+template <typename R, bool WANT>
+__device__ __forceinline__ void lepton_events(const StepArgs<R>& a, uint32_t phase, int kind, const EventRing<R>* ring,
+                                              uint32_t p, uint32_t take, EventSums<R>& es) {
+  const SpeciesDev<R>& sp = a.sp[kind];
   const SpeciesDev<R>& dst = a.sp[2];  // photon children are appended to the photon species
   const int lane = threadIdx.x & 31;
   const bool ev = (uint32_t)lane < take;
-  const uint32_t p = (head + (uint32_t)lane) & (uint32_t)(kRing - 1);
   uint32_t i = 0;
   R x = (R)0, y = (R)0, z = (R)0, u[3] = {(R)0, (R)0, (R)0}, eta = (R)0;
   if (ev) {
@@ -277,11 +292,24 @@ __device__ __forceinline__ void lepton_events(const StepArgs<R>& a, uint32_t pha
   bool child = false;
   R kx = (R)0, ky = (R)0, kz = (R)0, emitted = (R)0, def = (R)0;
   Tau<R> tau = Tau<R>::one(), ctau = Tau<R>::one();
+  // whether there is a photon is known before its energy: the append slots are asked for first, and
+  // their answer comes while the energies are searched
+  XiSampler<R> xs;
+  Uniform<R> U[4];
   if (ev) {
-    Uniform<R> U[4];
-    draw4r<R>(a.seed, a.scenario, sp.id[i], a.step, (uint64_t)KIND, 0, U);
-    R xi;
-    if (sample_xi<R>(a.tab, eta, U[0].u, U[0].v, xi)) {
+    const uint32_t id = sp.id[i];
+    xs.prepare(a.tab, eta);
+    draw4r<R>(a.seed, a.scenario, id, a.step, (uint64_t)kind, 0, U);
+    child = xs.above_cut(U[0].u);
+  }
+  const unsigned childm = __ballot_sync(kFull, child);
+  const uint32_t nc = (uint32_t)__popc(childm);
+  const int leader = __ffs(childm) - 1;
+  uint32_t base = 0;
+  if (lane == leader) base = atomicAdd(&dst.cnt->n_app, nc);
+  if (ev) {
+    if (child) {
+      const R xi = xs.sample(a.tab, eta, U[0].u, U[0].v);
       const R eps = xi * gam;
       const R um = Num<R>::sqrt_(u2);
       const R ium = (R)1 / um;
@@ -300,7 +328,6 @@ __device__ __forceinline__ void lepton_events(const StepArgs<R>& a, uint32_t pha
       emitted = eps;
       gam = gf;
       ctau = Tau<R>::fresh(-Num<R>::log_(U[2].u));
-      child = true;
     } else {
       // no photon: the event is not a child after all
       atomicAnd(&sp.evmask[i >> 5], ~(1u << (i & 31u)));
@@ -308,25 +335,19 @@ __device__ __forceinline__ void lepton_events(const StepArgs<R>& a, uint32_t pha
     }
     tau = Tau<R>::fresh(-Num<R>::log_(U[1].u));
   }
-  const unsigned childm = __ballot_sync(kFull, child);
-  const uint32_t nc = (uint32_t)__popc(childm);
-  if (a.want) {
+  if (WANT) {
     const KSum<R> se = warp_ksum<R>(emitted), sd = warp_ksum<R>(def), sg = warp_ksum<R>(ev ? gam : (R)0);
     if (lane == 0) {
-      EventSums<R>& es = ring->sums;
       es.emit_e.merge(se);
       es.emit_def.merge(sd);
       es.emit_n += nc;
       es.drop += take - nc;
-      es.e[KIND].merge(sg);
-      es.n[KIND] += take;
+      es.e[kind].merge(sg);
+      es.n[kind] += take;
       if (!a.drain) { es.e[2].merge(se); es.n[2] += nc; }
     }
   }
   if (childm) {
-    const int leader = __ffs(childm) - 1;
-    uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(&dst.cnt->n_app, nc);
     base = __shfl_sync(kFull, base, leader);
     if (child) {
       const uint32_t slot = base + (uint32_t)__popc(childm & ((1u << lane) - 1u));
@@ -334,7 +355,7 @@ __device__ __forceinline__ void lepton_events(const StepArgs<R>& a, uint32_t pha
         dst.ax[slot] = x; dst.ay[slot] = y; dst.az[slot] = z;
         dst.aux[slot] = kx; dst.auy[slot] = ky; dst.auz[slot] = kz;
         ctau.store(dst.atau + slot);
-        dst.aparent[slot] = i | ((uint32_t)KIND << 31);
+        dst.aparent[slot] = i | ((uint32_t)kind << 31);
         if (dst.aw) dst.aw[slot] = sp.w ? sp.w[i] : (R)1;  // the photon stands for as many
       } else {
         atomicOr(&dst.cnt->err, 1u << QED_ERR_CAPACITY);
@@ -369,9 +390,10 @@ __device__ __forceinline__ R photon_advance(const StepScalars<R>& S, const TabDe
   return chi;
 }
 
-template <typename R, bool G, int FC>
+template <typename R, bool G, int FC, bool WANT>
 __device__ __forceinline__ void photon_chunk(const StepArgs<R>& a, const StepScalars<R>& S, const R* lnT,
-                                             uint32_t chunk, uint32_t n, int lane, Acc<R>& acc, EventQueue<R>& q,
+                                             uint32_t chunk, uint32_t n, int lane, RunSums<R>& sums, uint32_t& pushed_ph,
+                                             uint32_t& tau_ph, EventQueue<R>& q,
                                              R x, R y, R z, R k0, R k1, R k2, const double* tau_src) {
   const SpeciesDev<R>& sp = a.sp[2];
   const uint32_t i = chunk * 32u + (uint32_t)lane;
@@ -383,10 +405,10 @@ __device__ __forceinline__ void photon_chunk(const StepArgs<R>& a, const StepSca
   R eps, ie;
   int oor;
   const R chi = photon_advance<R, G, FC>(S, a.tab, lnT, a.dt_r, a.win_v_r, x, y, z, k, tau, eps, ie, oor);
-  if (alive) acc.pushed_ph++;
+  if (alive) pushed_ph++;
   // a photon outside any field keeps its optical depth: only its position is stored
   const bool tau_moves = alive && chi > (R)0;
-  if (tau_moves) acc.tau_ph++;
+  if (tau_moves) tau_ph++;
 
   // a photon whose optical depth ran out always converts: its pair is counted here
   const bool ev = alive && a.pairs && tau.used_up();
@@ -403,24 +425,24 @@ __device__ __forceinline__ void photon_chunk(const StepArgs<R>& a, const StepSca
   if (alive) {
     sp.x[i] = x; sp.y[i] = y; sp.z[i] = z;  // k is unchanged between events
     if (!ev && tau_moves) tau.store(sp.tau + i);
-    if (a.want) {
-      if (oor > 0) acc.oor_chi++;
-      if (!ev) { acc.e[2].add(eps); acc.n[2]++; }
+    if (WANT) {
+      if (oor > 0) sums.oor++;
+      if (!ev) { sums.e.add(eps); sums.n++; }
     }
   }
 }
 
-// Takes `take` (<= 32) events from the ring, starting at `head`, one per lane: pair creation
+// Takes `take` (<= 32) events, one per lane (lane l: entry p of ring `src`): pair creation
 // by a photon (Sec. 3): the energy split from the inverse CDF of P_f, the electron and the
 // positron along k with fresh optical depths, appended to their species' append regions; the
 // photon is annihilated (its optical depth becomes +inf, a hole until compaction).  Inlined
 // for the same reason as lepton_events.
-template <typename R>
-__device__ __forceinline__ void photon_events(const StepArgs<R>& a, EventRing<R>* ring, uint32_t head, uint32_t take) {
+template <typename R, bool WANT>
+__device__ __forceinline__ void photon_events(const StepArgs<R>& a, const EventRing<R>* ring, uint32_t p, uint32_t take,
+                                              EventSums<R>& es) {
   const SpeciesDev<R>& sp = a.sp[2];
   const int lane = threadIdx.x & 31;
   const bool ev = (uint32_t)lane < take;
-  const uint32_t p = (head + (uint32_t)lane) & (uint32_t)(kRing - 1);
   uint32_t i = 0;
   R x = (R)0, y = (R)0, z = (R)0, k[3] = {(R)0, (R)0, (R)1}, chi = (R)0;
   if (ev) {
@@ -435,6 +457,11 @@ __device__ __forceinline__ void photon_events(const StepArgs<R>& a, EventRing<R>
   R ue[3] = {(R)0, (R)0, (R)0}, up[3] = {(R)0, (R)0, (R)0};
   R converted = (R)0, def = (R)0, gm = (R)0, gp = (R)0;
   Tau<R> te = Tau<R>::one(), tp = Tau<R>::one();
+  uint32_t be = 0, bp = 0;  // append slots, asked for first
+  if (lane == 0) {
+    be = atomicAdd(&a.sp[0].cnt->n_app, take);
+    bp = atomicAdd(&a.sp[1].cnt->n_app, take);
+  }
   if (ev) {
     Uniform<R> U[4];
     draw4r<R>(a.seed, a.scenario, sp.id[i], a.step, (uint64_t)QED_PHOTON, 0, U);
@@ -457,12 +484,10 @@ __device__ __forceinline__ void photon_events(const StepArgs<R>& a, EventRing<R>
     te = Tau<R>::fresh(-Num<R>::log_(U[1].u));
     tp = Tau<R>::fresh(-Num<R>::log_(U[2].u));
   }
-  const unsigned evm = __ballot_sync(kFull, ev);
-  if (a.want) {
+  if (WANT) {
     const KSum<R> se = warp_ksum<R>(converted), sd = warp_ksum<R>(def);
     const KSum<R> s0 = warp_ksum<R>(gm), s1 = warp_ksum<R>(gp);
     if (lane == 0) {
-      EventSums<R>& es = ring->sums;
       es.pair_e.merge(se);
       es.pair_def.merge(sd);
       es.pair_n += take;
@@ -470,14 +495,8 @@ __device__ __forceinline__ void photon_events(const StepArgs<R>& a, EventRing<R>
       es.e[1].merge(s1); es.n[1] += take;
     }
   }
-  const int leader = __ffs(evm) - 1;
-  uint32_t be = 0, bp = 0;
-  if (lane == leader) {
-    be = atomicAdd(&a.sp[0].cnt->n_app, take);
-    bp = atomicAdd(&a.sp[1].cnt->n_app, take);
-  }
-  be = __shfl_sync(kFull, be, leader);
-  bp = __shfl_sync(kFull, bp, leader);
+  be = __shfl_sync(kFull, be, 0);
+  bp = __shfl_sync(kFull, bp, 0);
   if (ev) {
     const uint32_t r = (uint32_t)lane;  // the events fill lanes 0 .. take-1
     const SpeciesDev<R>& de = a.sp[0];
@@ -524,6 +543,9 @@ struct TileBuf;
 #ifndef QED_STEP_MIN_BLOCKS
 #define QED_STEP_MIN_BLOCKS 3
 #endif
+#ifndef QED_BATCH_MIN_BLOCKS
+#define QED_BATCH_MIN_BLOCKS 3
+#endif
 constexpr int kStages = QED_STAGES;  // tile copies in flight per block
 constexpr uint32_t kWaitLimit = 1u << 16;  // mbarrier polls (<= 20 us each) before a copy is declared lost
 
@@ -533,6 +555,9 @@ struct TileBuf {
   double tau[kTile];
 };
 
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ uint32_t floor16(uint32_t b) { return b & ~15u; }
 
 // Tile t of the step (over the concatenated species) -> species and tile index in it.
@@ -542,8 +567,7 @@ __device__ __forceinline__ void decode_tile(uint32_t t, uint32_t T0, uint32_t T1
   else { s = 2; j = t - T0 - T1; }
 }
 
-// Source arrays of species s, selected with constant indices (no dynamic indexing of the
-// kernel parameters, which would copy them to local memory).
+// Source arrays of a species.
 template <typename R>
 struct TileSrc {
   const R *x, *y, *z, *ux, *uy, *uz;
@@ -554,16 +578,26 @@ __device__ __forceinline__ TileSrc<R> tile_src(const SpeciesDev<R>& p) {
   return {p.x, p.y, p.z, p.ux, p.uy, p.uz, p.tau};
 }
 
+// Tiles of a photon window's conversions, each a share of its groups of 1024 photons: about two
+// groups per warp, and at most one tile per block.
+__device__ __forceinline__ uint32_t conversion_tiles(uint32_t win_n, uint32_t nblk) {
+  return min(nblk, ((win_n >> 10) + 15u) / 16u);
+}
+
 // Thread 0 issues the bulk copies of the block's k-th tile into stage k % kStages.
 template <typename R>
 __device__ __forceinline__ void issue_tile(const StepArgs<R>& a, TileBuf<R>* buf, uint64_t* bar, uint32_t k, uint32_t n0,
                                         uint32_t n1, uint32_t n2, uint32_t win_n, uint32_t blk, uint32_t nblk) {
   const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 - win_n + kTile - 1) / kTile;
   const uint32_t t = blk + k * nblk;
-  if (t >= T0 + T1 + T2) return;
+  if (t >= T0 + T1 + T2) {
+    // a tile of a photon window's conversions: nothing to copy
+    if (t < T0 + T1 + T2 + conversion_tiles(win_n, nblk)) mbar_arrive(&bar[k % kStages]);
+    return;
+  }
   int s; uint32_t j;
   decode_tile(t, T0, T1, s, j);
-  const TileSrc<R> src = s == 0 ? tile_src(a.sp[0]) : (s == 1 ? tile_src(a.sp[1]) : tile_src(a.sp[2]));
+  const TileSrc<R> src = tile_src(a.sp[s]);
   const uint32_t ns = s == 0 ? n0 : (s == 1 ? n1 : n2);
   const uint32_t first = (s == 2 ? win_n : 0u) + j * kTile;
   const uint32_t valid = min((uint32_t)kTile, ns - first);
@@ -585,20 +619,15 @@ __device__ __forceinline__ void issue_tile(const StepArgs<R>& a, TileBuf<R>* buf
   if (bt) bulk_load(b.tau, src.tau + first, bt, bb);
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 // barrier among the compute warps only (the producer warp does not take part)
 __device__ __forceinline__ void compute_warps_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kBlock) : "memory"); }
 
 // Fixed-order block reduction of the ledger partials in the working precision: compensated
 // sums are combined pairwise (two-sum), counts as integers; only the block totals become FP64
 // (an FP64 shuffle tree here took a quarter of the kernel on GB300's slow FP64 pipe).
-// W warps take part: the whole block (CW = false, every thread calls this), or the compute warps
-// only (CW = true, synchronised by their named barrier; the producer warp holds no sums, and its
-// zeros would change nothing).
+// (The multi-step passes; every thread of their W warps calls this.)
 constexpr int kCounts = 8;
-template <typename R, int W, bool CW = false>
+template <typename R, int W>
 __device__ __forceinline__ void write_ledger_partial(const Acc<R>& acc, double* ledger_part, uint32_t blk) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   KSum<R> f[7] = {acc.e[0], acc.e[1], acc.e[2], acc.emit_e, acc.emit_def, acc.pair_e, acc.pair_def};
@@ -623,8 +652,7 @@ __device__ __forceinline__ void write_ledger_partial(const Acc<R>& acc, double* 
     for (int q = 0; q < 7; ++q) s_fr[warp][q] = f[q];
     for (int q = 0; q < kCounts; ++q) s_cr[warp][q] = c[q];
   }
-  if (CW) compute_warps_sync();
-  else __syncthreads();
+  __syncthreads();
   if (threadIdx.x < kLedgerN) {
     const int k = threadIdx.x;
     int fs = -1, cs = -1;  // where ledger field k comes from
@@ -648,14 +676,39 @@ __device__ __forceinline__ void write_ledger_partial(const Acc<R>& acc, double* 
     }
     ledger_part[(size_t)blk * kLedgerN + k] = t;
   }
-  if (CW) compute_warps_sync();  // s_fr and s_cr are reused by the next slot's partial
+}
+
+// The block's ledger partial from its compute warps' sums (threads 0 .. kLedgerN - 1, after a barrier):
+// combined in warp order in the working precision, as write_ledger_partial does.
+template <typename R>
+__device__ __forceinline__ void write_step_partial(const EventRing<R>* ring, double* ledger_part, uint32_t blk) {
+  const int k = threadIdx.x;
+  if (k >= kLedgerN) return;
+  KSum<R> t;
+  uint32_t n = 0;
+  for (int w = 0; w < kWarps; ++w) {
+    const EventSums<R>& es = ring[w].sums;
+    switch (k) {
+      case kN0: case kN1: case kN2: n += es.n[k - kN0]; break;
+      case kE0: case kE1: case kE2: t.merge(es.e[k - kE0]); break;
+      case kEmitN: n += es.emit_n; break;
+      case kEmitE: t.merge(es.emit_e); break;
+      case kDrop: n += es.drop; break;
+      case kEmitDef: t.merge(es.emit_def); break;
+      case kPairN: n += es.pair_n; break;
+      case kPairE: t.merge(es.pair_e); break;
+      case kPairDef: t.merge(es.pair_def); break;
+      case kOorEta: n += es.oor_eta; break;
+      default: n += es.oor_chi; break;
+    }
+  }
+  ledger_part[(size_t)blk * kLedgerN + k] = n ? (double)n : t.value();
 }
 
 // The photon push counters of a block: summed over its warps in shared memory, then added to the
 // scenario's work counters (the e+- pushes follow from the particle counts).
-template <typename R>
-__device__ __forceinline__ void add_work(const Acc<R>& acc, uint32_t* s_work, int lane) {
-  const uint32_t p = __reduce_add_sync(kFull, acc.pushed_ph), t = __reduce_add_sync(kFull, acc.tau_ph);
+__device__ __forceinline__ void add_work(uint32_t pushed_ph, uint32_t tau_ph, uint32_t* s_work, int lane) {
+  const uint32_t p = __reduce_add_sync(kFull, pushed_ph), t = __reduce_add_sync(kFull, tau_ph);
   if (lane == 0 && p) {
     atomicAdd(&s_work[0], p);
     atomicAdd(&s_work[1], t);
@@ -666,133 +719,263 @@ __device__ __forceinline__ void flush_work(uint32_t* s_work, unsigned long long*
   if (s_work[1]) atomicAdd(&work[5], (unsigned long long)s_work[1]);
 }
 
-// The block's tiles of species SP, global tiles [t_lo, t_hi) over its particles [base, n), with the
-// block's tile count k running on; field class FC.  Events are taken 32 at a time and all of them after the species'
-// last tile.  False if a wait gave up (the events left in the ring are then not taken).  One loop
-// per species and field class, so no tile decodes its species or dispatches on the field (on
-// GB300 this took 10% off the head-on job's per-step kernel).  Species indices stay compile-time
-// constants (no dynamic indexing of the kernel parameters, which would copy them to local memory).
-template <typename R, bool G, int FC, int SP>
-__device__ __forceinline__ bool species_tiles(const StepArgs<R>& a, const StepScalars<R>& S, const R* lnh, const R* lnT,
-                                              TileBuf<R>* buf, uint64_t* full, uint64_t* empty, uint32_t& k,
-                                              uint32_t blk, uint32_t nblk, uint32_t t_lo, uint32_t t_hi, uint32_t base,
-                                              uint32_t n, int lane, int warp, Acc<R>& acc, EventQueue<R>& q) {
+// A run of tiles of one (slot, species): global tiles [g_lo, g_hi) of the step's tile space, which
+// hold the species' particles [base, n); slot_lo is the slot's first tile (batches).  s = 3: tiles
+// without particles, for the conversions that a photon window found among its first n photons.
+struct TileRun {
+  int slot = 0, s = -1;
+  uint32_t g_lo = 0, g_hi = 0, slot_lo = 0;
+  uint32_t n = 0, base = 0;
+};
+
+// What a block's compute warps share: the tile pipeline and the event rings.
+template <typename R>
+struct StepPipe {
+  TileBuf<R>* buf;
+  uint64_t *full, *empty;
+  EventRing<R>* ring;
+  const R *lnh, *lnT;
+  int* abort;
+  uint32_t blk, nblk;
+};
+
+// The state of one compute warp.
+template <typename R>
+struct WarpState {
+  EventQueue<R> q;
+  uint32_t pushed_ph = 0, tau_ph = 0;  // (per lane) photons pushed; those in a field
+  uint32_t k = 0;        // tiles the block has passed
+  bool stopped = false;  // a wait gave up: no more waits or work, but every barrier is kept
+};
+
+// Waits for the data of the block's tile w.k; false once a wait gave up.
+template <typename R>
+__device__ __forceinline__ bool tile_ready(const StepPipe<R>& P, WarpState<R>& w) {
+  if (!w.stopped && (*P.abort || !mbar_wait_bounded(&P.full[w.k % kStages], (w.k / kStages) & 1u, kWaitLimit))) {
+    *P.abort = 1;
+    w.stopped = true;
+  }
+  return !w.stopped;
+}
+
+// Tiles of one run, from the block's w.k-th on, until 32 events wait (true: take them and call again)
+// or the block's tiles of the run are done.  Compiled per field class FC and species SP, so no tile
+// dispatches on either (and the species' arrays are constants); the events' code, which is long, is
+// kept out of it.
+template <typename R, bool G, int FC, int SP, bool WANT>
+__device__ __forceinline__ bool run_tiles(const StepArgs<R>& A, const StepScalars<R>& S, const StepPipe<R>& P,
+                                          const TileRun& run, WarpState<R>& w, RunSums<R>& sums) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t n = run.n, base = SP == 2 ? run.base : 0u;
   const uint32_t last = n > base ? (n - base - 1u) / (uint32_t)kTile : 0u;  // the only tile that can be ragged
   const uint32_t valid = n - base - last * (uint32_t)kTile;
   const uint32_t in_r = floor16(valid * (uint32_t)sizeof(R)) / (uint32_t)sizeof(R);
   const uint32_t in_t = floor16(valid * 8u) / 8u;
   const bool ragged = in_r < valid || in_t < valid;
   const uint32_t r = threadIdx.x;
-  for (;; ++k) {
-    const uint32_t t = blk + k * nblk;
-    const bool more = t < t_hi;
-    if (more) {
-      const int st = (int)(k % kStages);
-      if (!mbar_wait_bounded(&full[st], (k / kStages) & 1u, kWaitLimit)) return false;
-      const uint32_t j = t - t_lo;
-      TileBuf<R>& b = buf[st];
-      if (ragged && j == last) {
-        const TileSrc<R> g = tile_src(a.sp[SP]);
-        const uint32_t gi = base + j * kTile + r;
-        if (r >= in_r && r < valid) {
-          b.x[r] = g.x[gi]; b.y[r] = g.y[gi]; b.z[r] = g.z[gi];
-          b.ux[r] = g.ux[gi]; b.uy[r] = g.uy[gi]; b.uz[r] = g.uz[gi];
-        }
-        if (r >= in_t && r < valid) b.tau[r] = g.tau[gi];
-        compute_warps_sync();
+  for (;; ++w.k) {
+    const uint32_t g = P.blk + w.k * P.nblk;
+    if (g >= run.g_hi) return false;
+    if (w.q.count >= 32u) return true;
+    if (!tile_ready(P, w)) continue;
+    const int st = (int)(w.k % kStages);
+    TileBuf<R>& b = P.buf[st];
+    const uint32_t j = g - run.g_lo;
+    // the ragged remainder of a species' last tile: each thread reads its own particle
+    if (ragged && j == last && r < valid && (r >= in_r || r >= in_t)) {
+      const SpeciesDev<R>& gs = A.sp[SP];
+      const uint32_t gi = base + j * kTile + r;
+      if (r >= in_r) {
+        b.x[r] = gs.x[gi]; b.y[r] = gs.y[gi]; b.z[r] = gs.z[gi];
+        b.ux[r] = gs.ux[gi]; b.uy[r] = gs.uy[gi]; b.uz[r] = gs.uz[gi];
       }
-      const uint32_t chunk = base / 32u + j * kWarps + warp;
-      if (SP == 2)
-        photon_chunk<R, G, FC>(a, S, lnT, chunk, n, lane, acc, q, b.x[r], b.y[r], b.z[r], b.ux[r], b.uy[r], b.uz[r],
-                               &b.tau[r]);
-      else
-        lepton_chunk<R, G, FC>(a, S, lnh, SP == 0 ? QED_ELECTRON : QED_POSITRON, chunk, n, lane, acc, q, b.x[r],
-                               b.y[r], b.z[r], b.ux[r], b.uy[r], b.uz[r], &b.tau[r]);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[st]);
+      if (r >= in_t) b.tau[r] = gs.tau[gi];
     }
-    while (q.count >= 32u || (!more && q.count > 0u)) {
-      const uint32_t take = min(q.count, 32u);
-      if (SP == 0) lepton_events<R, QED_ELECTRON>(a, S.phase[0], q.r, q.head, take);
-      else if (SP == 1) lepton_events<R, QED_POSITRON>(a, S.phase[1], q.r, q.head, take);
-      else photon_events<R>(a, q.r, q.head, take);
-      q.head = (q.head + take) & (uint32_t)(kRing - 1);
-      q.count -= take;
-    }
-    if (!more) return true;
+    const uint32_t chunk = base / 32u + j * kWarps + warp;
+    if constexpr (SP == 2)
+      photon_chunk<R, G, FC, WANT>(A, S, P.lnT, chunk, n, lane, sums, w.pushed_ph, w.tau_ph, w.q, b.x[r], b.y[r], b.z[r],
+                                   b.ux[r], b.uy[r], b.uz[r], &b.tau[r]);
+    else
+      lepton_chunk<R, G, FC, SP, WANT>(A, S, P.lnh, chunk, n, lane, sums, w.q, b.x[r], b.y[r], b.z[r], b.ux[r], b.uy[r],
+                                       b.uz[r], &b.tau[r]);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&P.empty[st]);
   }
-}
-template <typename R, bool G, int FC>
-__device__ __forceinline__ bool species_pass(const StepArgs<R>& a, const StepScalars<R>& S, const R* lnh, const R* lnT,
-                                             TileBuf<R>* buf, uint64_t* full, uint64_t* empty, uint32_t& k,
-                                             uint32_t blk, uint32_t nblk, uint32_t T0, uint32_t T1, uint32_t ttot,
-                                             uint32_t n0, uint32_t n1, uint32_t n2, uint32_t win_n, int lane,
-                                             int warp, Acc<R>& acc, EventQueue<R>& q) {
-  return species_tiles<R, G, FC, 0>(a, S, lnh, lnT, buf, full, empty, k, blk, nblk, 0u, T0, 0u, n0, lane, warp, acc,
-                                    q) &&
-         species_tiles<R, G, FC, 1>(a, S, lnh, lnT, buf, full, empty, k, blk, nblk, T0, T0 + T1, 0u, n1, lane, warp,
-                                    acc, q) &&
-         species_tiles<R, G, FC, 2>(a, S, lnh, lnT, buf, full, empty, k, blk, nblk, T0 + T1, ttot, win_n, n2, lane,
-                                    warp, acc, q);
 }
 
-// The conversions that the photon window found for this step: the groups of 1024 photons whose
-// flag has the step's bit, one group per warp at a time (one mask word per lane).  Makes the step's
-// event-mask words and counts of the group and takes the events (photon_events), as if the photons
-// had been pushed by this step.  A converted photon waits with its step and its chi in the place of
-// its optical depth, at its position after the push.
+// The conversions that the photon window found for this step, as a run without particles: its T tiles
+// share the window's groups of 1024 photons, neighbouring groups with different warps; a group whose
+// flag has the step's bit is done by the whole warp (one mask word per lane).  Makes the step's event-mask words and counts of the
+// group and queues the events, as if the photons had been pushed by this step.  A converted photon
+// waits with its step and its chi in the place of its optical depth, at its position after the
+// push.  Returns true when 32 events wait, with its place kept in `c`.
+struct ConversionState {
+  bool open = false;
+  uint32_t first = 0, next = 0, w = 0, m = 0;
+  unsigned todo = 0;
+};
 template <typename R>
-__device__ __forceinline__ void window_events(const StepArgs<R>& a, uint32_t phase, uint32_t win_n, uint32_t blk,
-                                              uint32_t nblk, int lane, int warp, EventQueue<R>& q) {
+__device__ __forceinline__ bool run_conversions(const StepArgs<R>& a, const StepScalars<R>& S, const StepPipe<R>& P,
+                                                const TileRun& run, WarpState<R>& ws, ConversionState& c) {
   const SpeciesDev<R>& sp = a.sp[2];
-  const uint32_t groups = win_n >> 10, W = nblk * kWarps, me = blk * kWarps + warp;
-  const uint32_t bit = 1u << a.win_s;
-  for (uint32_t g0 = 0; g0 < groups; g0 += 32u * W) {
-    const uint32_t mine = g0 + (uint32_t)lane * W + me;  // neighbouring groups go to different warps
-    const uint32_t fl = mine < groups ? sp.wflag[mine] : 0u;
-    unsigned todo = __ballot_sync(kFull, (fl & bit) != 0u);
-    if ((fl & bit) && !(fl >> a.win_s >> 1)) sp.wflag[mine] = 0u;  // the group's last step with conversions
-    while (todo) {
-      const uint32_t g = g0 + (uint32_t)(__ffs(todo) - 1) * W + me;
-      todo &= todo - 1u;
-      const uint32_t w = g * 32u + (uint32_t)lane;
-      uint32_t m = 0;
-      for (uint32_t left = sp.cmask[w]; left; left &= left - 1u) {
-        const uint32_t b = (uint32_t)__ffs(left) - 1u;
-        if (Tau<R>::load(sp.tau + w * 32u + b).window_step() == a.win_s) m |= 1u << b;
-      }
-      sp.evmask[w] = m;
-      const uint32_t c = __reduce_add_sync(kFull, (uint32_t)__popc(m));
-      if (lane == 0) {
-        count_events(sp, phase, g * 32u, c);
-        atomicAdd(&sp.cnt->n_dead, c);
-      }
-      while (__any_sync(kFull, m != 0u)) {
-        const bool ev = m != 0u;
-        uint32_t i = 0;
-        R x = (R)0, y = (R)0, z = (R)0, k0 = (R)0, k1 = (R)0, k2 = (R)0, chi = (R)0;
-        if (ev) {
-          i = w * 32u + (uint32_t)__ffs(m) - 1u;
-          x = sp.x[i]; y = sp.y[i]; z = sp.z[i];
-          k0 = sp.ux[i]; k1 = sp.uy[i]; k2 = sp.uz[i];
-          chi = Tau<R>::load(sp.tau + i).window_chi();
-          m &= m - 1u;
-        }
-        enqueue_event<R>(q, __ballot_sync(kFull, ev), ev, lane, i, x, y, z, k0, k1, k2, chi);
-        __syncwarp();
-        if (q.count >= 32u) {
-          photon_events<R>(a, q.r, q.head, 32u);
-          q.head = (q.head + 32u) & (uint32_t)(kRing - 1);
-          q.count -= 32u;
-        }
-      }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t groups = run.n >> 10, stride = (run.g_hi - run.g_lo) * kWarps;
+  for (;;) {
+    if (!c.open) {
+      const uint32_t t = P.blk + ws.k * P.nblk;
+      if (t >= run.g_hi) return false;
+      if (!tile_ready(P, ws)) { ++ws.k; continue; }
+      c.first = c.next = (t - run.g_lo) * kWarps + (uint32_t)warp;
+      c.open = true;
     }
+    while (__any_sync(kFull, c.m != 0u) || c.todo || c.next < groups) {
+      if (!__any_sync(kFull, c.m != 0u)) {
+        if (!c.todo) {  // the flags of the warp's next 32 groups
+          c.first = c.next;
+          c.next += 32u * stride;
+          const uint32_t mine = c.first + (uint32_t)lane * stride, bit = 1u << a.win_s;
+          const uint32_t fl = mine < groups ? sp.wflag[mine] : 0u;
+          c.todo = __ballot_sync(kFull, (fl & bit) != 0u);
+          if ((fl & bit) && !(fl >> a.win_s >> 1)) sp.wflag[mine] = 0u;  // the group's last step with conversions
+          continue;
+        }
+        const uint32_t g = c.first + (uint32_t)(__ffs(c.todo) - 1) * stride;
+        c.todo &= c.todo - 1u;
+        c.w = g * 32u + (uint32_t)lane;
+        for (uint32_t left = sp.cmask[c.w]; left; left &= left - 1u) {
+          const uint32_t b = (uint32_t)__ffs(left) - 1u;
+          if (Tau<R>::load(sp.tau + c.w * 32u + b).window_step() == a.win_s) c.m |= 1u << b;
+        }
+        sp.evmask[c.w] = c.m;
+        const uint32_t cnt = __reduce_add_sync(kFull, (uint32_t)__popc(c.m));
+        if (lane == 0) {
+          count_events(sp, S.phase[2], g * 32u, cnt);
+          atomicAdd(&sp.cnt->n_dead, cnt);
+        }
+      }
+      const bool ev = c.m != 0u;
+      uint32_t i = 0;
+      R x = (R)0, y = (R)0, z = (R)0, k0 = (R)0, k1 = (R)0, k2 = (R)0, chi = (R)0;
+      if (ev) {
+        i = c.w * 32u + (uint32_t)__ffs(c.m) - 1u;
+        x = sp.x[i]; y = sp.y[i]; z = sp.z[i];
+        k0 = sp.ux[i]; k1 = sp.uy[i]; k2 = sp.uz[i];
+        chi = Tau<R>::load(sp.tau + i).window_chi();
+        c.m &= c.m - 1u;
+      }
+      enqueue_event<R>(ws.q, __ballot_sync(kFull, ev), ev, lane, i, x, y, z, k0, k1, k2, chi);
+      __syncwarp();
+      if (ws.q.count >= 32u) return true;
+    }
+    c.open = false;
+    if (lane == 0) mbar_arrive(&P.empty[ws.k % kStages]);
+    ++ws.k;
   }
-  if (q.count) {
-    photon_events<R>(a, q.r, q.head, q.count);
-    q.head = (q.head + q.count) & (uint32_t)(kRing - 1);
-    q.count = 0;
+}
+
+// The lanes' sums of a run into the warp's (fixed shuffle order).
+template <typename R>
+__device__ __forceinline__ void fold_run_sums(const RunSums<R>& sums, int s, EventSums<R>& es) {
+  KSum<R> t = sums.e;
+  for (int off = 16; off > 0; off >>= 1) {
+    KSum<R> o;
+    o.s = __shfl_down_sync(kFull, t.s, off);
+    o.c = __shfl_down_sync(kFull, t.c, off);
+    t.merge(o);
   }
+  const uint32_t n = __reduce_add_sync(kFull, sums.n), oor = __reduce_add_sync(kFull, sums.oor);
+  if ((threadIdx.x & 31) == 0) {
+    es.e[s].merge(t);
+    es.n[s] += n;
+    if (s == 2) es.oor_chi += oor;
+    else es.oor_eta += oor;
+  }
+}
+
+// The block's tiles of one run of leptons and all their events (every compute warp of the block calls
+// this): a warp takes 32 events whenever it has them, and what is left in the block's rings is
+// taken together, 32 per warp: eight rings with fewer than 32 each make at most eight batches.
+template <typename R, bool G, bool WANT>
+__device__ __forceinline__ void run_leptons(const StepArgs<R>& A, const StepScalars<R>& S, const StepPipe<R>& P,
+                                            const TileRun& run, WarpState<R>& w) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  RunSums<R> sums;
+  for (bool more = true; more;) {
+    if (!G && S.kind == QED_FIELD_PLANE_LP)
+      more = run.s == 0 ? run_tiles<R, G, G ? kFieldAny : kFieldLP, 0, WANT>(A, S, P, run, w, sums)
+                        : run_tiles<R, G, G ? kFieldAny : kFieldLP, 1, WANT>(A, S, P, run, w, sums);
+    else if (!G && S.kind == QED_FIELD_PLANE_CP)
+      more = run.s == 0 ? run_tiles<R, G, G ? kFieldAny : kFieldCP, 0, WANT>(A, S, P, run, w, sums)
+                        : run_tiles<R, G, G ? kFieldAny : kFieldCP, 1, WANT>(A, S, P, run, w, sums);
+    else
+      more = run.s == 0 ? run_tiles<R, G, kFieldAny, 0, WANT>(A, S, P, run, w, sums)
+                        : run_tiles<R, G, kFieldAny, 1, WANT>(A, S, P, run, w, sums);
+    const EventRing<R>* src = w.q.r;
+    uint32_t p = w.q.head + (uint32_t)lane, take = 32u;
+    if (more) {  // 32 of the warp's own
+      w.q.head += 32u;
+      w.q.count -= 32u;
+    } else {
+      if (w.stopped) w.q.count = 0;  // (an unfinished step: QED_ERR_TIMEOUT)
+      if (lane == 0) { w.q.r->head = w.q.head; w.q.r->count = w.q.count; }
+      compute_warps_sync();
+      uint32_t inc = lane < kWarps ? P.ring[lane].count : 0u;
+#pragma unroll
+      for (int off = 1; off < kWarps; off <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, inc, off);
+        if (lane >= off) inc += t;
+      }
+      const uint32_t total = __shfl_sync(kFull, inc, kWarps - 1), e0 = (uint32_t)warp * 32u;
+      take = total > e0 ? min(32u, total - e0) : 0u;
+      const uint32_t e = e0 + (uint32_t)lane;
+      uint32_t j = 0, before = 0;
+#pragma unroll
+      for (int t = 0; t < kWarps - 1; ++t) {
+        const uint32_t upto = __shfl_sync(kFull, inc, t);
+        if (e >= upto) { j = (uint32_t)t + 1u; before = upto; }
+      }
+      src = P.ring + j;
+      p = src->head + e - before;
+    }
+    if (take) lepton_events<R, WANT>(A, S.phase[run.s], run.s, src, p & (uint32_t)(kRing - 1), take, w.q.r->sums);
+  }
+  compute_warps_sync();  // every ring has been read
+  w.q.count = 0;
+  if (WANT) fold_run_sums(sums, run.s, w.q.r->sums);
+}
+
+// The block's tiles of one run of photons, or of a window's conversions, and the warp's events.
+template <typename R, bool G, bool WANT>
+__device__ __forceinline__ void run_photons(const StepArgs<R>& A, const StepScalars<R>& S, const StepPipe<R>& P,
+                                            const TileRun& run, WarpState<R>& w) {
+  RunSums<R> sums;
+  ConversionState conv;
+  for (bool more = true; more;) {
+    if (run.s == 3) {
+      more = false;
+      if constexpr (sizeof(R) == 4) more = run_conversions(A, S, P, run, w, conv);
+    } else if (!G && S.kind == QED_FIELD_PLANE_LP) {
+      more = run_tiles<R, G, G ? kFieldAny : kFieldLP, 2, WANT>(A, S, P, run, w, sums);
+    } else if (!G && S.kind == QED_FIELD_PLANE_CP) {
+      more = run_tiles<R, G, G ? kFieldAny : kFieldCP, 2, WANT>(A, S, P, run, w, sums);
+    } else {
+      more = run_tiles<R, G, kFieldAny, 2, WANT>(A, S, P, run, w, sums);
+    }
+    if (w.stopped) w.q.count = 0;
+    const uint32_t take = min(w.q.count, 32u);
+    if (take)
+      photon_events<R, WANT>(A, w.q.r, (w.q.head + (threadIdx.x & 31u)) & (uint32_t)(kRing - 1), take, w.q.r->sums);
+    w.q.head += take;
+    w.q.count -= take;
+  }
+  if (WANT && run.s == 2) fold_run_sums(sums, 2, w.q.r->sums);
+}
+
+template <typename R, bool G, bool WANT>
+__device__ __forceinline__ void run_species(const StepArgs<R>& A, const StepScalars<R>& S, const StepPipe<R>& P,
+                                            const TileRun& run, WarpState<R>& w) {
+  if (run.s < 2) run_leptons<R, G, WANT>(A, S, P, run, w);
+  else run_photons<R, G, WANT>(A, S, P, run, w);
 }
 
 // The step over one scenario, run by block `blk` of the `nblk` blocks given to it: block blk
@@ -800,9 +983,9 @@ __device__ __forceinline__ void window_events(const StepArgs<R>& a, uint32_t pha
 // Warp roles: warps 0-7 compute (warp w takes 32-particle chunk w of each tile); warp 8 is the
 // producer: its first lane issues the bulk copies of tile k into stage k % kStages once the 8
 // compute warps have released that stage (mbarrier `empty`, one arrival per warp); compute warps
-// wait only for their tile's data (mbarrier `full`), never for each other.  Each compute warp
-// keeps its events in its own ring (see EventRing) and takes them between tiles.
-template <typename R, bool G>
+// wait only for their tile's data (mbarrier `full`), and for each other once per species, to share
+// out the events left in their rings.
+template <typename R, bool G, bool WANT>
 __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, uint32_t nblk, unsigned char* smem_raw) {
   TileBuf<R>* buf = reinterpret_cast<TileBuf<R>*>(smem_raw);
   EventRing<R>* ring = reinterpret_cast<EventRing<R>*>(buf + kStages);
@@ -812,7 +995,6 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
   __shared__ __align__(8) uint64_t empty[kStages];
   __shared__ StepScalars<R> S;
   __shared__ int s_abort;
-
   __shared__ uint32_t s_work[2];
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -834,14 +1016,15 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
   const uint32_t n0 = a.sp[0].cnt->n, n1 = a.sp[1].cnt->n, n2 = a.sp[2].cnt->n;
   const uint32_t win_n = sizeof(R) == 4 && a.win_s >= 0 ? a.sp[2].cnt->win_n : 0u;
   const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 - win_n + kTile - 1) / kTile;
-  const uint32_t ttot = T0 + T1 + T2;
-  if (threadIdx.x < 3) S.phase[threadIdx.x] = (threadIdx.x == 0 ? a.sp[0] : (threadIdx.x == 1 ? a.sp[1] : a.sp[2])).cnt->phase;
+  const uint32_t T3 = conversion_tiles(win_n, nblk);
+  const uint32_t ttot = T0 + T1 + T2 + T3;
+  if (threadIdx.x < 3) S.phase[threadIdx.x] = a.sp[threadIdx.x].cnt->phase;
   if (threadIdx.x == kBlock)
     for (uint32_t k = 0; k < (uint32_t)kStages; ++k) issue_tile(a, buf, full, k, n0, n1, n2, win_n, blk, nblk);
   __syncthreads();
   pdl_launch();
 
-  Acc<R> acc;
+  WarpState<R> w;
   if (warp == kWarps) {
     // ---------------- producer
     if (lane == 0) {
@@ -863,46 +1046,31 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
     }
   } else {
     // ---------------- compute warps
-    EventQueue<R> q{ring + warp, 0u, 0u};
-    if (lane == 0) q.r->sums = EventSums<R>{};
+    w.q = EventQueue<R>{ring + warp, 0u, 0u};
+    if (lane == 0) w.q.r->sums = EventSums<R>{};
     __syncwarp();
-    if constexpr (sizeof(R) == 4)
-      if (win_n) window_events<R>(a, S.phase[2], win_n, blk, nblk, lane, warp, q);
-    // one loop per species and field class: no per-tile dispatch (a grid-field instantiation
-    // only ever sees the general class)
-    uint32_t k = 0;
-    bool ok;
-    if (!G && S.kind == QED_FIELD_PLANE_LP)
-      ok = species_pass<R, G, G ? kFieldAny : kFieldLP>(a, S, s_lnh, s_lnT, buf, full, empty, k, blk, nblk, T0, T1,
-                                                        ttot, n0, n1, n2, win_n, lane, warp, acc, q);
-    else if (!G && S.kind == QED_FIELD_PLANE_CP)
-      ok = species_pass<R, G, G ? kFieldAny : kFieldCP>(a, S, s_lnh, s_lnT, buf, full, empty, k, blk, nblk, T0, T1,
-                                                        ttot, n0, n1, n2, win_n, lane, warp, acc, q);
-    else
-      ok = species_pass<R, G, kFieldAny>(a, S, s_lnh, s_lnT, buf, full, empty, k, blk, nblk, T0, T1, ttot, n0, n1, n2,
-                                         win_n, lane, warp, acc, q);
-    if (!ok) s_abort = 1;
-    // a wait that gave up leaves the step unfinished (QED_ERR_TIMEOUT): events still in the
-    // ring are not taken
-    __syncwarp();
-    if (a.want && lane == 0) {
-      const EventSums<R>& es = q.r->sums;
-      for (int c = 0; c < 3; ++c) { acc.e[c].merge(es.e[c]); acc.n[c] += es.n[c]; }
-      acc.emit_e = es.emit_e; acc.emit_def = es.emit_def;
-      acc.pair_e = es.pair_e; acc.pair_def = es.pair_def;
-      acc.emit_n = es.emit_n; acc.drop = es.drop; acc.pair_n = es.pair_n;
+    const StepPipe<R> P{buf, full, empty, ring, s_lnh, s_lnT, &s_abort, blk, nblk};
+    TileRun run;
+    for (run.s = 0; run.s < 4; ++run.s) {
+      run.g_lo = run.g_hi;
+      run.g_hi += run.s == 0 ? T0 : (run.s == 1 ? T1 : (run.s == 2 ? T2 : T3));
+      run.n = run.s == 0 ? n0 : (run.s == 1 ? n1 : (run.s == 2 ? n2 : win_n));
+      run.base = run.s == 2 ? win_n : 0u;
+      if (blk + w.k * nblk < run.g_hi) run_species<R, G, WANT>(a, S, P, run, w);  // (the same for every warp)
     }
-    add_work(acc, s_work, lane);
+    add_work(w.pushed_ph, w.tau_ph, s_work, lane);
   }
   __syncthreads();
   if (threadIdx.x == 0) flush_work(s_work, a.work);
-  if (a.want) write_ledger_partial<R, kWarps + 1>(acc, a.ledger_part, blk);
+  if (WANT) write_step_partial<R>(ring, a.ledger_part, blk);
 }
 
-template <typename R, bool G>
-__global__ void __launch_bounds__(kStepThreads, sizeof(R) == 4 ? QED_STEP_MIN_BLOCKS : 1) step_kernel(const StepArgs<R> a) {
+// WANT: the step's ledger can be read (the last step of a run).
+template <typename R, bool G, bool WANT>
+__global__ void __launch_bounds__(kStepThreads, sizeof(R) == 4 ? QED_STEP_MIN_BLOCKS : 1)
+step_kernel(const __grid_constant__ StepArgs<R> a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  step_body<R, G>(a, blockIdx.x, gridDim.x, smem_raw);
+  step_body<R, G, WANT>(a, blockIdx.x, gridDim.x, smem_raw);
 }
 
 // ----------------------------------------------------------------------------- multi-step
@@ -1547,18 +1715,17 @@ __device__ __forceinline__ void window_batch(const StepArgs<float>& a, const Win
   __syncwarp();  // the ring slots read above may be refilled
 }
 
+// A warp's chunks chunk, chunk + nw, ... below `chunks`; the ring is empty after it.  Returns the
+// lane's pushes.
 template <bool G, int WC>
-__device__ __forceinline__ void window_body(const StepArgs<float>& a, int K, uint32_t blk, uint32_t nblk, WinShared& sh,
-                                            const float2* cell) {
+__device__ __forceinline__ uint32_t window_chunks(const StepArgs<float>& a, int K, uint32_t chunk, uint32_t chunks,
+                                                  uint32_t nw, WinShared& sh, const float2* cell) {
   const SpeciesDev<float>& sp = a.sp[2];
-  const uint32_t nwin = sp.cnt->n & ~1023u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t nw = nblk * (kFuseThreads / 32), chunks = nwin >> 5;
   const float dt = a.dt_r;
   WinRing& ring = sh.ring[warp];
   uint32_t head = 0, count = 0;  // warp-uniform
   uint32_t pushed = 0;
-  uint32_t chunk = blk * (kFuseThreads / 32) + warp;
   // the next chunk's state is loaded while the current one is stepped
   PState<float> nxt{};
   auto load = [&](uint32_t c) {
@@ -1631,16 +1798,33 @@ __device__ __forceinline__ void window_body(const StepArgs<float>& a, int K, uin
       }
     }
   }
-  pushed = __reduce_add_sync(kFull, pushed);
-  if (lane == 0 && pushed) atomicAdd(&sh.pushed, pushed);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (sh.pushed) {
-      atomicAdd(&a.work[1], (unsigned long long)sh.pushed);
-      atomicAdd(&a.work[4], (unsigned long long)sh.pushed);
-    }
-    if (blk == 0) sp.cnt->win_n = nwin;
+  return pushed;
+}
+
+template <bool G>
+__device__ __forceinline__ uint32_t window_photons(const StepArgs<float>& a, int K, uint32_t chunk, uint32_t chunks,
+                                                   uint32_t nw, WinShared& sh, const float2* cell) {
+  switch (a.field.kind) {
+    case QED_FIELD_PLANE_LP: return window_chunks<G, kWinLP>(a, K, chunk, chunks, nw, sh, cell);
+    case QED_FIELD_PLANE_CP: return window_chunks<G, kWinCP>(a, K, chunk, chunks, nw, sh, cell);
+    case QED_FIELD_ROTATING_E: return window_chunks<G, kWinRotating>(a, K, chunk, chunks, nw, sh, cell);
+    case QED_FIELD_UNIFORM: return window_chunks<G, kWinUniform>(a, K, chunk, chunks, nw, sh, cell);
+    default:
+      if constexpr (G) return window_chunks<G, kWinGrid>(a, K, chunk, chunks, nw, sh, cell);
+      return 0;
   }
+}
+
+__device__ __forceinline__ void load_cells(const TabDev<float>& tab, float2* cell) {
+  for (int k = threadIdx.x; k + 1 < tab.n_chi; k += blockDim.x) cell[k] = make_float2(tab.ln_T[k], tab.ln_T[k + 1]);
+}
+__device__ __forceinline__ float2 window_pair(int kind, const StepScalars<float>& S) {
+  return kind == QED_FIELD_ROTATING_E ? make_float2(S.E[0], S.E[1]) : make_float2(S.phi_ref, S.phi_ref_mod);
+}
+__device__ __forceinline__ void add_window_work(const StepArgs<float>& a, uint32_t pushed) {
+  if (!pushed) return;
+  atomicAdd(&a.work[1], (unsigned long long)pushed);
+  atomicAdd(&a.work[4], (unsigned long long)pushed);
 }
 
 // Shared memory: WinShared, then the T table's cells (n_chi - 1 of them).
@@ -1651,22 +1835,26 @@ __global__ void __launch_bounds__(kFuseThreads) window_kernel(const StepArgs<flo
   extern __shared__ __align__(128) unsigned char smem_raw[];
   WinShared& sh = *reinterpret_cast<WinShared*>(smem_raw);
   float2* cell = reinterpret_cast<float2*>(smem_raw + sizeof(WinShared));
-  for (int k = threadIdx.x; k + 1 < a.tab.n_chi; k += blockDim.x) cell[k] = make_float2(a.tab.ln_T[k], a.tab.ln_T[k + 1]);
-  const int kind = a.field.kind;
+  load_cells(a.tab, cell);
   if ((int)threadIdx.x < K) {
     StepScalars<float>& S = sh.S[threadIdx.x];
     make_scalars<float>(a.field, a.t0 + (double)(a.step + threadIdx.x) * a.dt, a.win_x0, a.win_v, S);
-    sh.pair[threadIdx.x] = kind == QED_FIELD_ROTATING_E ? make_float2(S.E[0], S.E[1]) : make_float2(S.phi_ref, S.phi_ref_mod);
+    sh.pair[threadIdx.x] = window_pair(a.field.kind, S);
   }
   if (threadIdx.x == 0) sh.pushed = 0;
   pdl_wait();
   __syncthreads();
   pdl_launch();
-  if (G) window_body<G, kWinGrid>(a, K, blockIdx.x, gridDim.x, sh, cell);
-  else if (kind == QED_FIELD_PLANE_LP) window_body<G, kWinLP>(a, K, blockIdx.x, gridDim.x, sh, cell);
-  else if (kind == QED_FIELD_PLANE_CP) window_body<G, kWinCP>(a, K, blockIdx.x, gridDim.x, sh, cell);
-  else if (kind == QED_FIELD_ROTATING_E) window_body<G, kWinRotating>(a, K, blockIdx.x, gridDim.x, sh, cell);
-  else window_body<G, kWinUniform>(a, K, blockIdx.x, gridDim.x, sh, cell);
+  constexpr uint32_t W = kFuseThreads / 32;
+  const uint32_t nwin = a.sp[2].cnt->n & ~1023u;
+  const uint32_t pushed = __reduce_add_sync(
+      kFull, window_photons<G>(a, K, blockIdx.x * W + (threadIdx.x >> 5), nwin >> 5, gridDim.x * W, sh, cell));
+  if ((threadIdx.x & 31) == 0 && pushed) atomicAdd(&sh.pushed, pushed);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    add_window_work(a, sh.pushed);
+    if (blockIdx.x == 0) a.sp[2].cnt->win_n = nwin;
+  }
 }
 
 template <typename R>
@@ -1748,13 +1936,28 @@ __device__ __forceinline__ int slot_of_block(const uint32_t* blocks, int S, uint
   return lo;
 }
 
+template <typename R>
+__device__ __forceinline__ bool is_call_end(const BatchCtl<R>& c, int end) {
+  return end == kBatchCallEnd || (end == kBatchGroupEnd && c.tot[1] != 0u);
+}
+// Steps of a slot's photon window when the batch's spans W: up to the step before its last (whose
+// ledger is kept), 0 if that leaves fewer than 2.  end: where the batch's window ends.
+template <typename R>
+__device__ __forceinline__ uint32_t win_steps(const BatchCtl<R>& c, uint32_t remaining, int W, int end) {
+  const uint32_t w = (uint32_t)W - (is_call_end(c, end) ? 1u : 0u);
+  const uint32_t k = remaining > 0u ? min(w, remaining - 1u) : 0u;
+  return k >= 2u ? k : 0u;
+}
+
 // ---- per-step path of a batch: one tile space over all live slots
 // The tile schedule (one block) lays the live slots' tiles end to end (slot order, species order
 // inside a slot) and evaluates every slot's per-step field
-// scalars once.  want: the batch call's last step (the ledgers of all live slots can be read after
-// it; a slot that ends with this step keeps its ledger too).
+// scalars once.  win_w, win_end, win_s: the batch's photon window and the step's place in it (-1:
+// none).  end: the ledgers of all live slots can be read after the call's last step; a slot that
+// ends with this step keeps its ledger too.
 template <typename R>
-__global__ void __launch_bounds__(1024) batch_tiles_kernel(const BatchCtl<R> c, int want) {
+__global__ void __launch_bounds__(1024) batch_tiles_kernel(const BatchCtl<R> c, int end, int win_w, int win_end,
+                                                           int win_s) {
   pdl_wait();
   pdl_launch();
   const int per = (c.S + blockDim.x - 1) / blockDim.x;
@@ -1765,12 +1968,18 @@ __global__ void __launch_bounds__(1024) batch_tiles_kernel(const BatchCtl<R> c, 
     q.live = c.remaining[sl] > 0u ? 1u : 0u;
     if (q.live) {
       const StepArgs<R>& a = c.args[sl];
+      const uint32_t rem = c.remaining[sl];
+      // the slot's place in its photon window (its own may be shorter than the batch's)
+      const bool in = win_s >= 0 && (uint32_t)win_s < win_steps(c, rem + (uint32_t)win_s, win_w, win_end);
+      if (in) q.win_n = a.sp[2].cnt->win_n;
       for (int k = 0; k < 3; ++k) {
         q.n[k] = a.sp[k].cnt->n;
-        q.T[k] = (q.n[k] + kTile - 1) / kTile;
-        tiles += q.T[k];
+        q.T[k] = (q.n[k] - (k == 2 ? q.win_n : 0u) + kTile - 1) / kTile;
       }
-      c.args[sl].want = want || c.remaining[sl] == 1u;
+      q.T[3] = conversion_tiles(q.win_n, (uint32_t)c.target_blocks);
+      for (int k = 0; k < 4; ++k) tiles += q.T[k];
+      c.args[sl].want = rem == 1u || is_call_end(c, end);
+      c.args[sl].win_s = in ? win_s : -1;
       StepScalars<R>& S = static_cast<StepScalars<R>*>(c.scal)[sl];
       make_scalars<R>(a.field, a.t0 + (double)a.step * a.dt, a.win_x0, a.win_v, S);
       for (int k = 0; k < 3; ++k) S.phase[k] = a.sp[k].cnt->phase;
@@ -1782,20 +1991,14 @@ __global__ void __launch_bounds__(1024) batch_tiles_kernel(const BatchCtl<R> c, 
   for (int sl = s0; sl < s1; ++sl) {
     SlotPlan& q = c.splan[sl];
     q.tile_base = tb;
-    tb += q.T[0] + q.T[1] + q.T[2];
+    tb += q.T[0] + q.T[1] + q.T[2] + q.T[3];
     c.live[sl] = q.live;
   }
   if (threadIdx.x == 0) c.tot[0] = ttot;
 }
 
-// The run of tiles of one (slot, species) that global tile g of the batch step lies in: its tiles
-// are [g_lo, g_hi) of the tile space, slot_lo the slot's first.  A block's tiles increase, so the
-// slot cursor only moves forward and the run is looked up again only when g leaves it.
-struct TileRun {
-  int slot = 0, s = -1;
-  uint32_t g_lo = 0, g_hi = 0, slot_lo = 0;
-  uint32_t n = 0;  // particles of the species (the step's parents)
-};
+// The run that global tile g of the batch step lies in.  A block's tiles increase, so the slot cursor
+// only moves forward and the run is looked up again only when g leaves it.
 __device__ __forceinline__ void find_run(const SlotPlan* sp, int S, uint32_t g, TileRun& r) {
   if (g >= r.g_lo && g < r.g_hi) return;
   int cur = r.slot;
@@ -1804,9 +2007,12 @@ __device__ __forceinline__ void find_run(const SlotPlan* sp, int S, uint32_t g, 
   const uint32_t local = g - q.tile_base, T0 = q.T[0], T1 = q.T[1];
   r.slot = cur;
   r.slot_lo = q.tile_base;
+  r.base = 0;
+  const uint32_t T2 = q.T[2];
   if (local < T0) { r.s = 0; r.g_lo = q.tile_base; r.g_hi = r.g_lo + T0; r.n = q.n[0]; }
   else if (local < T0 + T1) { r.s = 1; r.g_lo = q.tile_base + T0; r.g_hi = r.g_lo + T1; r.n = q.n[1]; }
-  else { r.s = 2; r.g_lo = q.tile_base + T0 + T1; r.g_hi = r.g_lo + q.T[2]; r.n = q.n[2]; }
+  else if (local < T0 + T1 + T2) { r.s = 2; r.g_lo = q.tile_base + T0 + T1; r.g_hi = r.g_lo + T2; r.n = q.n[2]; r.base = q.win_n; }
+  else { r.s = 3; r.g_lo = q.tile_base + T0 + T1 + T2; r.g_hi = r.g_lo + q.T[3]; r.n = q.win_n; }  // conversions
 }
 
 // Producer (thread kBlock): bulk copies of the block's k-th tile, global tile g, into stage
@@ -1816,10 +2022,14 @@ __device__ __forceinline__ void issue_batch_tile(const BatchCtl<R>& c, TileBuf<R
                                                  uint32_t g, TileRun& run, TileSrc<R>& src) {
   if (!(g >= run.g_lo && g < run.g_hi)) {
     find_run(c.splan, c.S, g, run);
-    src = tile_src(c.args[run.slot].sp[run.s]);
+    if (run.s < 3) src = tile_src(c.args[run.slot].sp[run.s]);
+  }
+  if (run.s == 3) {  // nothing to copy
+    mbar_arrive(&bar[k % kStages]);
+    return;
   }
   const TileSrc<R>& sp = src;
-  const uint32_t first = (g - run.g_lo) * kTile;
+  const uint32_t first = run.base + (g - run.g_lo) * kTile;
   const uint32_t valid = min((uint32_t)kTile, run.n - first);
   const uint32_t br = floor16(valid * (uint32_t)sizeof(R)), bt = floor16(valid * 8u);
   TileBuf<R>& b = buf[k % kStages];
@@ -1836,81 +2046,6 @@ __device__ __forceinline__ void issue_batch_tile(const BatchCtl<R>& c, TileBuf<R
   if (bt) bulk_load(b.tau, sp.tau + first, bt, bb);
 }
 
-// The block's tiles of one run (slot, species SP: global tiles [run.g_lo, run.g_hi)), the block's
-// tile count k running on; field class FC.  Events are taken 32 at a time and all of them after
-// the run's last tile.  Once a wait gave up (`stopped`) the tiles are passed over.
-template <typename R, bool G, int FC, int SP>
-__device__ __forceinline__ void run_tiles(const StepArgs<R>& A, const StepScalars<R>& S, const R* lnh, const R* lnT,
-                                          TileBuf<R>* buf, uint64_t* full, uint64_t* empty, uint32_t& k, uint32_t blk,
-                                          uint32_t nblk, const TileRun& run, int lane, int warp, Acc<R>& acc,
-                                          EventQueue<R>& q, bool& stopped, int& s_abort) {
-  const uint32_t n = run.n;
-  const uint32_t last = n ? (n - 1u) / (uint32_t)kTile : 0u;  // the only tile that can be ragged
-  const uint32_t valid = n - last * (uint32_t)kTile;
-  const uint32_t in_r = floor16(valid * (uint32_t)sizeof(R)) / (uint32_t)sizeof(R);
-  const uint32_t in_t = floor16(valid * 8u) / 8u;
-  const bool ragged = in_r < valid || in_t < valid;
-  const uint32_t r = threadIdx.x;
-  for (;; ++k) {
-    const uint32_t g = blk + k * nblk;
-    const bool more = g < run.g_hi;
-    if (more) {
-      const int st = (int)(k % kStages);
-      if (!stopped && (s_abort || !mbar_wait_bounded(&full[st], (k / kStages) & 1u, kWaitLimit))) {
-        s_abort = 1;
-        stopped = true;
-      }
-      if (stopped) continue;
-      TileBuf<R>& b = buf[st];
-      const uint32_t j = g - run.g_lo;
-      // the ragged remainder of a species' last tile: each thread reads its own particle
-      if (ragged && j == last && r < valid && (r >= in_r || r >= in_t)) {
-        const SpeciesDev<R>& gs = A.sp[SP];
-        const uint32_t gi = j * kTile + r;
-        if (r >= in_r) {
-          b.x[r] = gs.x[gi]; b.y[r] = gs.y[gi]; b.z[r] = gs.z[gi];
-          b.ux[r] = gs.ux[gi]; b.uy[r] = gs.uy[gi]; b.uz[r] = gs.uz[gi];
-        }
-        if (r >= in_t) b.tau[r] = gs.tau[gi];
-      }
-      const uint32_t chunk = j * kWarps + warp;
-      if (SP == 2)
-        photon_chunk<R, G, FC>(A, S, lnT, chunk, n, lane, acc, q, b.x[r], b.y[r], b.z[r], b.ux[r], b.uy[r], b.uz[r],
-                               &b.tau[r]);
-      else
-        lepton_chunk<R, G, FC>(A, S, lnh, SP == 0 ? QED_ELECTRON : QED_POSITRON, chunk, n, lane, acc, q, b.x[r],
-                               b.y[r], b.z[r], b.ux[r], b.uy[r], b.uz[r], &b.tau[r]);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[st]);
-    }
-    if (stopped) {
-      if (!more) return;
-      continue;
-    }
-    while (q.count >= 32u || (!more && q.count > 0u)) {
-      const uint32_t take = min(q.count, 32u);
-      if (SP == 0) lepton_events<R, QED_ELECTRON>(A, S.phase[0], q.r, q.head, take);
-      else if (SP == 1) lepton_events<R, QED_POSITRON>(A, S.phase[1], q.r, q.head, take);
-      else photon_events<R>(A, q.r, q.head, take);
-      q.head = (q.head + take) & (uint32_t)(kRing - 1);
-      q.count -= take;
-    }
-    if (!more) return;
-  }
-}
-template <typename R, bool G, int FC>
-__device__ __forceinline__ void run_species(const StepArgs<R>& A, const StepScalars<R>& S, const R* lnh, const R* lnT,
-                                            TileBuf<R>* buf, uint64_t* full, uint64_t* empty, uint32_t& k,
-                                            uint32_t blk, uint32_t nblk, const TileRun& run, int lane, int warp,
-                                            Acc<R>& acc, EventQueue<R>& q, bool& stopped, int& s_abort) {
-  if (run.s == 0)
-    run_tiles<R, G, FC, 0>(A, S, lnh, lnT, buf, full, empty, k, blk, nblk, run, lane, warp, acc, q, stopped, s_abort);
-  else if (run.s == 1)
-    run_tiles<R, G, FC, 1>(A, S, lnh, lnT, buf, full, empty, k, blk, nblk, run, lane, warp, acc, q, stopped, s_abort);
-  else
-    run_tiles<R, G, FC, 2>(A, S, lnh, lnT, buf, full, empty, k, blk, nblk, run, lane, warp, acc, q, stopped, s_abort);
-}
-
 // One batch step of every live slot in one persistent launch.  Block blk takes the global tiles
 // blk, blk + G, blk + 2G, ... (G = gridDim.x), whatever slot they belong to, so every block gets
 // an equal share of tiles in one wave.  Inside a slot, block blk takes exactly the slot-local
@@ -1921,7 +2056,7 @@ __device__ __forceinline__ void run_species(const StepArgs<R>& A, const StepScal
 // barrier) when their tiles move on to the next slot, after taking the events queued for it and
 // writing its ledger partial.
 template <typename R, bool G>
-__global__ void __launch_bounds__(kStepThreads, sizeof(R) == 4 ? QED_STEP_MIN_BLOCKS : 1)
+__global__ void __launch_bounds__(kStepThreads, sizeof(R) == 4 ? QED_BATCH_MIN_BLOCKS : 1)
 batch_step_kernel(const BatchCtl<R> c) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   TileBuf<R>* buf = reinterpret_cast<TileBuf<R>*>(smem_raw);
@@ -1979,40 +2114,32 @@ batch_step_kernel(const BatchCtl<R> c) {
     return;  // the producer takes part in no later barrier
   }
   // ---------------- compute warps
-  EventQueue<R> q{ring + warp, 0u, 0u};
-  Acc<R> acc;
-  if (lane == 0) q.r->sums = EventSums<R>{};
+  WarpState<R> w;
+  w.q = EventQueue<R>{ring + warp, 0u, 0u};
+  if (lane == 0) w.q.r->sums = EventSums<R>{};
   __syncwarp();
+  const StepPipe<R> P{buf, full, empty, ring, s_lnh, s_lnT, &s_abort, blk, nblk};
   TileRun run;
   int cur = -1;
   uint32_t part = 0;
-  bool stopped = false;  // a wait gave up: no more waits or work, but every slot barrier is kept
   const int nw = (int)(sizeof(StepArgs<R>) / 8), ns = (int)(sizeof(StepScalars<R>) / 8);
   static_assert(sizeof(StepArgs<R>) % 8 == 0 && sizeof(StepScalars<R>) % 8 == 0, "8-byte words");
   auto flush_slot = [&]() {
-    __syncwarp();
-    add_work(acc, s_work, lane);
-    if (A.want) {
-      if (lane == 0) {
-        const EventSums<R>& es = q.r->sums;
-        for (int k = 0; k < 3; ++k) { acc.e[k].merge(es.e[k]); acc.n[k] += es.n[k]; }
-        acc.emit_e = es.emit_e; acc.emit_def = es.emit_def;
-        acc.pair_e = es.pair_e; acc.pair_def = es.pair_def;
-        acc.emit_n = es.emit_n; acc.drop = es.drop; acc.pair_n = es.pair_n;
-        q.r->sums = EventSums<R>{};
-      }
-      __syncwarp();
-      write_ledger_partial<R, kWarps, true>(acc, A.ledger_part, part);
-    }
-    acc = Acc<R>{};
-    compute_warps_sync();  // every warp has added its work
+    add_work(w.pushed_ph, w.tau_ph, s_work, lane);
+    w.pushed_ph = w.tau_ph = 0;
+    compute_warps_sync();  // every warp has added its work and its sums
     if (threadIdx.x == 0) {
       flush_work(s_work, A.work);
       s_work[0] = s_work[1] = 0;
     }
+    if (A.want) {
+      write_step_partial<R>(ring, A.ledger_part, part);
+      compute_warps_sync();
+      if (lane == 0) w.q.r->sums = EventSums<R>{};
+    }
   };
-  for (uint32_t k = 0;;) {
-    const uint32_t g = blk + k * nblk;
+  for (;;) {
+    const uint32_t g = blk + w.k * nblk;
     if (g >= ttot) break;
     find_run(c.splan, c.S, g, run);
     if (run.slot != cur) {
@@ -2023,28 +2150,22 @@ batch_step_kernel(const BatchCtl<R> c) {
           static_cast<const StepScalars<R>*>(c.scal) + run.slot);
       unsigned long long* da = reinterpret_cast<unsigned long long*>(&A);
       unsigned long long* ds = reinterpret_cast<unsigned long long*>(&S);
-      for (int w = threadIdx.x; w < nw; w += kBlock) da[w] = sa[w];
-      for (int w = threadIdx.x; w < ns; w += kBlock) ds[w] = ss[w];
+      for (int q = threadIdx.x; q < nw; q += kBlock) da[q] = sa[q];
+      for (int q = threadIdx.x; q < ns; q += kBlock) ds[q] = ss[q];
       compute_warps_sync();
       cur = run.slot;
       part = g - run.slot_lo;  // < G: the block's first tile of the slot
     }
-    // the block's tiles of this run (one slot, one species), compiled for its species and field
-    // class (a batch with a grid field runs the grid-capable instantiation: the general class only)
-    if (!G && S.kind == QED_FIELD_PLANE_LP)
-      run_species<R, G, G ? kFieldAny : kFieldLP>(A, S, s_lnh, s_lnT, buf, full, empty, k, blk, nblk, run, lane, warp,
-                                                  acc, q, stopped, s_abort);
-    else if (!G && S.kind == QED_FIELD_PLANE_CP)
-      run_species<R, G, G ? kFieldAny : kFieldCP>(A, S, s_lnh, s_lnT, buf, full, empty, k, blk, nblk, run, lane, warp,
-                                                  acc, q, stopped, s_abort);
-    else
-      run_species<R, G, kFieldAny>(A, S, s_lnh, s_lnT, buf, full, empty, k, blk, nblk, run, lane, warp, acc, q, stopped,
-                                   s_abort);
+    // (a batch with a grid field runs the grid-capable instantiation: the general class only)
+    if (A.want) run_species<R, G, true>(A, S, P, run, w);
+    else run_species<R, G, false>(A, S, P, run, w);
   }
-  // a wait that gave up leaves the step unfinished (QED_ERR_TIMEOUT): events still in the ring
+  // a wait that gave up leaves the step unfinished (QED_ERR_TIMEOUT): events still in the rings
   // are not taken
   if (cur >= 0) flush_slot();
 }
+
+constexpr int kMaxScatterSlots = 4096;  // slots of a batch at most
 
 // Per-slot plan (one block per live slot): the exclusive prefixes of its species' coarse event
 // counts, the merge plan, the slot's ledger (from its partials 0 .. min(its tiles, G) - 1) where it
@@ -2084,7 +2205,6 @@ __global__ void __launch_bounds__(256) batch_plan_kernel(const BatchCtl<R> c, in
 // The new particles of every live slot, ranked and moved into place (place_child) by a grid that
 // strides through all slots' children together; the first threads of block 0 then set each
 // slot's counters and advance its step.
-constexpr int kMaxScatterSlots = 4096;
 template <typename R>
 __global__ void __launch_bounds__(256) batch_scatter_kernel(const BatchCtl<R> c) {
   __shared__ uint32_t s_base[kMaxScatterSlots + 1];
@@ -2119,6 +2239,85 @@ __global__ void __launch_bounds__(256) batch_scatter_kernel(const BatchCtl<R> c)
       c.args[sl].step = a.step + 1;  // the slot's next step
       c.remaining[sl] -= 1u;
     }
+}
+
+// A photon window in a batch (24 scenarios of 1e3 to 2e5 electrons, 256 steps on GB300: 106 -> 82 ms
+// with it, 57 ms with the block-wide event batches and the guides): first the field scalars of every live slot's window steps (one thread
+// each, 16 per slot) and the photons it takes, then the photons of all slots, in units of 4096 that
+// a persistent grid strides through (a unit lies in one slot; its 8 warps share its chunks).
+__global__ void __launch_bounds__(128) batch_window_prepare_kernel(const BatchCtl<float> c, int W, int end) {
+  pdl_wait();
+  pdl_launch();
+  const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x), sl = t / kWinMax, k = t % kWinMax;
+  if (sl >= c.S) return;
+  const StepArgs<float>& a = c.args[sl];
+  const uint32_t rem = c.remaining[sl];
+  if (rem == 0u) return;
+  const uint32_t K = win_steps(c, rem, W, end);
+  if (k == 0) a.sp[2].cnt->win_n = K ? a.sp[2].cnt->n & ~1023u : 0u;
+  if ((uint32_t)k < K)
+    make_scalars<float>(a.field, a.t0 + (double)(a.step + k) * a.dt, a.win_x0, a.win_v,
+                        static_cast<StepScalars<float>*>(c.wscal)[sl * kWinMax + k]);
+}
+
+constexpr uint32_t kUnitChunks = 128;  // chunks of 32 photons per unit
+template <bool G>
+__global__ void __launch_bounds__(kFuseThreads) batch_window_kernel(const BatchCtl<float> c, int W, int end) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  WinShared& sh = *reinterpret_cast<WinShared*>(smem_raw);
+  float2* cell = reinterpret_cast<float2*>(smem_raw + sizeof(WinShared));
+  __shared__ __align__(16) StepArgs<float> A;
+  __shared__ uint32_t s_base[kMaxScatterSlots + 1];  // exclusive prefix of the slots' units
+  load_cells(c.tab, cell);
+  pdl_wait();
+  pdl_launch();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = (c.S + kFuseThreads - 1) / kFuseThreads;
+  const int s0 = threadIdx.x * per, s1 = min(c.S, s0 + per);
+  uint32_t mine = 0;
+  for (int sl = s0; sl < s1; ++sl) {
+    uint32_t u = 0;
+    if (c.remaining[sl] > 0u) u = ((c.args[sl].sp[2].cnt->win_n >> 5) + kUnitChunks - 1) / kUnitChunks;
+    s_base[sl] = u;
+    mine += u;
+  }
+  __syncthreads();
+  uint32_t tot;
+  uint32_t run = block_exclusive_scan(mine, &tot);
+  for (int sl = s0; sl < s1; ++sl) { const uint32_t u = s_base[sl]; s_base[sl] = run; run += u; }
+  if (threadIdx.x == 0) s_base[c.S] = tot;
+  __syncthreads();
+  int cur = -1, K = 0;
+  uint32_t pushed = 0;
+  for (uint32_t u = blockIdx.x; u < tot; u += gridDim.x) {
+    int lo = cur < 0 ? 0 : cur, hi = c.S;  // s_base[lo] <= u < s_base[hi]
+    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (s_base[mid] <= u) lo = mid; else hi = mid; }
+    if (lo != cur) {
+      if (cur >= 0) {
+        pushed = __reduce_add_sync(kFull, pushed);
+        if (lane == 0) add_window_work(A, pushed);
+        pushed = 0;
+      }
+      __syncthreads();
+      const unsigned long long* src = reinterpret_cast<const unsigned long long*>(c.args + lo);
+      for (int w = threadIdx.x; w < (int)(sizeof(StepArgs<float>) / 8); w += kFuseThreads)
+        reinterpret_cast<unsigned long long*>(&A)[w] = src[w];
+      K = (int)win_steps(c, c.remaining[lo], W, end);
+      const StepScalars<float>* ws = static_cast<const StepScalars<float>*>(c.wscal) + lo * kWinMax;
+      const unsigned long long* wsrc = reinterpret_cast<const unsigned long long*>(ws);
+      for (int w = threadIdx.x; w < K * (int)(sizeof(StepScalars<float>) / 8); w += kFuseThreads)
+        reinterpret_cast<unsigned long long*>(sh.S)[w] = wsrc[w];
+      if ((int)threadIdx.x < K) sh.pair[threadIdx.x] = window_pair(ws[threadIdx.x].kind, ws[threadIdx.x]);
+      __syncthreads();
+      cur = lo;
+    }
+    const uint32_t c0 = (u - s_base[cur]) * kUnitChunks;
+    pushed += window_photons<G>(A, K, c0 + warp, min(c0 + kUnitChunks, A.sp[2].cnt->win_n >> 5), kFuseThreads / 32, sh, cell);
+  }
+  if (cur >= 0) {
+    pushed = __reduce_add_sync(kFull, pushed);
+    if (lane == 0) add_window_work(A, pushed);
+  }
 }
 
 // Multi-step passes in a batch (when fuse_k >= 2): every live slot probes up to
@@ -2389,9 +2588,9 @@ static size_t step_smem(int n_eta, int n_chi) {
 template <typename R>
 static int step_blocks_per_sm(size_t smem) {
   if (smem > 48 * 1024)
-    cudaFuncSetAttribute(step_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(step_kernel<R, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int b = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, step_kernel<R, false>, kStepThreads, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, step_kernel<R, false, false>, kStepThreads, smem);
   return b > 0 ? b : 1;
 }
 
@@ -2410,23 +2609,31 @@ void launch_step(const StepArgs<R>& a, int grid, int block, size_t smem_unused, 
   const size_t smem = step_smem<R>(a.tab.n_eta, a.tab.n_chi);
   // the grid-capable instantiation runs in waves if it fits fewer blocks per SM; the analytic-field
   // one sets the persistent grid size
-  if (a.field.kind == QED_FIELD_GRID) {
-    if (smem > 48 * 1024)
-      cudaFuncSetAttribute(step_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(step_kernel<R, true>, grid, kStepThreads, smem, s, a);
-  } else {
-    if (smem > 48 * 1024)
-      cudaFuncSetAttribute(step_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(step_kernel<R, false>, grid, kStepThreads, smem, s, a);
-  }
+  const bool g = a.field.kind == QED_FIELD_GRID;
+  const auto k = a.want ? (g ? step_kernel<R, true, true> : step_kernel<R, false, true>)
+                        : (g ? step_kernel<R, true, false> : step_kernel<R, false, false>);
+  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  launch_pdl(k, grid, kStepThreads, smem, s, a);
   count_launch();
 }
 
 #endif
 
 #if QED_PART(2)
+void launch_batch_window(const BatchCtl<float>& c, int n_chi, int W, BatchEnd end, cudaStream_t s) {
+  launch_pdl(batch_window_prepare_kernel, (c.S * kWinMax + 127) / 128, 128, 0, s, c, W, (int)end);
+  const size_t smem = window_smem(n_chi);
+  const auto k = c.grid_fields ? batch_window_kernel<true> : batch_window_kernel<false>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int b = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, kFuseThreads, smem);
+  launch_pdl(k, sm_count() * std::max(b, 1), kFuseThreads, smem, s, c, W, (int)end);
+  count_launch(2);
+}
+
 template <typename R>
-void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, bool want, cudaStream_t s) {
+void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, BatchEnd end, int win_w, BatchEnd win_end, int win_s,
+                       cudaStream_t s) {
   const size_t smem = step_smem<R>(n_eta, n_chi);
   if (smem + sizeof(StepArgs<R>) + sizeof(StepScalars<R>) > 40 * 1024) {
     cudaFuncSetAttribute(batch_step_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -2448,7 +2655,7 @@ void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, bool want, cu
     count_launch(5);
   }
   // the per-step path: one tile space over all live slots, strided by a persistent grid
-  launch_pdl(batch_tiles_kernel<R>, 1, 1024, 0, s, c, want ? 1 : 0);
+  launch_pdl(batch_tiles_kernel<R>, 1, 1024, 0, s, c, (int)end, win_w, (int)win_end, win_s);
   if (c.grid_fields) launch_pdl(batch_step_kernel<R, true>, c.target_blocks, kStepThreads, smem, s, c);
   else launch_pdl(batch_step_kernel<R, false>, c.target_blocks, kStepThreads, smem, s, c);
   launch_pdl(batch_plan_kernel<R>, c.S, 256, 0, s, c, c.target_blocks);
@@ -2767,8 +2974,8 @@ QED_INSTANTIATE_STEP(float)
 QED_INSTANTIATE_STEP(double)
 #endif
 #if QED_PART(2)
-template void launch_batch_step<float>(const BatchCtl<float>&, int, int, bool, cudaStream_t);
-template void launch_batch_step<double>(const BatchCtl<double>&, int, int, bool, cudaStream_t);
+template void launch_batch_step<float>(const BatchCtl<float>&, int, int, BatchEnd, int, BatchEnd, int, cudaStream_t);
+template void launch_batch_step<double>(const BatchCtl<double>&, int, int, BatchEnd, int, BatchEnd, int, cudaStream_t);
 #endif
 #if QED_PART(3)
 #define QED_INSTANTIATE(R)                                                                                       \

@@ -96,3 +96,36 @@ def test_windows_respect_the_switches(tables):
             qed.check(sp)
             out.append([s.save() for s in sp])
         assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("graph_steps", [0, 8, 32])
+def test_batch_windows_match_single_runs(tables, graph_steps):
+    # slots of every field, with different steps left, advanced by calls that end inside and at the
+    # end of a graph: each slot's particles and ledger are those of its own run
+    kinds = ["uniform", "rotating", "lp", "cp", "lp", "rotating"]
+    sizes = [(1023, 40), (5000, 37), (3071, 17), (2048, 2), (1100, 1), (20000, 40)]
+    first = 5
+
+    def params(k):
+        return qed.StepParams(dt=DT, t0=-10 * DT, seed=11, scenario=k, field=field(kinds[k]), window_x0=100.0,
+                              window_v=-0.5)
+
+    refs = []
+    for k, (n_g, steps) in enumerate(sizes):
+        sp = population(20 + k, 400, n_g, weights=k == 1)
+        qed.run(tables, sp, params(k), first, steps)
+        refs.append((sp, qed.work_read(sp[0])))
+    batch = qed.Batch(tables, qed.MIXED, len(sizes) + 1)
+    batch.config(0, graph_steps)
+    mix = [population(20 + k, 400, n_g, weights=k == 1) for k, (n_g, _) in enumerate(sizes)]
+    for k, sp in enumerate(mix):
+        batch.attach(k, sp, params(k), first, sizes[k][1])
+    for n in (8, 1, 2, 16, 3, 32):
+        batch.run(n)
+    assert np.all(batch.remaining() == 0)
+    for k, ((ref, wr), sp) in enumerate(zip(refs, mix)):
+        qed.check(sp)
+        for a, b in zip(ref, sp):
+            assert np.array_equal(a.save(), b.save()), f"slot {k}"
+        assert qed.read_ledger(ref) == qed.read_ledger(sp)
+        assert wr == qed.work_read(sp[0])
