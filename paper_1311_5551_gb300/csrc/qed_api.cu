@@ -319,6 +319,7 @@ struct qed_species {
   void* other_w = nullptr;
   uint32_t* seg_count = nullptr;
   uint32_t* seg_prefix = nullptr;
+  uint32_t* merge_counts = nullptr;  // digit counts of merging's sort (1/16 word per particle)
   int last_drain = 0;
 };
 
@@ -651,7 +652,7 @@ namespace {
 // then becomes the species' arrays.  The second set (and the scan scratch) is allocated at the
 // first compaction.
 template <typename R>
-qed_status compact_impl(qed_species* sp, SpeciesDev<R>& cur, cudaStream_t s) {
+qed_status ensure_second_set(qed_species* sp, const SpeciesDev<R>& cur, cudaStream_t s) {
   const size_t cap = sp->cap, segs = cap / 2048 + 2;
   if (!sp->alt_mem.ptr) {
     Carver cv;
@@ -659,6 +660,7 @@ qed_status compact_impl(qed_species* sp, SpeciesDev<R>& cur, cudaStream_t s) {
     cv.add(&b.x, cap); cv.add(&b.y, cap); cv.add(&b.z, cap); cv.add(&b.ux, cap); cv.add(&b.uy, cap);
     cv.add(&b.uz, cap); cv.add(&b.tau, cap); cv.add(&b.id, cap);
     cv.add(&sp->seg_count, segs); cv.add(&sp->seg_prefix, segs + 1);
+    cv.add(&sp->merge_counts, 256 * (cap / 4096 + 2));
     qed_status st = sp->alt_mem.get(cv.total(), sp->have_alloc ? &sp->alloc_copy : nullptr, s);
     if (st != QED_OK) return st;
     cv.bind(sp->alt_mem.ptr);
@@ -671,6 +673,13 @@ qed_status compact_impl(qed_species* sp, SpeciesDev<R>& cur, cudaStream_t s) {
     if (st != QED_OK) return st;
     sp->other_w = sp->alt_wmem.ptr;
   }
+  return QED_OK;
+}
+
+template <typename R>
+qed_status compact_impl(qed_species* sp, SpeciesDev<R>& cur, cudaStream_t s) {
+  qed_status st = ensure_second_set(sp, cur, s);
+  if (st != QED_OK) return st;
   SpeciesDev<R> out = cur;
   out.x = (R*)sp->other[0]; out.y = (R*)sp->other[1]; out.z = (R*)sp->other[2];
   out.ux = (R*)sp->other[3]; out.uy = (R*)sp->other[4]; out.uz = (R*)sp->other[5];
@@ -749,10 +758,15 @@ extern "C" qed_status qed_species_merge(qed_species* sp, const qed_merge_params*
       return fail(QED_ERR_INVALID_ARG, "qed_species_merge: cells must be finite, > 0 and at least one per axis");
     cells *= (uint64_t)m->n_cells[a];
     md.origin[a] = m->origin[a]; md.cell[a] = m->cell[a]; md.n_cells[a] = m->n_cells[a];
+    md.inv_cell[a] = (float)(1.0 / m->cell[a]);
   }
   if (cells > 0xffffffffull || 6ull * m->n_face * m->n_face > 0xffffull || (uint64_t)m->n_sub * 2200 > 0xffffull)
     return fail(QED_ERR_INVALID_ARG, "qed_species_merge: too many bins for the 64-bit group key");
   md.n_face = m->n_face; md.n_sub = m->n_sub; md.min_group = m->min_group;
+  md.n_dir = 6ull * m->n_face * m->n_face;
+  md.n_en = 2200ull * m->n_sub;
+  md.none = cells * md.n_dir * md.n_en;  // < 2^64: each factor is bounded above
+  while (md.bits < 64 && (md.none >> md.bits) != 0) ++md.bits;
   cudaStream_t s = as_stream(stream);
   DevCounters c;
   qed_status st = read_counters(sp, c, s);
@@ -761,23 +775,33 @@ extern "C" qed_status qed_species_merge(qed_species* sp, const qed_merge_params*
   if (c.n < 3) return QED_OK;
   st = ensure_weights(sp, s);  // merged particles carry weights other than 1
   if (st != QED_OK) return st;
+  // The first buffer of (key, index) pairs comes from the allocator the species was created with (the
+  // library does not allocate on its own behalf) and is given back before the call returns; the
+  // second one lies in the species' second array set, which the compaction below fills afterwards (the
+  // sort's counts are beside that set).
+  st = sp->precision == QED_MIXED ? ensure_second_set(sp, sp->f, s) : ensure_second_set(sp, sp->d, s);
+  if (st != QED_OK) return st;
   uint32_t N = 1;
   while (N < c.n) N <<= 1;
-  // sort scratch through the allocator the species was created with (the library does not
-  // allocate on its own behalf)
   const size_t bytes = (size_t)N * 12 + 256;
   DeviceBlock scratch;
   st = scratch.get(bytes, sp->have_alloc ? &sp->alloc_copy : nullptr, s);
   if (st != QED_OK) return st;
   char* tmp = static_cast<char*>(scratch.ptr);
-  uint64_t* keys = reinterpret_cast<uint64_t*>(tmp);
-  uint32_t* idx = reinterpret_cast<uint32_t*>(tmp + (size_t)N * 8);
   unsigned long long* groups = reinterpret_cast<unsigned long long*>(tmp + (size_t)N * 12 + 128);
-  cudaError_t e = cudaMemsetAsync(groups, 0, 8, s);
+  MergeScratch w;
+  w.keys[0] = tmp;
+  w.idx[0] = reinterpret_cast<uint32_t*>(tmp + (size_t)N * 8);
+  w.keys[1] = sp->other_tau;
+  w.idx[1] = sp->other_id;
+  w.hist = sp->merge_counts;
+  w.totals = w.hist + 256 * (sp->cap / 4096 + 1);
+  w.count = reinterpret_cast<uint32_t*>(groups + 1);
+  cudaError_t e = cudaMemsetAsync(groups, 0, 16, s);
   if (e != cudaSuccess) { scratch.release(); return cuda_fail(e, "cudaMemsetAsync"); }
   const int massless = sp->kind == QED_PHOTON ? 1 : 0;
-  if (sp->precision == QED_MIXED) launch_merge<float>(sp->f, md, keys, idx, N, massless, groups, s);
-  else launch_merge<double>(sp->d, md, keys, idx, N, massless, groups, s);
+  if (sp->precision == QED_MIXED) launch_merge<float>(sp->f, md, w, c.n, massless, groups, s);
+  else launch_merge<double>(sp->d, md, w, c.n, massless, groups, s);
   unsigned long long g = 0;
   e = read_on(&g, groups, 8, s);
   scratch.release();  // ordered after the merge kernels on s

@@ -248,10 +248,21 @@ void launch_totals(const SpeciesDev<R>& sp, int massless, double* partials, int 
 struct MergeDev {
   double origin[3], cell[3];
   int n_cells[3], n_face, n_sub, min_group;
+  uint64_t n_dir, n_en;  // direction and energy bins
+  uint64_t none;         // cells * n_dir * n_en: the key of a photon that is not merged
+  int bits;              // of the keys 0 .. none
+  float inv_cell[3];     // 1/cell (the FP32 filter of the keys)
+};
+// Two buffers of n keys (32 or 64 bits, as M.bits needs) and indices; 256 counts per 4096 photons
+// and 256 totals; two zeroed counters.
+struct MergeScratch {
+  void* keys[2];
+  uint32_t* idx[2];
+  uint32_t *hist, *totals, *count;
 };
 template <typename R>
-void launch_merge(const SpeciesDev<R>& sp, const MergeDev& m, uint64_t* keys, uint32_t* idx, uint32_t N,
-                  int massless, unsigned long long* groups, cudaStream_t s);
+void launch_merge(const SpeciesDev<R>& sp, const MergeDev& m, const MergeScratch& w, uint32_t n, int massless,
+                  unsigned long long* groups, cudaStream_t s);
 
 // Device images of a table set (defined with qed_tables in qed_api.cu).
 struct TablesDev {

@@ -2507,22 +2507,39 @@ __global__ void __launch_bounds__(1024) compact_scan_kernel(const SpeciesDev<R> 
 template <typename R>
 __global__ void __launch_bounds__(256) compact_scatter_kernel(const SpeciesDev<R> sp, SpeciesDev<R> out,
                                                               const uint32_t* seg_prefix) {
+  // warp w moves the segment's particles [256 w, 256 w + 256), 32 at a time: its survivors are counted
+  // first, so the block synchronises once per segment (2.4e6 of 3e6 photons: 106 -> 60 us on GB300
+  // against a block-wide scan for every 256)
+  __shared__ uint32_t s_w[8];
   const uint32_t n = sp.cnt->n, nseg = (n + kSeg - 1) / kSeg;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kRounds = kSeg / 256;
   for (uint32_t g = blockIdx.x; g < nseg; g += gridDim.x) {
+    const uint32_t first = g * kSeg + (uint32_t)warp * (kRounds * 32u) + (uint32_t)lane;
+    unsigned keep[kRounds];
+    uint32_t mine = 0;
+#pragma unroll
+    for (int q = 0; q < kRounds; ++q) {
+      const uint32_t i = first + 32u * q;
+      keep[q] = __ballot_sync(kFull, i < n && !Tau<R>::load(sp.tau + i).dead());
+      mine += (uint32_t)__popc(keep[q]);
+    }
+    __syncthreads();  // the last segment's counts have been read
+    if (lane == 0) s_w[warp] = mine;
+    __syncthreads();
     uint32_t base = seg_prefix[g];
-    for (uint32_t i0 = g * kSeg; i0 < min(n, (g + 1) * kSeg); i0 += blockDim.x) {
-      const uint32_t i = i0 + threadIdx.x;
-      const bool keep = i < n && !Tau<R>::load(sp.tau + i).dead();
-      uint32_t tot;
-      const uint32_t ex = block_exclusive_scan(keep ? 1u : 0u, &tot);
-      if (keep) {
-        const uint32_t o = base + ex;
+    for (int w = 0; w < warp; ++w) base += s_w[w];
+#pragma unroll
+    for (int q = 0; q < kRounds; ++q) {
+      const uint32_t i = first + 32u * q;
+      if (keep[q] >> lane & 1u) {
+        const uint32_t o = base + (uint32_t)__popc(keep[q] & ((1u << lane) - 1u));
         out.x[o] = sp.x[i]; out.y[o] = sp.y[i]; out.z[o] = sp.z[i];
         out.ux[o] = sp.ux[i]; out.uy[o] = sp.uy[i]; out.uz[o] = sp.uz[i];
         out.tau[o] = sp.tau[i]; out.id[o] = sp.id[i];
         if (sp.w) out.w[o] = sp.w[i];
       }
-      base += tot;
+      base += (uint32_t)__popc(keep[q]);
     }
   }
 }
@@ -2818,7 +2835,7 @@ __global__ void __launch_bounds__(256) totals_kernel(const SpeciesDev<R> sp, int
 
 // Group key of a photon for merging, or ~0 when it is not merged: position cell, cube-face
 // direction bin and binary-exponent energy bin, from exact operations only (divisions, floor,
-// frexp) in double, so that it equals the key any other IEEE double implementation computes.
+// frexp) in double, so that it names the same groups as any other IEEE double implementation.
 __device__ uint64_t merge_key_dev(const double x[3], const double k[3], const MergeDev& M) {
   uint64_t cell = 0;
   for (int a = 2; a >= 0; --a) {
@@ -2845,92 +2862,407 @@ __device__ uint64_t merge_key_dev(const double x[3], const double k[3], const Me
   int sub = (int)floor((mant - 0.5) * 2.0 * M.n_sub);
   if (sub >= M.n_sub) sub = M.n_sub - 1;
   const uint64_t en = (uint64_t)(e2 + 1100) * (uint64_t)M.n_sub + (uint64_t)sub;
-  return (cell << 32) | (dir << 16) | en;
+  return (cell * M.n_dir + dir) * M.n_en + en;  // < M.none
 }
 
-template <typename R>
-__global__ void merge_key_kernel(const SpeciesDev<R> sp, MergeDev M, uint64_t* keys, uint32_t* idx, uint32_t N) {
-  const uint32_t n = sp.cnt->n;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-    uint64_t key = ~0ull;
-    if (i < n && !Tau<R>::load(sp.tau + i).dead()) {
-      const double x[3] = {(double)sp.x[i], (double)sp.y[i], (double)sp.z[i]};
-      const double k[3] = {(double)sp.ux[i], (double)sp.uy[i], (double)sp.uz[i]};
-      key = merge_key_dev(x, k, M);
+// The same key from FP32 arithmetic, for FP32 particles: true where no bin edge is near enough for the
+// rounding to matter (the bounds below are several times the worst error), so the bins are those of
+// the exact operations.  GB300's FP64 pipe made the exact key of 3e6 photons take 620 us (five
+// divisions, a square root and the conversions); with this filter, where about 1 in 1e4 photons
+// needs the exact one, it is 30 us.
+__device__ __forceinline__ bool sure_floor(float t, float err, int& b) {
+  const float f = floorf(t);
+  b = (int)f;
+  return t - f > err && t - f < 1.0f - err;  // false for NaN and for |t| too large for its fraction
+}
+__device__ bool merge_key_fast(const float x[3], const float k[3], const MergeDev& M, uint64_t& key) {
+  uint64_t cell = 0;
+  bool out = false;
+#pragma unroll
+  for (int a = 2; a >= 0; --a) {
+    const float o = (float)M.origin[a], inv = M.inv_cell[a];
+    int c;
+    if (!sure_floor((x[a] - o) * inv, 1e-6f + 1e-6f * (fabsf(x[a]) + fabsf(o)) * inv, c)) return false;
+    out = out || c < 0 || c >= M.n_cells[a];
+    cell = cell * (uint64_t)M.n_cells[a] + (uint64_t)(uint32_t)c;
+  }
+  const float ka[3] = {fabsf(k[0]), fabsf(k[1]), fabsf(k[2])};
+  int ax = 0;
+  float m = ka[0];
+  if (ka[1] > m) { ax = 1; m = ka[1]; }
+  if (ka[2] > m) { ax = 2; m = ka[2]; }
+  if (!(m > 1e-15f && m < 1e15f)) return false;  // (zero momenta, and squares that would leave the range)
+  if (out) { key = ~0ull; return true; }
+  const float kx = ax == 0 ? k[0] : (ax == 1 ? k[1] : k[2]);
+  const int face = 2 * ax + (kx < 0.0f ? 1 : 0);
+  const float im = 1.0f / m, half = 0.5f * (float)M.n_face;
+  int fb[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const float v = q == 0 ? (ax == 0 ? k[1] : k[0]) : (ax == 2 ? k[1] : k[2]);
+    if (v == 0.0f) {  // exactly the middle
+      fb[q] = M.n_face / 2;
+    } else {
+      if (!sure_floor((v * im + 1.0f) * half, 2e-6f * (float)M.n_face, fb[q])) return false;
+      if (fb[q] < 0 || fb[q] >= M.n_face) return false;
     }
-    keys[i] = key;
+  }
+  const uint64_t dir = ((uint64_t)face * M.n_face + fb[0]) * M.n_face + fb[1];
+  const float e = sqrtf(fmaf(k[0], k[0], fmaf(k[1], k[1], k[2] * k[2])));
+  const int bits = __float_as_int(e);
+  const int e2 = (bits >> 23) - 126;                                      // e = mant 2^e2, mant in [1/2, 1)
+  const float mant = __int_as_float((bits & 0x7fffff) | 0x3f000000);
+  int sub;
+  const float n_sub = (float)M.n_sub;
+  if (!sure_floor((mant - 0.5f) * 2.0f * n_sub, 2e-6f * n_sub, sub)) return false;  // (power-of-two edges among them)
+  const uint64_t en = (uint64_t)(e2 + 1100) * (uint64_t)M.n_sub + (uint64_t)sub;
+  key = (cell * M.n_dir + dir) * M.n_en + en;
+  return true;
+}
+
+template <typename R, typename K>
+__global__ void merge_key_kernel(const SpeciesDev<R> sp, MergeDev M, K* keys, uint32_t* idx, uint32_t n) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    uint64_t key = ~0ull;
+    if (!Tau<R>::load(sp.tau + i).dead()) {
+      bool sure = false;
+      if constexpr (sizeof(R) == 4) {
+        const float x[3] = {sp.x[i], sp.y[i], sp.z[i]}, k[3] = {sp.ux[i], sp.uy[i], sp.uz[i]};
+        sure = merge_key_fast(x, k, M, key);
+      }
+      if (!sure) {
+        const double x[3] = {(double)sp.x[i], (double)sp.y[i], (double)sp.z[i]};
+        const double k[3] = {(double)sp.ux[i], (double)sp.uy[i], (double)sp.uz[i]};
+        key = merge_key_dev(x, k, M);
+      }
+    }
+    keys[i] = key == ~0ull ? (K)M.none : (K)key;
     idx[i] = i;
   }
 }
 
-// One compare-exchange pass of a bitonic sort of (key, index) pairs (N a power of two): the
-// result is ordered by key, and by index within a key.
-__global__ void bitonic_pass_kernel(uint64_t* keys, uint32_t* idx, uint32_t N, uint32_t k, uint32_t j) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-    const uint32_t l = i ^ j;
-    if (l <= i) continue;
-    const bool asc = (i & k) == 0u;
-    const uint64_t ka = keys[i], kb = keys[l];
-    const uint32_t ia = idx[i], ib = idx[l];
-    const bool greater = ka > kb || (ka == kb && ia > ib);
-    if (greater == asc) {
-      keys[i] = kb; keys[l] = ka;
-      idx[i] = ib; idx[l] = ia;
+// ----------------------------------------------------------------------------- radix sort
+// Stable sort of (key, index) pairs by 8 bits at a time, least significant first, so equal keys keep
+// their order (by index).  A pass is three launches: digit counts per segment of 4096 pairs, their
+// prefixes (one block per digit), and the scatter, which ranks a segment's pairs by warp match and
+// per-warp counts.  Memory-bound: a pass reads the keys twice and the indices once and writes both,
+// 20 B per pair with 32-bit keys, and the merging bins in use need 29 bits, so 4 passes; the bitonic
+// network before it took log2(n)(log2(n)+1)/2 passes of 24 B (253 at 3e6 photons).
+constexpr uint32_t kSortItems = 16;                          // pairs per thread
+constexpr uint32_t kSortSeg = 256 * kSortItems;
+template <typename K>
+__device__ __forceinline__ uint32_t digit_of(K key, int shift) { return (uint32_t)(key >> shift) & 255u; }
+
+template <typename K>
+__global__ void __launch_bounds__(256) radix_count_kernel(const K* keys, uint32_t n, int shift, uint32_t* hist) {
+  __shared__ uint32_t s_h[256];
+  s_h[threadIdx.x] = 0;
+  __syncthreads();
+  const uint32_t first = blockIdx.x * kSortSeg, last = min(n, first + kSortSeg);
+  for (uint32_t i = first + threadIdx.x; i < last; i += 256) atomicAdd(&s_h[digit_of(keys[i], shift)], 1u);
+  __syncthreads();
+  hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s_h[threadIdx.x];
+}
+
+// Block d: exclusive prefixes of digit d's counts over the segments; totals[d] their sum.
+__global__ void __launch_bounds__(256) radix_scan_kernel(uint32_t* hist, uint32_t segs, uint32_t* totals) {
+  uint32_t* h = hist + (size_t)blockIdx.x * segs;
+  uint32_t base = 0;
+  for (uint32_t k0 = 0; k0 < segs; k0 += 1024) {
+    uint32_t v[4], sum = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t k = k0 + threadIdx.x * 4 + q;
+      v[q] = k < segs ? h[k] : 0u;
+      sum += v[q];
     }
+    uint32_t tot;
+    uint32_t run = base + block_exclusive_scan(sum, &tot);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t k = k0 + threadIdx.x * 4 + q;
+      if (k < segs) h[k] = run;
+      run += v[q];
+    }
+    base += tot;
+  }
+  if (threadIdx.x == 0) totals[blockIdx.x] = base;
+}
+
+template <typename K>
+__global__ void __launch_bounds__(256) radix_scatter_kernel(const K* keys, const uint32_t* idx, K* keys_out,
+                                                            uint32_t* idx_out, uint32_t n, int shift, const uint32_t* hist,
+                                                            const uint32_t* totals) {
+  __shared__ uint32_t s_c[8][256];  // per warp and digit: pairs seen, then where the warp's begin
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int w = 0; w < 8; ++w) s_c[w][threadIdx.x] = 0;
+  __syncthreads();
+  // warp w takes the segment's pairs [512 w, 512 w + 512), 32 consecutive ones at a time
+  const uint32_t first = blockIdx.x * kSortSeg + (uint32_t)warp * (kSortItems * 32u) + (uint32_t)lane;
+  K key[kSortItems];
+  uint32_t id[kSortItems], rank[kSortItems];
+#pragma unroll
+  for (uint32_t q = 0; q < kSortItems; ++q) {
+    const uint32_t i = first + 32u * q;
+    key[q] = i < n ? keys[i] : (K)0;
+    id[q] = i < n ? idx[i] : 0u;
+  }
+#pragma unroll
+  for (uint32_t q = 0; q < kSortItems; ++q) {
+    const bool in = first + 32u * q < n;
+    const uint32_t d = in ? digit_of(key[q], shift) : 256u;
+    const unsigned same = __match_any_sync(kFull, d);
+    const uint32_t before = in ? s_c[warp][d] : 0u;
+    __syncwarp();
+    if (in && lane == __ffs(same) - 1) s_c[warp][d] = before + (uint32_t)__popc(same);
+    __syncwarp();
+    rank[q] = before + (uint32_t)__popc(same & ((1u << lane) - 1u));
+  }
+  __syncthreads();
+  // thread d: where digit d's pairs of each warp begin
+  uint32_t run = block_exclusive_scan(totals[threadIdx.x], nullptr) + hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x];
+  for (int w = 0; w < 8; ++w) {
+    const uint32_t c = s_c[w][threadIdx.x];
+    s_c[w][threadIdx.x] = run;
+    run += c;
+  }
+  __syncthreads();
+#pragma unroll
+  for (uint32_t q = 0; q < kSortItems; ++q) {
+    if (first + 32u * q >= n) continue;
+    const uint32_t o = s_c[warp][digit_of(key[q], shift)] + rank[q];
+    keys_out[o] = key[q];
+    idx_out[o] = id[q];
   }
 }
 
-// One thread per group (at the group's first sorted position): groups of at least min_group
-// photons become two (the two lowest indices) that carry the group's weight, momentum and energy;
-// the others become holes (tau = +inf) that compaction removes.
+// ----------------------------------------------------------------------------- merging groups
+// First positions of the groups in the sorted order (any order): heads[0 .. *count).
+template <typename K>
+__global__ void merge_heads_kernel(const K* keys, uint32_t n, K none, uint32_t* heads, uint32_t* count) {
+  const int lane = threadIdx.x & 31;
+  for (uint32_t p0 = blockIdx.x * blockDim.x; p0 < n; p0 += gridDim.x * blockDim.x) {
+    const uint32_t p = p0 + threadIdx.x;
+    const bool head = p < n && keys[p] != none && (p == 0 || keys[p - 1] != keys[p]);
+    const unsigned m = __ballot_sync(kFull, head);
+    if (!m) continue;
+    uint32_t base = 0;
+    if (lane == 0) base = atomicAdd(count, (uint32_t)__popc(m));
+    base = __shfl_sync(kFull, base, 0);
+    if (head) heads[base + (uint32_t)__popc(m & ((1u << lane) - 1u))] = p;
+  }
+}
+
+// A float as a double by integer operations (conversions share the FP64 pipe); the few that are
+// neither zero nor normal are converted (a call, so that nothing converts ahead of the test).
+__device__ __noinline__ double widen_rare(float v) { return (double)v; }
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = (uint32_t)__float_as_int(v), e = b & 0x7f800000u;
+  if (e == 0x7f800000u || (e == 0u && (b & 0x7fffffffu) != 0u)) return widen_rare(v);
+  if (e == 0u) return __hiloint2double((int)b, 0);
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+// sqrt of a double to its last bit or the one beside it, by two Newton steps from the FP32 reciprocal
+// root (Heron's rule; 7 FP64 operations against about 25); outside FP32's range the function.
+__device__ __forceinline__ double root_newton(double v) {
+  const float f = __double2float_rn(v);
+  if (!(f > 1e-30f && f < 1e30f)) return sqrt(v);
+  const float y = rsqrtf(f);
+  const double h = widen(0.5f * y);
+  double s = v * widen(y);
+  s = fma(fma(-s, s, v), h, s);
+  return fma(fma(-s, s, v), h, s);
+}
+
+constexpr int kMergeSums = 8;  // W, E, P[3], X[3]
+// One member's share of the group's sums.
 template <typename R>
-__global__ void merge_groups_kernel(SpeciesDev<R> sp, MergeDev M, const uint64_t* keys, const uint32_t* idx, uint32_t N,
-                                    int massless, unsigned long long* groups) {
-  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
-    const uint64_t key = keys[p];
-    if (key == ~0ull || (p > 0 && keys[p - 1] == key)) continue;
-    uint32_t q = p + 1;
-    while (q < N && keys[q] == key) ++q;
-    if ((int)(q - p) < M.min_group) continue;
-    double W = 0.0, E = 0.0, P[3] = {0.0, 0.0, 0.0}, X[3] = {0.0, 0.0, 0.0};
-    for (uint32_t r = p; r < q; ++r) {
-      const uint32_t i = idx[r];
-      const double w = sp.w ? (double)sp.w[i] : 1.0;
-      const double k[3] = {(double)sp.ux[i], (double)sp.uy[i], (double)sp.uz[i]};
-      const double x[3] = {(double)sp.x[i], (double)sp.y[i], (double)sp.z[i]};
-      const double k2 = k[0] * k[0] + k[1] * k[1] + k[2] * k[2];
-      W += w;
-      E += w * (massless ? sqrt(k2) : sqrt(1.0 + k2));
-      for (int c = 0; c < 3; ++c) { P[c] += w * k[c]; X[c] += w * x[c]; }
+__device__ __forceinline__ void merge_member(const SpeciesDev<R>& sp, uint32_t i, int massless, double v[kMergeSums]) {
+  const R w = sp.w ? sp.w[i] : (R)1;
+  const double k[3] = {widen(sp.ux[i]), widen(sp.uy[i]), widen(sp.uz[i])};
+  const double x[3] = {widen(sp.x[i]), widen(sp.y[i]), widen(sp.z[i])};
+  double e2 = k[0] * k[0] + k[1] * k[1] + k[2] * k[2];
+  if (!massless) e2 = 1.0 + e2;
+  v[0] = 1.0;
+  v[1] = sizeof(R) == 8 ? sqrt(e2) : root_newton(e2);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) { v[2 + c] = k[c]; v[5 + c] = x[c]; }
+  if (w != (R)1) {  // (unweighted photons: 7 multiplications by one)
+    const double wd = widen(w);
+    v[0] = wd;
+#pragma unroll
+    for (int c = 1; c < kMergeSums; ++c) v[c] = wd * v[c];
+  }
+}
+// The group's survivor number `which` (0 or 1), particle i, from the group's sums.
+template <typename R>
+__device__ void merge_survivor(SpeciesDev<R>& sp, uint32_t i, int which, int massless, const double t[kMergeSums]) {
+  const double W = t[0], E = t[1], *P = t + 2, *X = t + 5;
+  // both members get energy E/W; massive ones sit on the mass shell, |u|^2 = (E/W)^2 - 1
+  const double et = E / W, mv[3] = {P[0] / W, P[1] / W, P[2] / W};
+  const double m2 = mv[0] * mv[0] + mv[1] * mv[1] + mv[2] * mv[2];
+  const double d2 = (massless ? et * et : et * et - 1.0) - m2;
+  const double dl = d2 > 0.0 ? sqrt(d2) : 0.0;
+  int ax = 0;
+  for (int c = 1; c < 3; ++c)
+    if (fabs(mv[c]) < fabs(mv[ax])) ax = c;
+  double e[3] = {0.0, 0.0, 0.0};
+  e[ax] = 1.0;
+  double dv[3] = {mv[1] * e[2] - mv[2] * e[1], mv[2] * e[0] - mv[0] * e[2], mv[0] * e[1] - mv[1] * e[0]};
+  const double dn = sqrt(dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2]);
+  if (dn > 0.0) {
+    for (int c = 0; c < 3; ++c) dv[c] *= dl / dn;
+  } else {
+    for (int c = 0; c < 3; ++c) dv[c] = 0.0;
+    dv[ax] = dl;
+  }
+  const double sg = which == 0 ? 1.0 : -1.0;
+  sp.ux[i] = (R)(mv[0] + sg * dv[0]); sp.uy[i] = (R)(mv[1] + sg * dv[1]); sp.uz[i] = (R)(mv[2] + sg * dv[2]);
+  sp.x[i] = (R)(X[0] / W); sp.y[i] = (R)(X[1] / W); sp.z[i] = (R)(X[2] / W);
+  if (sp.w) sp.w[i] = (R)(0.5 * W);
+}
+
+// Groups of at least min_group photons become two (the two lowest indices) that carry the group's
+// weight, momentum and energy; the others become holes (tau = +inf) that compaction removes.  FP64
+// species: a warp per group, 32 members at a time, sums in index order (lane c adds sum c of the
+// 32), so the results are those of a plain loop.  Mixed: eight lanes per group, each sums its own
+// members and the eight are added in a fixed order; groups of more than kMergeBig members, of which
+// a few hold most of the photons, are left to merge_big_kernel, a block each.  Bound by the FP64
+// pipe, which is why it sees no conversions and no square roots of the mixed path (3e6 photons, 3e4
+// groups on GB300: 408 us, and 378 us for the big ones side by side with 2e6 of the photons; the whole
+// merge, with its upload, 15.6 -> 1.48 ms).
+constexpr uint32_t kMergeBig = 256;
+template <typename R, typename K>
+__global__ void __launch_bounds__(128) merge_groups_kernel(SpeciesDev<R> sp, MergeDev M, const K* keys, const uint32_t* idx,
+                                                           uint32_t n, const uint32_t* heads, const uint32_t* count,
+                                                           uint32_t* big, uint32_t* n_big, int massless,
+                                                           unsigned long long* groups) {
+  constexpr bool kOrdered = sizeof(R) == 8;
+  constexpr int L = kOrdered ? 32 : 8;  // lanes per group
+  __shared__ double s_v[kOrdered ? 4 : 1][kMergeSums][33];
+  const int lane = threadIdx.x & (L - 1), row = kOrdered ? threadIdx.x >> 5 : 0;
+  const unsigned shift = threadIdx.x & (32u - L) & 31u;  // of the group's lanes in a warp's ballot
+  const uint32_t nh = *count, stride = gridDim.x * (128u / L);
+  uint32_t merged = 0, removed = 0;
+  // (the groups of a warp go through their members together)
+  for (uint32_t h0 = blockIdx.x * (128u / L) + (threadIdx.x & ~31u) / L; h0 < nh; h0 += stride) {
+    const uint32_t h = h0 + (threadIdx.x & 31u) / L;
+    bool open = h < nh, whole = open;
+    const uint32_t p = open ? heads[h] : 0u;
+    const K key = keys[p];
+    double acc[kMergeSums];  // ordered: sum `lane` in acc[0]; else the lane's own
+#pragma unroll
+    for (int c = 0; c < kMergeSums; ++c) acc[c] = 0.0;
+    uint32_t size = 0;
+    for (uint32_t r = p + (uint32_t)lane; __any_sync(kFull, open); r += L) {
+      const bool in = open && r < n && keys[r] == key;
+      const unsigned m = __ballot_sync(kFull, in) >> shift;
+      const uint32_t here = (uint32_t)__popc(L == 32 ? m : m & ((1u << (L & 31)) - 1u));  // (the members come first)
+      size += here;
+      if (here < (uint32_t)L) {
+        open = false;
+        whole = whole && size >= (uint32_t)M.min_group;
+      }
+      if (!kOrdered && size > kMergeBig) {
+        if (whole && lane == 0) big[atomicAdd(n_big, 1u)] = p;
+        open = whole = false;
+      }
+      double v[kMergeSums];
+#pragma unroll
+      for (int c = 0; c < kMergeSums; ++c) v[c] = 0.0;
+      if (in && whole) merge_member<R>(sp, idx[r], massless, v);
+      if (kOrdered) {
+#pragma unroll
+        for (int c = 0; c < kMergeSums; ++c) s_v[row][c][lane] = v[c];
+        __syncwarp();
+        if (lane < kMergeSums)
+          for (uint32_t t = 0; t < here; ++t) acc[0] += s_v[row][lane][t];
+        __syncwarp();
+      } else {
+#pragma unroll
+        for (int c = 0; c < kMergeSums; ++c) acc[c] += v[c];
+      }
     }
-    // both members get energy E/W; massive ones sit on the mass shell, |u|^2 = (E/W)^2 - 1
-    const double et = E / W, mv[3] = {P[0] / W, P[1] / W, P[2] / W};
-    const double m2 = mv[0] * mv[0] + mv[1] * mv[1] + mv[2] * mv[2];
-    const double d2 = (massless ? et * et : et * et - 1.0) - m2;
-    const double dl = d2 > 0.0 ? sqrt(d2) : 0.0;
-    int ax = 0;
-    for (int c = 1; c < 3; ++c)
-      if (fabs(mv[c]) < fabs(mv[ax])) ax = c;
-    double e[3] = {0.0, 0.0, 0.0};
-    e[ax] = 1.0;
-    double dv[3] = {mv[1] * e[2] - mv[2] * e[1], mv[2] * e[0] - mv[0] * e[2], mv[0] * e[1] - mv[1] * e[0]};
-    const double dn = sqrt(dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2]);
-    if (dn > 0.0) {
-      for (int c = 0; c < 3; ++c) dv[c] *= dl / dn;
-    } else {
-      for (int c = 0; c < 3; ++c) dv[c] = 0.0;
-      dv[ax] = dl;
+    double t[kMergeSums];
+#pragma unroll
+    for (int c = 0; c < kMergeSums; ++c) {
+      if (kOrdered) {
+        t[c] = __shfl_sync(kFull, acc[0], c);
+      } else {
+        double a = acc[c];
+        for (int off = L / 2; off > 0; off >>= 1) a += __shfl_xor_sync(kFull, a, off);
+        t[c] = a;
+      }
     }
-    for (int t = 0; t < 2; ++t) {
-      const uint32_t i = idx[p + t];
-      const double sg = t == 0 ? 1.0 : -1.0;
-      sp.ux[i] = (R)(mv[0] + sg * dv[0]); sp.uy[i] = (R)(mv[1] + sg * dv[1]); sp.uz[i] = (R)(mv[2] + sg * dv[2]);
-      sp.x[i] = (R)(X[0] / W); sp.y[i] = (R)(X[1] / W); sp.z[i] = (R)(X[2] / W);
-      if (sp.w) sp.w[i] = (R)(0.5 * W);
+    if (!whole) continue;
+    for (uint32_t r = p + 2u + (uint32_t)lane; r < p + size; r += L) Tau<R>::infinite().store(sp.tau + idx[r]);
+    ++merged;
+    removed += size - 2u;
+    if (lane < 2) merge_survivor<R>(sp, idx[p + (uint32_t)lane], lane, massless, t);
+  }
+  if (lane == 0 && merged) {
+    atomicAdd(&sp.cnt->n_dead, removed);
+    atomicAdd(groups, (unsigned long long)merged);
+  }
+}
+
+// The groups of more than kMergeBig members of the mixed path, one block each.
+template <typename R, typename K>
+__global__ void __launch_bounds__(512) merge_big_kernel(SpeciesDev<R> sp, MergeDev M, const K* keys, const uint32_t* idx,
+                                                        uint32_t n, const uint32_t* big, const uint32_t* n_big, int massless,
+                                                        unsigned long long* groups) {
+  __shared__ uint32_t s_end;
+  __shared__ double s_t[16][kMergeSums];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t nb = *n_big;
+  for (uint32_t b = blockIdx.x; b < nb; b += gridDim.x) {
+    const uint32_t p = big[b];
+    const K key = keys[p];
+    if (warp == 0) {
+      // the group's end, 32 probes at a time: keys[lo] belongs to it, keys[hi] (if any) does not
+      uint32_t lo = p, hi = n;
+      while (hi - lo > 1) {
+        const uint32_t step = (hi - lo + 32u) / 33u, q = lo + step * (uint32_t)(lane + 1);
+        const uint32_t c = (uint32_t)__popc(__ballot_sync(kFull, q < hi && keys[q] == key));
+        if (lo + step * (c + 1u) < hi) hi = lo + step * (c + 1u);
+        lo += step * c;
+      }
+      if (lane == 0) s_end = lo + 1u;
     }
-    for (uint32_t r = p + 2; r < q; ++r) Tau<R>::infinite().store(sp.tau + idx[r]);
-    atomicAdd(&sp.cnt->n_dead, q - p - 2);
-    atomicAdd(groups, 1ull);
+    __syncthreads();
+    const uint32_t end = s_end;
+    if (end - p < (uint32_t)M.min_group) { __syncthreads(); continue; }
+    double acc[kMergeSums];
+#pragma unroll
+    for (int c = 0; c < kMergeSums; ++c) acc[c] = 0.0;
+    for (uint32_t r = p + threadIdx.x; r < end; r += 512u) {
+      double v[kMergeSums];
+      merge_member<R>(sp, idx[r], massless, v);
+#pragma unroll
+      for (int c = 0; c < kMergeSums; ++c) acc[c] += v[c];
+    }
+#pragma unroll
+    for (int c = 0; c < kMergeSums; ++c) {
+      double a = acc[c];
+      for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(kFull, a, off);
+      if (lane == 0) s_t[warp][c] = a;
+    }
+    __syncthreads();  // the sums are there, and every member has been read
+    for (uint32_t r = p + 2u + threadIdx.x; r < end; r += 512u) Tau<R>::infinite().store(sp.tau + idx[r]);
+    if (threadIdx.x < 2) {
+      double t[kMergeSums];
+      for (int c = 0; c < kMergeSums; ++c) {
+        t[c] = 0.0;
+        for (int w = 0; w < 16; ++w) t[c] += s_t[w][c];
+      }
+      merge_survivor<R>(sp, idx[p + threadIdx.x], (int)threadIdx.x, massless, t);
+    }
+    if (threadIdx.x == 0) {
+      atomicAdd(&sp.cnt->n_dead, end - p - 2u);
+      atomicAdd(groups, 1ull);
+    }
+    __syncthreads();
   }
 }
 
@@ -2947,19 +3279,44 @@ void launch_totals(const SpeciesDev<R>& sp, int massless, double* partials, int 
   count_launch();
 }
 
+// Sorts the n (key, index) pairs of a[0]; returns which of the two buffers holds the result.
+template <typename K>
+static int radix_sort(K* keys[2], uint32_t* idx[2], uint32_t n, int bits, uint32_t* hist, uint32_t* totals, cudaStream_t s) {
+  const uint32_t segs = (n + kSortSeg - 1) / kSortSeg;
+  int cur = 0;
+  for (int shift = 0; shift < bits; shift += 8, cur ^= 1) {
+    radix_count_kernel<K><<<segs, 256, 0, s>>>(keys[cur], n, shift, hist);
+    radix_scan_kernel<<<256, 256, 0, s>>>(hist, segs, totals);
+    radix_scatter_kernel<K><<<segs, 256, 0, s>>>(keys[cur], idx[cur], keys[cur ^ 1], idx[cur ^ 1], n, shift, hist, totals);
+    count_launch(3);
+  }
+  return cur;
+}
+
+template <typename R, typename K>
+static void merge_with_keys(const SpeciesDev<R>& sp, const MergeDev& m, const MergeScratch& w, uint32_t n, int massless,
+                            unsigned long long* groups, cudaStream_t s) {
+  K* keys[2] = {static_cast<K*>(w.keys[0]), static_cast<K*>(w.keys[1])};
+  uint32_t* idx[2] = {w.idx[0], w.idx[1]};
+  merge_key_kernel<R, K><<<small_grid(n), 256, 0, s>>>(sp, m, keys[0], idx[0], n);
+  const int at = radix_sort<K>(keys, idx, n, m.bits, w.hist, w.totals, s);
+  uint32_t* heads = idx[at ^ 1];  // the other buffer is free now
+  merge_heads_kernel<K><<<small_grid(n), 256, 0, s>>>(keys[at], n, (K)m.none, heads, w.count);
+  uint32_t* big = static_cast<uint32_t*>(w.keys[at ^ 1]);  // (so is its keys' buffer)
+  merge_groups_kernel<R, K><<<sm_count() * 8, 128, 0, s>>>(sp, m, keys[at], idx[at], n, heads, w.count, big, w.count + 1,
+                                                           massless, groups);
+  count_launch(3);
+  if (sizeof(R) == 4) {
+    merge_big_kernel<R, K><<<sm_count() * 2, 512, 0, s>>>(sp, m, keys[at], idx[at], n, big, w.count + 1, massless, groups);
+    count_launch();
+  }
+}
+
 template <typename R>
-void launch_merge(const SpeciesDev<R>& sp, const MergeDev& m, uint64_t* keys, uint32_t* idx, uint32_t N,
-                  int massless, unsigned long long* groups, cudaStream_t s) {
-  const int grid = sm_count() * 8;
-  merge_key_kernel<R><<<grid, 256, 0, s>>>(sp, m, keys, idx, N);
-  int launches = 1;
-  for (uint32_t k = 2; k <= N; k <<= 1)
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      bitonic_pass_kernel<<<grid, 256, 0, s>>>(keys, idx, N, k, j);
-      ++launches;
-    }
-  merge_groups_kernel<R><<<grid, 256, 0, s>>>(sp, m, keys, idx, N, massless, groups);
-  count_launch(launches + 1);
+void launch_merge(const SpeciesDev<R>& sp, const MergeDev& m, const MergeScratch& w, uint32_t n, int massless,
+                  unsigned long long* groups, cudaStream_t s) {
+  if (m.bits <= 32) merge_with_keys<R, uint32_t>(sp, m, w, n, massless, groups, s);
+  else merge_with_keys<R, uint64_t>(sp, m, w, n, massless, groups, s);
 }
 
 #endif
@@ -2988,7 +3345,7 @@ template void launch_batch_step<double>(const BatchCtl<double>&, int, int, Batch
   template void launch_compact<R>(const SpeciesDev<R>&, const SpeciesDev<R>&, uint32_t*, uint32_t*, cudaStream_t); \
   template void launch_fill<R>(R*, size_t, R, cudaStream_t);                                                     \
   template void launch_totals<R>(const SpeciesDev<R>&, int, double*, int, cudaStream_t);                         \
-  template void launch_merge<R>(const SpeciesDev<R>&, const MergeDev&, uint64_t*, uint32_t*, uint32_t, int,        \
+  template void launch_merge<R>(const SpeciesDev<R>&, const MergeDev&, const MergeScratch&, uint32_t, int,         \
                                 unsigned long long*, cudaStream_t);
 QED_INSTANTIATE(float)
 QED_INSTANTIATE(double)

@@ -173,3 +173,43 @@ def test_merge_scratch_comes_from_the_callers_allocator(tables):
     assert len(live) == len(log) - 1  # weights and the compaction's second set stay with the species
     g.close()
     assert not live, "every block is given back when the species is freed"
+
+
+@pytest.mark.parametrize("prec", [qed.FP64, qed.MIXED])
+@pytest.mark.parametrize("n,cells", [(3, 2), (33, 2), (4095, 4), (4096, 64), (4097, 1500), (20011, 4), (70001, 700)])
+def test_merge_sizes_match_oracle(tables, prec, n, cells):
+    # around the sort's segments (4096) with 32-bit (few cells) and 64-bit keys, groups from one
+    # member to a few hundred, converted photons among them
+    rng = np.random.default_rng(n)
+    m = max(1, n // 40)
+    centre = rng.integers(0, m, n) * (rng.random(n) < 0.9)
+    x = rng.uniform(-9, 9, (m, 3))[centre] + rng.normal(size=(n, 3)) * 1e-3
+    d = rng.normal(size=(m, 3))[centre]
+    k = d / np.linalg.norm(d, axis=1, keepdims=True) * (10.0 ** rng.uniform(-2, 3, m))[centre][:, None]
+    k = k * rng.uniform(0.98, 1.02, (n, 1))
+    tau = rng.uniform(0.1, 3.0, n)
+    tau[::17] = np.inf
+    w = rng.uniform(0.5, 4.0, n)
+    if prec == qed.MIXED:
+        x, k, w, tau = (a.astype(np.float32).astype(np.float64) for a in (x, k, w, tau))
+    grid = dict(origin=(-10.0,) * 3, cell=(20.0 / cells,) * 3, n_cells=(cells,) * 3)
+    ids = np.arange(n, dtype=np.uint32)
+    # the library leaves converted photons out of the groups (and removes them); the oracle merges
+    # what it is given: the living
+    alive = np.isfinite(tau)
+    ref = o.Species(n + 4)
+    ref.set(x[alive], k[alive], tau=tau[alive], ids=ids[alive], w=w[alive])
+    g_ref = ref.merge(**grid, n_face=6, n_sub=2, min_group=4)
+    g = qed.Species(qed.PHOTON, prec, n + 5, 16)
+    g.upload(x, k, tau=tau, ids=ids, next_id=n)
+    g.set_weights(w)
+    assert g.merge(**grid, n_face=6, n_sub=2, min_group=4) == g_ref
+    a = g.download()
+    assert np.array_equal(a["id"], ref.get("id"))
+    if prec == qed.FP64:
+        assert np.array_equal(a["x"], ref.x()) and np.array_equal(a["u"], ref.u())
+        assert np.array_equal(g.weights(), ref.get("w"))
+    else:
+        np.testing.assert_allclose(a["x"], ref.x(), rtol=1e-6, atol=1e-5)
+        np.testing.assert_allclose(a["u"], ref.u(), rtol=1e-6, atol=1e-6 * np.abs(ref.u()).max())
+        np.testing.assert_allclose(g.weights(), ref.get("w"), rtol=1e-6)
