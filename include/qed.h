@@ -216,7 +216,9 @@ qed_status qed_species_merge(qed_species* sp, const qed_merge_params* params, ui
  *                        axis); shape = 2: triangular-shaped cloud (quadratic weights over the
  *                        nearest node and its two neighbours).  Stencil nodes outside the grid
  *                        contribute nothing, so fields fall to zero outside it.  The fields do
- *                        not depend on t: the caller updates the grid between steps.
+ *                        not depend on t: the caller updates the grid between calls.  A mixed
+ *                        single-scenario call with particles enough packs a shape = 1 grid by cells
+ *                        for its own use (at most 256 MB, from sp[0]'s allocator, kept with sp[0]).
  * ------------------------------------------------------------------------------------------ */
 typedef enum {
   QED_FIELD_UNIFORM = 0, QED_FIELD_ROTATING_E = 1, QED_FIELD_PLANE_LP = 2, QED_FIELD_PLANE_CP = 3,

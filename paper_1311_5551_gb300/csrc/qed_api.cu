@@ -311,6 +311,10 @@ struct qed_species {
   DeviceBlock wmem;
   // second array set for compaction (allocated at the first compaction)
   DeviceBlock alt_mem, alt_wmem;
+  // packed grid of the calls that pass this species as sp[0] (see grid_workspace)
+  DeviceBlock cell_mem;
+  std::vector<DeviceBlock> old_cells;  // outgrown ones (calls on other streams may still read them)
+  bool use_cells = false;  // the call under way packed its grid
   qed_allocator alloc_copy{};
   bool have_alloc = false;
   void* other[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
@@ -452,6 +456,8 @@ extern "C" qed_status qed_species_alloc(qed_kind kind, qed_precision precision, 
 
 extern "C" void qed_species_free(qed_species* sp) {
   if (!sp) return;
+  sp->cell_mem.release();
+  for (DeviceBlock& b : sp->old_cells) b.release();
   sp->alt_wmem.release();
   sp->alt_mem.release();
   sp->wmem.release();
@@ -861,6 +867,43 @@ template <typename R> const TabDev<R>& tab_of(const qed_tables* t);
 template <> const TabDev<float>& tab_of<float>(const qed_tables* t) { return t->d32; }
 template <> const TabDev<double>& tab_of<double>(const qed_tables* t) { return t->d64; }
 
+// Room for the packed form of a cloud-in-cell grid field (pack_grid_kernel) in the electron species, from
+// its allocator: kept while the species lives, and at least doubled when a grid needs more, up to
+// kMaxPacked bytes (so all of them take at most twice that).  Larger grids, and calls under stream capture that would have to allocate, gather from the grid.
+constexpr size_t kMaxPacked = size_t(256) << 20;
+bool grid_workspace(qed_species* e, const qed_field_desc& f, cudaStream_t s) {
+  if (f.kind != QED_FIELD_GRID || f.shape != 1 || e->precision != QED_MIXED) return false;
+  for (int c = 0; c < 3; ++c)
+    if ((size_t)f.n[c] > kMaxPacked / 192) return false;  // (so the product below cannot overflow)
+  const size_t row = ((size_t)f.n[0] + 1) * ((size_t)f.n[1] + 1);
+  if (row > kMaxPacked / 192) return false;
+  const size_t bytes = 256 + 192 * row * ((size_t)f.n[2] + 1);
+  if (bytes > kMaxPacked) return false;
+  if (e->cell_mem.ptr && e->cell_mem.bytes >= bytes) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  DeviceBlock grown;
+  const size_t get = std::min(kMaxPacked, std::max(bytes, 2 * e->cell_mem.bytes));
+  if (grown.get(get, e->have_alloc ? &e->alloc_copy : nullptr, s) != QED_OK) {
+    cudaGetLastError();
+    return false;
+  }
+  if (e->cell_mem.ptr) e->old_cells.push_back(e->cell_mem);
+  e->cell_mem = grown;
+  return true;
+}
+
+// Packs the grid of a single-scenario call of n steps, if that pays, for make_args to pass on.
+template <typename R>
+StepArgs<R> make_args(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t step);
+void pack_grid(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t n, cudaStream_t s) {
+  sp[0]->use_cells = n > 0 && grid_workspace(sp[0], p.field, s);
+  if (sp[0]->use_cells) launch_pack_grid(make_args<float>(T, sp, p, p.step), n, s);
+}
+
 template <typename R>
 StepArgs<R> make_args(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t step) {
   StepArgs<R> a{};
@@ -880,6 +923,10 @@ StepArgs<R> make_args(const qed_tables* T, qed_species* const* sp, const qed_ste
   a.plan = sp[0]->plan;
   a.work = sp[0]->work;
   a.win_s = -1;
+  if (sp[0]->use_cells) {
+    a.field.packed = static_cast<uint32_t*>(sp[0]->cell_mem.ptr);
+    a.field.cells = static_cast<char*>(sp[0]->cell_mem.ptr) + 256;
+  }
   return a;
 }
 
@@ -1274,8 +1321,10 @@ extern "C" qed_status qed_run(const qed_tables* T, qed_species* const* sp, const
   st = sync_weights(sp, s);
   if (st != QED_OK) return st;
   NvtxRange range("qed_run");
+  pack_grid(T, sp, *p, n_steps, s);
   if (sp[0]->precision == QED_MIXED) do_steps<float>(T, sp, *p, p->step, n_steps, true, s);
   else do_steps<double>(T, sp, *p, p->step, n_steps, true, s);
+  sp[0]->use_cells = false;
   QED_CUDA(cudaGetLastError());
   return QED_OK;
 }
@@ -1340,8 +1389,10 @@ extern "C" qed_status qed_run_multistep(const qed_tables* T, qed_species* const*
   st = sync_weights(sp, s);
   if (st != QED_OK) return st;
   NvtxRange range("qed_run_multistep");
+  pack_grid(T, sp, *p, n_steps, s);
   st = sp[0]->precision == QED_MIXED ? run_multi<float>(T, sp, *p, n_steps, chunk, s)
                                      : run_multi<double>(T, sp, *p, n_steps, chunk, s);
+  sp[0]->use_cells = false;
   if (st != QED_OK) return st;
   QED_CUDA(cudaGetLastError());
   return QED_OK;

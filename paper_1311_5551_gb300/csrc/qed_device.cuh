@@ -160,6 +160,7 @@ struct StepScalars {
   // grid gather
   const R* grid;
   size_t gN;       // values per component
+  const R* cells;  // the grid packed by cells (NULL: gather from the grid itself)
   int gn[3], shape;
   R gorg[3], ginv[3];
 };
@@ -176,6 +177,7 @@ __device__ void make_scalars(const FieldDev& f, double t, double win_x0, double 
   S.phi_ref = (R)0;
   S.phi_ref_mod = (R)0;
   S.grid = nullptr;
+  S.cells = nullptr;
   if (f.kind == QED_FIELD_GRID) {
     S.grid = static_cast<const R*>(f.grid);
     S.shape = f.shape;
@@ -273,6 +275,50 @@ __device__ __forceinline__ void gather_fields(const StepScalars<R>& S, const R s
   B[2] = gather_component<R, W>(S.grid + 5 * S.gN, S.gn, half[0], half[1], node[2]);
 }
 
+// Cloud-in-cell weights on a grid packed by cells: a component's eight node values of a cell lie side
+// by side (zero where a node is outside), cells from index -1 to n - 1 on every axis, x fastest, so
+// a component is one 32-byte read instead of eight scattered ones.  Same products and
+// order as gather_component, and so the same bits (a node outside adds an exact zero).
+__device__ __forceinline__ void load_cell(const float* p, float v[8]) {
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+      : "l"(p));
+}
+__device__ __forceinline__ float gather_cell(const float* C, const int n[3], const AxisWeights<float, 2>& ax,
+                                             const AxisWeights<float, 2>& ay, const AxisWeights<float, 2>& az) {
+  using R = float;
+  const unsigned cx = (unsigned)(ax.i0 + 1), cy = (unsigned)(ay.i0 + 1), cz = (unsigned)(az.i0 + 1);
+  if (cx > (unsigned)n[0] || cy > (unsigned)n[1] || cz > (unsigned)n[2]) return (R)0;
+  R v[8];
+  load_cell(C + 8 * (((size_t)cz * (size_t)(n[1] + 1) + cy) * (size_t)(n[0] + 1) + cx), v);
+  R t = (R)0;
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const R wzy = az.w[k] * ay.w[j];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) t = Num<R>::fma_(wzy * ax.w[i], v[4 * k + 2 * j + i], t);
+    }
+  return t;
+}
+__device__ __forceinline__ void gather_cells(const StepScalars<float>& S, const float s[3], float E[3], float B[3]) {
+  using R = float;
+  AxisWeights<R, 2> node[3], half[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    node[a] = axis_weights<R, 2>(s[a]);
+    half[a] = axis_weights<R, 2>(s[a] - (R)0.5);
+  }
+  const size_t N = 8 * grid_cells(S.gn);
+  E[0] = gather_cell(S.cells + 0 * N, S.gn, half[0], node[1], node[2]);
+  E[1] = gather_cell(S.cells + 1 * N, S.gn, node[0], half[1], node[2]);
+  E[2] = gather_cell(S.cells + 2 * N, S.gn, node[0], node[1], half[2]);
+  B[0] = gather_cell(S.cells + 3 * N, S.gn, node[0], half[1], half[2]);
+  B[1] = gather_cell(S.cells + 4 * N, S.gn, half[0], node[1], half[2]);
+  B[2] = gather_cell(S.cells + 5 * N, S.gn, half[0], half[1], node[2]);
+}
+
 template <typename R>
 __device__ __forceinline__ void grid_field_at(const StepScalars<R>& S, R x, R y, R z, R E[3], R B[3]) {
   E[0] = E[1] = E[2] = B[0] = B[1] = B[2] = (R)0;
@@ -281,6 +327,9 @@ __device__ __forceinline__ void grid_field_at(const StepScalars<R>& S, R x, R y,
 #pragma unroll
   for (int a = 0; a < 3; ++a)
     if (!(s[a] > (R)-3 && s[a] < (R)S.gn[a] + (R)2)) return;
+  if constexpr (sizeof(R) == 4) {
+    if (S.cells) { gather_cells(S, s, E, B); return; }
+  }
   if (S.shape == 1) gather_fields<R, 2>(S, s, E, B);
   else gather_fields<R, 3>(S, s, E, B);
 }

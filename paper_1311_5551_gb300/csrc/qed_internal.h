@@ -127,7 +127,12 @@ struct FieldDev {
   int n[3];
   int shape;
   double origin[3], spacing[3];
+  // the grid packed by cells for this call (see pack_grid_kernel), and whether it was; NULL: not
+  void* cells;
+  uint32_t* packed;
 };
+// Cells of a packed grid component, and the bytes of a whole packed grid.
+QED_HD constexpr size_t grid_cells(const int n[3]) { return ((size_t)n[0] + 1) * ((size_t)n[1] + 1) * ((size_t)n[2] + 1); }
 
 // Host: descriptor -> device form, and its validation (shared by every entry point that steps).
 FieldDev field_dev(const qed_field_desc& f);
@@ -196,6 +201,9 @@ struct BatchCtl {
   int fuse_k;            // multi-step stretch per batch step (0: per-step only)
 };
 
+// Packs a.field's grid into a.field.cells if the run of `steps` steps has particles enough to gain by
+// it, and writes to a.field.packed whether it has.
+void launch_pack_grid(const StepArgs<float>& a, uint64_t steps, cudaStream_t s);
 template <typename R>
 void launch_step(const StepArgs<R>& a, int grid, int block, size_t smem, cudaStream_t s);
 template <typename R>

@@ -978,6 +978,12 @@ __device__ __forceinline__ void run_species(const StepArgs<R>& A, const StepScal
   else run_photons<R, G, WANT>(A, S, P, run, w);
 }
 
+// The call's packed grid, if it has one (after pdl_wait: pack_grid_kernel writes the flag).
+template <typename R>
+__device__ __forceinline__ const R* packed_cells(const FieldDev& f) {
+  return sizeof(R) == 4 && f.cells && *f.packed ? static_cast<const R*>(f.cells) : nullptr;
+}
+
 // The step over one scenario, run by block `blk` of the `nblk` blocks given to it: block blk
 // takes the scenario's tiles blk, blk + nblk, ... and writes ledger partial number blk.
 // Warp roles: warps 0-7 compute (warp w takes 32-particle chunk w of each tile); warp 8 is the
@@ -1019,6 +1025,7 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
   const uint32_t T3 = conversion_tiles(win_n, nblk);
   const uint32_t ttot = T0 + T1 + T2 + T3;
   if (threadIdx.x < 3) S.phase[threadIdx.x] = a.sp[threadIdx.x].cnt->phase;
+  if (G && threadIdx.x == 0) S.cells = packed_cells<R>(a.field);
   if (threadIdx.x == kBlock)
     for (uint32_t k = 0; k < (uint32_t)kStages; ++k) issue_tile(a, buf, full, k, n0, n1, n2, win_n, blk, nblk);
   __syncthreads();
@@ -1322,6 +1329,44 @@ __global__ void selftest_wait_kernel(uint32_t polls, uint32_t* bits) {
 }
 
 
+// ----------------------------------------------------------------------------- packed grids
+// Packs a cloud-in-cell grid by cells for one call (the caller updates its grid between calls).  A
+// gather straight from the grid is 48 scattered 4-byte reads per particle, and the L1's one look-up
+// per lane and read bounds it: on GB300 60 us for 4e5 particles on a grid of 48^3 nodes; packed it is
+// 6 reads of 32 bytes, 20 us.  Packing writes 192 bytes per cell, so it pays from about a third of a
+// particle-step per cell on (48^3: break-even at 3e4 particles, 64^3: 1e5); with fewer it is skipped.  (The FP64 path is
+// bound by the FP64 pipe and gains nothing: 375 us a step against 391 with the packing.)  One thread per component and cell; blocks
+// stand for 256 cells of one z layer of one component.
+__global__ void __launch_bounds__(256) pack_grid_kernel(const StepArgs<float> a, uint64_t steps) {
+  pdl_wait();
+  pdl_launch();
+  const FieldDev& f = a.field;
+  const uint64_t cells = grid_cells(f.n);
+  const uint64_t particles = (uint64_t)a.sp[0].cnt->n + a.sp[1].cnt->n + a.sp[2].cnt->n;
+  const bool on = particles * min(steps, (uint64_t)1 << 20) >= cells / 3u;
+  if (blockIdx.x + blockIdx.y + blockIdx.z + threadIdx.x == 0) *f.packed = on ? 1u : 0u;
+  if (!on) return;
+  const int nx = f.n[0], ny = f.n[1], nz = f.n[2];
+  const uint32_t q = blockIdx.x * 256u + threadIdx.x, layer = (uint32_t)(nx + 1) * (uint32_t)(ny + 1);
+  if (q >= layer) return;
+  const int y = (int)(q / (uint32_t)(nx + 1)) - 1, x = (int)(q % (uint32_t)(nx + 1)) - 1;
+  const size_t N = (size_t)nx * ny * nz;
+  const float* grid = static_cast<const float*>(f.grid) + blockIdx.z * N;
+  for (int z = (int)blockIdx.y - 1; z < nz; z += (int)gridDim.y) {
+    float v[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int i = x + (t & 1), j = y + (t >> 1 & 1), k = z + (t >> 2);
+      const bool in = i >= 0 && i < nx && j >= 0 && j < ny && k >= 0 && k < nz;
+      v[t] = in ? grid[((size_t)k * ny + j) * nx + i] : 0.0f;
+    }
+    float4* out = reinterpret_cast<float4*>(static_cast<float*>(f.cells) +
+                                            8 * (blockIdx.z * cells + (uint64_t)(z + 1) * layer + q));
+    out[0] = make_float4(v[0], v[1], v[2], v[3]);
+    out[1] = make_float4(v[4], v[5], v[6], v[7]);
+  }
+}
+
 // ----------------------------------------------------------------------------- finalisation
 // Block-wide exclusive scan of one value per thread (blockDim.x <= 1024, multiple of 32).
 __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
@@ -1542,7 +1587,12 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const StepArgs<
       return r;
     });
   clear_other_counts(a, P, first, stride);
-  if (a.want && blockIdx.x == gridDim.x - 1) reduce_ledger(a, nparts);
+  if (a.want && blockIdx.x == gridDim.x - 1) {
+    // (blocks without a tile have nothing to add)
+    uint32_t tiles = 0;
+    for (int s = 0; s < 3; ++s) tiles += (n[s] + kTile - 1) / kTile;
+    reduce_ledger(a, (int)min((uint32_t)nparts, tiles));
+  }
   // the last block to get here sets the counters: by then every block has read them
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1843,6 +1893,7 @@ __global__ void __launch_bounds__(kFuseThreads) window_kernel(const StepArgs<flo
   }
   if (threadIdx.x == 0) sh.pushed = 0;
   pdl_wait();
+  if (G && (int)threadIdx.x < K) sh.S[threadIdx.x].cells = packed_cells<float>(a.field);
   __syncthreads();
   pdl_launch();
   constexpr uint32_t W = kFuseThreads / 32;
@@ -2743,6 +2794,17 @@ void launch_selftest_wait(uint32_t polls, uint32_t* bits, cudaStream_t s) {
 template <typename R>
 void launch_finalize(const StepArgs<R>& a, int step_grid, cudaStream_t s) {
   launch_pdl(finalize_kernel<R>, sm_count(), kFinalThreads, 0, s, a, step_grid);
+  count_launch();
+}
+
+void launch_pack_grid(const StepArgs<float>& a, uint64_t steps, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  const size_t layer = ((size_t)a.field.n[0] + 1) * ((size_t)a.field.n[1] + 1);
+  const size_t gx = (layer + 255) / 256, room = std::max<size_t>(1, (size_t)sm_count() * 8 / (6 * gx));
+  cfg.gridDim = dim3((unsigned)gx, (unsigned)std::min<size_t>((size_t)a.field.n[2] + 1, room), 6);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchKernelEx(&cfg, pack_grid_kernel, a, steps);
   count_launch();
 }
 

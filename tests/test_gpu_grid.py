@@ -125,3 +125,36 @@ def test_grid_scenario_in_a_batch(tables):
     assert np.all(b.remaining() == 0)
     for a, s in zip(ref, mix[0]):
         assert np.array_equal(a.save(), s.save())
+
+
+@pytest.mark.parametrize("N", [(1, 1, 1), (2, 3, 5), (13, 11, 9), (40, 3, 33)])
+@pytest.mark.parametrize("n,steps", [(37, 1), (5000, 1), (3001, 19)])
+def test_packed_grid_matches_the_grid(tables, N, n, steps):
+    # single-scenario runs gather from the grid packed by cells where that pays, batches from the grid
+    # itself: the same particles bit for bit, inside, at the edges and outside (every node weight and
+    # the nodes that do not exist are exercised), for grids of one node to a few thousand
+    prec = qed.MIXED
+    org, spc = (-20.0, 5.0, 100.0), (3.0e4, 2.5e4, 4.0e4)
+    rng = np.random.default_rng(n + N[0])
+    fq = qed.Field(kind=qed.FIELD_GRID, grid=dev_grid(random_grid(N, 3), prec), shape=1, origin=org, spacing=spc)
+    x = np.stack([rng.uniform(org[a] - 3 * spc[a], org[a] + (N[a] + 2) * spc[a], n) for a in range(3)], axis=1)
+    u = rng.normal(size=(n, 3)) * 300.0
+    xg, kg = rng.permutation(x), rng.normal(size=(n, 3)) * 10.0 ** rng.uniform(-1, 4, (n, 1))
+    out = []
+    for batched in (False, True):
+        sp = [qed.Species(qed.ELECTRON, prec, 4 * n + 64, 4 * n + 64), qed.Species(qed.POSITRON, prec, 4 * n + 64, 4 * n + 64),
+              qed.Species(qed.PHOTON, prec, 30 * n + 64, 8 * n + 64)]
+        sp[0].upload(x, u)
+        sp[0].init_tau(2)
+        sp[2].upload(xg, kg)
+        sp[2].init_tau(2)
+        p = qed.StepParams(dt=2.0e3, seed=2, field=fq)
+        if batched:
+            b = qed.Batch(tables, prec, 1)
+            b.attach(0, sp, p, 0, steps)
+            b.run(steps)
+        else:
+            qed.run(tables, sp, p, 0, steps)
+        qed.check(sp)
+        out.append([s.save() for s in sp])
+    assert all(np.array_equal(a, c) for a, c in zip(*out))
