@@ -155,6 +155,7 @@ struct StepArgs {
                              // per-step photon pushes in a field
   int want;                  // somebody can read this step's ledger: keep its sums
   int win_s;                 // step of the photon window this step belongs to (-1: none)
+  uint32_t* counter;         // allocation-free step: the caller's photon counter (else NULL)
 };
 
 // What one batch step does with a slot, written by the tile schedule at the start of the step:

@@ -1600,6 +1600,13 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const StepArgs<
     if (atomicAdd(&a.plan->ticket, 1u) == gridDim.x - 1) {
       a.plan->ticket = 0u;
       finish_counters(a, P, n);
+      if (a.counter) {  // the allocation-free step: the caller's photon count, next id and error bits
+        a.counter[0] = a.sp[3].cnt->n;
+        a.counter[1] = a.sp[3].cnt->next_id;
+        uint32_t err = 0;
+        for (int k = 0; k < 4; ++k) err |= *(volatile uint32_t*)&a.sp[k].cnt->err;
+        a.counter[2] |= err;
+      }
     }
   }
 }
@@ -2653,20 +2660,37 @@ static size_t step_smem(int n_eta, int n_chi) {
          (size_t)(n_eta + n_chi) * sizeof(R);
 }
 
-template <typename R>
-static int step_blocks_per_sm(size_t smem) {
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(step_kernel<R, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int b = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, step_kernel<R, false, false>, kStepThreads, smem);
-  return b > 0 ? b : 1;
-}
+// Resident blocks per SM of a kernel at a given dynamic shared memory size, with its limit raised to
+// it (never lowered: another thread may be about to launch with more): asked of the runtime once per
+// kernel, device and size (the queries took a third of a one-step call's 12 us on the host).  Any
+// thread; two that ask at once find the same.
+struct Residency {
+  std::atomic<uint64_t> known[128];  // per device: size << 16 | blocks (0: not asked yet)
+  std::atomic<uint64_t> limit[128];  // per device: the largest size asked for
+  template <typename F>
+  int operator()(F kernel, int threads, size_t smem) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::atomic<uint64_t>* slot = dev >= 0 && dev < 128 ? &known[dev] : nullptr;
+    const uint64_t have = slot ? slot->load(std::memory_order_relaxed) : 0;
+    if (have && (have >> 16) == smem) return (int)(have & 0xffffu);
+    if (!slot || smem > limit[dev].load()) {
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (slot) limit[dev].store(smem);
+    }
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess || b < 1) return 1;
+    if (slot) slot->store((uint64_t)smem << 16 | (uint64_t)b, std::memory_order_relaxed);
+    return b;
+  }
+};
 
 #if QED_PART(1)
 int step_grid_size(int precision) {
   // occupancy for the paper's table sizes (256 eta, 256 chi)
-  const int b = precision == QED_MIXED ? step_blocks_per_sm<float>(step_smem<float>(256, 256))
-                                       : step_blocks_per_sm<double>(step_smem<double>(256, 256));
+  static Residency mixed, fp64;
+  const int b = precision == QED_MIXED ? mixed(step_kernel<float, false, false>, kStepThreads, step_smem<float>(256, 256))
+                                       : fp64(step_kernel<double, false, false>, kStepThreads, step_smem<double>(256, 256));
   return sm_count() * b;
 }
 
@@ -2680,7 +2704,8 @@ void launch_step(const StepArgs<R>& a, int grid, int block, size_t smem_unused, 
   const bool g = a.field.kind == QED_FIELD_GRID;
   const auto k = a.want ? (g ? step_kernel<R, true, true> : step_kernel<R, false, true>)
                         : (g ? step_kernel<R, true, false> : step_kernel<R, false, false>);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static Residency known[4];
+  known[(a.want ? 2 : 0) + (g ? 1 : 0)](k, kStepThreads, smem);  // (raises the shared memory limit)
   launch_pdl(k, grid, kStepThreads, smem, s, a);
   count_launch();
 }
@@ -2692,10 +2717,8 @@ void launch_batch_window(const BatchCtl<float>& c, int n_chi, int W, BatchEnd en
   launch_pdl(batch_window_prepare_kernel, (c.S * kWinMax + 127) / 128, 128, 0, s, c, W, (int)end);
   const size_t smem = window_smem(n_chi);
   const auto k = c.grid_fields ? batch_window_kernel<true> : batch_window_kernel<false>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int b = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, kFuseThreads, smem);
-  launch_pdl(k, sm_count() * std::max(b, 1), kFuseThreads, smem, s, c, W, (int)end);
+  static Residency known[2];
+  launch_pdl(k, sm_count() * known[c.grid_fields != 0](k, kFuseThreads, smem), kFuseThreads, smem, s, c, W, (int)end);
   count_launch(2);
 }
 
@@ -2703,10 +2726,9 @@ template <typename R>
 void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, BatchEnd end, int win_w, BatchEnd win_end, int win_s,
                        cudaStream_t s) {
   const size_t smem = step_smem<R>(n_eta, n_chi);
-  if (smem + sizeof(StepArgs<R>) + sizeof(StepScalars<R>) > 40 * 1024) {
-    cudaFuncSetAttribute(batch_step_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(batch_step_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  }
+  const auto k = c.grid_fields ? batch_step_kernel<R, true> : batch_step_kernel<R, false>;
+  static Residency known[2];
+  known[c.grid_fields != 0](k, kStepThreads, smem);  // (raises the shared memory limit)
   if (c.fuse_k >= 2) {
     const size_t fsm = (size_t)(n_eta + n_chi) * sizeof(R);
     const int fgrid = c.target_blocks + c.S;
@@ -2724,8 +2746,7 @@ void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, BatchEnd end,
   }
   // the per-step path: one tile space over all live slots, strided by a persistent grid
   launch_pdl(batch_tiles_kernel<R>, 1, 1024, 0, s, c, (int)end, win_w, (int)win_end, win_s);
-  if (c.grid_fields) launch_pdl(batch_step_kernel<R, true>, c.target_blocks, kStepThreads, smem, s, c);
-  else launch_pdl(batch_step_kernel<R, false>, c.target_blocks, kStepThreads, smem, s, c);
+  launch_pdl(k, c.target_blocks, kStepThreads, smem, s, c);
   launch_pdl(batch_plan_kernel<R>, c.S, 256, 0, s, c, c.target_blocks);
   launch_pdl(batch_scatter_kernel<R>, sm_count() * 4, 256, 0, s, c);
   count_launch(4);
@@ -2741,9 +2762,8 @@ size_t step_scalars_bytes(int precision) {
 // grid of the multi-step kernels: every SM full, never more blocks than ledger partials
 template <typename R, bool G, bool C>
 static int fused_grid(int max_parts, size_t smem) {
-  int b = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fused_kernel<R, G, C>, kFuseThreads, smem);
-  return std::max(1, std::min(max_parts, sm_count() * std::max(b, 1)));
+  static Residency known;
+  return std::max(1, std::min(max_parts, sm_count() * known(fused_kernel<R, G, C>, kFuseThreads, smem)));
 }
 
 template <typename R>
@@ -2778,11 +2798,10 @@ int fuse_max_steps() { return kMaxFuse; }
 
 void launch_window(const StepArgs<float>& a, int K, cudaStream_t s) {
   const size_t smem = window_smem(a.tab.n_chi);
-  const auto k = a.field.kind == QED_FIELD_GRID ? window_kernel<true> : window_kernel<false>;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int b = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, kFuseThreads, smem);
-  launch_pdl(k, sm_count() * std::max(b, 1), kFuseThreads, smem, s, a, K);
+  const bool g = a.field.kind == QED_FIELD_GRID;
+  const auto k = g ? window_kernel<true> : window_kernel<false>;
+  static Residency known[2];
+  launch_pdl(k, sm_count() * known[g](k, kFuseThreads, smem), kFuseThreads, smem, s, a, K);
   count_launch();
 }
 

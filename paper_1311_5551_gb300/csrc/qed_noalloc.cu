@@ -62,14 +62,6 @@ __global__ void noalloc_begin_kernel(DevCounters* c, uint32_t* counts, uint32_t 
   c[3].next_id = photon_counter[1];
 }
 
-__global__ void noalloc_end_kernel(const DevCounters* c, uint32_t* photon_counter) {
-  photon_counter[0] = c[3].n;
-  photon_counter[1] = c[3].next_id;
-  uint32_t err = 0;
-  for (int k = 0; k < 4; ++k) err |= c[k].err;
-  photon_counter[2] |= err;
-}
-
 template <typename R>
 void bind_species(SpeciesDev<R>& s, DevCounters* cnt, uint32_t* masks, uint32_t* counts, size_t cap) {
   s.cnt = cnt;
@@ -114,6 +106,7 @@ qed_status run_noalloc(const TablesDev& tv, const qed_soa* e, size_t n, const qe
   a.dt_r = (R)p->dt; a.win_v_r = (R)p->window_v;
   a.seed = p->seed; a.scenario = p->scenario; a.step = p->step;
   a.win_s = -1;
+  a.counter = counter;
   a.emit = 1; a.pairs = 0; a.drain = 1; a.recoil_energy = p->recoil_energy ? 1 : 0;
   a.ledger_part = reinterpret_cast<double*>(base + kOffLedger);
   a.ledger = a.ledger_part + kMaxGrid * kLedgerN;
@@ -123,8 +116,7 @@ qed_status run_noalloc(const TablesDev& tv, const qed_soa* e, size_t n, const qe
   const int grid = std::min(step_grid_size(sizeof(R) == 4 ? QED_MIXED : QED_FP64), (int)kMaxGrid);
   launch_step<R>(a, grid, 256, 0, s);
   launch_finalize<R>(a, grid, s);
-  noalloc_end_kernel<<<1, 1, 0, s>>>(cnt, counter);
-  count_launch(2);
+  count_launch();
   const cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return set_error(QED_ERR_CUDA, cudaGetErrorString(err));
   return QED_OK;

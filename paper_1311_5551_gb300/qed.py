@@ -37,6 +37,7 @@ class TableParams(C.Structure):
 
 
 _dp = C.POINTER(C.c_double)
+_D3, _I3, _P4 = C.c_double * 3, C.c_int32 * 3, C.c_void_p * 4
 
 
 class TableArrays(C.Structure):
@@ -241,9 +242,10 @@ def _torch():
 
 
 def _stream_ptr(stream):
-    torch = _torch()
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the current stream's handle, without the object around it (a few microseconds per call)
+        torch = _torch()
+        return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return C.c_void_p(stream.cuda_stream)
 
 
@@ -496,9 +498,8 @@ class Field:
                 raise ValueError("grid must be a contiguous CUDA tensor of shape (6, nz, ny, nx)")
             ptr = self.grid.data_ptr()
             n = (self.grid.shape[3], self.grid.shape[2], self.grid.shape[1])
-        return FieldDesc(self.kind, (C.c_double * 3)(*self.E), (C.c_double * 3)(*self.B), self.E0, self.omega,
-                         self.phase0, self.phi_start, self.phi_len, ptr, (C.c_int32 * 3)(*n), int(self.shape),
-                         (C.c_double * 3)(*self.origin), (C.c_double * 3)(*self.spacing))
+        return FieldDesc(self.kind, _D3(*self.E), _D3(*self.B), self.E0, self.omega, self.phase0, self.phi_start,
+                         self.phi_len, ptr, _I3(*n), int(self.shape), _D3(*self.origin), _D3(*self.spacing))
 
 
 @dataclass
@@ -531,7 +532,7 @@ def _check_grid(fld, precision):
 
 
 def _sp_array(species):
-    return (C.c_void_p * 4)(*[s._h if s is not None else None for s in species])
+    return _P4(*[s._h if s is not None else None for s in species])
 
 
 def run(tables: Tables, species, params: StepParams, step: int, n_steps: int = 1, stream=None):
@@ -562,6 +563,28 @@ def read_ledger(species, stream=None) -> dict:
 _SOA_KEYS = ("x", "y", "z", "ux", "uy", "uz", "tau", "id")
 
 
+def _noalloc_args_plain(torch, cur, rbytes, electrons, n, photons, photon_counter) -> bool:
+    """True when every argument of step_emit_noalloc is as it should be, found the short way (a time
+    loop makes this check once per step); False leaves the answer, and its words, to the full one."""
+    real = torch.float32 if rbytes == 4 else torch.float64
+    dev = torch.device("cuda", cur)
+    x = photons.get("x")
+    if x is None:
+        return False
+    for arrays, length in ((electrons, n), (photons, x.numel())):
+        for k in _SOA_KEYS:
+            t = arrays.get(k)
+            if t is None or t.device != dev or not t.is_contiguous() or t.numel() < length:
+                return False
+            if k == "tau":
+                if t.element_size() != 8:
+                    return False
+            elif t.dtype != (torch.int32 if k == "id" else real):
+                return False
+    c = photon_counter
+    return c is not None and c.device == dev and c.is_contiguous() and c.dtype == torch.int32 and c.numel() >= 3
+
+
 def noalloc_arg_errors(precision: int, electrons: dict, n: int, photons: dict, photon_counter,
                        require_cuda: bool = True) -> list[str]:
     """Why the arguments of step_emit_noalloc would let the kernels read or write outside the
@@ -580,6 +603,8 @@ def noalloc_arg_errors(precision: int, electrons: dict, n: int, photons: dict, p
     if require_cuda:
         torch = _torch()
         cur = torch.cuda.current_device() if torch.cuda.is_available() else None
+        if not errs and cur is not None and _noalloc_args_plain(torch, cur, rbytes, electrons, n, photons, photon_counter):
+            return errs
 
     def check(name, t, min_len, nbytes, floating):
         if t is None:
