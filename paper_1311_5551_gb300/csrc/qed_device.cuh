@@ -592,6 +592,16 @@ __device__ __forceinline__ void bracket2(const R* A, int n, bool rising, R v, ui
 template <typename R>
 __device__ __forceinline__ int guide_bin(R v, R scale) { return min((int)(v * (scale * (R)kGuide)), kGuide - 1); }
 
+// Events in quads: where a warp has few, four neighbouring lanes take one event together, each its part
+// of the logarithms, square roots, exponentials and quotients (kQuad lanes hold the same event).
+constexpr int kQuad = 4;
+// Lane j of the quad's v (the quad's four lanes call this together).
+template <typename R>
+__device__ __forceinline__ R quad_get(R v, int j) {
+  const int base = (int)(threadIdx.x & 28u);
+  return __shfl_sync(0xfu << base, v, base + j);
+}
+
 // Photon energy fraction xi = 2chi/eta (Sec. 3) by inverting the two bracketing P_chi rows: what
 // does not depend on the draw is loaded first (it overlaps the random numbers).
 template <typename R>
@@ -599,8 +609,8 @@ struct XiSampler {
   int i, o;
   R w, p0[2], qn[2], zlo[2], zhi[2];
 
-  __device__ __forceinline__ void prepare(const TabDev<R>& T, R eta) {
-    grid_pos(Num<R>::log_(eta), T.ln_eta_min, T.inv_d_eta, T.n_eta, i, w, o);
+  __device__ __forceinline__ void prepare(const TabDev<R>& T, R ln_eta) {
+    grid_pos(ln_eta, T.ln_eta_min, T.inv_d_eta, T.n_eta, i, w, o);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const auto a = node_pair<R>(T.head, 2 * (i + r)), z = node_pair<R>(T.head, 2 * (i + r) + 1);
@@ -614,6 +624,8 @@ struct XiSampler {
   // Both rows inverted and blended: xi linear in P between the bracketing nodes j, j + 1; the
   // complement Q is used when U > 1/2 (the same interpolation, precise near P = 1).  (Loops over
   // the rows and nodes, not unrolled: the event path is long, straight and mostly fetched anew.)
+  // L lanes hold the draw: 1, or a quad, lane 2 r + t of it taking node t of row r.
+  template <int L = 1>
   __device__ __forceinline__ R sample(const TabDev<R>& T, R eta, R U, R V) const {
     const bool lower = U <= (R)0.5;
     const int n = T.n_xi;
@@ -624,22 +636,37 @@ struct XiSampler {
     bracket2<R>(A, n, lower, v, __ldg(g), __ldg(g + kGuide), j0, j1);
     const auto e0 = node_pair<R>(A, j0), e1 = node_pair<R>(A, n + j1);
     R xr[2];
+    if constexpr (L == 1) {
 #pragma unroll 1
-    for (int r = 0; r < 2; ++r) {
+      for (int r = 0; r < 2; ++r) {
+        const R lo = r ? e1.x : e0.x, hi = r ? e1.y : e0.y;
+        const R pz = r ? p0[1] : p0[0], qz = r ? qn[1] : qn[0], zl = r ? zlo[1] : zlo[0], zh = r ? zhi[1] : zhi[0];
+        const bool lo0 = U <= pz, hi1 = !lo0 && V <= qz;
+        const int j = lo0 ? 0 : (hi1 ? n - 1 : (r ? j1 : j0));
+        R x01[2];
+#pragma unroll 1
+        for (int t = 0; t < 2; ++t) {
+          const R z = zl + (R)(j + t) * (zh - zl) / (R)(n - 1);
+          const R xx = (R)1 / ((R)1 + Num<R>::exp_(-z));
+          if (t == 0) x01[0] = xx; else x01[1] = xx;
+        }
+        const R frac = lower ? (U - lo) / (hi - lo) : (lo - V) / (lo - hi);
+        const R x = lo0 || hi1 ? x01[0] : x01[0] + frac * (x01[1] - x01[0]);
+        if (r == 0) xr[0] = x; else xr[1] = x;
+      }
+    } else {
+      const int q = (int)(threadIdx.x & 3u), r = q >> 1, t = q & 1;
       const R lo = r ? e1.x : e0.x, hi = r ? e1.y : e0.y;
       const R pz = r ? p0[1] : p0[0], qz = r ? qn[1] : qn[0], zl = r ? zlo[1] : zlo[0], zh = r ? zhi[1] : zhi[0];
       const bool lo0 = U <= pz, hi1 = !lo0 && V <= qz;
       const int j = lo0 ? 0 : (hi1 ? n - 1 : (r ? j1 : j0));
-      R x01[2];
-#pragma unroll 1
-      for (int t = 0; t < 2; ++t) {
-        const R z = zl + (R)(j + t) * (zh - zl) / (R)(n - 1);
-        const R xx = (R)1 / ((R)1 + Num<R>::exp_(-z));
-        if (t == 0) x01[0] = xx; else x01[1] = xx;
-      }
+      const R z = zl + (R)(j + t) * (zh - zl) / (R)(n - 1);
+      const R xx = (R)1 / ((R)1 + Num<R>::exp_(-z));
+      const R x0 = quad_get(xx, 2 * r), x1 = quad_get(xx, 2 * r + 1);
       const R frac = lower ? (U - lo) / (hi - lo) : (lo - V) / (lo - hi);
-      const R x = lo0 || hi1 ? x01[0] : x01[0] + frac * (x01[1] - x01[0]);
-      if (r == 0) xr[0] = x; else xr[1] = x;
+      const R x = lo0 || hi1 ? x0 : x0 + frac * (x1 - x0);
+      xr[0] = quad_get(x, 0);
+      xr[1] = quad_get(x, 2);
     }
     R x = ((R)1 - w) * xr[0];
     if (w > (R)0) x += w * xr[1];
@@ -653,18 +680,19 @@ struct XiSampler {
 template <typename R>
 __device__ __forceinline__ bool sample_xi(const TabDev<R>& T, R eta, R U, R V, R& xi) {
   XiSampler<R> s;
-  s.prepare(T, eta);
+  s.prepare(T, Num<R>::log_(eta));
   if (!s.above_cut(U)) return false;
   xi = s.sample(T, eta, U, V);
   return true;
 }
 
 // Positron energy fraction f (Sec. 3, App. B): U < 1/2 maps to f <= 1/2 through V = 2U,
-// U >= 1/2 to f >= 1/2 through V = 2(1 - U).
-template <typename R>
-__device__ __forceinline__ R sample_f(const TabDev<R>& T, R chi, R U, R Vc) {
+// U >= 1/2 to f >= 1/2 through V = 2(1 - U).  L lanes hold the draw: 1, or a quad, lane 2 r + t of it
+// taking node t of row r.
+template <typename R, int L = 1>
+__device__ __forceinline__ R sample_f(const TabDev<R>& T, R ln_chi, R U, R Vc) {
   int i, o; R w;
-  grid_pos(Num<R>::log_(chi), T.ln_chi_min, T.inv_d_chi, T.n_chi, i, w, o);
+  grid_pos(ln_chi, T.ln_chi_min, T.inv_d_chi, T.n_chi, i, w, o);
   const bool lower = U < (R)0.5;
   const R V = lower ? (R)2 * U : (R)2 * Vc;
   const int n = T.n_f;
@@ -673,13 +701,22 @@ __device__ __forceinline__ R sample_f(const TabDev<R>& T, R chi, R U, R Vc) {
   int j[2];
   bracket2<R>(P, n, true, V, __ldg(g), __ldg(g + kGuide), j[0], j[1]);
   R fr[2];
+  if constexpr (L == 1) {
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int lo = j[r];
+    for (int r = 0; r < 2; ++r) {
+      const int lo = j[r];
+      const auto e = node_pair<R>(P, r * n + lo);
+      const R frac = (V - e.x) / (e.y - e.x);
+      const R f0 = (R)0.5 * (R)lo / (R)(n - 1), f1 = (R)0.5 * (R)(lo + 1) / (R)(n - 1);
+      fr[r] = f0 + frac * (f1 - f0);
+    }
+  } else {
+    const int q = (int)(threadIdx.x & 3u), r = q >> 1, lo = r ? j[1] : j[0];
     const auto e = node_pair<R>(P, r * n + lo);
-    const R frac = (V - e.x) / (e.y - e.x);
-    const R f0 = (R)0.5 * (R)lo / (R)(n - 1), f1 = (R)0.5 * (R)(lo + 1) / (R)(n - 1);
-    fr[r] = f0 + frac * (f1 - f0);
+    const R frac = (V - e.x) / (e.y - e.x), ft = (R)0.5 * (R)(lo + (q & 1)) / (R)(n - 1);
+    const R f0 = quad_get(ft, 2 * r), f = f0 + frac * (quad_get(ft, 2 * r + 1) - f0);
+    fr[0] = quad_get(f, 0);
+    fr[1] = quad_get(f, 2);
   }
   R fh = ((R)1 - w) * fr[0];
   if (w > (R)0) fh += w * fr[1];

@@ -29,9 +29,15 @@ namespace qedlib {
 
 namespace {
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kBlock = 256;            // compute threads of a step block (one tile of particles)
-constexpr int kWarps = kBlock / 32;    // compute warps
-constexpr int kStepThreads = kBlock + 32;  // plus one producer warp that issues the tile copies
+// Compute threads of a step block (one tile of particles), compute warps, and all threads: plus one
+// producer warp that issues the tile copies.  FP64 blocks are half as large, and two of them share an SM: a
+// warp instruction holds the SM's one FP64 pipe for 16 cycles however few its lanes, so a small
+// population has to reach many SMs (1e4 particles are 40 tiles of 256).  On GB300 100 steps of 1e4
+// electrons in a field took 4.22 ms with tiles of 256 particles, 3.65 with 128, 3.57 with 64 and 3.48
+// with 32; 60 of 1e5 in a wave 2.58, 2.50, 2.56 and 2.88.
+template <typename R> constexpr int kTile = sizeof(R) == 4 ? 256 : 128;
+template <typename R> constexpr int kWarps = kTile<R> / 32;
+template <typename R> constexpr int kStepThreads = kTile<R> + 32;
 
 enum LedgerSlot {
   kN0 = 0, kN1, kN2, kE0, kE1, kE2, kEmitN, kEmitE, kDrop, kEmitDef, kPairN, kPairE, kPairDef, kOorEta, kOorChi
@@ -298,7 +304,7 @@ __device__ __forceinline__ void lepton_events(const StepArgs<R>& a, uint32_t pha
   Uniform<R> U[4];
   if (ev) {
     const uint32_t id = sp.id[i];
-    xs.prepare(a.tab, eta);
+    xs.prepare(a.tab, Num<R>::log_(eta));
     draw4r<R>(a.seed, a.scenario, id, a.step, (uint64_t)kind, 0, U);
     child = xs.above_cut(U[0].u);
   }
@@ -363,6 +369,111 @@ __device__ __forceinline__ void lepton_events(const StepArgs<R>& a, uint32_t pha
     }
   }
   if (ev) {
+    sp.ux[i] = u[0]; sp.uy[i] = u[1]; sp.uz[i] = u[2];
+    tau.store(sp.tau + i);
+  }
+  __syncwarp();  // the ring slots read above may be refilled by the next chunk
+}
+
+// The same for at most kFew events, entry p of the ring on a quad's four lanes.
+template <typename R, bool WANT>
+__device__ __forceinline__ void lepton_events_quads(const StepArgs<R>& a, uint32_t phase, int kind,
+                                                    const EventRing<R>* ring, uint32_t p, uint32_t take, EventSums<R>& es) {
+  const SpeciesDev<R>& sp = a.sp[kind];
+  const SpeciesDev<R>& dst = a.sp[2];  // photon children are appended to the photon species
+  const int lane = threadIdx.x & 31, part = lane % kQuad;
+  const bool ev = (uint32_t)(lane / kQuad) < take, lead = ev && part == 0;
+  uint32_t i = 0;
+  R x = (R)0, y = (R)0, z = (R)0, u[3] = {(R)0, (R)0, (R)0}, eta = (R)0;
+  if (ev) {
+    i = ring->i[p];
+    x = ring->v[0][p]; y = ring->v[1][p]; z = ring->v[2][p];
+    u[0] = ring->v[3][p]; u[1] = ring->v[4][p]; u[2] = ring->v[5][p];
+    eta = ring->v[6][p];
+  }
+  // gamma from u after the push, as the push computed it
+  const R u2 = dot3<R>(u, u);
+  const R root = Num<R>::sqrt_(part == 1 ? u2 : (R)1 + u2);  // (what root_inv_ gives on the FP64 path)
+  R gam = quad_get(root, 0);
+  const R um = quad_get(root, 1);
+  R lnU1 = (R)0, lnU2 = (R)0;
+  bool child = false;
+  R kx = (R)0, ky = (R)0, kz = (R)0, emitted = (R)0, def = (R)0;
+  Tau<R> tau = Tau<R>::one(), ctau = Tau<R>::one();
+  // whether there is a photon is known before its energy: the append slots are asked for first, and
+  // their answer comes while the energies are searched
+  XiSampler<R> xs;
+  Uniform<R> U[4];
+  if (ev) {
+    const uint32_t id = sp.id[i];
+    draw4r<R>(a.seed, a.scenario, id, a.step, (uint64_t)kind, 0, U);
+    const R ln = Num<R>::log_(part == 0 ? eta : (part == 1 ? U[1].u : U[2].u));
+    xs.prepare(a.tab, quad_get(ln, 0));
+    lnU1 = quad_get(ln, 1);
+    lnU2 = quad_get(ln, 2);
+    child = xs.above_cut(U[0].u);
+  }
+  const unsigned childm = __ballot_sync(kFull, child && part == 0);
+  const uint32_t nc = (uint32_t)__popc(childm);
+  const int leader = __ffs(childm) - 1;
+  uint32_t base = 0;
+  if (lane == leader) base = atomicAdd(&dst.cnt->n_app, nc);
+  if (ev) {
+    if (child) {
+      const R xi = xs.template sample<kQuad>(a.tab, eta, U[0].u, U[0].v);
+      const R eps = xi * gam;
+      const R ium = (R)1 / um;
+      const R h0 = u[0] * ium, h1 = u[1] * ium, h2 = u[2] * ium;
+      kx = eps * h0; ky = eps * h1; kz = eps * h2;
+      // recoil p_f = p_i - (h nu/c) phat_i (Sec. 3), or energy-conserving on request
+      R umf;
+      if (a.recoil_energy) { const R gf = gam - eps; umf = gf > (R)1 ? Num<R>::sqrt_(gf * gf - (R)1) : (R)0; }
+      else umf = um > eps ? um - eps : (R)0;
+      u[0] = umf * h0; u[1] = umf * h1; u[2] = umf * h2;
+      const R gf = Num<R>::sqrt_((R)1 + umf * umf);
+      // energy defect (gamma_f + eps) - gamma_i (Sec. 3.1); for the momentum-conserving recoil
+      // written without cancellation as 2 eps / ((gamma_i + |u_i|)(gamma_f + gamma_i - eps))
+      if (!a.recoil_energy && um > eps) def = (R)2 * eps / ((gam + um) * (gf + gam - eps));
+      else def = (gf + eps) - gam;
+      emitted = eps;
+      gam = gf;
+      ctau = Tau<R>::fresh(-lnU2);
+    } else if (lead) {
+      // no photon: the event is not a child after all
+      atomicAnd(&sp.evmask[i >> 5], ~(1u << (i & 31u)));
+      count_events(sp, phase, i >> 5, 0xffffffffu);
+    }
+    tau = Tau<R>::fresh(-lnU1);
+  }
+  if (WANT) {
+    const KSum<R> se = warp_ksum<R>(part == 0 ? emitted : (R)0), sd = warp_ksum<R>(part == 0 ? def : (R)0),
+                  sg = warp_ksum<R>(lead ? gam : (R)0);
+    if (lane == 0) {
+      es.emit_e.merge(se);
+      es.emit_def.merge(sd);
+      es.emit_n += nc;
+      es.drop += take - nc;
+      es.e[kind].merge(sg);
+      es.n[kind] += take;
+      if (!a.drain) { es.e[2].merge(se); es.n[2] += nc; }
+    }
+  }
+  if (childm) {
+    base = __shfl_sync(kFull, base, leader);
+    if (child && lead) {
+      const uint32_t slot = base + (uint32_t)__popc(childm & ((1u << lane) - 1u));
+      if (slot < dst.acap) {
+        dst.ax[slot] = x; dst.ay[slot] = y; dst.az[slot] = z;
+        dst.aux[slot] = kx; dst.auy[slot] = ky; dst.auz[slot] = kz;
+        ctau.store(dst.atau + slot);
+        dst.aparent[slot] = i | ((uint32_t)kind << 31);
+        if (dst.aw) dst.aw[slot] = sp.w ? sp.w[i] : (R)1;  // the photon stands for as many
+      } else {
+        atomicOr(&dst.cnt->err, 1u << QED_ERR_CAPACITY);
+      }
+    }
+  }
+  if (lead) {
     sp.ux[i] = u[0]; sp.uy[i] = u[1]; sp.uz[i] = u[2];
     tau.store(sp.tau + i);
   }
@@ -465,7 +576,7 @@ __device__ __forceinline__ void photon_events(const StepArgs<R>& a, const EventR
   if (ev) {
     Uniform<R> U[4];
     draw4r<R>(a.seed, a.scenario, sp.id[i], a.step, (uint64_t)QED_PHOTON, 0, U);
-    const R f = sample_f<R>(a.tab, chi, U[0].u, U[0].v);
+    const R f = sample_f<R>(a.tab, Num<R>::log_(chi), U[0].u, U[0].v);
     R se = (R)1 - f, sq = f;  // the positron takes f h nu (Sec. 3)
     if (a.recoil_energy && eps >= (R)2) {
       const R g1 = (R)1 + f * (eps - (R)2), g0 = (R)1 + ((R)1 - f) * (eps - (R)2);
@@ -526,8 +637,87 @@ __device__ __forceinline__ void photon_events(const StepArgs<R>& a, const EventR
   __syncwarp();  // the ring slots read above may be refilled by the next chunk
 }
 
-// One pipeline stage: a tile of 256 consecutive particles of one species (8 warp chunks).
-constexpr int kTile = kBlock;
+// The same for at most kFew events, entry p of the ring on a quad's four lanes: the even lanes take the
+// electron, the odd ones the positron.
+template <typename R, bool WANT>
+__device__ __forceinline__ void photon_events_quads(const StepArgs<R>& a, const EventRing<R>* ring, uint32_t p, uint32_t take,
+                                                    EventSums<R>& es) {
+  const SpeciesDev<R>& sp = a.sp[2];
+  const int lane = threadIdx.x & 31, part = lane % kQuad, c = part & 1;
+  const uint32_t r = (uint32_t)(lane / kQuad);  // the event among those taken
+  const bool ev = r < take, lead = ev && part == 0;
+  uint32_t i = 0;
+  R x = (R)0, y = (R)0, z = (R)0, k[3] = {(R)0, (R)0, (R)1}, chi = (R)0;
+  if (ev) {
+    i = ring->i[p];
+    x = ring->v[0][p]; y = ring->v[1][p]; z = ring->v[2][p];
+    k[0] = ring->v[3][p]; k[1] = ring->v[4][p]; k[2] = ring->v[5][p];
+    chi = ring->v[6][p];
+  }
+  // the photon energy as the push computed it
+  R eps, ie;
+  Num<R>::root_inv_(dot3<R>(k, k), eps, ie);
+  // the lane's particle: its share of k, gamma and optical depth; the positron's gamma
+  R share = (R)0, gam = (R)0, gp = (R)0, converted = (R)0, def = (R)0;
+  Tau<R> tau = Tau<R>::one();
+  uint32_t be = 0, bp = 0;  // append slots, asked for first
+  if (lane == 0) {
+    be = atomicAdd(&a.sp[0].cnt->n_app, take);
+    bp = atomicAdd(&a.sp[1].cnt->n_app, take);
+  }
+  if (ev) {
+    Uniform<R> U[4];
+    draw4r<R>(a.seed, a.scenario, sp.id[i], a.step, (uint64_t)QED_PHOTON, 0, U);
+    const R ln = Num<R>::log_(part == 0 ? chi : (part == 1 ? U[1].u : U[2].u));
+    const R f = sample_f<R, kQuad>(a.tab, quad_get(ln, 0), U[0].u, U[0].v);
+    const bool keep = a.recoil_energy && eps >= (R)2;
+    const R fc = c ? f : (R)1 - f;  // the positron takes f h nu (Sec. 3)
+    share = fc;
+    if (keep) {
+      const R g1 = (R)1 + fc * (eps - (R)2);
+      share = Num<R>::sqrt_(g1 * g1 - (R)1) * ie;
+    }
+    const R pc = share * eps;
+    gam = Num<R>::sqrt_((R)1 + pc * pc);
+    gp = quad_get(gam, 1);
+    const R inv = (R)1 / (gam + pc), inv_p = quad_get(inv, 1);
+    tau = Tau<R>::fresh(-quad_get(ln, 1 + c));
+    // defect (gamma_- + gamma_+) - eps (Sec. 3.1); for the momentum split it is exactly
+    // 1/(gamma_- + p_-) + 1/(gamma_+ + p_+), written so to avoid cancellation
+    def = keep ? (gam + gp) - eps : inv + inv_p;
+    converted = eps;
+  }
+  if (WANT) {
+    const KSum<R> se = warp_ksum<R>(lead ? converted : (R)0), sd = warp_ksum<R>(lead ? def : (R)0);
+    const KSum<R> s0 = warp_ksum<R>(lead ? gam : (R)0), s1 = warp_ksum<R>(lead ? gp : (R)0);
+    if (lane == 0) {
+      es.pair_e.merge(se);
+      es.pair_def.merge(sd);
+      es.pair_n += take;
+      es.e[0].merge(s0); es.n[0] += take;
+      es.e[1].merge(s1); es.n[1] += take;
+    }
+  }
+  be = __shfl_sync(kFull, be, 0);
+  bp = __shfl_sync(kFull, bp, 0);
+  if (ev && part < 2) {
+    const SpeciesDev<R>& d = c ? a.sp[1] : a.sp[0];
+    const uint32_t s = (c ? bp : be) + r;
+    if (s < d.acap) {
+      d.ax[s] = x; d.ay[s] = y; d.az[s] = z;
+      d.aux[s] = share * k[0]; d.auy[s] = share * k[1]; d.auz[s] = share * k[2];
+      tau.store(d.atau + s);
+      d.aparent[s] = i;
+      if (d.aw) d.aw[s] = sp.w ? sp.w[i] : (R)1;
+    } else {
+      atomicOr(&d.cnt->err, 1u << QED_ERR_CAPACITY);
+    }
+  }
+  if (lead) Tau<R>::infinite().store(sp.tau + i);  // the photon is annihilated
+  __syncwarp();  // the ring slots read above may be refilled by the next chunk
+}
+
+// One pipeline stage: a tile of consecutive particles of one species, a chunk of 32 per compute warp.
 
 template <typename R>
 struct TileBuf;
@@ -551,8 +741,8 @@ constexpr uint32_t kWaitLimit = 1u << 16;  // mbarrier polls (<= 20 us each) bef
 
 template <typename R>
 struct TileBuf {
-  R x[kTile], y[kTile], z[kTile], ux[kTile], uy[kTile], uz[kTile];
-  double tau[kTile];
+  R x[kTile<R>], y[kTile<R>], z[kTile<R>], ux[kTile<R>], uy[kTile<R>], uz[kTile<R>];
+  double tau[kTile<R>];
 };
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -588,7 +778,7 @@ __device__ __forceinline__ uint32_t conversion_tiles(uint32_t win_n, uint32_t nb
 template <typename R>
 __device__ __forceinline__ void issue_tile(const StepArgs<R>& a, TileBuf<R>* buf, uint64_t* bar, uint32_t k, uint32_t n0,
                                         uint32_t n1, uint32_t n2, uint32_t win_n, uint32_t blk, uint32_t nblk) {
-  const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 - win_n + kTile - 1) / kTile;
+  const uint32_t T0 = (n0 + kTile<R> - 1) / kTile<R>, T1 = (n1 + kTile<R> - 1) / kTile<R>, T2 = (n2 - win_n + kTile<R> - 1) / kTile<R>;
   const uint32_t t = blk + k * nblk;
   if (t >= T0 + T1 + T2) {
     // a tile of a photon window's conversions: nothing to copy
@@ -599,8 +789,8 @@ __device__ __forceinline__ void issue_tile(const StepArgs<R>& a, TileBuf<R>* buf
   decode_tile(t, T0, T1, s, j);
   const TileSrc<R> src = tile_src(a.sp[s]);
   const uint32_t ns = s == 0 ? n0 : (s == 1 ? n1 : n2);
-  const uint32_t first = (s == 2 ? win_n : 0u) + j * kTile;
-  const uint32_t valid = min((uint32_t)kTile, ns - first);
+  const uint32_t first = (s == 2 ? win_n : 0u) + j * kTile<R>;
+  const uint32_t valid = min((uint32_t)kTile<R>, ns - first);
   // arrays start 16-byte aligned and tiles start at multiples of 256 particles, so every source
   // is 16-byte aligned; only whole 16-byte pieces are copied (no read past the last particle),
   // the ragged remainder of the last tile is read with plain loads by its threads
@@ -620,7 +810,8 @@ __device__ __forceinline__ void issue_tile(const StepArgs<R>& a, TileBuf<R>* buf
 }
 
 // barrier among the compute warps only (the producer warp does not take part)
-__device__ __forceinline__ void compute_warps_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kBlock) : "memory"); }
+template <typename R>
+__device__ __forceinline__ void compute_warps_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTile<R>) : "memory"); }
 
 // Fixed-order block reduction of the ledger partials in the working precision: compensated
 // sums are combined pairwise (two-sum), counts as integers; only the block totals become FP64
@@ -686,7 +877,7 @@ __device__ __forceinline__ void write_step_partial(const EventRing<R>* ring, dou
   if (k >= kLedgerN) return;
   KSum<R> t;
   uint32_t n = 0;
-  for (int w = 0; w < kWarps; ++w) {
+  for (int w = 0; w < kWarps<R>; ++w) {
     const EventSums<R>& es = ring[w].sums;
     switch (k) {
       case kN0: case kN1: case kN2: n += es.n[k - kN0]; break;
@@ -767,8 +958,8 @@ __device__ __forceinline__ bool run_tiles(const StepArgs<R>& A, const StepScalar
                                           const TileRun& run, WarpState<R>& w, RunSums<R>& sums) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t n = run.n, base = SP == 2 ? run.base : 0u;
-  const uint32_t last = n > base ? (n - base - 1u) / (uint32_t)kTile : 0u;  // the only tile that can be ragged
-  const uint32_t valid = n - base - last * (uint32_t)kTile;
+  const uint32_t last = n > base ? (n - base - 1u) / (uint32_t)kTile<R> : 0u;  // the only tile that can be ragged
+  const uint32_t valid = n - base - last * (uint32_t)kTile<R>;
   const uint32_t in_r = floor16(valid * (uint32_t)sizeof(R)) / (uint32_t)sizeof(R);
   const uint32_t in_t = floor16(valid * 8u) / 8u;
   const bool ragged = in_r < valid || in_t < valid;
@@ -784,14 +975,14 @@ __device__ __forceinline__ bool run_tiles(const StepArgs<R>& A, const StepScalar
     // the ragged remainder of a species' last tile: each thread reads its own particle
     if (ragged && j == last && r < valid && (r >= in_r || r >= in_t)) {
       const SpeciesDev<R>& gs = A.sp[SP];
-      const uint32_t gi = base + j * kTile + r;
+      const uint32_t gi = base + j * kTile<R> + r;
       if (r >= in_r) {
         b.x[r] = gs.x[gi]; b.y[r] = gs.y[gi]; b.z[r] = gs.z[gi];
         b.ux[r] = gs.ux[gi]; b.uy[r] = gs.uy[gi]; b.uz[r] = gs.uz[gi];
       }
       if (r >= in_t) b.tau[r] = gs.tau[gi];
     }
-    const uint32_t chunk = base / 32u + j * kWarps + warp;
+    const uint32_t chunk = base / 32u + j * kWarps<R> + warp;
     if constexpr (SP == 2)
       photon_chunk<R, G, FC, WANT>(A, S, P.lnT, chunk, n, lane, sums, w.pushed_ph, w.tau_ph, w.q, b.x[r], b.y[r], b.z[r],
                                    b.ux[r], b.uy[r], b.uz[r], &b.tau[r]);
@@ -819,13 +1010,13 @@ __device__ __forceinline__ bool run_conversions(const StepArgs<R>& a, const Step
                                                 const TileRun& run, WarpState<R>& ws, ConversionState& c) {
   const SpeciesDev<R>& sp = a.sp[2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t groups = run.n >> 10, stride = (run.g_hi - run.g_lo) * kWarps;
+  const uint32_t groups = run.n >> 10, stride = (run.g_hi - run.g_lo) * kWarps<R>;
   for (;;) {
     if (!c.open) {
       const uint32_t t = P.blk + ws.k * P.nblk;
       if (t >= run.g_hi) return false;
       if (!tile_ready(P, ws)) { ++ws.k; continue; }
-      c.first = c.next = (t - run.g_lo) * kWarps + (uint32_t)warp;
+      c.first = c.next = (t - run.g_lo) * kWarps<R> + (uint32_t)warp;
       c.open = true;
     }
     while (__any_sync(kFull, c.m != 0u) || c.todo || c.next < groups) {
@@ -892,9 +1083,16 @@ __device__ __forceinline__ void fold_run_sums(const RunSums<R>& sums, int s, Eve
   }
 }
 
+// Up to this many events per warp are taken in quads, on the FP64 path: what bounds a small step's events
+// there is the chain of FP64 instructions (350 of them for a batch of 1 to 32 events, at some 70
+// cycles each; in quads 150).  On GB300 100 steps of 1e4 electrons went from 3.65 to 3.0 ms; the
+// mixed path, whose registers are full, lost 2 to 5% to the second form in the kernel and has only one.
+template <typename R> constexpr uint32_t kFew = sizeof(R) == 8 ? 32 / kQuad : 0;
+
 // The block's tiles of one run of leptons and all their events (every compute warp of the block calls
 // this): a warp takes 32 events whenever it has them, and what is left in the block's rings is
-// taken together, 32 per warp: eight rings with fewer than 32 each make at most eight batches.
+// taken together, 32 per warp (or fewer, in quads): rings with fewer than 32 each make at most one
+// batch per warp.
 template <typename R, bool G, bool WANT>
 __device__ __forceinline__ void run_leptons(const StepArgs<R>& A, const StepScalars<R>& S, const StepPipe<R>& P,
                                             const TileRun& run, WarpState<R>& w) {
@@ -912,34 +1110,44 @@ __device__ __forceinline__ void run_leptons(const StepArgs<R>& A, const StepScal
                         : run_tiles<R, G, kFieldAny, 1, WANT>(A, S, P, run, w, sums);
     const EventRing<R>* src = w.q.r;
     uint32_t p = w.q.head + (uint32_t)lane, take = 32u;
+    [[maybe_unused]] bool few = false;
     if (more) {  // 32 of the warp's own
       w.q.head += 32u;
       w.q.count -= 32u;
     } else {
       if (w.stopped) w.q.count = 0;  // (an unfinished step: QED_ERR_TIMEOUT)
       if (lane == 0) { w.q.r->head = w.q.head; w.q.r->count = w.q.count; }
-      compute_warps_sync();
-      uint32_t inc = lane < kWarps ? P.ring[lane].count : 0u;
+      compute_warps_sync<R>();
+      uint32_t inc = lane < kWarps<R> ? P.ring[lane].count : 0u;
 #pragma unroll
-      for (int off = 1; off < kWarps; off <<= 1) {
+      for (int off = 1; off < kWarps<R>; off <<= 1) {
         const uint32_t t = __shfl_up_sync(kFull, inc, off);
         if (lane >= off) inc += t;
       }
-      const uint32_t total = __shfl_sync(kFull, inc, kWarps - 1), e0 = (uint32_t)warp * 32u;
-      take = total > e0 ? min(32u, total - e0) : 0u;
-      const uint32_t e = e0 + (uint32_t)lane;
+      const uint32_t total = __shfl_sync(kFull, inc, kWarps<R> - 1);
+      if constexpr (kFew<R> != 0) few = total <= (uint32_t)kWarps<R> * kFew<R>;
+      const uint32_t each = few ? kFew<R> : 32u, e0 = (uint32_t)warp * each;
+      take = total > e0 ? min(each, total - e0) : 0u;
+      const uint32_t e = e0 + (uint32_t)(few ? lane / kQuad : lane);
       uint32_t j = 0, before = 0;
 #pragma unroll
-      for (int t = 0; t < kWarps - 1; ++t) {
+      for (int t = 0; t < kWarps<R> - 1; ++t) {
         const uint32_t upto = __shfl_sync(kFull, inc, t);
         if (e >= upto) { j = (uint32_t)t + 1u; before = upto; }
       }
       src = P.ring + j;
       p = src->head + e - before;
     }
+    if constexpr (kFew<R> != 0) {
+      if (few) {
+        if (take)
+          lepton_events_quads<R, WANT>(A, S.phase[run.s], run.s, src, p & (uint32_t)(kRing - 1), take, w.q.r->sums);
+        continue;
+      }
+    }
     if (take) lepton_events<R, WANT>(A, S.phase[run.s], run.s, src, p & (uint32_t)(kRing - 1), take, w.q.r->sums);
   }
-  compute_warps_sync();  // every ring has been read
+  compute_warps_sync<R>();  // every ring has been read
   w.q.count = 0;
   if (WANT) fold_run_sums(sums, run.s, w.q.r->sums);
 }
@@ -963,8 +1171,14 @@ __device__ __forceinline__ void run_photons(const StepArgs<R>& A, const StepScal
     }
     if (w.stopped) w.q.count = 0;
     const uint32_t take = min(w.q.count, 32u);
-    if (take)
+    const bool few = take <= kFew<R>;
+    if (take && !few)
       photon_events<R, WANT>(A, w.q.r, (w.q.head + (threadIdx.x & 31u)) & (uint32_t)(kRing - 1), take, w.q.r->sums);
+    if constexpr (kFew<R> != 0) {
+      if (take && few)
+        photon_events_quads<R, WANT>(A, w.q.r, (w.q.head + (threadIdx.x & 31u) / kQuad) & (uint32_t)(kRing - 1), take,
+                                     w.q.r->sums);
+    }
     w.q.head += take;
     w.q.count -= take;
   }
@@ -986,8 +1200,8 @@ __device__ __forceinline__ const R* packed_cells(const FieldDev& f) {
 
 // The step over one scenario, run by block `blk` of the `nblk` blocks given to it: block blk
 // takes the scenario's tiles blk, blk + nblk, ... and writes ledger partial number blk.
-// Warp roles: warps 0-7 compute (warp w takes 32-particle chunk w of each tile); warp 8 is the
-// producer: its first lane issues the bulk copies of tile k into stage k % kStages once the 8
+// Warp roles: all warps but the last compute (warp w takes 32-particle chunk w of each tile); the last is
+// the producer: its first lane issues the bulk copies of tile k into stage k % kStages once the
 // compute warps have released that stage (mbarrier `empty`, one arrival per warp); compute warps
 // wait only for their tile's data (mbarrier `full`), and for each other once per species, to share
 // out the events left in their rings.
@@ -995,7 +1209,7 @@ template <typename R, bool G, bool WANT>
 __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, uint32_t nblk, unsigned char* smem_raw) {
   TileBuf<R>* buf = reinterpret_cast<TileBuf<R>*>(smem_raw);
   EventRing<R>* ring = reinterpret_cast<EventRing<R>*>(buf + kStages);
-  R* s_lnh = reinterpret_cast<R*>(ring + kWarps);
+  R* s_lnh = reinterpret_cast<R*>(ring + kWarps<R>);
   R* s_lnT = s_lnh + a.tab.n_eta;
   __shared__ __align__(8) uint64_t full[kStages];
   __shared__ __align__(8) uint64_t empty[kStages];
@@ -1006,10 +1220,10 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // what does not depend on the step before: barriers, rate tables (fixed after their upload) and
   // the field scalars of this step
-  if (threadIdx.x == kBlock) {
+  if (threadIdx.x == kTile<R>) {
     for (int st = 0; st < kStages; ++st) {
       mbar_init(&full[st], 1);
-      mbar_init(&empty[st], kWarps);
+      mbar_init(&empty[st], kWarps<R>);
     }
     mbar_fence_init();
     s_abort = 0;
@@ -1021,18 +1235,18 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
   pdl_wait();
   const uint32_t n0 = a.sp[0].cnt->n, n1 = a.sp[1].cnt->n, n2 = a.sp[2].cnt->n;
   const uint32_t win_n = sizeof(R) == 4 && a.win_s >= 0 ? a.sp[2].cnt->win_n : 0u;
-  const uint32_t T0 = (n0 + kTile - 1) / kTile, T1 = (n1 + kTile - 1) / kTile, T2 = (n2 - win_n + kTile - 1) / kTile;
+  const uint32_t T0 = (n0 + kTile<R> - 1) / kTile<R>, T1 = (n1 + kTile<R> - 1) / kTile<R>, T2 = (n2 - win_n + kTile<R> - 1) / kTile<R>;
   const uint32_t T3 = conversion_tiles(win_n, nblk);
   const uint32_t ttot = T0 + T1 + T2 + T3;
   if (threadIdx.x < 3) S.phase[threadIdx.x] = a.sp[threadIdx.x].cnt->phase;
   if (G && threadIdx.x == 0) S.cells = packed_cells<R>(a.field);
-  if (threadIdx.x == kBlock)
+  if (threadIdx.x == kTile<R>)
     for (uint32_t k = 0; k < (uint32_t)kStages; ++k) issue_tile(a, buf, full, k, n0, n1, n2, win_n, blk, nblk);
   __syncthreads();
   pdl_launch();
 
   WarpState<R> w;
-  if (warp == kWarps) {
+  if (warp == kWarps<R>) {
     // ---------------- producer
     if (lane == 0) {
       uint32_t k = kStages;
@@ -1074,7 +1288,7 @@ __device__ __forceinline__ void step_body(const StepArgs<R>& a, uint32_t blk, ui
 
 // WANT: the step's ledger can be read (the last step of a run).
 template <typename R, bool G, bool WANT>
-__global__ void __launch_bounds__(kStepThreads, sizeof(R) == 4 ? QED_STEP_MIN_BLOCKS : 1)
+__global__ void __launch_bounds__(kStepThreads<R>, sizeof(R) == 4 ? QED_STEP_MIN_BLOCKS : 256 / kTile<double>)
 step_kernel(const __grid_constant__ StepArgs<R> a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   step_body<R, G, WANT>(a, blockIdx.x, gridDim.x, smem_raw);
@@ -1590,7 +1804,7 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const StepArgs<
   if (a.want && blockIdx.x == gridDim.x - 1) {
     // (blocks without a tile have nothing to add)
     uint32_t tiles = 0;
-    for (int s = 0; s < 3; ++s) tiles += (n[s] + kTile - 1) / kTile;
+    for (int s = 0; s < 3; ++s) tiles += (n[s] + kTile<R> - 1) / kTile<R>;
     reduce_ledger(a, (int)min((uint32_t)nparts, tiles));
   }
   // the last block to get here sets the counters: by then every block has read them
@@ -1945,7 +2159,7 @@ __global__ void __launch_bounds__(1024) batch_schedule_kernel(const BatchCtl<R> 
     const int sl = threadIdx.x * per + q;
     if (sl >= c.S || c.remaining[sl] == 0u) continue;
     const StepArgs<R>& a = c.args[sl];
-    for (int k = 0; k < 3; ++k) mine += (a.sp[k].cnt->n + kTile - 1) / kTile;
+    for (int k = 0; k < 3; ++k) mine += (a.sp[k].cnt->n + kTile<R> - 1) / kTile<R>;
   }
   atomicAdd(&s_tiles, mine);
   __syncthreads();
@@ -1959,7 +2173,7 @@ __global__ void __launch_bounds__(1024) batch_schedule_kernel(const BatchCtl<R> 
     if (live) {
       const StepArgs<R>& a = c.args[sl];
       uint32_t t = 0;
-      for (int k = 0; k < 3; ++k) t += (a.sp[k].cnt->n + kTile - 1) / kTile;
+      for (int k = 0; k < 3; ++k) t += (a.sp[k].cnt->n + kTile<R> - 1) / kTile<R>;
       if (t > 0) {
         b = (uint32_t)(c.target_blocks * (double)t / total + 0.5);
         b = max(1u, min(b, min(t, (uint32_t)c.max_parts)));
@@ -1977,7 +2191,7 @@ __global__ void __launch_bounds__(1024) batch_schedule_kernel(const BatchCtl<R> 
     if (c.live[sl]) {
       const StepArgs<R>& a = c.args[sl];
       uint32_t t = 0;
-      for (int k = 0; k < 3; ++k) t += (a.sp[k].cnt->n + kTile - 1) / kTile;
+      for (int k = 0; k < 3; ++k) t += (a.sp[k].cnt->n + kTile<R> - 1) / kTile<R>;
       if (t > 0) {
         uint32_t b = (uint32_t)(c.target_blocks * (double)t / total + 0.5);
         run += max(1u, min(b, min(t, (uint32_t)c.max_parts)));
@@ -2032,7 +2246,7 @@ __global__ void __launch_bounds__(1024) batch_tiles_kernel(const BatchCtl<R> c, 
       if (in) q.win_n = a.sp[2].cnt->win_n;
       for (int k = 0; k < 3; ++k) {
         q.n[k] = a.sp[k].cnt->n;
-        q.T[k] = (q.n[k] - (k == 2 ? q.win_n : 0u) + kTile - 1) / kTile;
+        q.T[k] = (q.n[k] - (k == 2 ? q.win_n : 0u) + kTile<R> - 1) / kTile<R>;
       }
       q.T[3] = conversion_tiles(q.win_n, (uint32_t)c.target_blocks);
       for (int k = 0; k < 4; ++k) tiles += q.T[k];
@@ -2073,7 +2287,7 @@ __device__ __forceinline__ void find_run(const SlotPlan* sp, int S, uint32_t g, 
   else { r.s = 3; r.g_lo = q.tile_base + T0 + T1 + T2; r.g_hi = r.g_lo + q.T[3]; r.n = q.win_n; }  // conversions
 }
 
-// Producer (thread kBlock): bulk copies of the block's k-th tile, global tile g, into stage
+// Producer (thread kTile<R>): bulk copies of the block's k-th tile, global tile g, into stage
 // k % kStages; as issue_tile, with the arrays of the tile's run (kept while the run lasts).
 template <typename R>
 __device__ __forceinline__ void issue_batch_tile(const BatchCtl<R>& c, TileBuf<R>* buf, uint64_t* bar, uint32_t k,
@@ -2087,8 +2301,8 @@ __device__ __forceinline__ void issue_batch_tile(const BatchCtl<R>& c, TileBuf<R
     return;
   }
   const TileSrc<R>& sp = src;
-  const uint32_t first = run.base + (g - run.g_lo) * kTile;
-  const uint32_t valid = min((uint32_t)kTile, run.n - first);
+  const uint32_t first = run.base + (g - run.g_lo) * kTile<R>;
+  const uint32_t valid = min((uint32_t)kTile<R>, run.n - first);
   const uint32_t br = floor16(valid * (uint32_t)sizeof(R)), bt = floor16(valid * 8u);
   TileBuf<R>& b = buf[k % kStages];
   uint64_t* bb = &bar[k % kStages];
@@ -2114,12 +2328,12 @@ __device__ __forceinline__ void issue_batch_tile(const BatchCtl<R>& c, TileBuf<R
 // barrier) when their tiles move on to the next slot, after taking the events queued for it and
 // writing its ledger partial.
 template <typename R, bool G>
-__global__ void __launch_bounds__(kStepThreads, sizeof(R) == 4 ? QED_BATCH_MIN_BLOCKS : 1)
+__global__ void __launch_bounds__(kStepThreads<R>, sizeof(R) == 4 ? QED_BATCH_MIN_BLOCKS : 256 / kTile<double>)
 batch_step_kernel(const BatchCtl<R> c) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   TileBuf<R>* buf = reinterpret_cast<TileBuf<R>*>(smem_raw);
   EventRing<R>* ring = reinterpret_cast<EventRing<R>*>(buf + kStages);
-  R* s_lnh = reinterpret_cast<R*>(ring + kWarps);
+  R* s_lnh = reinterpret_cast<R*>(ring + kWarps<R>);
   R* s_lnT = s_lnh + c.tab.n_eta;
   __shared__ __align__(8) uint64_t full[kStages];
   __shared__ __align__(8) uint64_t empty[kStages];
@@ -2132,10 +2346,10 @@ batch_step_kernel(const BatchCtl<R> c) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int k = threadIdx.x; k < c.tab.n_eta; k += blockDim.x) s_lnh[k] = c.tab.ln_h[k];
   for (int k = threadIdx.x; k < c.tab.n_chi; k += blockDim.x) s_lnT[k] = c.tab.ln_T[k];
-  if (threadIdx.x == kBlock) {
+  if (threadIdx.x == kTile<R>) {
     for (int st = 0; st < kStages; ++st) {
       mbar_init(&full[st], 1);
-      mbar_init(&empty[st], kWarps);
+      mbar_init(&empty[st], kWarps<R>);
     }
     mbar_fence_init();
     s_abort = 0;
@@ -2147,11 +2361,11 @@ batch_step_kernel(const BatchCtl<R> c) {
   pdl_launch();
   TileRun prun;  // producer's run of tiles and its arrays
   TileSrc<R> psrc{};
-  if (threadIdx.x == kBlock)
+  if (threadIdx.x == kTile<R>)
     for (uint32_t k = 0; k < (uint32_t)kStages && blk + k * nblk < ttot; ++k)
       issue_batch_tile(c, buf, full, k, blk + k * nblk, prun, psrc);
 
-  if (warp == kWarps) {
+  if (warp == kWarps<R>) {
     // ---------------- producer
     if (lane == 0) {
       uint32_t k = kStages;
@@ -2185,14 +2399,14 @@ batch_step_kernel(const BatchCtl<R> c) {
   auto flush_slot = [&]() {
     add_work(w.pushed_ph, w.tau_ph, s_work, lane);
     w.pushed_ph = w.tau_ph = 0;
-    compute_warps_sync();  // every warp has added its work and its sums
+    compute_warps_sync<R>();  // every warp has added its work and its sums
     if (threadIdx.x == 0) {
       flush_work(s_work, A.work);
       s_work[0] = s_work[1] = 0;
     }
     if (A.want) {
       write_step_partial<R>(ring, A.ledger_part, part);
-      compute_warps_sync();
+      compute_warps_sync<R>();
       if (lane == 0) w.q.r->sums = EventSums<R>{};
     }
   };
@@ -2202,15 +2416,15 @@ batch_step_kernel(const BatchCtl<R> c) {
     find_run(c.splan, c.S, g, run);
     if (run.slot != cur) {
       if (cur >= 0) flush_slot();
-      compute_warps_sync();  // every warp is done with the previous slot's arguments
+      compute_warps_sync<R>();  // every warp is done with the previous slot's arguments
       const unsigned long long* sa = reinterpret_cast<const unsigned long long*>(c.args + run.slot);
       const unsigned long long* ss = reinterpret_cast<const unsigned long long*>(
           static_cast<const StepScalars<R>*>(c.scal) + run.slot);
       unsigned long long* da = reinterpret_cast<unsigned long long*>(&A);
       unsigned long long* ds = reinterpret_cast<unsigned long long*>(&S);
-      for (int q = threadIdx.x; q < nw; q += kBlock) da[q] = sa[q];
-      for (int q = threadIdx.x; q < ns; q += kBlock) ds[q] = ss[q];
-      compute_warps_sync();
+      for (int q = threadIdx.x; q < nw; q += kTile<R>) da[q] = sa[q];
+      for (int q = threadIdx.x; q < ns; q += kTile<R>) ds[q] = ss[q];
+      compute_warps_sync<R>();
       cur = run.slot;
       part = g - run.slot_lo;  // < G: the block's first tile of the slot
     }
@@ -2502,7 +2716,7 @@ __global__ void sample_kernel(const TabDev<R> tab, int which, size_t n, const do
       out[i] = good ? (double)xi : 0.0;
       ok[i] = good ? 1 : 0;
     } else {
-      out[i] = (double)sample_f<R>(tab, (R)param[i], u, v);
+      out[i] = (double)sample_f<R>(tab, Num<R>::log_((R)param[i]), u, v);
       ok[i] = 1;
     }
   }
@@ -2656,7 +2870,7 @@ static void launch_pdl(void (*k)(P...), int grid, int block, size_t smem, cudaSt
 // then ln h and ln T
 template <typename R>
 static size_t step_smem(int n_eta, int n_chi) {
-  return (size_t)kStages * sizeof(TileBuf<R>) + (size_t)kWarps * sizeof(EventRing<R>) +
+  return (size_t)kStages * sizeof(TileBuf<R>) + (size_t)kWarps<R> * sizeof(EventRing<R>) +
          (size_t)(n_eta + n_chi) * sizeof(R);
 }
 
@@ -2689,8 +2903,8 @@ struct Residency {
 int step_grid_size(int precision) {
   // occupancy for the paper's table sizes (256 eta, 256 chi)
   static Residency mixed, fp64;
-  const int b = precision == QED_MIXED ? mixed(step_kernel<float, false, false>, kStepThreads, step_smem<float>(256, 256))
-                                       : fp64(step_kernel<double, false, false>, kStepThreads, step_smem<double>(256, 256));
+  const int b = precision == QED_MIXED ? mixed(step_kernel<float, false, false>, kStepThreads<float>, step_smem<float>(256, 256))
+                                       : fp64(step_kernel<double, false, false>, kStepThreads<double>, step_smem<double>(256, 256));
   return sm_count() * b;
 }
 
@@ -2705,8 +2919,8 @@ void launch_step(const StepArgs<R>& a, int grid, int block, size_t smem_unused, 
   const auto k = a.want ? (g ? step_kernel<R, true, true> : step_kernel<R, false, true>)
                         : (g ? step_kernel<R, true, false> : step_kernel<R, false, false>);
   static Residency known[4];
-  known[(a.want ? 2 : 0) + (g ? 1 : 0)](k, kStepThreads, smem);  // (raises the shared memory limit)
-  launch_pdl(k, grid, kStepThreads, smem, s, a);
+  known[(a.want ? 2 : 0) + (g ? 1 : 0)](k, kStepThreads<R>, smem);  // (raises the shared memory limit)
+  launch_pdl(k, grid, kStepThreads<R>, smem, s, a);
   count_launch();
 }
 
@@ -2728,7 +2942,7 @@ void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, BatchEnd end,
   const size_t smem = step_smem<R>(n_eta, n_chi);
   const auto k = c.grid_fields ? batch_step_kernel<R, true> : batch_step_kernel<R, false>;
   static Residency known[2];
-  known[c.grid_fields != 0](k, kStepThreads, smem);  // (raises the shared memory limit)
+  known[c.grid_fields != 0](k, kStepThreads<R>, smem);  // (raises the shared memory limit)
   if (c.fuse_k >= 2) {
     const size_t fsm = (size_t)(n_eta + n_chi) * sizeof(R);
     const int fgrid = c.target_blocks + c.S;
@@ -2746,7 +2960,7 @@ void launch_batch_step(const BatchCtl<R>& c, int n_eta, int n_chi, BatchEnd end,
   }
   // the per-step path: one tile space over all live slots, strided by a persistent grid
   launch_pdl(batch_tiles_kernel<R>, 1, 1024, 0, s, c, (int)end, win_w, (int)win_end, win_s);
-  launch_pdl(k, c.target_blocks, kStepThreads, smem, s, c);
+  launch_pdl(k, c.target_blocks, kStepThreads<R>, smem, s, c);
   launch_pdl(batch_plan_kernel<R>, c.S, 256, 0, s, c, c.target_blocks);
   launch_pdl(batch_scatter_kernel<R>, sm_count() * 4, 256, 0, s, c);
   count_launch(4);
