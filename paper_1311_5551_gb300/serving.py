@@ -68,6 +68,14 @@ class Scheduler:
             out.append(r)
         return out
 
+    def defer(self, r: Request):
+        """Takes back the admission of r: it is the first in the queue again."""
+        del self.running[r.slot]
+        self.in_use -= r.footprint
+        self.free.append(r.slot)
+        r.slot, r.admitted = -1, math.nan
+        self.pending.appendleft(r)
+
     def complete(self, slot: int, now: float) -> Request:
         r = self.running.pop(slot)
         r.done = now
@@ -212,6 +220,9 @@ def serve(qed, tables, requests, precision, slots: int = 64, budget_bytes: int =
         future.append(Request(k, t, w.n, w.n_steps, footprint(w, prec_bytes, caps), w))
     species = {}
     served_units = 0
+    # An admission that fits the budget can still find no block of its size where the allocator's free
+    # memory is split up: the request waits until a running one has given its blocks back.
+    waiting_for_memory = False
     t0 = time.perf_counter()
     rounds = 0
     while True:
@@ -223,9 +234,18 @@ def serve(qed, tables, requests, precision, slots: int = 64, budget_bytes: int =
         if admit_until is not None:
             while future and future[0].arrival > admit_until:
                 future.popleft()  # arrivals after the window are not part of the run
-        for r in sched.admit(now):
+        late = []  # admitted requests that found no memory, and those behind them
+        for r in [] if waiting_for_memory else sched.admit(now):
             w = r.payload.workload() if hasattr(r.payload, "workload") else r.payload
-            sp = make_species(qed, w, precision)
+            try:
+                sp = None if late else make_species(qed, w, precision)
+            except qed.QedError as e:
+                if e.code != qed.QED_ERR_OOM or not species:
+                    raise
+                sp = None
+            if sp is None:
+                late.append(r)
+                continue
             xr = w.x.copy()
             xr[:, 0] -= w.window_x0
             sp[0].upload(xr, w.u)
@@ -235,6 +255,9 @@ def serve(qed, tables, requests, precision, slots: int = 64, budget_bytes: int =
             batch.attach(r.slot, sp, p, 0, w.n_steps)
             qed.work_read(sp[0], reset=True)
             species[r.slot] = sp
+        for r in reversed(late):
+            sched.defer(r)
+        waiting_for_memory = waiting_for_memory or bool(late)
         if not sched.running:
             if sched.idle() and not future:
                 break
@@ -257,6 +280,7 @@ def serve(qed, tables, requests, precision, slots: int = 64, budget_bytes: int =
                 batch.detach(slot)
                 for s in sp:
                     s.close()
+                waiting_for_memory = False
     wall = time.perf_counter() - t0
     # work done on requests still running when the run stopped (a request waiting in the queue
     # has done none)

@@ -327,3 +327,66 @@ def test_rotating_field_recipe():
     period = 2 * math.pi / w.field.omega  # lambda / c in the time unit
     assert w.dt == pytest.approx(period / 200.0, rel=1e-12)
     assert w.field.omega == pytest.approx(2 * math.pi * 299792458.0 / 0.8e-6 * W.TIME_UNIT_S, rel=1e-9)
+
+
+def test_serving_waits_for_memory_that_the_budget_does_not_show(monkeypatch):
+    # an admission whose allocation fails is first in the queue again and runs after another finished
+    from types import SimpleNamespace
+
+    from paper_1311_5551_gb300 import qed, serving
+
+    blocks = {"held": 0}  # the allocator holds two requests at a time, whatever the budget says
+
+    class Store:
+        open = False
+
+        def __init__(self):
+            if blocks["held"] == 6:
+                raise qed.QedError(qed.QED_ERR_OOM, "no block")
+            blocks["held"] += 1
+            self.open = True
+
+        def upload(self, x, u):
+            pass
+
+        def init_tau(self, seed, scenario):
+            pass
+
+        def close(self):
+            blocks["held"] -= self.open
+            self.open = False
+
+        __del__ = close
+
+    class Batch:
+        def __init__(self, tables, precision, slots):
+            self.left = [0] * slots
+
+        def attach(self, slot, sp, p, step, n):
+            self.left[slot] = n
+
+        def detach(self, slot):
+            self.left[slot] = 0
+
+        def run(self, n):
+            self.left = [max(0, k - n) for k in self.left]
+
+        def remaining(self):
+            return self.left
+
+        def close(self):
+            pass
+
+    fake = SimpleNamespace(MIXED=0, Batch=Batch, QedError=qed.QedError, QED_ERR_OOM=qed.QED_ERR_OOM,
+                           StepParams=lambda **k: None, Field=lambda **k: None, read_ledger=lambda sp: {},
+                           work_read=lambda sp, reset=False: (1, 0, 0))
+    monkeypatch.setattr(serving, "make_species", lambda q, w, prec: [Store() for _ in range(3)])
+    w = SimpleNamespace(n=4, n_steps=10, x=np.zeros((4, 3)), u=np.zeros((4, 3)), window_x0=0.0, window_v=0.0, dt=1.0,
+                        seed=1, field=SimpleNamespace(as_dict=dict), extra={})
+    fin, st = serving.serve(fake, None, [(0.0, w)] * 5, 0, slots=4, chunk=5, max_wall=30.0)
+    assert sorted(r.rid for r in fin) == [0, 1, 2, 3, 4] and st["still_running"] == st["queued"] == 0
+    assert [r.rid for r in fin][:2] == [0, 1] and blocks["held"] == 0
+    # with nothing running there is nothing to wait for
+    blocks["held"] = 6
+    with pytest.raises(qed.QedError):
+        serving.serve(fake, None, [(0.0, w)], 0, slots=4, chunk=5, max_wall=30.0)
