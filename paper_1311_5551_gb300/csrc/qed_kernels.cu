@@ -34,7 +34,7 @@ constexpr unsigned kFull = 0xffffffffu;
 // warp instruction holds the SM's one FP64 pipe for 16 cycles however few its lanes, so a small
 // population has to reach many SMs (1e4 particles are 40 tiles of 256).  On GB300 100 steps of 1e4
 // electrons in a field took 4.22 ms with tiles of 256 particles, 3.65 with 128, 3.57 with 64 and 3.48
-// with 32; 60 of 1e5 in a wave 2.58, 2.50, 2.56 and 2.88.
+// with 32; 20 of 1e5 in a wave 2.58, 2.50, 2.56 and 2.88.
 template <typename R> constexpr int kTile = sizeof(R) == 4 ? 256 : 128;
 template <typename R> constexpr int kWarps = kTile<R> / 32;
 template <typename R> constexpr int kStepThreads = kTile<R> + 32;
@@ -791,7 +791,7 @@ __device__ __forceinline__ void issue_tile(const StepArgs<R>& a, TileBuf<R>* buf
   const uint32_t ns = s == 0 ? n0 : (s == 1 ? n1 : n2);
   const uint32_t first = (s == 2 ? win_n : 0u) + j * kTile<R>;
   const uint32_t valid = min((uint32_t)kTile<R>, ns - first);
-  // arrays start 16-byte aligned and tiles start at multiples of 256 particles, so every source
+  // arrays start 16-byte aligned and tiles start at multiples of 128 particles, so every source
   // is 16-byte aligned; only whole 16-byte pieces are copied (no read past the last particle),
   // the ragged remainder of the last tile is read with plain loads by its threads
   const uint32_t br = floor16(valid * (uint32_t)sizeof(R)), bt = floor16(valid * 8u);
