@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <mutex>
 
 #include "qed_device.cuh"
 
@@ -2878,10 +2879,9 @@ static size_t step_smem(int n_eta, int n_chi) {
 // Resident blocks per SM of a kernel at a given dynamic shared memory size, with its limit raised to
 // it (never lowered: another thread may be about to launch with more): asked of the runtime once per
 // kernel, device and size (the queries took a third of a one-step call's 12 us on the host).  Any
-// thread; two that ask at once find the same.
+// thread; the limit is compared and raised under a lock.
 struct Residency {
   std::atomic<uint64_t> known[128];  // per device: size << 16 | blocks (0: not asked yet)
-  std::atomic<uint64_t> limit[128];  // per device: the largest size asked for
   template <typename F>
   int operator()(F kernel, int threads, size_t smem) {
     int dev = 0;
@@ -2889,10 +2889,11 @@ struct Residency {
     std::atomic<uint64_t>* slot = dev >= 0 && dev < 128 ? &known[dev] : nullptr;
     const uint64_t have = slot ? slot->load(std::memory_order_relaxed) : 0;
     if (have && (have >> 16) == smem) return (int)(have & 0xffffu);
-    if (!slot || smem > limit[dev].load()) {
+    static std::mutex m;  // (one for all that ask for the same kernel type)
+    std::lock_guard<std::mutex> lock(m);
+    cudaFuncAttributes fa{};
+    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes < smem)
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (slot) limit[dev].store(smem);
-    }
     int b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess || b < 1) return 1;
     if (slot) slot->store((uint64_t)smem << 16 | (uint64_t)b, std::memory_order_relaxed);
