@@ -591,6 +591,19 @@ __device__ __forceinline__ void bracket2(const R* A, int n, bool rising, R v, ui
 // Guide entry of a draw v in [0, 1/scale].
 template <typename R>
 __device__ __forceinline__ int guide_bin(R v, R scale) { return min((int)(v * (scale * (R)kGuide)), kGuide - 1); }
+// The guide entries of v in two neighbouring rows of n nodes.  The step draws in (0, 1); ANY: v is a
+// caller's number, and one outside [0, 1/scale] (or NaN), which the guides do not cover, takes the
+// whole rows.
+template <bool ANY, typename R>
+__device__ __forceinline__ void guide_entries(const uint32_t* g, R v, R scale, int n, uint32_t& ga, uint32_t& gb) {
+  if (ANY && !(v >= (R)0 && v * scale <= (R)1)) {
+    ga = gb = (uint32_t)(n - 2) << 16;
+    return;
+  }
+  const uint32_t* e = g + guide_bin<R>(v, scale);
+  ga = __ldg(e);
+  gb = __ldg(e + kGuide);
+}
 
 // Events in quads: where a warp has few, four neighbouring lanes take one event together, each its part
 // of the logarithms, square roots, exponentials and quotients (kQuad lanes hold the same event).
@@ -624,16 +637,18 @@ struct XiSampler {
   // Both rows inverted and blended: xi linear in P between the bracketing nodes j, j + 1; the
   // complement Q is used when U > 1/2 (the same interpolation, precise near P = 1).  (Loops over
   // the rows and nodes, not unrolled: the event path is long, straight and mostly fetched anew.)
-  // L lanes hold the draw: 1, or a quad, lane 2 r + t of it taking node t of row r.
-  template <int L = 1>
+  // L lanes hold the draw: 1, or a quad, lane 2 r + t of it taking node t of row r.  ANY: see
+  // guide_entries.
+  template <int L = 1, bool ANY = false>
   __device__ __forceinline__ R sample(const TabDev<R>& T, R eta, R U, R V) const {
     const bool lower = U <= (R)0.5;
     const int n = T.n_xi;
     const R* A = (lower ? T.P2 : T.Q2) + 2 * (size_t)i * (size_t)n;
     const R v = lower ? U : V;
-    const uint32_t* g = (lower ? T.gP : T.gQ) + (size_t)i * kGuide + guide_bin<R>(v, (R)2);
+    uint32_t g0, g1;
+    guide_entries<ANY, R>((lower ? T.gP : T.gQ) + (size_t)i * kGuide, v, (R)2, n, g0, g1);
     int j0, j1;
-    bracket2<R>(A, n, lower, v, __ldg(g), __ldg(g + kGuide), j0, j1);
+    bracket2<R>(A, n, lower, v, g0, g1, j0, j1);
     const auto e0 = node_pair<R>(A, j0), e1 = node_pair<R>(A, n + j1);
     R xr[2];
     if constexpr (L == 1) {
@@ -676,20 +691,20 @@ struct XiSampler {
   }
 };
 
-// xi for (eta, U); false when U is below the cut-off.
+// xi for (eta, U), any U; false when U is below the cut-off.
 template <typename R>
 __device__ __forceinline__ bool sample_xi(const TabDev<R>& T, R eta, R U, R V, R& xi) {
   XiSampler<R> s;
   s.prepare(T, Num<R>::log_(eta));
   if (!s.above_cut(U)) return false;
-  xi = s.sample(T, eta, U, V);
+  xi = s.template sample<1, true>(T, eta, U, V);
   return true;
 }
 
 // Positron energy fraction f (Sec. 3, App. B): U < 1/2 maps to f <= 1/2 through V = 2U,
 // U >= 1/2 to f >= 1/2 through V = 2(1 - U).  L lanes hold the draw: 1, or a quad, lane 2 r + t of it
-// taking node t of row r.
-template <typename R, int L = 1>
+// taking node t of row r.  ANY: see guide_entries.
+template <typename R, int L = 1, bool ANY = false>
 __device__ __forceinline__ R sample_f(const TabDev<R>& T, R ln_chi, R U, R Vc) {
   int i, o; R w;
   grid_pos(ln_chi, T.ln_chi_min, T.inv_d_chi, T.n_chi, i, w, o);
@@ -697,9 +712,10 @@ __device__ __forceinline__ R sample_f(const TabDev<R>& T, R ln_chi, R U, R Vc) {
   const R V = lower ? (R)2 * U : (R)2 * Vc;
   const int n = T.n_f;
   const R* P = T.F2 + 2 * (size_t)i * (size_t)n;
-  const uint32_t* g = T.gF + (size_t)i * kGuide + guide_bin<R>(V, (R)1);
+  uint32_t g0, g1;
+  guide_entries<ANY, R>(T.gF + (size_t)i * kGuide, V, (R)1, n, g0, g1);
   int j[2];
-  bracket2<R>(P, n, true, V, __ldg(g), __ldg(g + kGuide), j[0], j[1]);
+  bracket2<R>(P, n, true, V, g0, g1, j[0], j[1]);
   R fr[2];
   if constexpr (L == 1) {
 #pragma unroll

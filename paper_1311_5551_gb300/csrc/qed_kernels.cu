@@ -2718,7 +2718,7 @@ __global__ void sample_kernel(const TabDev<R> tab, int which, size_t n, const do
       out[i] = good ? (double)xi : 0.0;
       ok[i] = good ? 1 : 0;
     } else {
-      out[i] = (double)sample_f<R>(tab, Num<R>::log_((R)param[i]), u, v);
+      out[i] = (double)sample_f<R, 1, true>(tab, Num<R>::log_((R)param[i]), u, v);
       ok[i] = 1;
     }
   }

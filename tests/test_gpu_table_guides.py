@@ -115,3 +115,25 @@ def test_samples_through_guides(n_xi, n_f, broken):
     ref = np.array([f_ref(arrays, spec, e, u) for e, u in zip(eta, U)])
     fine = np.isfinite(ref)
     np.testing.assert_allclose(got[fine], ref[fine], rtol=1e-12)
+
+
+@pytest.mark.parametrize("prec", [qed.FP64, qed.MIXED])
+def test_draws_outside_the_unit_interval(prec):
+    # the diagnostic takes any number as the draw: outside [0, 1] it extrapolates from the row's first
+    # or last bracket, as the plain search does, and a NaN gives a NaN
+    qbuild.build()
+    spec, arrays = make(64, 33, np.random.default_rng(5), False)
+    tables = qed.Tables(spec, arrays)
+    U = np.repeat([-1e30, -1e6, -0.5, -1.0 / 512, -1e-9, 0.0, 1.0, 1 + 1e-6, 1.5, 3.0, 1e6, 1e30, np.inf, -np.inf, np.nan], 40)
+    par = 10.0 ** np.random.default_rng(6).uniform(-2, 2, len(U))
+    got, ok = qed.sample(tables, prec, 0, par, U)
+    for e, u, g, k in zip(par, U, got, ok):
+        r = xi_ref(arrays, spec, e, u)
+        assert k == (r is not None)
+        if r is not None:
+            np.testing.assert_allclose(g, r, rtol=1e-12 if prec == qed.FP64 else 1e-4)
+    if prec == qed.FP64:
+        got, _ = qed.sample(tables, prec, 1, par, U)
+        with np.errstate(all="ignore"):
+            ref = np.array([f_ref(arrays, spec, e, u) for e, u in zip(par, U)])
+        np.testing.assert_allclose(got, ref, rtol=1e-12)
