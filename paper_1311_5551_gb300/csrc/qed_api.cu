@@ -1,6 +1,7 @@
 // qed_api.cu -- the C ABI of include/qed.h: object lifetimes, device memory through the
 // caller's allocator, host <-> device transfers and the launch sequence of one step.
 #include <cuda_runtime.h>
+#include <stdint.h>
 #include <string.h>
 
 #include <algorithm>
@@ -871,13 +872,19 @@ template <> const TabDev<double>& tab_of<double>(const qed_tables* t) { return t
 // its allocator: kept while the species lives, and at least doubled when a grid needs more, up to
 // kMaxPacked bytes (so all of them take at most twice that).  Larger grids, and calls under stream capture that would have to allocate, gather from the grid.
 constexpr size_t kMaxPacked = size_t(256) << 20;
+// The block holds the flag, then the cells.  The step reads cells 32 bytes at a time, while an allocator
+// may give any block that is aligned to 16: the cells start at the first multiple of 256 beyond the flag.
+constexpr size_t kCellsOffset = 512;  // (at most)
+char* packed_cells_of(const qed_species* e) {
+  return reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(e->cell_mem.ptr) + kCellsOffset - 1) & ~uintptr_t(255));
+}
 bool grid_workspace(qed_species* e, const qed_field_desc& f, cudaStream_t s) {
   if (f.kind != QED_FIELD_GRID || f.shape != 1 || e->precision != QED_MIXED) return false;
   for (int c = 0; c < 3; ++c)
     if ((size_t)f.n[c] > kMaxPacked / 192) return false;  // (so the product below cannot overflow)
   const size_t row = ((size_t)f.n[0] + 1) * ((size_t)f.n[1] + 1);
   if (row > kMaxPacked / 192) return false;
-  const size_t bytes = 256 + 192 * row * ((size_t)f.n[2] + 1);
+  const size_t bytes = kCellsOffset + 192 * row * ((size_t)f.n[2] + 1);
   if (bytes > kMaxPacked) return false;
   if (e->cell_mem.ptr && e->cell_mem.bytes >= bytes) return true;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -925,7 +932,7 @@ StepArgs<R> make_args(const qed_tables* T, qed_species* const* sp, const qed_ste
   a.win_s = -1;
   if (sp[0]->use_cells) {
     a.field.packed = static_cast<uint32_t*>(sp[0]->cell_mem.ptr);
-    a.field.cells = static_cast<char*>(sp[0]->cell_mem.ptr) + 256;
+    a.field.cells = packed_cells_of(sp[0]);
   }
   return a;
 }

@@ -1,0 +1,86 @@
+"""The memory of the packed grid that single-scenario runs in a cloud-in-cell field take from the
+electron species' allocator: which blocks they accept and when they take one."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1311_5551_gb300 import build as qbuild  # noqa: E402
+from paper_1311_5551_gb300 import qed  # noqa: E402
+
+N, ORG, SPC = (13, 11, 9), (-20.0, 5.0, 100.0), (3.0e4, 2.5e4, 4.0e4)
+
+
+@pytest.fixture(scope="module")
+def tables():
+    qbuild.build()
+    return qed.Tables()
+
+
+class Pool:
+    """A qed_allocator over torch's: blocks start `shift` bytes after a 256-byte boundary."""
+
+    def __init__(self, shift=0):
+        self.shift, self.live, self.log = shift, {}, []
+
+        @C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p)
+        def alloc(nbytes, stream, user):
+            t = torch.empty(int(nbytes) + 512, dtype=torch.uint8, device="cuda")
+            ptr = ((t.data_ptr() + 255) & ~255) + self.shift
+            self.live[ptr] = t
+            self.log.append((int(nbytes), int(stream or 0)))
+            return ptr
+
+        @C.CFUNCTYPE(None, C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p)
+        def free(ptr, nbytes, stream, user):
+            del self.live[int(ptr)]
+
+        self._keep = (alloc, free)
+        self.allocator = qed.Allocator(alloc, free, None)
+
+
+def grid(n, seed):
+    rng = np.random.default_rng(seed)
+    return torch.tensor(rng.normal(size=(6, n[2], n[1], n[0])) * 1e-3, dtype=torch.float32, device="cuda")
+
+
+def field(g):
+    return qed.Field(kind=qed.FIELD_GRID, grid=g, shape=1, origin=ORG, spacing=SPC)
+
+
+def fresh(n, seed, allocator=None):
+    rng = np.random.default_rng(seed)
+    x = np.stack([rng.uniform(ORG[a] - 3 * SPC[a], ORG[a] + (N[a] + 2) * SPC[a], n) for a in range(3)], axis=1)
+    u = rng.normal(size=(n, 3)) * 300.0
+    sp = [qed.Species(qed.ELECTRON, qed.MIXED, 4 * n + 64, 4 * n + 64, allocator=allocator),
+          qed.Species(qed.POSITRON, qed.MIXED, 4 * n + 64, 4 * n + 64, allocator=allocator),
+          qed.Species(qed.PHOTON, qed.MIXED, 30 * n + 64, 8 * n + 64, allocator=allocator)]
+    sp[0].upload(x, u)
+    sp[0].init_tau(seed)
+    sp[2].upload(rng.permutation(x), rng.normal(size=(n, 3)) * 10.0 ** rng.uniform(-1, 4, (n, 1)))
+    sp[2].init_tau(seed)
+    return sp
+
+
+def params(g):
+    return qed.StepParams(dt=2.0e3, seed=2, field=field(g))
+
+
+@pytest.mark.parametrize("shift", [16, 48, 240])
+def test_blocks_aligned_to_16_bytes(tables, shift):
+    # an allocator promises no more than the 16 bytes that the tile copies need
+    g = grid(N, 1)
+    out = []
+    for pool in (None, Pool(shift)):
+        sp = fresh(3001, 5, pool.allocator if pool else None)
+        qed.run(tables, sp, params(g), 0, 5)
+        qed.check(sp)
+        out.append([s.save() for s in sp])
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
+    assert len(pool.log) == 4  # three species and the packed grid
