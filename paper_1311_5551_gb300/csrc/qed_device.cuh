@@ -233,8 +233,11 @@ __device__ __forceinline__ AxisWeights<R, W> axis_weights(R s) {
 }
 
 // One component: sum of w_x w_y w_z * value over the stencil nodes that exist.
+// Plain loads, here and of packed cells: a step's blocks can start while the kernel that writes the
+// grid still runs (they wait for it before they read), so its values are not read-only for the
+// lifetime of the step's kernel, which is what non-coherent loads ask for.
 template <typename R, int W>
-__device__ __forceinline__ R gather_component(const R* __restrict__ G, const int n[3], const AxisWeights<R, W>& ax,
+__device__ __forceinline__ R gather_component(const R* G, const int n[3], const AxisWeights<R, W>& ax,
                                               const AxisWeights<R, W>& ay, const AxisWeights<R, W>& az) {
   R v = (R)0;
 #pragma unroll
@@ -251,7 +254,7 @@ __device__ __forceinline__ R gather_component(const R* __restrict__ G, const int
       for (int i = 0; i < W; ++i) {
         const int ix = ax.i0 + i;
         if (ix < 0 || ix >= n[0]) continue;
-        v = Num<R>::fma_(wzy * ax.w[i], __ldg(row + ix), v);
+        v = Num<R>::fma_(wzy * ax.w[i], row[ix], v);
       }
     }
   }
@@ -280,9 +283,9 @@ __device__ __forceinline__ void gather_fields(const StepScalars<R>& S, const R s
 // a component is one 32-byte read instead of eight scattered ones.  Same products and
 // order as gather_component, and so the same bits (a node outside adds an exact zero).
 __device__ __forceinline__ void load_cell(const float* p, float v[8]) {
-  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-      : "l"(p));
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "l"(p));
 }
 __device__ __forceinline__ float gather_cell(const float* C, const int n[3], const AxisWeights<float, 2>& ax,
                                              const AxisWeights<float, 2>& ay, const AxisWeights<float, 2>& az) {

@@ -84,3 +84,27 @@ def test_blocks_aligned_to_16_bytes(tables, shift):
         out.append([s.save() for s in sp])
     assert all(np.array_equal(a, b) for a, b in zip(*out))
     assert len(pool.log) == 4  # three species and the packed grid
+
+
+@pytest.mark.parametrize("shape", [1, 2])
+@pytest.mark.parametrize("steps", [1, 3])
+def test_grid_updated_between_calls(tables, shape, steps):
+    # the loop of a PIC code: the caller's kernels rewrite one grid in place between calls; the same
+    # particles as with every call's fields in a tensor of their own
+    out = []
+    for in_place in (False, True):
+        sp = fresh(3001, 6)
+        g = grid(N, 9)
+        keep = []
+        for k in range(12):
+            p = params(g)
+            p.field.shape = shape
+            qed.run(tables, sp, p, k * steps, steps)
+            keep.append(g)
+            if in_place:
+                g.mul_(-0.75)
+            else:
+                g = g * -0.75
+        qed.check(sp)
+        out.append([s.save() for s in sp])
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
