@@ -898,6 +898,7 @@ bool grid_workspace(qed_species* e, const qed_field_desc& f, cudaStream_t s) {
     cudaGetLastError();
     return false;
   }
+  grown.stream = e->mem.stream;  // released with the species, when the call's stream may be gone
   if (e->cell_mem.ptr) e->old_cells.push_back(e->cell_mem);
   e->cell_mem = grown;
   return true;

@@ -27,7 +27,7 @@ class Pool:
     """A qed_allocator over torch's: blocks start `shift` bytes after a 256-byte boundary."""
 
     def __init__(self, shift=0):
-        self.shift, self.live, self.log = shift, {}, []
+        self.shift, self.live, self.log, self.freed = shift, {}, [], []
 
         @C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p)
         def alloc(nbytes, stream, user):
@@ -40,6 +40,7 @@ class Pool:
         @C.CFUNCTYPE(None, C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p)
         def free(ptr, nbytes, stream, user):
             del self.live[int(ptr)]
+            self.freed.append((int(nbytes), int(stream or 0)))
 
         self._keep = (alloc, free)
         self.allocator = qed.Allocator(alloc, free, None)
@@ -108,3 +109,23 @@ def test_grid_updated_between_calls(tables, shape, steps):
         qed.check(sp)
         out.append([s.save() for s in sp])
     assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+def test_packed_grid_is_released_on_the_species_stream(tables):
+    # a run may use a stream that is destroyed before the species: the room it took for the packed grid
+    # is given back on the stream the species was created on
+    pool = Pool()
+    sp = fresh(3001, 7, pool.allocator)
+    home = torch.cuda.current_stream().cuda_stream
+    other = torch.cuda.Stream()
+    g = grid(N, 1)
+    torch.cuda.synchronize()
+    qed.run(tables, sp, params(g), 0, 2, stream=other)
+    other.synchronize()
+    nbytes, stream = pool.log[3]
+    assert stream == other.cuda_stream != home
+    del other
+    for s in sp:
+        s.close()
+    assert not pool.live and (nbytes, home) in pool.freed
+    assert all(s == home for _, s in pool.freed)
