@@ -894,7 +894,10 @@ bool grid_workspace(qed_species* e, const qed_field_desc& f, cudaStream_t s) {
   }
   DeviceBlock grown;
   const size_t get = std::min(kMaxPacked, std::max(bytes, 2 * e->cell_mem.bytes));
+  std::string message = g_err;
   if (grown.get(get, e->have_alloc ? &e->alloc_copy : nullptr, s) != QED_OK) {
+    // refused: the run does without, so the refusal is no error of this call
+    g_err.swap(message);
     cudaGetLastError();
     return false;
   }

@@ -24,13 +24,17 @@ def tables():
 
 
 class Pool:
-    """A qed_allocator over torch's: blocks start `shift` bytes after a 256-byte boundary."""
+    """A qed_allocator over torch's: blocks start `shift` bytes after a 256-byte boundary; after `blocks`
+    of them it refuses."""
 
-    def __init__(self, shift=0):
-        self.shift, self.live, self.log, self.freed = shift, {}, [], []
+    def __init__(self, shift=0, blocks=1 << 30):
+        self.shift, self.live, self.log, self.freed, self.refused = shift, {}, [], [], 0
 
         @C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p)
         def alloc(nbytes, stream, user):
+            if len(self.log) >= blocks:
+                self.refused += 1
+                return None
             t = torch.empty(int(nbytes) + 512, dtype=torch.uint8, device="cuda")
             ptr = ((t.data_ptr() + 255) & ~255) + self.shift
             self.live[ptr] = t
@@ -129,3 +133,21 @@ def test_packed_grid_is_released_on_the_species_stream(tables):
         s.close()
     assert not pool.live and (nbytes, home) in pool.freed
     assert all(s == home for _, s in pool.freed)
+
+
+def test_refused_packed_grid_is_no_error(tables):
+    # an allocator that gives no room for the packed grid: the run gathers from the grid itself, with the
+    # same particles, and the thread's last error message stays what it was
+    g = grid(N, 1)
+    out = []
+    for pool in (Pool(), Pool(blocks=3)):
+        sp = fresh(3001, 8, pool.allocator)
+        with pytest.raises(qed.QedError):
+            qed.Species(7, qed.MIXED, 10, 10)
+        message = qed.lib().qed_last_error()
+        qed.run(tables, sp, params(g), 0, 5)
+        assert qed.lib().qed_last_error() == message
+        qed.check(sp)
+        out.append([s.save() for s in sp])
+    assert pool.refused >= 1
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
