@@ -316,6 +316,7 @@ struct qed_species {
   DeviceBlock cell_mem;
   std::vector<DeviceBlock> old_cells;  // outgrown ones (calls on other streams may still read them)
   bool use_cells = false;  // the call under way packed its grid
+  size_t cells_refused = SIZE_MAX;  // the least room for one that the allocator has refused
   qed_allocator alloc_copy{};
   bool have_alloc = false;
   void* other[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
@@ -887,6 +888,9 @@ bool grid_workspace(qed_species* e, const qed_field_desc& f, cudaStream_t s) {
   const size_t bytes = kCellsOffset + 192 * row * ((size_t)f.n[2] + 1);
   if (bytes > kMaxPacked) return false;
   if (e->cell_mem.ptr && e->cell_mem.bytes >= bytes) return true;
+  // asked once: a refusal may be slow (an allocator that first empties its caches), and a time loop comes
+  // here at every step
+  if (bytes >= e->cells_refused) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
@@ -899,6 +903,7 @@ bool grid_workspace(qed_species* e, const qed_field_desc& f, cudaStream_t s) {
     // refused: the run does without, so the refusal is no error of this call
     g_err.swap(message);
     cudaGetLastError();
+    e->cells_refused = bytes;
     return false;
   }
   grown.stream = e->mem.stream;  // released with the species, when the call's stream may be gone

@@ -151,3 +151,19 @@ def test_refused_packed_grid_is_no_error(tables):
         out.append([s.save() for s in sp])
     assert pool.refused >= 1
     assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+def test_refusing_allocator_is_asked_once(tables):
+    pool = Pool(blocks=3)
+    sp = fresh(3001, 9, pool.allocator)
+    g = grid(N, 1)
+    for k in range(6):
+        qed.run(tables, sp, params(g), k, 1)
+    qed.check(sp)
+    assert pool.refused == 1
+    big = qed.StepParams(dt=2.0e3, seed=2, field=field(grid((20, 20, 20), 1)))
+    qed.run(tables, sp, big, 6, 1)
+    assert pool.refused == 1  # no more than was refused before
+    small = qed.StepParams(dt=2.0e3, seed=2, field=field(grid((4, 4, 4), 1)))
+    qed.run(tables, sp, small, 7, 1)
+    assert pool.refused == 2
