@@ -217,8 +217,13 @@ qed_status qed_species_merge(qed_species* sp, const qed_merge_params* params, ui
  *                        nearest node and its two neighbours).  Stencil nodes outside the grid
  *                        contribute nothing, so fields fall to zero outside it.  The fields do
  *                        not depend on t: the caller updates the grid between calls.  A mixed
- *                        single-scenario call with particles enough packs a shape = 1 grid by cells
- *                        for its own use (at most 256 MB, from sp[0]'s allocator, kept with sp[0]).
+ *                        single-scenario run on a shape = 1 grid whose species can hold particles
+ *                        enough (capacities times steps at least a third of the cells) takes room
+ *                        to pack the grid by cells for its own use from sp[0]'s allocator: 192
+ *                        bytes per cell, at most 256 MB, kept with sp[0], outgrown room too (in
+ *                        all at most twice that).  An allocator that returns NULL declines: the
+ *                        run gathers from the grid itself, with the same results, and sp[0] does
+ *                        not ask for as much again.
  * ------------------------------------------------------------------------------------------ */
 typedef enum {
   QED_FIELD_UNIFORM = 0, QED_FIELD_ROTATING_E = 1, QED_FIELD_PLANE_LP = 2, QED_FIELD_PLANE_CP = 3,

@@ -916,7 +916,11 @@ bool grid_workspace(qed_species* e, const qed_field_desc& f, cudaStream_t s) {
 template <typename R>
 StepArgs<R> make_args(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t step);
 void pack_grid(const qed_tables* T, qed_species* const* sp, const qed_step_params& p, uint64_t n, cudaStream_t s) {
-  sp[0]->use_cells = n > 0 && grid_workspace(sp[0], p.field, s);
+  // (the particles held are counted on the device, by the packing kernel: here, whether the species could
+  // hold enough)
+  const bool can = n > 0 && p.field.kind == QED_FIELD_GRID &&
+                   packing_pays((uint64_t)sp[0]->cap + sp[1]->cap + sp[2]->cap, n, grid_cells(p.field.n));
+  sp[0]->use_cells = can && grid_workspace(sp[0], p.field, s);
   if (sp[0]->use_cells) launch_pack_grid(make_args<float>(T, sp, p, p.step), n, s);
 }
 

@@ -134,6 +134,11 @@ struct FieldDev {
 // Cells of a packed grid component, and the bytes of a whole packed grid.
 QED_HD constexpr size_t grid_cells(const int n[3]) { return ((size_t)n[0] + 1) * ((size_t)n[1] + 1) * ((size_t)n[2] + 1); }
 
+// Whether a run of `steps` steps over that many particles gains by packing its grid (see pack_grid_kernel).
+QED_HD constexpr bool packing_pays(uint64_t particles, uint64_t steps, uint64_t cells) {
+  return particles * (steps < (1u << 20) ? steps : 1u << 20) >= cells / 3u;
+}
+
 // Host: descriptor -> device form, and its validation (shared by every entry point that steps).
 FieldDev field_dev(const qed_field_desc& f);
 qed_status check_field(const qed_field_desc& f, const char* who);

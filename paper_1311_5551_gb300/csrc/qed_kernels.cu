@@ -1559,7 +1559,7 @@ __global__ void __launch_bounds__(256) pack_grid_kernel(const StepArgs<float> a,
   const FieldDev& f = a.field;
   const uint64_t cells = grid_cells(f.n);
   const uint64_t particles = (uint64_t)a.sp[0].cnt->n + a.sp[1].cnt->n + a.sp[2].cnt->n;
-  const bool on = particles * min(steps, (uint64_t)1 << 20) >= cells / 3u;
+  const bool on = packing_pays(particles, steps, cells);
   if (blockIdx.x + blockIdx.y + blockIdx.z + threadIdx.x == 0) *f.packed = on ? 1u : 0u;
   if (!on) return;
   const int nx = f.n[0], ny = f.n[1], nz = f.n[2];

@@ -167,3 +167,20 @@ def test_refusing_allocator_is_asked_once(tables):
     small = qed.StepParams(dt=2.0e3, seed=2, field=field(grid((4, 4, 4), 1)))
     qed.run(tables, sp, small, 7, 1)
     assert pool.refused == 2
+
+
+def test_no_room_is_taken_where_packing_cannot_pay(tables):
+    # packing pays from a third of a particle-step per cell on: species that cannot hold as many take no
+    # room in a one-step call, and do in a longer one
+    g = grid((40, 40, 40), 1)
+    cap = 2000
+    for steps, blocks in ((1, 3), (3, 3), (4, 4)):  # 41^3 / 3 cells against 3 x 2000 particles a step
+        pool = Pool()
+        sp = [qed.Species(k, qed.MIXED, cap, 100, allocator=pool.allocator)
+              for k in (qed.ELECTRON, qed.POSITRON, qed.PHOTON)]
+        rng = np.random.default_rng(1)
+        sp[0].upload(rng.uniform(0, 1e6, (50, 3)), rng.normal(size=(50, 3)) * 10)
+        sp[0].init_tau(1)
+        qed.run(tables, sp, params(g), 0, steps)
+        qed.check(sp)
+        assert len(pool.log) == blocks, (steps, pool.log)
