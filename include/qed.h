@@ -155,7 +155,7 @@ qed_status qed_species_restore(qed_species* sp, const void* src, size_t bytes, v
 /* Initial optical depths, Sec. 3: tau = -ln U with U from the Philox stream
  * (key = (seed, scenario), counter = (id, 0, kind, 1)). */
 qed_status qed_species_init_tau(qed_species* sp, uint64_t seed, uint64_t scenario, void* stream);
-/* Stable removal of converted photons (tau = +inf).  Uses the species' scratch arrays. */
+/* Stable removal of converted photons (tau = +inf), into the species' second array set. */
 qed_status qed_species_compact(qed_species* sp, void* stream);
 
 /* Macroparticle weights (the physical particles a macroparticle stands for).  Uploads set
@@ -185,8 +185,12 @@ qed_status qed_species_totals(qed_species* sp, double out[5], void* stream);
  * total weight W, momentum P and energy E: energy E/W each, momenta P/W + d and P/W - d with d
  * perpendicular to P.  They are the group's two lowest-index photons (keeping ids and optical
  * depths); the others are removed and the remaining photons keep their order.  *groups_out:
- * groups merged.  Takes temporary device memory of 12 bytes per photon from the allocator the
- * species was created with (released before the call returns); synchronises. */
+ * groups merged.  Takes temporary device memory of 12 bytes per photon, their number rounded up to
+ * a power of two, from the allocator the species was created with (released before the call
+ * returns), and sorts in it and in the species' second array set, which the first compaction or
+ * merge allocates (as large as the arrays) and the species keeps; a first merge that finds no
+ * room for both at once takes them in turn.  QED_ERR_OOM leaves the particles as they were.
+ * Synchronises. */
 typedef struct {
   double origin[3], cell[3];
   int32_t n_cells[3];

@@ -325,7 +325,6 @@ struct qed_species {
   void* other_w = nullptr;
   uint32_t* seg_count = nullptr;
   uint32_t* seg_prefix = nullptr;
-  uint32_t* merge_counts = nullptr;  // digit counts of merging's sort (1/16 word per particle)
   int last_drain = 0;
 };
 
@@ -668,7 +667,6 @@ qed_status ensure_second_set(qed_species* sp, const SpeciesDev<R>& cur, cudaStre
     cv.add(&b.x, cap); cv.add(&b.y, cap); cv.add(&b.z, cap); cv.add(&b.ux, cap); cv.add(&b.uy, cap);
     cv.add(&b.uz, cap); cv.add(&b.tau, cap); cv.add(&b.id, cap);
     cv.add(&sp->seg_count, segs); cv.add(&sp->seg_prefix, segs + 1);
-    cv.add(&sp->merge_counts, 256 * (cap / 4096 + 2));
     qed_status st = sp->alt_mem.get(cv.total(), sp->have_alloc ? &sp->alloc_copy : nullptr, s);
     if (st != QED_OK) return st;
     cv.bind(sp->alt_mem.ptr);
@@ -682,6 +680,15 @@ qed_status ensure_second_set(qed_species* sp, const SpeciesDev<R>& cur, cudaStre
     sp->other_w = sp->alt_wmem.ptr;
   }
   return QED_OK;
+}
+
+void drop_second_set(qed_species* sp) {
+  sp->alt_wmem.release();
+  sp->alt_mem.release();
+  for (void*& p : sp->other) p = nullptr;
+  sp->other_tau = nullptr;
+  sp->other_id = nullptr;
+  sp->other_w = nullptr;
 }
 
 template <typename R>
@@ -783,27 +790,50 @@ extern "C" qed_status qed_species_merge(qed_species* sp, const qed_merge_params*
   if (c.n < 3) return QED_OK;
   st = ensure_weights(sp, s);  // merged particles carry weights other than 1
   if (st != QED_OK) return st;
-  // The first buffer of (key, index) pairs comes from the allocator the species was created with (the
-  // library does not allocate on its own behalf) and is given back before the call returns; the
-  // second one lies in the species' second array set, which the compaction below fills afterwards (the
-  // sort's counts are beside that set).
+  // The sort's two buffers of (key, index) pairs: the first comes from the allocator the species was
+  // created with (the library does not allocate on its own behalf) and is given back before the call
+  // returns; the second, and the sort's counts, lie in the species' second array set, which the
+  // compaction below fills afterwards.  Where the first merge finds no room for both at once, both buffers
+  // come from the allocator, before the second set takes its room (which is larger).
+  const size_t n = c.n, counts = 256 * ((n + 4095) / 4096 + 1) * sizeof(uint32_t);
+  const bool had_set = sp->alt_mem.ptr != nullptr;
   st = sp->precision == QED_MIXED ? ensure_second_set(sp, sp->f, s) : ensure_second_set(sp, sp->d, s);
   if (st != QED_OK) return st;
-  uint32_t N = 1;
-  while (N < c.n) N <<= 1;
-  const size_t bytes = (size_t)N * 12 + 256;
+  size_t N = 1;
+  while (N < n) N <<= 1;
+  const bool counts_in_set = sp->cap * elem_bytes(sp) >= counts;
+  const qed_allocator* alloc = sp->have_alloc ? &sp->alloc_copy : nullptr;
   DeviceBlock scratch;
-  st = scratch.get(bytes, sp->have_alloc ? &sp->alloc_copy : nullptr, s);
-  if (st != QED_OK) return st;
-  char* tmp = static_cast<char*>(scratch.ptr);
-  unsigned long long* groups = reinterpret_cast<unsigned long long*>(tmp + (size_t)N * 12 + 128);
   MergeScratch w;
-  w.keys[0] = tmp;
-  w.idx[0] = reinterpret_cast<uint32_t*>(tmp + (size_t)N * 8);
-  w.keys[1] = sp->other_tau;
-  w.idx[1] = sp->other_id;
-  w.hist = sp->merge_counts;
-  w.totals = w.hist + 256 * (sp->cap / 4096 + 1);
+  char* tmp = nullptr;  // two counters of the groups, and what follows them
+  std::string message = g_err;
+  st = scratch.get(N * 12 + 256 + (counts_in_set ? 0 : counts), alloc, s);
+  if (st == QED_OK) {
+    char* base = static_cast<char*>(scratch.ptr);
+    w.keys[0] = base;
+    w.idx[0] = reinterpret_cast<uint32_t*>(base + N * 8);
+    w.keys[1] = sp->other_tau;
+    w.idx[1] = sp->other_id;
+    tmp = base + N * 12 + 128;
+    w.hist = static_cast<uint32_t*>(counts_in_set ? sp->other[0] : tmp + 128);
+  } else {
+    if (had_set) return st;
+    cudaGetLastError();
+    drop_second_set(sp);
+    Carver cv;
+    char* keys[2];
+    const size_t key = md.bits <= 32 ? 4 : 8;
+    for (int k = 0; k < 2; ++k) { cv.add(&keys[k], n * key); cv.add(&w.idx[k], n); }
+    cv.add(&w.hist, counts / sizeof(uint32_t));
+    cv.add(&tmp, 16);
+    st = scratch.get(cv.total(), alloc, s);
+    if (st != QED_OK) return st;
+    cv.bind(scratch.ptr);
+    for (int k = 0; k < 2; ++k) w.keys[k] = keys[k];
+    g_err.swap(message);
+  }
+  w.totals = w.hist + 256 * ((n + 4095) / 4096);
+  unsigned long long* groups = reinterpret_cast<unsigned long long*>(tmp);
   w.count = reinterpret_cast<uint32_t*>(groups + 1);
   cudaError_t e = cudaMemsetAsync(groups, 0, 16, s);
   if (e != cudaSuccess) { scratch.release(); return cuda_fail(e, "cudaMemsetAsync"); }

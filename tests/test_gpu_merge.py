@@ -213,3 +213,61 @@ def test_merge_sizes_match_oracle(tables, prec, n, cells):
         np.testing.assert_allclose(a["x"], ref.x(), rtol=1e-6, atol=1e-5)
         np.testing.assert_allclose(a["u"], ref.u(), rtol=1e-6, atol=1e-6 * np.abs(ref.u()).max())
         np.testing.assert_allclose(g.weights(), ref.get("w"), rtol=1e-6)
+
+
+@pytest.mark.parametrize("prec", [qed.FP64, qed.MIXED])
+@pytest.mark.parametrize("cells", [2, 1500])  # 32-bit and 64-bit keys
+def test_first_merge_fits_where_its_parts_fit_in_turn(tables, prec, cells):
+    # the sort's scratch and the second array set need not be there at once: a pool that holds the
+    # larger of the two is enough for the first merge, with the same result; one that does not hold the
+    # second set refuses and leaves the particles as they were
+    import ctypes as C
+
+    class Pool:
+        def __init__(self, limit):
+            self.limit, self.live, self.log, self.used = limit, {}, [], 0
+
+            @C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p)
+            def alloc(nbytes, stream, user):
+                if self.used + nbytes > self.limit:
+                    return None
+                t = torch.empty(int(nbytes), dtype=torch.uint8, device="cuda")
+                self.live[t.data_ptr()] = t
+                self.used += nbytes
+                self.log.append(int(nbytes))
+                return t.data_ptr()
+
+            @C.CFUNCTYPE(None, C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p)
+            def free(ptr, nbytes, stream, user):
+                del self.live[int(ptr)]
+                self.used -= nbytes
+
+            self._keep = (alloc, free)
+            self.allocator = qed.Allocator(alloc, free, None)
+
+    x, k, w, tau = photon_inputs(8, n_groups=900, f32=prec == qed.MIXED)
+    n = len(x)
+    grid = dict(origin=(-30.0 - 60.0 * (cells // 2 - 1),) * 3, cell=(60.0,) * 3, n_cells=(cells,) * 3, n_face=8, n_sub=4,
+                min_group=3)
+
+    def merged(limit):
+        pool = Pool(limit)
+        g = qed.Species(qed.PHOTON, prec, n + 16, 16, allocator=pool.allocator)
+        g.upload(x, k, tau=tau)
+        g.set_weights(w)
+        before = g.save()
+        try:
+            groups = g.merge(**grid)
+        except qed.QedError as e:
+            assert e.code == qed.QED_ERR_OOM
+            groups = None
+        return pool.log, pool.used, groups, before, g.save()
+
+    log, _, groups, _, ref = merged(1 << 40)
+    assert groups > 10
+    species, weights, second, second_w, scratch = log
+    _, used, got, _, out = merged(species + weights + max(scratch, second + second_w))
+    assert got == groups and np.array_equal(out, ref)
+    assert used == species + weights + second + second_w
+    _, _, got, before, out = merged(species + weights + second - 1)
+    assert got is None and np.array_equal(out, before)
