@@ -3360,17 +3360,6 @@ __device__ __forceinline__ double widen(float v) {
   return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
 __device__ __forceinline__ double widen(double v) { return v; }
-// sqrt of a double to its last bit or the one beside it, by two Newton steps from the FP32 reciprocal
-// root (Heron's rule; 7 FP64 operations against about 25); outside FP32's range the function.
-__device__ __forceinline__ double root_newton(double v) {
-  const float f = __double2float_rn(v);
-  if (!(f > 1e-30f && f < 1e30f)) return sqrt(v);
-  const float y = rsqrtf(f);
-  const double h = widen(0.5f * y);
-  double s = v * widen(y);
-  s = fma(fma(-s, s, v), h, s);
-  return fma(fma(-s, s, v), h, s);
-}
 
 constexpr int kMergeSums = 8;  // W, E, P[3], X[3]
 // One member's share of the group's sums.
@@ -3382,7 +3371,7 @@ __device__ __forceinline__ void merge_member(const SpeciesDev<R>& sp, uint32_t i
   double e2 = k[0] * k[0] + k[1] * k[1] + k[2] * k[2];
   if (!massless) e2 = 1.0 + e2;
   v[0] = 1.0;
-  v[1] = sizeof(R) == 8 ? sqrt(e2) : root_newton(e2);
+  v[1] = sqrt(e2);
 #pragma unroll
   for (int c = 0; c < 3; ++c) { v[2 + c] = k[c]; v[5 + c] = x[c]; }
   if (w != (R)1) {  // (unweighted photons: 7 multiplications by one)
@@ -3425,10 +3414,12 @@ __device__ void merge_survivor(SpeciesDev<R>& sp, uint32_t i, int which, int mas
 // species: a warp per group, 32 members at a time, sums in index order (lane c adds sum c of the
 // 32), so the results are those of a plain loop.  Mixed: eight lanes per group, each sums its own
 // members and the eight are added in a fixed order; groups of more than kMergeBig members, of which
-// a few hold most of the photons, are left to merge_big_kernel, a block each.  Bound by the FP64
-// pipe, which is why it sees no conversions and no square roots of the mixed path (3e6 photons, 3e4
-// groups on GB300: 408 us, and 378 us for the big ones side by side with 2e6 of the photons; the whole
-// merge, with its upload, 15.6 -> 1.48 ms).
+// a few hold most of the photons, are left to merge_big_kernel, a block each.  The mixed path's
+// conversions are integer operations (widen), which keeps them off the FP64 pipe.  3e6 photons, 3e4
+// groups on GB300: 434 us, and 384 us for the big ones with 2e6 of the photons; the whole merge, with
+// its upload, 15.6 -> 1.51 ms.  The FP64 pipe is busy for about half of that (4.6e6 and 4.0e6 warp
+// instructions, each 16 cycles of an SM's pipe: 235 and 203 us); the rest is the wait for the members'
+// scattered reads (440 MB each from DRAM, 15% of its rate; 12% and 8% of the issue slots used).
 constexpr uint32_t kMergeBig = 256;
 template <typename R, typename K>
 __global__ void __launch_bounds__(128) merge_groups_kernel(SpeciesDev<R> sp, MergeDev M, const K* keys, const uint32_t* idx,
