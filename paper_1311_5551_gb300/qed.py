@@ -243,9 +243,13 @@ def _torch():
 
 def _stream_ptr(stream):
     if stream is None:
-        # the current stream's handle, without the object around it (a few microseconds per call)
+        # the current stream's handle, without the object around it (a few microseconds per call) where
+        # this PyTorch has the function, which is not part of its public interface
         torch = _torch()
-        return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return C.c_void_p(raw(torch.cuda.current_device()))
+        stream = torch.cuda.current_stream()
     return C.c_void_p(stream.cuda_stream)
 
 

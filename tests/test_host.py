@@ -390,3 +390,18 @@ def test_serving_waits_for_memory_that_the_budget_does_not_show(monkeypatch):
     blocks["held"] = 6
     with pytest.raises(qed.QedError):
         serving.serve(fake, None, [(0.0, w)], 0, slots=4, chunk=5, max_wall=30.0)
+
+
+@pytest.mark.parametrize("raw", [True, False])
+def test_current_stream_with_and_without_the_raw_handle(monkeypatch, raw):
+    # the short way to the current stream's handle is a private function of PyTorch: without it the
+    # public one is asked, with the same answer
+    from types import SimpleNamespace
+
+    from paper_1311_5551_gb300 import qed
+
+    cuda = SimpleNamespace(current_device=lambda: 3, current_stream=lambda: SimpleNamespace(cuda_stream=0x1230))
+    private = SimpleNamespace(_cuda_getCurrentRawStream=lambda d: 0x1230 if d == 3 else 0) if raw else SimpleNamespace()
+    monkeypatch.setattr(qed, "_torch", lambda: SimpleNamespace(_C=private, cuda=cuda))
+    assert qed._stream_ptr(None).value == 0x1230
+    assert qed._stream_ptr(SimpleNamespace(cuda_stream=0x99)).value == 0x99
