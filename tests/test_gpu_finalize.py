@@ -86,3 +86,36 @@ def test_counts_are_cleared_between_populations(tables):
     for seed, ns in enumerate([(60000, 1500), (40, 10), (50, 1), (65000, 2000), (33000, 33000)]):
         load(sp, ns, seed)
         step_and_check(tables, sp, p, seed, (lambda k: qed.run(tables, sp, p, k)) if seed % 3 else in_batch)
+
+
+@pytest.mark.parametrize("parent", [qed.ELECTRON, qed.PHOTON])
+def test_order_beyond_1024_coarse_groups(tables, parent):
+    # more than 1024 x 32768 parents: the merge's prefixes stand for two coarse groups each.  Every 37th
+    # parent has an event; a child starts at its parent's position, which tells whose it is
+    n = 34_000_037
+    i = torch.arange(n, device="cuda", dtype=torch.int64)
+    x = torch.stack([(i % 4099).float() * 3.0, (i % 509).float(), (i // 37).float()], dim=1)
+    u = torch.zeros((n, 3), device="cuda")
+    u[:, 0] = 1e3 if parent == qed.ELECTRON else 1e5
+    has = i % 37 == 5
+    tau = torch.where(has, 1e-12, 1e3).double()
+    want = int(has.sum())
+    cap = {k: n if k == parent else want + 10 for k in (qed.ELECTRON, qed.POSITRON, qed.PHOTON)}
+    sp = [qed.Species(k, qed.MIXED, cap[k], want + 10) for k in (qed.ELECTRON, qed.POSITRON, qed.PHOTON)]
+    src = sp[0 if parent == qed.ELECTRON else 2]
+    src.upload(x, u, tau=tau)
+    qed.run(tables, sp, qed.StepParams(dt=10.0, seed=4, field=qed.Field(B=(0.0, 0.0, 1e-3))), 0, 1)
+    qed.check(sp)
+    led = qed.read_ledger(sp)
+    at = src.download()["x"][5::37]  # the parents after the push, in order
+    if parent == qed.ELECTRON:
+        kids = [sp[2].download()]
+        assert led["emitted_n"] + led["dropped_n"] == want and len(kids[0]["id"]) == led["emitted_n"] > 0.9 * want
+    else:
+        kids = [sp[0].download(), sp[1].download()]
+        assert led["pairs_n"] == want and all(len(c["id"]) == want for c in kids)
+    for c in kids:
+        who = np.round(c["x"][:, 2]).astype(np.int64)
+        assert np.all(np.diff(who) > 0)
+        assert np.array_equal(c["x"], at[who])
+        assert np.array_equal(c["id"], np.arange(len(who), dtype=np.uint32))
