@@ -50,7 +50,7 @@ typedef enum { QED_ELECTRON = 0, QED_POSITRON = 1, QED_PHOTON = 2 } qed_kind;
 typedef enum { QED_FP64 = 0, QED_MIXED = 1 } qed_precision;
 
 /* Device memory provider.  alloc(bytes, stream, user) returns device memory or NULL;
- * free(ptr, bytes, stream, user) releases it.  A NULL allocator uses cudaMallocAsync and
+ * free(ptr, bytes, stream, user) releases it.  Blocks are aligned to 16 bytes at least.  A NULL allocator uses cudaMallocAsync and
  * cudaFreeAsync on the given stream. */
 typedef struct {
   void* (*alloc)(size_t bytes, void* stream, void* user);
@@ -189,8 +189,7 @@ qed_status qed_species_totals(qed_species* sp, double out[5], void* stream);
  * a power of two, from the allocator the species was created with (released before the call
  * returns), and sorts in it and in the species' second array set, which the first compaction or
  * merge allocates (as large as the arrays) and the species keeps; a first merge that finds no
- * room for both at once takes them in turn.  QED_ERR_OOM leaves the particles as they were.
- * Synchronises. */
+ * room for both at once takes them in turn.  Synchronises. */
 typedef struct {
   double origin[3], cell[3];
   int32_t n_cells[3];
@@ -299,13 +298,15 @@ qed_status qed_check(qed_species* const* sp, int n_species, void* stream);
  * Batches: many independent scenarios (for example a parameter scan of collisions, or the
  * requests of a serving loop), each with its own species, field and steps, advanced together.
  * Each batch step is four launches for all scenarios: a tile schedule that lays the live
- * scenarios' 256-particle tiles end to end in one tile space, the step (a persistent grid that
- * strides through that space, so every block gets an equal share in one wave), and the two
- * merge kernels (per-scenario plan and the ordered scatter, which strides
- * through all scenarios together); qed_batch_run replays them from a captured CUDA graph.  A
- * scenario gives the same particles alone or in any mix, and, with the default grid, the same
- * ledger bit for bit as qed_run (block p of the grid takes the same tiles of the scenario either
- * way).
+ * scenarios' tiles (256 particles, QED_FP64 128) end to end in one tile space, the step (a
+ * persistent grid that strides through that space, so every block gets an equal share in one
+ * wave), and the two merge kernels (per-scenario plan and the ordered scatter, which strides
+ * through all scenarios together); in the mixed path two more every 16 steps take the photons
+ * held through those steps, as qed_run does (not beside multi-step passes), and multi-step passes
+ * add five to each step.  qed_batch_run replays them from a captured CUDA graph.  Grid fields are
+ * gathered from the caller's grid (no packing).  A scenario gives the same particles alone or in any
+ * mix, and, with the default grid, the same ledger bit for bit as qed_run (block p of the grid
+ * takes the same tiles of the scenario either way).
  * ------------------------------------------------------------------------------------------ */
 typedef struct qed_batch qed_batch;
 qed_status qed_batch_create(const qed_tables* tables, qed_precision precision, int slots,
@@ -330,7 +331,8 @@ qed_status qed_batch_config(qed_batch* b, int target_blocks, int graph_steps);
  * event-free stretch of up to chunk steps in one pass (as qed_run_multistep, decided on the device
  * per slot, no host synchronisation), then the regular step, so one batch step advances a slot by
  * one to chunk + 1 steps; particles are identical to qed_run's.  Run batch steps until
- * qed_batch_remaining reports zero. */
+ * qed_batch_remaining reports zero.  While it is on, photons go one step at a time in the regular
+ * steps. */
 qed_status qed_batch_multistep(qed_batch* b, int chunk);
 /* Autotuner: times candidate (blocks, graph steps) on the live batch, trial_steps real batch
  * steps each, and keeps the fastest; the chosen values are returned.  Synchronises. */
@@ -401,8 +403,8 @@ qed_status qed_philox(size_t n, const uint64_t* ctr, const uint64_t key[2], uint
 qed_status qed_work_read(qed_species* electrons, uint64_t out[3], int reset, void* stream);
 /* As qed_work_read, plus out[3] e+- pushes and out[4] photon pushes made by passes over several
  * steps (the multi-step passes of qed_run_multistep and, in the mixed path, the photon windows of
- * every run of more than two steps; already counted in out[0] and out[1]), and out[5] photon pushes of the per-step kernel in a
- * field, whose optical depth changed and was written back (a photon outside every field keeps
+ * every run of more than two steps; already counted in out[0] and out[1]), and out[5] photon
+ * pushes of the per-step kernel in a field, whose optical depth changed and was written back (a photon outside every field keeps
  * its optical depth, and the step stores only its position). */
 qed_status qed_work_read_split(qed_species* electrons, uint64_t out[6], int reset, void* stream);
 /* Step-kernel timing: while enabled, every step-kernel launch is bracketed by CUDA events on its

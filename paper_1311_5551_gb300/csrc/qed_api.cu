@@ -901,7 +901,8 @@ template <> const TabDev<double>& tab_of<double>(const qed_tables* t) { return t
 
 // Room for the packed form of a cloud-in-cell grid field (pack_grid_kernel) in the electron species, from
 // its allocator: kept while the species lives, and at least doubled when a grid needs more, up to
-// kMaxPacked bytes (so all of them take at most twice that).  Larger grids, and calls under stream capture that would have to allocate, gather from the grid.
+// kMaxPacked bytes (so all of them take at most twice that).  Larger grids, calls under stream capture that
+// would have to allocate, and species whose allocator refuses gather from the grid.
 constexpr size_t kMaxPacked = size_t(256) << 20;
 // The block holds the flag, then the cells.  The step reads cells 32 bytes at a time, while an allocator
 // may give any block that is aligned to 16: the cells start at the first multiple of 256 beyond the flag.

@@ -107,7 +107,8 @@ struct SpeciesDev {
   R* aw;  // [acap]
 };
 
-// Finalisation plan written by the first finalisation kernel.
+// What a step's merge needs to know.  finalize_kernel's blocks each make their own (of the stored one
+// they use the ticket); in batches the plan kernel stores it for the scatter.
 struct FinalizePlan {
   uint32_t n_old[3];        // destination counts before the merge (e-, e+, photon destination)
   uint32_t next_id_old[3];
@@ -164,8 +165,8 @@ struct StepArgs {
 };
 
 // What one batch step does with a slot, written by the tile schedule at the start of the step:
-// the slot's 256-particle tiles occupy [tile_base, tile_base + T[0] + T[1] + T[2]) of the batch
-// step's tile space (species in order e-, e+, photons); n are the particles held (the step's
+// the slot's tiles (256 particles, FP64 128) occupy [tile_base, tile_base + T[0] + .. + T[3]) of the batch
+// step's tile space (species in order e-, e+, photons, then T[3]); n are the particles held (the step's
 // parents).  Inside a photon window the photon tiles start at photon win_n, and T[3] tiles without
 // particles follow, which share the conversions that the window found.
 struct SlotPlan {
@@ -191,7 +192,7 @@ struct BatchCtl {
   uint32_t* remaining;   // [S] steps left per slot (0: idle)
   uint32_t* live;        // [S] slot takes part in the current batch step (set by the schedule)
   uint32_t* blocks;      // [S+1] exclusive prefix of the step-kernel blocks per slot (multi-step)
-  SlotPlan* splan;       // [S] tile and range layout of the current batch step
+  SlotPlan* splan;       // [S] tile layout of the current batch step
   void* scal;            // [S] per-slot field scalars of the current step (StepScalars<R>)
   uint32_t* tot;         // [kBatchTotals] sizes of the current batch step's spaces
   void* wscal;           // [S * kWinMax] field scalars of the current photon window's steps (mixed path)

@@ -265,7 +265,7 @@ __device__ __forceinline__ void lepton_chunk(const StepArgs<R>& a, const StepSca
   }
 }
 
-// Takes `take` (<= 32) events, one per lane (lane l: entry p of ring `src`): photon emission
+// Takes `take` (<= 32) events, one per lane (each lane's is entry p of `ring`): photon emission
 // by an e+- (Sec. 3): photon energy from the inverse CDF of P_chi, recoil, fresh optical depths
 // for the emitter and the photon, the photon appended to the photon species' append region.
 // A chain of dependent loads and special functions, with scattered table reads: its latency counts
@@ -544,7 +544,7 @@ __device__ __forceinline__ void photon_chunk(const StepArgs<R>& a, const StepSca
   }
 }
 
-// Takes `take` (<= 32) events, one per lane (lane l: entry p of ring `src`): pair creation
+// Takes `take` (<= 32) events, one per lane (each lane's is entry p of `ring`): pair creation
 // by a photon (Sec. 3): the energy split from the inverse CDF of P_f, the electron and the
 // positron along k with fresh optical depths, appended to their species' append regions; the
 // photon is annihilated (its optical depth becomes +inf, a hole until compaction).  Inlined
@@ -1833,7 +1833,7 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const StepArgs<
 // advances every photon held (but for the last n mod 1024) by K steps in registers, with
 // photon_advance's own operations, and stops a photon at the step at which its optical depth runs
 // out; the K per-step kernels that follow push the leptons and the photons made since, and take the
-// conversions found for their step (window_events).  Particles, ids and order are those of the
+// conversions found for their step (run_conversions).  Particles, ids and order are those of the
 // per-step path: a conversion is taken at its step, and the merge ranks it by the photon's index.
 //
 // A step whose ledger can be read (the last of a run) belongs to no window: its sums are taken by
@@ -1952,7 +1952,7 @@ __device__ __forceinline__ int window_steps(const StepArgs<float>& a, const WinS
   return -1;
 }
 
-// Writes one stepped photon back; a converted one waits for its step (window_events).
+// Writes one stepped photon back; a converted one waits for its step (run_conversions).
 template <int WC>
 __device__ __forceinline__ void window_store(const StepArgs<float>& a, uint32_t i, const WinPhoton<WC>& p,
                                              const Tau<float>& tau0, int conv, float chi, int K, uint32_t& pushed) {
@@ -2149,7 +2149,7 @@ __device__ __forceinline__ void load_args(StepArgs<R>& dst, const StepArgs<R>* s
 }
 
 // One block: which slots step now and how many step-kernel blocks each gets (proportional to
-// its 256-particle tiles, at least one for a slot with work, at most its ledger partials).
+// its tiles, at least one for a slot with work, at most its ledger partials).
 template <typename R>
 __global__ void __launch_bounds__(1024) batch_schedule_kernel(const BatchCtl<R> c) {
   __shared__ unsigned long long s_tiles;

@@ -1,7 +1,7 @@
 // qed_noalloc.cu -- an allocation-free variant of the emission step for callers that must not
 // allocate device memory.
 //
-// The regular entry points keep their per-step scratch (event masks, prefix sums, the append
+// The regular entry points keep their per-step scratch (event masks and counts, the append
 // region of new photons, ledger partials, the merge plan, counters) inside species objects that
 // are allocated through a qed_allocator.  Some host codes cannot grant that: a simulation that has
 // reserved the whole device memory for its own pool, or a time loop that must not change its
